@@ -1,14 +1,21 @@
-"""ctypes binding of libresps.so: the same entry points as include/resps.h, taking torch
-tensors (device memory) and doing argument marshalling only -- every step of the path runs
-in the library's CUDA kernels.  There is no CPU fallback: if the shared library cannot be
-loaded, importing a symbol from here raises."""
+"""Binding of libresps.so: the same entry points as include/resps.h, taking torch tensors (device
+memory) and doing argument marshalling only -- every step of the path runs in the library's CUDA
+kernels.  The calls of a step are marshalled natively (the _call extension, csrc/call.cpp), everything
+else through ctypes.  There is no fallback: if one of the two shared libraries cannot be loaded,
+importing a symbol from here raises."""
 from __future__ import annotations
 
 import ctypes
 import os
+import types
 from typing import Optional, Sequence
 
 import torch
+
+try:
+    from . import _call
+except ImportError as e:  # not built yet, or not loadable: load() says so
+    _call, _call_error = None, e
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libresps.so")
@@ -64,6 +71,9 @@ def load() -> ctypes.CDLL:
     if not os.path.exists(LIB_PATH):
         raise ImportError(f"{LIB_PATH} is missing: run `python -m paper_2601_12212_b200.build` "
                           "(there is no fallback path)")
+    if _call is None:
+        raise ImportError("the _call extension cannot be imported: run `python -m paper_2601_12212_b200.build` "
+                          "(there is no fallback path)") from _call_error
     lib = ctypes.CDLL(LIB_PATH)
     vp, i32, i64, f32 = ctypes.c_void_p, ctypes.c_int, ctypes.c_int64, ctypes.c_float
     lib.resps_create.argtypes = [ctypes.POINTER(vp), ctypes.POINTER(RespsShape)]
@@ -99,6 +109,8 @@ def load() -> ctypes.CDLL:
     for name in EXPORTS:
         if name not in ("resps_strerror", "resps_workspace_bytes", "resps_scan_rows"):
             getattr(lib, name).restype = i32
+    lib.calls = types.SimpleNamespace(**{name: _call.bind(name, ctypes.cast(getattr(lib, name), vp).value)
+                                         for name in _call.names()})
     _lib = lib
     return lib
 
@@ -136,7 +148,9 @@ class Context:
         self.shape = RespsShape(n_q_heads, n_kv_heads, head_dim, vocab, max_batch, max_tt, max_k,
                                 max_depth)
         self._h = ctypes.c_void_p()
-        _check(load().resps_create(ctypes.byref(self._h), ctypes.byref(self.shape)), "resps_create")
+        lib = load()
+        _check(lib.resps_create(ctypes.byref(self._h), ctypes.byref(self.shape)), "resps_create")
+        self._calls, self._address = lib.calls, self._h.value
 
     @property
     def handle(self):
@@ -163,6 +177,7 @@ class Context:
         if self._h:
             load().resps_destroy(self._h)
             self._h = ctypes.c_void_p()
+            self._address = None
 
     def __del__(self):
         try:
@@ -177,58 +192,49 @@ STEP_DTYPE = torch.int32  # resps_step = 4 x int32 (tt, d, k, prefix_len): tenso
 def resps_tree_expand(ctx: Context, steps, batch: int, draft_logits, ld_b: int, ld_level: int,
                       ld_row: int, n_levels: int, n_slots: int, root_token, tokens, parent, depth,
                       position_ids, mask, retrieve, n_leaves, n_nodes, stream=None) -> None:
-    i32 = torch.int32
-    _check(load().resps_tree_expand(
-        ctx.handle, _ptr(steps, i32), batch, _ptr(draft_logits, torch.float32), ld_b, ld_level, ld_row,
-        n_levels, n_slots, _ptr(root_token, i32), _ptr(tokens, i32), _ptr(parent, i32),
-        _ptr(depth, i32), _ptr(position_ids, i32), _ptr(mask), _ptr(retrieve, i32),
-        _ptr(n_leaves, i32), _ptr(n_nodes, i32), _stream(stream)), "resps_tree_expand")
+    _check(ctx._calls.resps_tree_expand(
+        ctx._address, steps, batch, draft_logits, ld_b, ld_level, ld_row, n_levels, n_slots, root_token, tokens,
+        parent, depth, position_ids, mask, retrieve, n_leaves, n_nodes, stream),
+        "resps_tree_expand")
 
 
 def resps_tree_expand_begin(ctx: Context, steps, batch: int, n_slots: int) -> None:
-    _check(load().resps_tree_expand_begin(ctx.handle, _ptr(steps, torch.int32), batch, n_slots), "resps_tree_expand_begin")
+    _check(ctx._calls.resps_tree_expand_begin(ctx._address, steps, batch, n_slots), "resps_tree_expand_begin")
 
 
 def resps_tree_expand_level(ctx: Context, steps, batch: int, level: int, level_logits, ld_b: int, ld_row: int,
                             frontier_tokens, frontier_parent_slot, frontier_position_ids, frontier_node_index,
                             frontier_mask, frontier_score=None, stream=None) -> None:
-    i32 = torch.int32
-    _check(load().resps_tree_expand_level(
-        ctx.handle, _ptr(steps, i32), batch, level, _ptr(level_logits, torch.float32), ld_b, ld_row,
-        _ptr(frontier_tokens, i32), _ptr(frontier_parent_slot, i32), _ptr(frontier_position_ids, i32),
-        _ptr(frontier_node_index, i32), _ptr(frontier_mask), _ptr(frontier_score, torch.float64), _stream(stream)),
+    _check(ctx._calls.resps_tree_expand_level(
+        ctx._address, steps, batch, level, level_logits, ld_b, ld_row, frontier_tokens, frontier_parent_slot,
+        frontier_position_ids, frontier_node_index, frontier_mask, frontier_score, stream),
         "resps_tree_expand_level")
 
 
 def resps_tree_expand_finish(ctx: Context, steps, batch: int, root_token, tokens, parent, depth, position_ids, mask,
                              retrieve, n_leaves, n_nodes, stream=None) -> None:
-    i32 = torch.int32
-    _check(load().resps_tree_expand_finish(
-        ctx.handle, _ptr(steps, i32), batch, _ptr(root_token, i32), _ptr(tokens, i32), _ptr(parent, i32),
-        _ptr(depth, i32), _ptr(position_ids, i32), _ptr(mask), _ptr(retrieve, i32), _ptr(n_leaves, i32),
-        _ptr(n_nodes, i32), _stream(stream)), "resps_tree_expand_finish")
+    _check(ctx._calls.resps_tree_expand_finish(
+        ctx._address, steps, batch, root_token, tokens, parent, depth, position_ids, mask, retrieve, n_leaves, n_nodes,
+        stream),
+        "resps_tree_expand_finish")
 
 
 def resps_tree_attention(ctx: Context, steps, n_nodes, batch: int, q, o, lse, k_cache, v_cache,
                          kv_stride_seq: int, kv_stride_head: int, kv_stride_tok: int,
                          kv_capacity: int, mask, softmax_scale: float, stream=None) -> None:
-    i32, bf = torch.int32, torch.bfloat16
-    _check(load().resps_tree_attention(
-        ctx.handle, _ptr(steps, i32), _ptr(n_nodes, i32), batch, _ptr(q, bf), _ptr(o, bf),
-        _ptr(lse, torch.float32), _ptr(k_cache, bf), _ptr(v_cache, bf), kv_stride_seq, kv_stride_head,
-        kv_stride_tok, kv_capacity, _ptr(mask), float(softmax_scale), _stream(stream)),
+    _check(ctx._calls.resps_tree_attention(
+        ctx._address, steps, n_nodes, batch, q, o, lse, k_cache, v_cache, kv_stride_seq, kv_stride_head, kv_stride_tok,
+        kv_capacity, mask, softmax_scale, stream),
         "resps_tree_attention")
 
 
 def resps_verify_accept(ctx: Context, steps, n_nodes, batch: int, target_logits, ld_b: int,
                         ld_row: int, tokens, parent, target_argmax, accept_path, accept_len,
                         out_tokens, steps_next=None, stream=None) -> None:
-    i32 = torch.int32
-    _check(load().resps_verify_accept(
-        ctx.handle, _ptr(steps, i32), _ptr(n_nodes, i32), batch, _ptr(target_logits, torch.float32),
-        ld_b, ld_row, _ptr(tokens, i32), _ptr(parent, i32), _ptr(target_argmax, i32),
-        _ptr(accept_path, i32), _ptr(accept_len, i32), _ptr(out_tokens, i32), _ptr(steps_next, i32),
-        _stream(stream)), "resps_verify_accept")
+    _check(ctx._calls.resps_verify_accept(
+        ctx._address, steps, n_nodes, batch, target_logits, ld_b, ld_row, tokens, parent, target_argmax, accept_path,
+        accept_len, out_tokens, steps_next, stream),
+        "resps_verify_accept")
 
 
 def resps_verify_accept_sampled(ctx: Context, steps, n_nodes, batch: int, target_logits, ld_b: int, ld_row: int,
@@ -236,12 +242,11 @@ def resps_verify_accept_sampled(ctx: Context, steps, n_nodes, batch: int, target
                                 temperature: float, tokens, parent, u_accept, u_sample, accept_path, accept_len,
                                 out_tokens, steps_next=None, stream=None) -> None:
     """Acceptance under sampling (T > 0) for the tree of the last resps_tree_expand on this context."""
-    i32, f32, f64 = torch.int32, torch.float32, torch.float64
-    _check(load().resps_verify_accept_sampled(
-        ctx.handle, _ptr(steps, i32), _ptr(n_nodes, i32), batch, _ptr(target_logits, f32), ld_b, ld_row,
-        _ptr(draft_logits, f32), draft_ld_b, draft_ld_level, draft_ld_row, float(temperature), _ptr(tokens, i32),
-        _ptr(parent, i32), _ptr(u_accept, f64), _ptr(u_sample, f64), _ptr(accept_path, i32), _ptr(accept_len, i32),
-        _ptr(out_tokens, i32), _ptr(steps_next, i32), _stream(stream)), "resps_verify_accept_sampled")
+    _check(ctx._calls.resps_verify_accept_sampled(
+        ctx._address, steps, n_nodes, batch, target_logits, ld_b, ld_row, draft_logits, draft_ld_b, draft_ld_level,
+        draft_ld_row, temperature, tokens, parent, u_accept, u_sample, accept_path, accept_len, out_tokens, steps_next,
+        stream),
+        "resps_verify_accept_sampled")
 
 
 CONTROLLER_STATE_DTYPE = torch.int32  # resps_controller_state = (int32, int32, float32, int32): tensors [batch, 4]
@@ -258,49 +263,43 @@ def resps_controller_step(ctx: Context, policy: RespsPolicy, hidden_h, hidden_m,
                           interval: int, temperature: float, uniform, prev_accept_len, prev_elapsed_s, state, steps,
                           reward_avg, logits=None, action=None, stream=None) -> None:
     """One controller step (action cache, policy network, averaged reward); writes (TT, d, k) into `steps`."""
-    bf, i32, f32 = torch.bfloat16, torch.int32, torch.float32
-    _check(load().resps_controller_step(
-        ctx.handle, ctypes.byref(policy), _ptr(hidden_h, bf), _ptr(hidden_m, bf), _ptr(hidden_l, bf), ld_hidden, batch,
-        interval, float(temperature), _ptr(uniform, torch.float64), _ptr(prev_accept_len, i32),
-        _ptr(prev_elapsed_s, f32), _ptr(state, i32), _ptr(steps, i32), _ptr(reward_avg, f32), _ptr(logits, f32),
-        _ptr(action, i32), _stream(stream)), "resps_controller_step")
+    _check(ctx._calls.resps_controller_step(
+        ctx._address, ctypes.addressof(policy), hidden_h, hidden_m, hidden_l, ld_hidden, batch, interval, temperature,
+        uniform, prev_accept_len, prev_elapsed_s, state, steps, reward_avg, logits, action, stream),
+        "resps_controller_step")
 
 
 def resps_row_scan_shard(ctx: Context, steps, batch: int, draft_logits, ld_b: int, ld_level: int, ld_row: int,
                          n_levels: int, n_slots: int, part_val, part_id, part_lse, stream=None) -> None:
-    _check(load().resps_row_scan_shard(
-        ctx.handle, _ptr(steps, torch.int32), batch, _ptr(draft_logits, torch.float32), ld_b, ld_level, ld_row,
-        n_levels, n_slots, _ptr(part_val, torch.float32), _ptr(part_id, torch.int32), _ptr(part_lse, torch.float64),
-        _stream(stream)), "resps_row_scan_shard")
+    _check(ctx._calls.resps_row_scan_shard(
+        ctx._address, steps, batch, draft_logits, ld_b, ld_level, ld_row, n_levels, n_slots, part_val, part_id,
+        part_lse, stream),
+        "resps_row_scan_shard")
 
 
 def resps_tree_expand_merge(ctx: Context, steps, batch: int, n_levels: int, n_slots: int, n_shards: int, all_val,
                             all_id, all_lse, shard_offset, root_token, tokens, parent, depth, position_ids, mask,
                             retrieve, n_leaves, n_nodes, stream=None) -> None:
-    i32 = torch.int32
-    _check(load().resps_tree_expand_merge(
-        ctx.handle, _ptr(steps, i32), batch, n_levels, n_slots, n_shards, _ptr(all_val, torch.float32),
-        _ptr(all_id, i32), _ptr(all_lse, torch.float64), _ptr(shard_offset, i32), _ptr(root_token, i32),
-        _ptr(tokens, i32), _ptr(parent, i32), _ptr(depth, i32), _ptr(position_ids, i32), _ptr(mask),
-        _ptr(retrieve, i32), _ptr(n_leaves, i32), _ptr(n_nodes, i32), _stream(stream)), "resps_tree_expand_merge")
+    _check(ctx._calls.resps_tree_expand_merge(
+        ctx._address, steps, batch, n_levels, n_slots, n_shards, all_val, all_id, all_lse, shard_offset, root_token,
+        tokens, parent, depth, position_ids, mask, retrieve, n_leaves, n_nodes, stream),
+        "resps_tree_expand_merge")
 
 
 def resps_target_argmax_shard(ctx: Context, n_nodes, batch: int, target_logits, ld_b: int, ld_row: int, part_key,
                               stream=None) -> None:
-    _check(load().resps_target_argmax_shard(
-        ctx.handle, _ptr(n_nodes, torch.int32), batch, _ptr(target_logits, torch.float32), ld_b, ld_row,
-        _ptr(part_key, torch.int64), _stream(stream)), "resps_target_argmax_shard")
+    _check(ctx._calls.resps_target_argmax_shard(
+        ctx._address, n_nodes, batch, target_logits, ld_b, ld_row, part_key, stream),
+        "resps_target_argmax_shard")
 
 
 def resps_verify_accept_merge(ctx: Context, steps, n_nodes, batch: int, n_shards: int, all_key, shard_offset, tokens,
                               parent, target_argmax, accept_path, accept_len, out_tokens, steps_next=None,
                               stream=None) -> None:
-    i32 = torch.int32
-    _check(load().resps_verify_accept_merge(
-        ctx.handle, _ptr(steps, i32), _ptr(n_nodes, i32), batch, n_shards, _ptr(all_key, torch.int64),
-        _ptr(shard_offset, i32), _ptr(tokens, i32), _ptr(parent, i32), _ptr(target_argmax, i32),
-        _ptr(accept_path, i32), _ptr(accept_len, i32), _ptr(out_tokens, i32), _ptr(steps_next, i32),
-        _stream(stream)), "resps_verify_accept_merge")
+    _check(ctx._calls.resps_verify_accept_merge(
+        ctx._address, steps, n_nodes, batch, n_shards, all_key, shard_offset, tokens, parent, target_argmax,
+        accept_path, accept_len, out_tokens, steps_next, stream),
+        "resps_verify_accept_merge")
 
 
 def shard_columns(vocab: int, n_shards: int, multiple: int = 4):
@@ -334,21 +333,19 @@ def resps_kv_compact(ctx: Context, steps, batch: int, accept_path, accept_len, k
                      stream=None) -> None:
     """k_cache_ptrs / v_cache_ptrs: int64 CUDA tensors holding n_layers device pointers.
     steps_advanced: `steps` was already advanced by resps_verify_accept (steps_next aliased it)."""
-    i32 = torch.int32
-    _check(load().resps_kv_compact(
-        ctx.handle, _ptr(steps, i32), int(bool(steps_advanced)), batch, _ptr(accept_path, i32),
-        _ptr(accept_len, i32), _ptr(k_cache_ptrs, torch.int64), _ptr(v_cache_ptrs, torch.int64), n_layers,
-        kv_stride_seq, kv_stride_head, kv_stride_tok, kv_capacity, _stream(stream)), "resps_kv_compact")
+    _check(ctx._calls.resps_kv_compact(
+        ctx._address, steps, bool(steps_advanced), batch, accept_path, accept_len, k_cache_ptrs, v_cache_ptrs,
+        n_layers, kv_stride_seq, kv_stride_head, kv_stride_tok, kv_capacity, stream),
+        "resps_kv_compact")
 
 
 def resps_target_argmax_static(n_nodes, batch: int, max_tt: int, vocab: int, target_logits, ld_b: int,
                                ld_row: int, target_argmax, stream=None) -> None:
     """Per-node arg-max with no context and no allocation (scratch is a fixed array inside the
     library).  For callers that may not call cudaMalloc; batch * max_tt <= 1024."""
-    i32 = torch.int32
-    _check(load().resps_target_argmax_static(
-        _ptr(n_nodes, i32), batch, max_tt, vocab, _ptr(target_logits, torch.float32), ld_b, ld_row,
-        _ptr(target_argmax, i32), _stream(stream)), "resps_target_argmax_static")
+    _check(load().calls.resps_target_argmax_static(
+        n_nodes, batch, max_tt, vocab, target_logits, ld_b, ld_row, target_argmax, stream),
+        "resps_target_argmax_static")
 
 
 def layer_pointer_table(caches: Sequence[torch.Tensor]) -> torch.Tensor:

@@ -1,9 +1,11 @@
-"""Builds libresps.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libresps.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _call (the Python
+side of its entry points, csrc/call.cpp) with the host compiler."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -23,6 +25,8 @@ def _newer(target: str, deps) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+CALL_SRC = os.path.join(CSRC, "call.cpp")
+CALL_LIB = os.path.join(HERE, "_call" + sysconfig.get_config_var("EXT_SUFFIX"))
 WAIT_TEST_LIB = os.path.join(HERE, "libresps_waittest.so")
 
 
@@ -33,7 +37,32 @@ def build(force: bool = False, verbose: bool = False, wait_test: bool = False) -
     nvcc = os.environ.get("NVCC", "nvcc")
     if wait_test:
         return _build_into(nvcc, os.path.join(OBJ, "waittest"), WAIT_TEST_LIB, ["-DRESPS_WAIT_TEST"], force, verbose)
-    return _build_into(nvcc, OBJ, LIB, [], force, verbose)
+    with ThreadPoolExecutor(max_workers=1) as ex:
+        call = ex.submit(_build_call, force, verbose)
+        lib = _build_into(nvcc, OBJ, LIB, [], force, verbose)
+        call.result()
+    return lib
+
+
+def _build_call(force: bool, verbose: bool) -> None:
+    if not (force or _newer(CALL_LIB, [CALL_SRC, os.path.join(ROOT, "include", "resps.h")])):
+        return
+    import torch
+    from torch.utils.cpp_extension import include_paths
+    libs = os.path.join(os.path.dirname(torch.__file__), "lib")
+    tmp = CALL_LIB + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", CALL_SRC, "-o", tmp,
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"]]
+    for d in include_paths("cuda"):
+        cmd += ["-isystem", d]
+    cmd += ["-L", libs, "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or res.returncode:
+        sys.stderr.write(" ".join(cmd) + "\n" + res.stdout + res.stderr)
+    if res.returncode:
+        raise RuntimeError("g++ failed for csrc/call.cpp")
+    os.replace(tmp, CALL_LIB)
 
 
 def _build_into(nvcc, OBJ, LIB, extra_flags, force, verbose) -> str:
