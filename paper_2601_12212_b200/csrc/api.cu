@@ -53,6 +53,8 @@ void carve(resps_ctx* c, Carver& cv) {
     const int64_t zero_end = cv.off;  // everything above must start as zero
     (void)zero_end;
     cv.take(w.node_row, nodes);
+    cv.take(w.tree_frontier, static_cast<int64_t>(s.max_batch) * RESPS_MAX_DEPTH * RESPS_MAX_K);
+    cv.take(w.tree_score, static_cast<int64_t>(s.max_batch) * RESPS_MAX_DEPTH * RESPS_MAX_K);
     cv.take(w.amax_local, nodes);
     cv.take(w.ctl_h1, static_cast<int64_t>(s.max_batch) * resps::controller_max_hidden());
     cv.take(w.samp_scratch, static_cast<int64_t>(resps::sampled_scratch_doubles(s.max_batch, s.vocab)));

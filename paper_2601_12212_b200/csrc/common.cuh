@@ -39,6 +39,8 @@ struct Workspace {
     unsigned int* amax_counter = nullptr;    // [max_batch][max_tt]
     int32_t* amax_local = nullptr;           // [max_batch][max_tt] shard-local arg-max ids (vocabulary sharding)
     int32_t* node_row = nullptr;             // [max_batch][max_tt] draft row behind every node's children (tree build)
+    int32_t* tree_frontier = nullptr;        // [max_batch][RESPS_MAX_DEPTH][RESPS_MAX_K] level form: frontiers so far
+    double* tree_score = nullptr;            // ... and their path scores
     float* ctl_h1 = nullptr;                 // controller: first hidden layer [max_batch][256]
     unsigned int* ctl_counter = nullptr;     // controller: hidden units done per sequence (self-resetting)
     double* samp_scratch = nullptr;          // acceptance under sampling: partial sums, then (p, q) of every token and sequence
@@ -103,7 +105,7 @@ cudaError_t launch_tree_build(const resps_ctx* ctx, const resps_step* d_steps, i
                               int n_levels, int n_slots, const int32_t* root_token,
                               int32_t* tokens, int32_t* parent, int32_t* depth, int32_t* position_ids,
                               uint64_t* mask, int32_t* retrieve, int32_t* n_leaves, int32_t* n_nodes,
-                              cudaStream_t st, bool after_scan);  // after_scan: a scan or merge kernel of the same call precedes it
+                              cudaStream_t st, bool after_scan);  // after_scan: a scan or merge kernel of the same call precedes it; else the level form's last call
 // Arg-max of every target row; with `walk` non-null and rows that allow the streaming kernel the
 // acceptance walk runs in the same kernel (returns true through `walked`).
 cudaError_t launch_row_argmax(const resps_ctx* ctx, const int32_t* d_n_nodes, int batch,

@@ -4,11 +4,13 @@
 // best TT-1 kept; Algorithm 2, tree-building loop).  One CTA per sequence; integer
 // and fp64 work on at most k + (d-1)k^2 candidates, all in shared memory.
 //
-// Every level's candidates are k lists (one per frontier member), each already in the method's
-// order because a scanned row is sorted; a candidate's rank inside its level is its place in its own
-// list plus, for every other list, a binary search (one thread per candidate and list).  Its rank in
-// the global rerank is its level rank plus binary searches over the other levels' sorted heads, and
-// only the first TT-1 of a level can be kept at all.
+// A level's candidates are k lists (one per frontier member), each already in the method's order
+// because a scanned row is sorted.  The next frontier is the k best of them: one warp takes the best
+// list head k times.  The rerank is a selection over all candidates by a histogram of the scores.
+//
+// Bound by latency: one CTA per sequence and a chain of small dependent steps.  What is kept short is
+// the chain, and what is avoided is work that grows with k^3: ranking every candidate of a level
+// against every other list (k^3 searches a level) took 598 us at TT=128, d=8, k=32 (7200 candidates).
 #include <cmath>
 
 #include "common.cuh"
@@ -16,12 +18,22 @@
 namespace resps {
 namespace {
 
-constexpr int kTreeThreads = 1024;
+constexpr int kTreeThreads = 512;
 constexpr unsigned kFull = 0xFFFFFFFFu;
-constexpr int kStride = 8;                       // rerank: level ranks between two coarse probes
-constexpr int kProbes = RESPS_MAX_TT / kStride;  // coarse probes per level
-constexpr int kTokPrefetch = 2;  // token ids of the first 2 x 1024 candidates travel in registers
-static_assert(kTreeThreads == 1024, "the node-index scan assumes 32 warps");
+constexpr int kLevelThreads = 256;  // a launch that ranks one level only (level form)
+constexpr int kBins = kTreeThreads;         // steps of score in the rerank's histogram
+constexpr int kTieList = 256;       // candidates of one step that are ranked by counting
+constexpr double kLowest = -1e30;   // log-probabilities stay finite
+
+struct TreeShared {
+    int kept[RESPS_MAX_TT];  // candidates kept by the rerank, in no order
+    int hist[kBins];
+    int list[kTieList];
+    int parent[RESPS_MAX_TT], depth[RESPS_MAX_TT], has_child[RESPS_MAX_TT], row[RESPS_MAX_TT];
+    int warp_sum[32];
+    int n_kept, n_list, cut, cut_before, cut_count;
+    long long low, high;
+};
 
 struct TreeArgs {
     const resps_step* steps;
@@ -41,12 +53,16 @@ struct TreeArgs {
     // the frontier after level j and stops; -1 builds the whole tree.
     int emit_level;
     FrontierOut fr;
+    // Frontiers of the levels ranked so far [batch][RESPS_MAX_DEPTH][RESPS_MAX_K] (level form: every call
+    // ranks one level and leaves its frontier here; use_state = 1 reads it).
+    int32_t* state_frontier;
+    double* state_score;
+    int use_state;
     int setup_before_wait;  // 1: a scan or merge kernel of the same call runs directly before this kernel
 };
 
-// Path scores are compared as integers: the map below keeps the order of finite doubles (and their
-// equality, zero being stored as +0); an integer key turns "at least" into "above key - 1", which
-// spares the searches the tie-break read.  The map is its own inverse.
+// Path scores as integers, for the warp-wide maximum and the shared-memory minimum: the map keeps the
+// order of finite doubles (and their equality, zero being stored as +0) and is its own inverse.
 __device__ __forceinline__ long long score_key(double s) {
     const long long bits = __double_as_longlong(s + 0.0);
     return bits ^ ((bits >> 63) & 0x7FFFFFFFFFFFFFFFll);
@@ -63,23 +79,6 @@ struct FastDiv {
     __device__ __forceinline__ int div(int e) const { return __float2int_rd((static_cast<float>(e) + 0.5f) * inv); }
 };
 
-// Leading entries of the descending key list `keys[0..n)` that are above `thr`; `top` is the largest
-// power of two <= n (0 for an empty list).  A fixed number of steps without data-dependent branches.
-//
-// Candidate order of the method: larger score first, equal scores by lower candidate index.  Two
-// candidates of different lists of a level, or of different levels, compare by index the same way
-// for the whole list, so "before (key, c)" is "key above thr" with thr = key - 1 where the list's
-// indices are the lower ones and thr = key otherwise.
-__device__ __forceinline__ int count_above(const long long* keys, int n, int top, long long thr) {
-    int pos = 0;
-    for (int half = top; half > 0; half >>= 1) {
-        const int t = pos + half;
-        if (t <= n && keys[t - 1] > thr) pos = t;
-    }
-    return pos;
-}
-__device__ __forceinline__ int pow2_floor(int n) { return (n > 0) ? (1 << (31 - __clz(n))) : 0; }
-
 __global__ void __launch_bounds__(kTreeThreads, 1) tree_build_kernel(const TreeArgs a) {
     // The step parameters were written at least two kernels ago (a scan or a merge kernel of the same
     // call always sits between their writer and this kernel, and every kernel of the library signals its
@@ -88,7 +87,7 @@ __global__ void __launch_bounds__(kTreeThreads, 1) tree_build_kernel(const TreeA
     // kernel precedes this one -- the last call of the level form -- the wait comes first.)
     if (!a.setup_before_wait) pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int b = blockIdx.x, tid = threadIdx.x;
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthreads = blockDim.x;
     const StepDims sd = clamp_step(a.steps[b], a.n_levels, a.n_slots, a.max_tt, a.max_k, a.vocab);
     const int k = sd.k, kk = k * k;
     const int d = (a.emit_level >= 0) ? min(sd.d, a.emit_level + 1) : sd.d;  // levels ranked by this launch
@@ -96,22 +95,15 @@ __global__ void __launch_bounds__(kTreeThreads, 1) tree_build_kernel(const TreeA
     const int m = min(sd.tt - 1, n_cand);
     const int n = m + 1;
 
-    long long* skey = reinterpret_cast<long long*>(smem_raw);             // [cand_cap] own log-prob (as a double), then the key of the path score
-    long long* head_key = skey + a.cand_cap;                              // [max_depth][max_tt] keys of a level's first ranks
-    double* fscore = reinterpret_cast<double*>(head_key + RESPS_MAX_DEPTH * RESPS_MAX_TT);  // [max_depth][max_k] frontier scores
-    int* node_of = reinterpret_cast<int*>(fscore + RESPS_MAX_DEPTH * RESPS_MAX_K);  // [cand_cap] rank counters, level rank, then node index
-    int* frontier = node_of + a.cand_cap;                                 // [max_depth][max_k]
-    int* s_parent = frontier + RESPS_MAX_DEPTH * RESPS_MAX_K;             // [max_tt] node -> parent node
-    int* s_flag = s_parent + RESPS_MAX_TT;                                // [max_tt] has-child flags
-    int* s_warp = s_flag + RESPS_MAX_TT;                                  // [2][32] scan scratch
-    int* probe = s_warp + 64;                                             // [max_depth][kProbes] rerank counters, coarse
-    int* fine = probe + RESPS_MAX_DEPTH * kProbes;                        // [max_depth][kStride] rerank counters, fine
-    int* n_coarse = fine + RESPS_MAX_DEPTH * kStride;                     // [max_depth] probes kept
-    int* n_fine = n_coarse + RESPS_MAX_DEPTH;                             // [max_depth] kept after the last kept probe
+    double* score = reinterpret_cast<double*>(smem_raw);                  // [cand_cap] own log-prob, then the path score
+    double* fscore = score + a.cand_cap;                                  // [max_depth][max_k] frontier scores
+    int* node_of = reinterpret_cast<int*>(fscore + RESPS_MAX_DEPTH * RESPS_MAX_K);  // [cand_cap] node index of a kept candidate
+    int* frontier = node_of + a.cand_cap;                                 // [max_depth][max_k] candidates
+    __shared__ TreeShared sh;
 
-    // The kernel is bound by instruction issue (one CTA of 32 warps), so index arithmetic by the
-    // run-time k, k^2 and d goes through an exact float reciprocal (operands stay below 2^22).
-    const FastDiv by_k(k), by_kk(kk), by_d(d);
+    // Index arithmetic by the run-time k and k^2 goes through an exact float reciprocal (operands stay
+    // below 2^22).
+    const FastDiv by_k(k), by_kk(kk);
     const int64_t row0 = static_cast<int64_t>(b) * a.max_rows;
     struct Cand {
         int level, list, place;  // level, list inside the level (frontier slot of the parent), place in the list
@@ -128,81 +120,127 @@ __global__ void __launch_bounds__(kTreeThreads, 1) tree_build_kernel(const TreeA
         }
         return r;
     };
+    auto parent_of = [&](int c) {  // the parent's place in the frontier arrays, -1: the root
+        if (c < k) return -1;
+        const int t = c - k, jm1 = by_kk.div(t);
+        return jm1 * RESPS_MAX_K + by_k.div(t - jm1 * kk);
+    };
     auto cand_row = [&](const Cand& r) { return (r.level == 0) ? 0 : 1 + (r.level - 1) * k + r.list; };
 
-    // ---- every candidate's own log-probability, in one round trip to global memory (the rows
-    // a level reads do not depend on the levels before it); the token ids of the first candidates
-    // come along in registers for the outputs at the end ---------------------------------------
-    const Cand own = decode(min(tid, n_cand - 1));  // candidate tid, reused by the later passes over candidates
-    int tok_pre[kTokPrefetch];
+#pragma unroll 1
+    for (int i = tid; i < kBins; i += nthreads) sh.hist[i] = 0;
+    if (tid < RESPS_MAX_TT) sh.kept[tid] = 0x7FFFFFFF, sh.has_child[tid] = 0, sh.row[tid] = -1;
+    if (tid == 0) sh.n_kept = 0;
+    // Level form: a call ranks one level, the last call none; what the calls before left in the workspace
+    // is read instead (levels >= 1; level 0 is the first row itself).
+    const int first_level = (a.emit_level >= 0) ? a.emit_level : 0;  // the first level this launch needs the rows of
+    const int c_first = (first_level == 0) ? 0 : k + (first_level - 1) * kk;
+    const int64_t state0 = static_cast<int64_t>(b) * RESPS_MAX_DEPTH * RESPS_MAX_K;
+    constexpr int kAhead = 4;  // candidates a thread loads together; the first ones are located before the wait
+    int64_t at_row[kAhead], at[kAhead];
+    auto locate = [&](int c0) {
 #pragma unroll
-    for (int i = 0; i < kTokPrefetch; ++i) tok_pre[i] = 0;
-    for (int i = tid; i < RESPS_MAX_DEPTH * (kProbes + kStride + 2); i += kTreeThreads) probe[i] = 0;
-    // the first pass of the per-level loops below has the same index arithmetic at every level
-    const int pair_i = by_k.div(tid), pair_p2 = tid - pair_i * k, pair_p = by_k.div(pair_i);  // pair tid = (candidate, list)
-    const int k_top = pow2_floor(k);
+        for (int u = 0; u < kAhead; ++u) {
+            const Cand r = decode(min(c0 + u * nthreads, n_cand - 1));
+            at_row[u] = row0 + cand_row(r);
+            at[u] = at_row[u] * a.max_k + r.place;
+        }
+    };
+    locate(c_first + tid);
+    const int own_parent = parent_of(tid);
     if (a.setup_before_wait) pdl_wait();  // the kernel before this one in the stream has completed: the scanned rows are there
     pdl_launch_dependents();
-    for (int c = tid, i = 0; c < n_cand; c += kTreeThreads, ++i) {
-        const Cand r = (i == 0) ? own : decode(c);
-        const int64_t row = row0 + cand_row(r);
-        const int64_t at = row * a.max_k + r.place;
-        if (i < kTokPrefetch && a.emit_level < 0) {
-#pragma unroll
-            for (int u = 0; u < kTokPrefetch; ++u)
-                if (u == i) tok_pre[u] = a.row_id[at];
-        }
-        // (+ 0.0 stores a zero as +0, so that equal scores have equal keys)
-        const double lp = fmin(static_cast<double>(a.row_val[at]) - a.row_lse[row], 0.0) + 0.0;
-        skey[c] = (c < k) ? score_key(lp) : __double_as_longlong(lp);
-        node_of[c] = (c < k) ? c : 0;  // level 0 is ranked as scanned; the other levels count from 0
+    if (a.emit_level >= 0 && a.emit_level >= sd.d) {
+        // (a sequence whose own d is below j + 1 has nothing at this level: its entries stay untouched)
+        if (tid == 0 && sd.clamped) atomicOr(a.status, RESPS_STATUS_STEP_CLAMPED);
+        return;
     }
-    __syncthreads();
-    // ---- level 0 ---------------------------------------------------------------
-    if (tid < k) {
-        frontier[tid] = tid;
-        fscore[tid] = key_score(skey[tid]);
-        head_key[tid] = skey[tid];
+    if (a.use_state) {
+        const int known = (a.emit_level >= 0) ? a.emit_level : d;  // levels ranked by earlier calls
+#pragma unroll 1
+        for (int i = tid; i < known * RESPS_MAX_K; i += nthreads) {
+            frontier[i] = a.state_frontier[state0 + i];
+            fscore[i] = a.state_score[state0 + i];
+        }
+    }
+    // ---- every candidate's own log-probability, in one round trip to global memory (the rows
+    // a level reads do not depend on the levels before it) ------------------------------------------
+#pragma unroll 1
+    for (int c0 = c_first + tid; c0 < n_cand; c0 += kAhead * nthreads) {
+        float val[kAhead];
+        double lse[kAhead];
+        if (c0 != c_first + tid) locate(c0);
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            if (c0 + u * nthreads < n_cand) val[u] = a.row_val[at[u]], lse[u] = a.row_lse[at_row[u]];
+        }
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int c = c0 + u * nthreads;
+            if (c < n_cand) score[c] = fmax(fmin(static_cast<double>(val[u]) - lse[u], 0.0), kLowest) + 0.0;
+        }
     }
     __syncthreads();
 
-    // ---- levels 1..d-1 -----------------------------------------------------------
-    for (int j = 1; j < d; ++j) {
-        const int base = k + (j - 1) * kk;
-        const double* fs = fscore + (j - 1) * RESPS_MAX_K;
-        // path score = own log-probability + the parent's path score, kept as its key
-        for (int i = tid; i < kk; i += kTreeThreads) {
-            const int p = (i == tid) ? pair_i : by_k.div(i);  // (pair_i = tid / k)
-            skey[base + i] = score_key(__longlong_as_double(skey[base + i]) + fs[p]);
+    // ---- frontiers: one warp walks the levels.  A level's candidates are k lists (one per frontier
+    // member) already in the method's order, because a scanned row is sorted, and only the k best of the
+    // level are needed: lane p holds the head of list p, and k times the best head is taken (ties by the
+    // lower lane, which has the lower candidate indices).  No block-wide barrier in the chain, no branch
+    // on a lane's own data, and the entry behind a head is made ready in the shadow of the reduction:
+    // about 150 cycles an entry (an insertion into the order of the heads took 420, a binary search of
+    // every candidate in every other list 4000-25000 a level, against 1900 for k = 10 and 4800 for k = 32).
+    if (warp == 0) {
+        if (first_level == 0) {
+            if (lane < k) frontier[lane] = lane, fscore[lane] = score[lane];
+            __syncwarp();
         }
-        __syncthreads();
-        // one thread per (candidate, other list): candidates of that list ranking before it
-        for (int e = tid; e < kk * k; e += kTreeThreads) {
-            int i = pair_i, p2 = pair_p2, p = pair_p;
-            if (e != tid) {
-                i = by_k.div(e), p2 = e - i * k;
-                p = by_k.div(i);
+        const int j0 = (a.use_state && a.emit_level < 0) ? d : max(first_level, 1);
+#pragma unroll 1
+        for (int j = j0; j < d; ++j) {
+            constexpr long long kNone = static_cast<long long>(0x8000000000000000ull);
+            const bool on = lane < k;
+            const int base = k + (j - 1) * kk;
+            const double parent = on ? fscore[(j - 1) * RESPS_MAX_K + lane] : 0.0;
+            const double* list = score + base + lane * k;
+            double head_score = on ? list[0] + parent : 0.0;
+            long long head = on ? score_key(head_score) : kNone;
+            double next = (on && k > 1) ? list[1] : 0.0;
+            int place = 0;
+            const unsigned lower_lanes = (1u << lane) - 1u;
+#pragma unroll 1
+            for (int r = 0; r < k; ++r) {
+                const int hi = static_cast<int>(head >> 32);
+                const int top_hi = __reduce_max_sync(kFull, hi);
+                unsigned best = __ballot_sync(kFull, hi == top_hi);
+                const double next_score = next + parent;
+                const long long next_key = (on && place + 1 < k) ? score_key(next_score) : kNone;
+                if (best & (best - 1)) {  // the same upper half more than once: the lower half decides
+                    const bool in = hi == top_hi;
+                    const unsigned lo = in ? static_cast<unsigned>(head) : 0u;
+                    const unsigned top_lo = __reduce_max_sync(kFull, lo);  // (every lane takes part)
+                    best = __ballot_sync(kFull, in && lo == top_lo);
+                }
+                const bool win = ((best >> lane) & 1u) && !(best & lower_lanes);
+                if (win) {
+                    frontier[j * RESPS_MAX_K + r] = base + lane * k + place;
+                    fscore[j * RESPS_MAX_K + r] = head_score;
+                }
+                head = win ? next_key : head;
+                head_score = win ? next_score : head_score;
+                place += win ? 1 : 0;
+                if (win) next = list[min(place + 1, k - 1)];
             }
-            if (p2 == p) continue;
-            const int c = base + i;
-            const int cnt = count_above(skey + base + p2 * k, k, k_top, skey[c] - ((p2 < p) ? 1 : 0));
-            if (cnt) atomicAdd(&node_of[c], cnt);
+            __syncwarp();
         }
-        __syncthreads();
-        // level rank = place in the own list + the counts; the k best form the next frontier
-        for (int i = tid; i < kk; i += kTreeThreads) {
-            const int c = base + i, p = (i == tid) ? pair_i : by_k.div(i);
-            const int rank = (i - p * k) + node_of[c];
-            const long long key = skey[c];
-            node_of[c] = rank;
-            if (rank < k) {
-                frontier[j * RESPS_MAX_K + rank] = c;
-                fscore[j * RESPS_MAX_K + rank] = key_score(key);
-            }
-            if (rank < RESPS_MAX_TT) head_key[j * RESPS_MAX_TT + rank] = key;
+        if (a.emit_level < 0) {
+            // a lower bound of the rerank's m-th best, if the frontiers alone hold m candidates: their
+            // worst member (the lower half of its key cleared)
+            const int mine = (lane < d) ? static_cast<int>(score_key(fscore[lane * RESPS_MAX_K + k - 1]) >> 32) : 0x7FFFFFFF;
+            const int least = __reduce_min_sync(kFull, mine);
+            if (lane == 0) sh.low = static_cast<long long>(least) << 32;
         }
-        __syncthreads();
     }
+    __syncthreads();
 
     if (a.emit_level >= 0) {
         // ---- level form: the frontier after level j, for the draft model's next pass ------------------
@@ -210,18 +248,21 @@ __global__ void __launch_bounds__(kTreeThreads, 1) tree_build_kernel(const TreeA
         // 1 + i k .. i k + k): token, the slot of its parent in the previous frontier, position id, the
         // ancestor-or-self mask over draft nodes (only while they fit 128 bits) and its score.
         const int j = a.emit_level;
-        if (j < sd.d && tid < k) {
+        if (tid < k) {
             const int c = frontier[j * RESPS_MAX_K + tid];
             const int64_t of = static_cast<int64_t>(b) * a.max_k + tid;
             const Cand r = decode(c);
             a.fr.tokens[of] = a.row_id[(row0 + cand_row(r)) * a.max_k + r.place];
-            a.fr.parent_slot[of] = (j == 0) ? -1 : ((c - (k + (j - 1) * kk)) / k);
+            a.fr.parent_slot[of] = (j == 0) ? -1 : r.list;
             a.fr.position_ids[of] = sd.L + j + 1;
             a.fr.node_index[of] = 1 + j * k + tid;
-            if (a.fr.score) a.fr.score[of] = key_score(skey[c]);
+            if (a.fr.score) a.fr.score[of] = fscore[j * RESPS_MAX_K + tid];
+            a.state_frontier[state0 + j * RESPS_MAX_K + tid] = c;
+            a.state_score[state0 + j * RESPS_MAX_K + tid] = fscore[j * RESPS_MAX_K + tid];
             unsigned long long lo = 1ull, hi = 0ull;  // the root
             if (1 + (j + 1) * k <= 128) {
                 int cc = c, slot = tid;
+#pragma unroll 1
                 for (int jj = j; jj >= 0; --jj) {
                     const int node = 1 + jj * k + slot;
                     if (node < 64)
@@ -229,7 +270,7 @@ __global__ void __launch_bounds__(kTreeThreads, 1) tree_build_kernel(const TreeA
                     else
                         hi |= 1ull << (node - 64);
                     if (jj > 0) {
-                        slot = (cc - (k + (jj - 1) * kk)) / k;
+                        slot = by_k.div(cc - (k + (jj - 1) * kk));
                         cc = frontier[(jj - 1) * RESPS_MAX_K + slot];
                     }
                 }
@@ -239,176 +280,229 @@ __global__ void __launch_bounds__(kTreeThreads, 1) tree_build_kernel(const TreeA
             a.fr.mask[of * 2 + 0] = lo;
             a.fr.mask[of * 2 + 1] = hi;
         }
-        // (a sequence whose own d is below j + 1 has nothing at this level: its entries stay untouched)
         if (tid == 0 && sd.clamped) atomicOr(a.status, RESPS_STATUS_STEP_CLAMPED);
         return;
     }
 
-    // ---- global rerank: keep the m best of all candidates -------------------------
-    // Inside a level the global rank grows with the level rank, so a level keeps a prefix of its
-    // sorted order and only the prefix length is needed.  A candidate's global rank is its level
-    // rank plus, per other level, a binary search over that level's first m scores (one thread per
-    // candidate and level).  Coarse pass: every kStride-th level rank; fine pass: the kStride-1
-    // ranks after the last probe that was kept.
-    const int mm = min(kk, m), m0 = min(k, m);
-    auto level_head = [&](int j) { return (j == 0) ? m0 : mm; };
-    const int mm_top = pow2_floor(mm), m0_top = pow2_floor(m0);
-    auto others_before = [&](int j, int i, int q) {  // of level q's first m, those before (level j, rank i)
-        const long long key = head_key[j * RESPS_MAX_TT + i];
-        return count_above(head_key + q * RESPS_MAX_TT, level_head(q), (q == 0) ? m0_top : mm_top, key - ((q < j) ? 1 : 0));
+    // ---- global rerank: keep the m best of all candidates -------------------------------------------
+    // A selection, not a sort: a histogram over equal steps of score between the best score (a first-level
+    // candidate: scores only fall along a path) and a lower bound of the m-th best finds the step in which
+    // the m-th best lies; the steps above are kept whole, and the few candidates inside it are ranked by
+    // counting.  The bound is the worst frontier member when the frontiers alone hold m candidates, else
+    // the worst candidate.  A step with many candidates is cut again; one whose candidates all tie is cut
+    // by index.  (Subtraction, product and truncation are monotone, so a better score is never in a later
+    // step.)
+    const bool bounded = d * k >= m;
+    double top = fscore[0], low = key_score(sh.low), inv = 0.0;
+    auto set_range = [&](double t, double l) {  // (the reciprocal need not be exact, only the same for all)
+        top = t, low = l;
+        inv = static_cast<double>(__fdividef(static_cast<float>(kBins), static_cast<float>(t - l)));
     };
-    const int n_probe = (mm + kStride - 1) / kStride;
-    const FastDiv by_probe(max(n_probe, 1)), by_fine(kStride - 1);
-    for (int e = tid; e < d * n_probe * d; e += kTreeThreads) {
-        const int slot = by_d.div(e), q = e - slot * d;
-        const int j = by_probe.div(slot), u = slot - j * n_probe;
-        if (q == j || u * kStride >= level_head(j)) continue;
-        const int cnt = others_before(j, u * kStride, q);
-        if (cnt) atomicAdd(&probe[j * kProbes + u], cnt);
-    }
-    __syncthreads();
-    for (int e = tid; e < d * n_probe; e += kTreeThreads) {
-        const int j = by_probe.div(e), u = e - j * n_probe;
-        if (u * kStride < level_head(j) && u * kStride + probe[j * kProbes + u] < m) atomicAdd(&n_coarse[j], 1);
-    }
-    __syncthreads();
-    for (int e = tid; e < d * (kStride - 1) * d; e += kTreeThreads) {
-        const int slot = by_d.div(e), q = e - slot * d;
-        const int j = by_fine.div(slot), w = slot - j * (kStride - 1) + 1;
-        const int kept = n_coarse[j];
-        const int i = (kept - 1) * kStride + w;
-        if (q == j || kept == 0 || i >= level_head(j)) continue;
-        const int cnt = others_before(j, i, q);
-        if (cnt) atomicAdd(&fine[j * kStride + w], cnt);
-    }
-    __syncthreads();
-    for (int e = tid; e < d * (kStride - 1); e += kTreeThreads) {
-        const int j = by_fine.div(e), w = e - j * (kStride - 1) + 1;
-        const int kept = n_coarse[j];
-        const int i = (kept - 1) * kStride + w;
-        if (kept > 0 && i < level_head(j) && i + fine[j * kStride + w] < m) atomicAdd(&n_fine[j], 1);
-    }
-    __syncthreads();
-    // level j keeps its first keep_of(j) ranks
-    auto keep_of = [&](int j) { return (n_coarse[j] > 0) ? (n_coarse[j] - 1) * kStride + 1 + n_fine[j] : 0; };
-
-    // ---- node index = 1 + kept candidates with a lower index ------------------------
-    const int lane = tid & 31, warp = tid >> 5;
-    int total = 0;
-    for (int c0 = 0, it = 0; c0 < n_cand; c0 += kTreeThreads, ++it) {
-        const int c = c0 + tid;
-        const int level = (it == 0) ? own.level : decode(min(c, n_cand - 1)).level;
-        const bool keep = (c < n_cand) && (node_of[c] < keep_of(level));
-        const unsigned bal = __ballot_sync(kFull, keep);
-        int* sw = s_warp + (it & 1) * 32;
-        if (lane == 0) sw[warp] = __popc(bal);
-        __syncthreads();
-        int inc = sw[lane];  // kTreeThreads / 32 == 32 warps
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(kFull, inc, o);
-            if (lane >= o) inc += t;
+    auto count = [&](int c, double s) {
+        int at = kBins;  // outside
+        if (s >= low && s <= top) {
+            at = max(min(__double2int_rz((top - s) * inv), kBins - 1), 0);  // (0 * inf counts as 0)
+            atomicAdd(&sh.hist[at], 1);
         }
-        const int before_warp = __shfl_sync(kFull, inc, warp) - __popc(bal);
-        const int chunk_total = __shfl_sync(kFull, inc, 31);
-        if (c < n_cand) node_of[c] = keep ? 1 + total + before_warp + __popc(bal & ((1u << lane) - 1u)) : 0;
-        total += chunk_total;
+        node_of[c] = at;
+    };
+    if (bounded) set_range(top, low);
+    double least = low;
+#pragma unroll 1
+    for (int c = tid, u = 0; c < n_cand; c += nthreads, ++u) {
+        const int parent = (u == 0) ? own_parent : parent_of(c);
+        double s = score[c];
+        if (parent >= 0) score[c] = s = s + fscore[parent];
+        if (bounded)
+            count(c, s);
+        else
+            least = fmin(least, s);
     }
+    if (!bounded) {
+        __syncthreads();
+        if (least < low) atomicMin(&sh.low, score_key(least));
+        __syncthreads();
+        set_range(top, key_score(sh.low));
+    }
+    int need = m;
+    constexpr int kMaxRounds = 256;  // (a round narrows the range of scores several hundredfold: never reached)
+#pragma unroll 1
+    for (int round = 0; need > 0 && round < kMaxRounds; ++round) {
+        if (round > 0 || !bounded)
+#pragma unroll 1
+            for (int c = tid; c < n_cand; c += nthreads) count(c, score[c]);
+        __syncthreads();
+        {  // the step in which the count reaches `need`; a warp's share of the steps is contiguous
+            const int mine = sh.hist[tid];
+            int incl = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += t;
+            }
+            if (lane == 31) sh.warp_sum[warp] = incl;
+            __syncthreads();
+            const int before_warp = __reduce_add_sync(kFull, lane < warp ? sh.warp_sum[lane] : 0);
+            const int before = before_warp + incl - mine;
+            if (before < need && before + mine >= need) sh.cut = tid, sh.cut_before = before, sh.cut_count = mine;
+            if (tid == 0) sh.n_list = 0, sh.low = score_key(top), sh.high = score_key(low);
+            sh.hist[tid] = 0;
+        }
+        __syncthreads();
+        const int cut = sh.cut, in_cut = sh.cut_count;
+        need -= sh.cut_before;
+        const bool whole = in_cut == need, again = !whole && in_cut > kTieList;
+#pragma unroll 1
+        for (int c0 = 0; c0 < n_cand; c0 += kTreeThreads) {
+            const int c = c0 + tid;
+            const int at = (c < n_cand) ? node_of[c] : kBins;
+            const bool keep = at < cut || (at == cut && whole);
+            const unsigned bal = __ballot_sync(kFull, keep);
+            if (bal) {  // one counter update per warp
+                int pos = 0;
+                if (lane == 0) pos = atomicAdd(&sh.n_kept, __popc(bal));
+                pos = __shfl_sync(kFull, pos, 0) + __popc(bal & ((1u << lane) - 1u));
+                if (keep) sh.kept[pos] = c;
+            }
+            if (c < n_cand) node_of[c] = 0;
+            if (at == cut && !whole) {
+                if (!again) {
+                    sh.list[atomicAdd(&sh.n_list, 1)] = c;
+                } else {
+                    atomicMin(&sh.low, score_key(score[c]));
+                    atomicMax(&sh.high, score_key(score[c]));
+                }
+            }
+        }
+        __syncthreads();
+        if (whole) break;
+        if (!again) {
+            if (tid < in_cut) {
+                const int c = sh.list[tid];
+                const double s = score[c];
+                int rank = 0;
+#pragma unroll 1
+                for (int i = 0; i < in_cut; ++i) {
+                    const int o = sh.list[i];
+                    rank += (score[o] > s || (score[o] == s && o < c)) ? 1 : 0;
+                }
+                if (rank < need) sh.kept[atomicAdd(&sh.n_kept, 1)] = c;
+            }
+            __syncthreads();
+            break;
+        }
+        set_range(key_score(sh.high), key_score(sh.low));
+        if (low == top) {  // equal scores: the lower indices
+#pragma unroll 1
+            for (int c0 = 0; need > 0 && c0 < n_cand; c0 += kTreeThreads) {
+                const int c = c0 + tid;
+                const bool tie = c < n_cand && score[c] == low;
+                const unsigned bal = __ballot_sync(kFull, tie);
+                __syncthreads();
+                if (lane == 0) sh.warp_sum[warp] = __popc(bal);
+                __syncthreads();
+                const int before = __reduce_add_sync(kFull, lane < warp ? sh.warp_sum[lane] : 0) + __popc(bal & ((1u << lane) - 1u));
+                if (tie && before < need) sh.kept[atomicAdd(&sh.n_kept, 1)] = c;
+                need -= __reduce_add_sync(kFull, lane < kTreeThreads / 32 ? sh.warp_sum[lane] : 0);
+            }
+            __syncthreads();
+            break;
+        }
+    }
+    if (tid >= RESPS_MAX_TT) return;  // at most 127 candidates are left: four warps and their own barrier
+    auto meet = [] { asm volatile("bar.sync 1, 128;" ::: "memory"); };
+
+    // ---- node index = 1 + kept candidates with a lower index ------------------------------------------
     const int64_t ob = static_cast<int64_t>(b) * a.max_tt;
-    __syncthreads();
+    int node = 0, token = 0, dep = 0;
+    Cand own = {0, 0, 0};
+    if (tid < m) {
+        const int c = sh.kept[tid];
+        own = decode(c);
+        token = a.row_id[(row0 + cand_row(own)) * a.max_k + own.place];  // on its way during what follows
+        dep = own.level + 1;
+        const int4* all = reinterpret_cast<const int4*>(sh.kept);
+#pragma unroll 1
+        for (int i = 0; i < (m + 3) / 4; ++i) {
+            const int4 v = all[i];
+            node += (v.x < c) + (v.y < c) + (v.z < c) + (v.w < c);
+        }
+        ++node;
+        node_of[c] = node;
+    } else if (tid == m) {
+        token = a.root_token[b];
+    }
+    meet();
+    int pn = -1;
+    if (tid < m) {
+        pn = (own.level == 0) ? 0 : node_of[frontier[(own.level - 1) * RESPS_MAX_K + own.list]];
+        sh.parent[node] = pn;
+        sh.has_child[pn] = 1;
+    } else if (tid == m) {
+        sh.parent[0] = -1;
+        sh.row[0] = 0;
+    }
     // The draft row every node's children were taken from (kept in the workspace for the acceptance
     // under sampling, which needs the draft distribution behind every tried child): the root's is row
     // (0, 0); the p-th member of the frontier after level j < d-1 was given row (j+1, p).
-    for (int i = tid; i < n; i += kTreeThreads) a.node_row[ob + i] = (i == 0) ? 0 : -1;
-    __syncthreads();
-    for (int e = tid; e < (d - 1) * k; e += kTreeThreads) {
+#pragma unroll 1
+    for (int e = tid; e < (d - 1) * k; e += RESPS_MAX_TT) {
         const int j = by_k.div(e), p = e - j * k;
         const int i = node_of[frontier[j * RESPS_MAX_K + p]];
-        if (i > 0) a.node_row[ob + i] = (j + 1) * RESPS_MAX_K + p;
+        if (i > 0) sh.row[i] = (j + 1) * RESPS_MAX_K + p;
     }
-    // `total` equals m by construction of the ranks.
-    for (int c = tid, it = 0; c < n_cand; c += kTreeThreads, ++it) {
-        const int i = node_of[c];
-        if (i == 0) continue;
-        const Cand r = (it == 0) ? own : decode(c);
-        const int pn = (r.level == 0) ? 0 : node_of[frontier[(r.level - 1) * RESPS_MAX_K + r.list]];
-        const int dep = r.level + 1;
-        int tok = 0;
-        if (it < kTokPrefetch) {
-#pragma unroll
-            for (int u = 0; u < kTokPrefetch; ++u)
-                if (u == it) tok = tok_pre[u];
-        } else {
-            tok = a.row_id[(row0 + cand_row(r)) * a.max_k + r.place];
-        }
-        a.tokens[ob + i] = tok;
-        a.parent[ob + i] = pn;
-        a.depth[ob + i] = dep;
-        a.position_ids[ob + i] = sd.L + dep;
-        s_parent[i] = pn;
-    }
-    if (tid == 0) {
-        a.tokens[ob] = a.root_token[b];
-        a.parent[ob] = -1;
-        a.depth[ob] = 0;
-        a.position_ids[ob] = sd.L;
-        s_parent[0] = -1;
-        a.n_nodes[b] = n;
-        if (sd.clamped || total != m) atomicOr(a.status, RESPS_STATUS_STEP_CLAMPED);
-    }
-    if (tid < RESPS_MAX_TT) s_flag[tid] = 0;
-    __syncthreads();
+    if (tid <= m) sh.depth[node] = dep;
+    meet();
 
-    // ---- ancestor masks, leaves, retrieve rows --------------------------------------
-    const int rs = a.max_depth + 1;
+    // ---- ancestor masks, leaves, retrieve rows (thread = node) ------------------------------------------
+    const bool leaf = tid < n && !sh.has_child[tid];
+    const unsigned bal = __ballot_sync(kFull, leaf);
+    if (lane == 0) sh.warp_sum[warp] = __popc(bal);
+    meet();
     if (tid < n) {
+        const int rs = a.max_depth + 1;
+        const int last = sh.depth[tid];
+        int row = __popc(bal & ((1u << lane) - 1u));
+#pragma unroll 1
+        for (int w = 0; w < warp; ++w) row += sh.warp_sum[w];
+        int32_t* path = a.retrieve + (ob + row) * rs;
         unsigned long long lo = 0ull, hi = 0ull;
-        int cur = tid, dep = 0;
-        while (cur >= 0 && dep <= RESPS_MAX_DEPTH) {
+        int cur = tid;
+#pragma unroll 1
+        for (int t = last; t >= 0; --t) {
+            const unsigned long long bit = 1ull << (cur & 63);
             if (cur < 64)
-                lo |= 1ull << cur;
+                lo |= bit;
             else
-                hi |= 1ull << (cur - 64);
-            cur = s_parent[cur];
-            ++dep;
+                hi |= bit;
+            if (leaf) path[t] = cur;
+            cur = sh.parent[cur];
         }
+        if (leaf)
+#pragma unroll 1
+            for (int t = last + 1; t < rs; ++t) path[t] = -1;
         a.mask[(ob + tid) * 2 + 0] = lo;
         a.mask[(ob + tid) * 2 + 1] = hi;
-        if (tid > 0) s_flag[s_parent[tid]] = 1;
+        a.node_row[ob + tid] = sh.row[tid];
+        // (these by the candidate's thread: the token id has been on its way since the candidate was known)
+        a.tokens[ob + node] = token;
+        a.parent[ob + node] = pn;
+        a.depth[ob + node] = dep;
+        a.position_ids[ob + node] = sd.L + dep;
     }
-    __syncthreads();
-    if (tid < RESPS_MAX_TT) {  // 4 warps: rank the leaves with ballots
-        const bool leaf = (tid < n) && !s_flag[tid];
-        const unsigned bal = __ballot_sync(kFull, leaf);
-        if ((tid & 31) == 0) s_warp[tid >> 5] = __popc(bal);
-        // named barrier over the first 128 threads only
-        asm volatile("bar.sync 1, 128;");
-        int row = __popc(bal & ((1u << (tid & 31)) - 1u));
-        for (int w = 0; w < (tid >> 5); ++w) row += s_warp[w];
-        if (leaf) {
-            int32_t* out = a.retrieve + (ob + row) * rs;
-            int len = 0;
-            for (int cur = tid; cur >= 0 && len < rs; cur = s_parent[cur]) ++len;
-            for (int t = len; t < rs; ++t) out[t] = -1;
-            int cur = tid;
-            for (int t = len - 1; t >= 0; --t) {
-                out[t] = cur;
-                cur = s_parent[cur];
-            }
-        }
-        if (tid == 0) a.n_leaves[b] = s_warp[0] + s_warp[1] + s_warp[2] + s_warp[3];
+    if (tid == 0) {
+        a.n_leaves[b] = sh.warp_sum[0] + sh.warp_sum[1] + sh.warp_sum[2] + sh.warp_sum[3];
+        a.n_nodes[b] = n;
+        if (sd.clamped || sh.n_kept != m) atomicOr(a.status, RESPS_STATUS_STEP_CLAMPED);
     }
 }
-
 }  // namespace
 
-constexpr size_t kTreeFixedSmem = sizeof(double) * (RESPS_MAX_DEPTH * RESPS_MAX_TT + RESPS_MAX_DEPTH * RESPS_MAX_K) +
-                                  sizeof(int) * (RESPS_MAX_DEPTH * RESPS_MAX_K + 2 * RESPS_MAX_TT + 64 +
-                                                 RESPS_MAX_DEPTH * (kProbes + kStride + 2));
-constexpr size_t kTreeSmemCap = 200 * 1024;
+constexpr int kMaxCandidates = 14944;  // k + (d-1) k^2: what shared memory holds (12 bytes each)
 
 static size_t tree_smem_bytes(int cand_cap) {
-    return static_cast<size_t>(cand_cap) * (sizeof(double) + sizeof(int)) + kTreeFixedSmem;
+    return static_cast<size_t>(cand_cap) * (sizeof(double) + sizeof(int)) +
+           RESPS_MAX_DEPTH * RESPS_MAX_K * (sizeof(double) + sizeof(int));
 }
 
 cudaError_t launch_tree_build(const resps_ctx* ctx, const resps_step* d_steps, int batch,
@@ -430,6 +524,8 @@ cudaError_t launch_tree_build(const resps_ctx* ctx, const resps_step* d_steps, i
     a.status = ctx->ws.status;
     a.cand_cap = s.max_k + (s.max_depth - 1) * s.max_k * s.max_k;
     a.emit_level = -1;
+    a.state_frontier = ctx->ws.tree_frontier, a.state_score = ctx->ws.tree_score;
+    a.use_state = after_scan ? 0 : 1;
     a.setup_before_wait = after_scan ? 1 : 0;
     a.fr = FrontierOut{};
     const size_t smem = tree_smem_bytes(a.cand_cap);
@@ -449,19 +545,19 @@ cudaError_t launch_tree_level(const resps_ctx* ctx, const resps_step* d_steps, i
     a.status = ctx->ws.status;
     a.cand_cap = s.max_k + (s.max_depth - 1) * s.max_k * s.max_k;
     a.emit_level = level;
+    a.state_frontier = ctx->ws.tree_frontier, a.state_score = ctx->ws.tree_score;
+    a.use_state = 1;
     a.setup_before_wait = 1;  // the scan of this level's rows runs directly before
     a.fr = out;
-    return launch_pdl(tree_build_kernel, dim3(batch), dim3(kTreeThreads), tree_smem_bytes(a.cand_cap), st, a);
+    return launch_pdl(tree_build_kernel, dim3(batch), dim3(kLevelThreads), tree_smem_bytes(a.cand_cap), st, a);
 }
 
 // Largest k + (d-1)k^2 the shared-memory arrays can hold.
-int tree_candidate_limit() {
-    return static_cast<int>((kTreeSmemCap - kTreeFixedSmem) / (sizeof(double) + sizeof(int)));
-}
+int tree_candidate_limit() { return kMaxCandidates; }
 
 cudaError_t tree_setup(resps_ctx*) {
     return cudaFuncSetAttribute(tree_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(kTreeSmemCap));
+                                static_cast<int>(tree_smem_bytes(kMaxCandidates)));
 }
 
 }  // namespace resps
