@@ -107,12 +107,12 @@ int64_t resps_workspace_bytes(const resps_ctx* ctx);
  * Returns INVALID_ARG for an unknown key.  (The paper has no counterpart.)
  */
 enum {
-    RESPS_DEBUG_ATTN_ROUNDS = 1,    /* rounds of work items the attention work list plans: 0 = its own choice */
-    RESPS_DEBUG_ATTN_MIN_TILES = 2, /* fewest 64-key tiles a split of the keys is given (default 2)           */
-    RESPS_DEBUG_ATTN_STAGGER = 3,   /* SM cycles the second half of a CTA starts behind the first (default 1000) */
-    RESPS_DEBUG_SCAN_SLICES = 4,    /* slices a logits row is cut into by the streaming scan: 0 = its own choice */
-    RESPS_DEBUG_ATTN_SINGLE = 5     /* single row tiles (both halves of a CTA on one tile) while no sequence has more
-                                       than this many (row tiles per KV head)^2 x key tiles (default 2000)           */
+    RESPS_DEBUG_ATTN_ROUNDS = 1,    /* the attention work list is cut for 1/value of the CTAs: 0 = for all             */
+    RESPS_DEBUG_ATTN_MIN_TILES = 2, /* fewest 64-key tiles a CTA of a cluster is given (default 2)                     */
+    RESPS_DEBUG_ATTN_CLUSTER = 3,   /* most CTAs per cluster of the attention kernel (1..8): 0 = its own choice        */
+    RESPS_DEBUG_SCAN_SLICES = 4,    /* slices a logits row is cut into by the streaming scan: 0 = its own choice       */
+    RESPS_DEBUG_ATTN_SINGLE = 5     /* key tiles a CTA must be spared before the groups are cut into equal ranges instead
+                                       of equal splits each (default 6)                                           */
 };
 int resps_debug_set(resps_ctx* ctx, int key, int value);
 

@@ -32,7 +32,7 @@ RESPS_STATUS_WAIT_TIMEOUT = 4
 RESPS_STATUS_STALE_PLAN = 8
 RESPS_DEBUG_ATTN_ROUNDS = 1
 RESPS_DEBUG_ATTN_MIN_TILES = 2
-RESPS_DEBUG_ATTN_STAGGER = 3
+RESPS_DEBUG_ATTN_CLUSTER = 3
 RESPS_DEBUG_SCAN_SLICES = 4
 RESPS_DEBUG_ATTN_SINGLE = 5
 

@@ -10,9 +10,10 @@
 
 namespace resps {
 int scan_chunk_max();
-int attention_item_rows();
-int attention_max_rounds();
 int attention_max_batch();
+int attention_place_rows();
+int attention_max_groups(int batch, int n_kv_heads, int max_tt, int group);
+int attention_max_items(int groups, int sm_count);
 }  // namespace resps
 
 namespace {
@@ -64,9 +65,10 @@ void carve(resps_ctx* c, Carver& cv) {
     cv.take(w.row_id, rows * s.max_k);
     cv.take(w.row_lse, rows);
     cv.take(w.amax_part, nodes * w.scan_splits);
-    cv.take(w.attn_plan, static_cast<int64_t>(resps::attention_plan_bytes(s.max_batch, w.attn_max_items)));
-    cv.take(w.attn_part_o, static_cast<int64_t>(w.attn_max_items) * resps::attention_item_rows() * s.head_dim);
-    cv.take(w.attn_part_ml, static_cast<int64_t>(w.attn_max_items) * resps::attention_item_rows());
+    cv.take(w.attn_plan, static_cast<int64_t>(resps::attention_plan_bytes(w.attn_max_items, w.attn_max_groups)));
+    const int64_t part_rows = static_cast<int64_t>(w.attn_max_items) * resps::attention_place_rows();
+    cv.take(w.attn_part_o, part_rows * s.head_dim);
+    cv.take(w.attn_part_ml, part_rows);
 }
 
 #define RESPS_CHECK_PTR(p) \
@@ -107,9 +109,12 @@ int resps_create(resps_ctx** out, const resps_shape* shape) {
 
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return RESPS_ERR_NO_DEVICE;
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return RESPS_ERR_NO_DEVICE;
-    if (prop.major != 10) return RESPS_ERR_NO_DEVICE;
+    // (two attributes, not cudaGetDeviceProperties: that call alone takes about 3 ms)
+    int major = 0, sm_count = 0;
+    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return RESPS_ERR_NO_DEVICE;
+    if (major != 10) return RESPS_ERR_NO_DEVICE;
 
     resps_ctx* c = new (std::nothrow) resps_ctx();
     if (!c) return RESPS_ERR_CUDA;
@@ -117,7 +122,7 @@ int resps_create(resps_ctx** out, const resps_shape* shape) {
     c->level_next = 0, c->level_slots = 1;
     c->shape = s;
     c->device = dev;
-    c->sm_count = prop.multiProcessorCount;
+    c->sm_count = sm_count;
     resps::Workspace& w = c->ws;
     // a scan CTA keeps its whole chunk in registers; up to 128 chunks per row (vocab <= 2^20)
     const int chunk = resps::scan_chunk_max();
@@ -129,11 +134,8 @@ int resps_create(resps_ctx** out, const resps_shape* shape) {
     }
     w.max_rows = 1 + (s.max_depth - 1) * s.max_k;
     const int G = s.n_q_heads / s.n_kv_heads;
-    const int item_rows = resps::attention_item_rows();
-    w.attn_grid = c->sm_count;
-    w.attn_min_tiles = 2;
-    w.attn_max_groups = s.max_batch * s.n_kv_heads * ((s.max_tt * G + item_rows / 2 - 1) / (item_rows / 2));  // single row tiles
-    w.attn_max_items = resps::attention_max_rounds() * w.attn_grid + w.attn_max_groups;
+    w.attn_max_groups = resps::attention_max_groups(s.max_batch, s.n_kv_heads, s.max_tt, G);
+    w.attn_max_items = resps::attention_max_items(w.attn_max_groups, c->sm_count);
 
     Carver dry;
     carve(c, dry);
@@ -181,8 +183,8 @@ int resps_debug_set(resps_ctx* ctx, int key, int value) {
     switch (key) {
         case RESPS_DEBUG_ATTN_ROUNDS: w.attn_rounds = std::max(0, value); break;
         case RESPS_DEBUG_ATTN_MIN_TILES: w.attn_min_tiles = std::max(1, value); break;
-        case RESPS_DEBUG_ATTN_SINGLE: w.attn_single = std::min(1 << 26, std::max(0, value)); break;
-        case RESPS_DEBUG_ATTN_STAGGER: w.attn_stagger = std::min(100000, std::max(0, value)); break;
+        case RESPS_DEBUG_ATTN_SINGLE: w.attn_stream = std::min(1 << 26, std::max(0, value)); break;
+        case RESPS_DEBUG_ATTN_CLUSTER: w.attn_cluster = std::max(0, value); break;
         case RESPS_DEBUG_SCAN_SLICES: w.scan_slices_hint = std::max(0, value); break;
 #ifdef RESPS_WAIT_TEST
         case 100: w.test_drop = value; break;  // test build only: which copy is left out (see common.cuh)

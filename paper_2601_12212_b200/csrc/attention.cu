@@ -7,32 +7,27 @@
 // so that Q K^T and P V are dense contractions: tcgen05.mma with the fp32
 // accumulators (S and O) in tensor memory.  K/V tiles of 64 keys are staged by TMA
 // (cp.async.bulk.tensor, one elected thread) into 128-byte-swizzled shared memory
-// through mbarrier rings (four stages each for K and V), Q tiles likewise (prefetched for the next item).
+// through mbarrier rings (four stages each for K and V), Q tiles likewise.
 //
-// A CTA runs two symmetric lanes.  A lane is an MMA-issuing warp, a softmax warpgroup
-// (one TMEM lane = one query row per thread) and a quarter of tensor memory (two S/P
-// buffers and one O accumulator).  The softmax warpgroup scales, applies the ancestor
-// bitmask (from registers, only on tiles that reach past the prefix), keeps the online
-// softmax state and writes P back into the tensor-memory columns S came from, from
-// where it is the A operand of P V.  P is kept as two bf16 terms (p = hi + lo): one
-// bf16 rounding of the weights alone would cost up to 2^-9 per weight, about 1 % of an
-// output row's rms in the worst element.
+// A CTA runs two symmetric lanes that take the key tiles of its range in turn.  A lane is an
+// MMA-issuing warp, a softmax warpgroup (one TMEM lane = one query row per thread) and a
+// quarter of tensor memory (two S/P buffers and one O accumulator).  The softmax warpgroup
+// scales, applies the ancestor bitmask (from registers, only on tiles that reach past the
+// prefix), keeps the online softmax state and writes P back into the tensor-memory columns S
+// came from, from where it is the A operand of P V.  P is kept as two bf16 terms (p = hi + lo):
+// one bf16 rounding of the weights alone would cost up to 2^-9 per weight, about 1 % of an
+// output row's rms in the worst element.  At the end the two lanes merge their results inside
+// the CTA (a lane reads the other's accumulator straight from tensor memory).
 //
-// A work item is (sequence, KV head, group of row tiles, range of key tiles).  With more
-// than 128 rows in the group, lane x takes row tile x over all key tiles ("row mode");
-// otherwise both lanes take the one row tile and alternate key tiles ("key mode") and
-// merge their two results inside the CTA (a lane reads the other's accumulator straight
-// from tensor memory).  The work list depends only on the step parameters, which are the
-// same for every layer of a step: a one-CTA kernel derives it once from the
-// device-resident parameters and leaves it in the workspace as a table (one 32-byte
-// descriptor per item), so nothing about a launch depends on (TT, d, k, L) and a CTA
-// learns its work from one load.  Items whose group has a single split write O directly;
-// all others write normalised partials that a second, small kernel combines.
+// The work list depends only on the step parameters, which are the same for every layer of a
+// step: a one-CTA kernel derives it once from the device-resident parameters and leaves it in
+// the workspace as a table, so nothing about a launch depends on (TT, d, k, L) and a CTA learns
+// its work from one load.  How the work is laid out is explained at the table.
 //
 // Every wait (mbarrier) is bounded: when it runs out the CTA raises
 // RESPS_STATUS_WAIT_TIMEOUT, stops issuing work, drains its copies in flight, frees
-// its tensor memory and returns.  Every barrier is used so that a waiter can never
-// fall two phases behind (a parity wait would then never return).
+// its tensor memory, meets the other CTAs of its cluster and returns.  Every barrier is used so
+// that a waiter can never fall two phases behind (a parity wait would then never return).
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -49,14 +44,14 @@ namespace {
 
 constexpr int kBM = 128;           // rows per row tile (one TMEM lane each)
 constexpr int kBN = 64;            // keys per tile
-// Ring depths.  Both must be even: in key mode the lanes take alternate tiles and a lane waits for
+// Ring depths.  Both must be even: the lanes take alternate tiles and a lane waits for
 // (and looks ahead at) the "full" barriers of its own tiles only, so the previous use of a stage
 // must have been its own too -- with an odd depth it would be the other lane's, which this lane has
 // not seen complete, and a parity wait cannot tell "not yet" from "one phase on".
 constexpr int kStagesK = 4;
 constexpr int kStagesV = 4;
-static_assert(kStagesK % 2 == 0 && kStagesV % 2 == 0, "ring depths must be even (key mode)");
-constexpr int kRowTiles = 2;       // row tiles per item
+static_assert(kStagesK % 2 == 0 && kStagesV % 2 == 0, "ring depths must be even");
+constexpr int kLanes = 2;
 constexpr int kSoftmaxThreads = 256;
 constexpr int kProducerWarp = 8;   // K and Q tiles
 constexpr int kMmaWarp0 = 9;       // lane x is issued by warp kMmaWarp0 + x
@@ -65,26 +60,46 @@ constexpr int kAttnThreads = 384;
 constexpr int kRegsSoftmax = 216;  // setmaxnreg: 256 x 216 + 128 x 72 = 384 x 168 <= 64 K registers
 constexpr int kRegsIssue = 72;
 constexpr int kSyncThreads = 320;  // softmax warps + the MMA warps meet at the end of an item
-constexpr int kMaxBatchSmem = 256;
+constexpr int kMaxBatch = 256;
+constexpr int kMaxCluster = 8;     // CTAs of a cluster (the portable limit)
+constexpr int kMaxGrid = 256;      // clusters x CTAs (one per SM)
+constexpr int kSnap = 2;           // mode stream: a cut this close to a group's edge (key tiles) is moved onto it
 constexpr int kTmemCols = 512;
-constexpr int kCombineThreads = 256;
-constexpr int kMaxRounds = 4;      // rounds of items the work list may plan for (long sequences only)
 constexpr uint32_t kWaitLimitCycles = kWaitTest ? 2000000u : 0x70000000u;  // bounded waits give up after ~1 s of SM clocks
 constexpr float kRescaleSlack = 8.0f;  // O is rescaled only when the running max grows by > 2^8
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
-// What the work list keeps per sequence (the combine kernels walk rows, not items) ...
-struct PlanSeq {
-    int n, L, mp, nfull, kt, s_row, s_key, item0;
+// How a layer's work is laid out, one of three ways (PlanHead::mode):
+//  whole   clusters of several CTAs, one group (sequence, KV head, row tile) per cluster.  The CTAs share
+//          the group's key tiles, leave normalised partial results in the workspace (L2), meet on an
+//          mbarrier and merge a share of the rows x columns each: one kernel does the layer.
+//  even    single CTAs; every group is cut into splits of at most T key tiles with the smallest T for which
+//          the splits fit one round of the grid; a second, small kernel combines the partials.
+//  stream  the same two kernels; the key tiles of all groups, one group after the other, are cut into equal
+//          contiguous ranges, one per CTA (a CTA may end one group and begin another).
+constexpr int kModeWhole = 0, kModeEven = 1, kModeStream = 2;
+
+struct PlanHead {
+    int mode, n_groups, pad[2];
 };
-// ... and per item: everything a CTA needs to start.
+// A cluster's (or CTA's) first item and its number of items.
+struct PlanCluster {
+    int first_item, n_items;
+};
+// For every item and CTA of the cluster everything the CTA needs to start.
 struct PlanItem {
-    int b_g;          // sequence | KV head << 16
-    int pair_splits;  // group index within the head | splits of the group << 16
-    int sp, first_item, t_begin, t_end;
-    int n, L;         // the sequence's tree size and prefix length
+    int b_g;             // sequence | KV head << 16
+    int tile_active;     // row tile of the KV head | CTAs that have key tiles of the item << 16
+    int t_begin, t_end;  // this CTA's key tiles (none: t_begin == t_end)
+    int n, L;            // the sequence's tree size and prefix length
+    int pieces;          // items the group is cut into
+    int pad;
 };
-static_assert(sizeof(PlanSeq) == 32 && sizeof(PlanItem) == 32, "two 16-byte loads each");
+// For the combine kernel: the partials of a group are those of consecutive items.
+struct PlanGroup {
+    int b_g, tile, n, first_item, pieces, pad[3];
+};
+static_assert(sizeof(PlanHead) == 16 && sizeof(PlanCluster) == 8 && sizeof(PlanItem) == 32 && sizeof(PlanGroup) == 32, "vector loads");
 
 struct AttnArgs {
     const resps_step* steps;
@@ -97,234 +112,282 @@ struct AttnArgs {
     const uint64_t* mask;
     float scale_log2;
     int Hq, Hkv, max_tt;
-    // Partials of split groups.  O is stored normalised (O / l, a convex combination of V rows) as
-    // fp16 times a per-row power of two that only differs from 1 when a value would leave the fp16
+    // Partials.  O is stored normalised (O / l, a convex combination of V rows) as
+    // fp16 times a power of two per half row that only differs from 1 when a value would leave the fp16
     // range: half the bytes of fp32, and 11 significant bits per element (2^-11, against the 2^-9
-    // of the final bf16 rounding).
-    uint4* part_o;    // [items][2 row tiles][D/8][128 rows]  eight fp16 each
-    float4* part_ml;  // [items][2 row tiles][128 rows]   (running max m, running sum l, l * row scale, -)
+    // of the final bf16 rounding).  Place = item x cluster size + CTA.
+    uint4* part_o;    // [places][D/8][128 rows]  eight fp16 each
+    float4* part_ml;  // [places][128 rows]   (running max m, running sum l, l * scale of each half row)
+    int cluster;      // CTAs per cluster (1: modes even and stream)
+    int clusters;     // clusters the work list is cut for (at most gridDim / cluster)
     int max_items;
-    int sched_grid;   // CTAs of the attention grid (the work list is balanced for it)
-    int min_tiles;    // smallest key-tile count worth a split of its own
-    int single_units; // single row tiles while no sequence has more than this many (row tiles)^2 x key tiles
-    int rounds;       // 0: the work list chooses its number of rounds; 1..kMaxRounds: as told (tests)
-    int stagger;      // cycles lane 1 starts behind lane 0 in row mode
+    int stream_gain;  // mode stream when it saves a CTA more than this many key tiles
+    int min_tiles;    // fewest key tiles a CTA is given
     int q_by_tma;     // 1: Q tiles come by TMA (128 % (Hq/Hkv) == 0), 0: by plain loads
     int plan_after_wait;  // 1: the work list was written by the kernel just before this one
     int test_drop;        // test build only: 1 = the CTA's first V copy is left out
     int32_t* status;
     // The work list, written by attention_plan_kernel.
-    int4* plan_head;             // (items, rows per group, -, -)
-    PlanSeq* plan_seq;       // [batch + 1]; entry [batch].item0 = items
-    PlanItem* plan_item;  // [max_items]
+    PlanHead* plan_head;
+    PlanCluster* plan_cluster;  // [kMaxGrid]
+    PlanItem* plan_first;       // [kMaxGrid] every CTA's first item once more (one load instead of two in a row)
+    PlanItem* plan_item;        // [max_items x cluster]
+    PlanGroup* plan_group;      // [groups]
 };
 
-// ---------------------------------------------------------------------------- work list
-// A group is (sequence, KV head, pair of row tiles).  A pair with more than 128 rows runs in row
-// mode and costs two units per key tile; the last pair of a head may have at most 128 rows, runs
-// in key mode and costs one.  Every group is cut into splits of at most T units, with the smallest
-// T for which the items fit one round of the grid (found by a short search; steps of 1/16), so
-// that the CTAs finish together whatever the mix of tree sizes and prefix lengths.
-// Groups are single row tiles instead, all in key mode, while no sequence has many row tiles per KV
-// head over a long prefix: items of half the size fill the grid where row-mode items (at least two key
-// tiles for each of two row tiles) cannot, and the two halves of a CTA merge into one partial; the
-// price is that K and V pass through L2 once per row tile instead of once per pair.  Measured
-// crossovers (per-call time, both groupings forced): 2 row tiles per KV head (8B shape, 60 nodes) --
-// single tiles ahead up to a prefix of 24 000, level at 32 000; 6 row tiles (70B shape, 96 nodes) --
-// ahead up to 3 000, 1.5 % behind from 4 000; ragged batch of 8 with up to 3 row tiles and prefixes up
-// to 8 000 -- ahead by 3 %.  All of them sit near (row tiles)^2 x key tiles = 2000 for the largest
-// sequence, which is the rule (`single_units`).  On the 8B-shaped workload with the prefix growing from
-// 1024 to 3010 this gives 480 us per step, against 510 already at 1837 with the first rule (at most two
-// units of work per CTA).
-struct Sched {
-    int group_rows;             // rows of a group: 256 (pairs of row tiles) or 128 (single tiles)
-    int n[kMaxBatchSmem];       // tree nodes (0 = sequence skipped)
-    int L[kMaxBatchSmem];
-    int mp[kMaxBatchSmem];      // row-tile pairs
-    int nfull[kMaxBatchSmem];   // pairs in row mode (mp or mp - 1)
-    int kt[kMaxBatchSmem];      // key tiles
-    int s_row[kMaxBatchSmem];   // splits of a row-mode group
-    int s_key[kMaxBatchSmem];   // splits of the key-mode group
-    int item0[kMaxBatchSmem + 1];
-};
-
-__device__ __forceinline__ int ceil_div(int a, int b) {  // a >= 0, b > 0: the unsigned division is the shorter one
+__host__ __device__ __forceinline__ int ceil_div(int a, int b) {  // a >= 0, b > 0: the unsigned division is the shorter one
     return static_cast<int>((static_cast<unsigned>(a) + static_cast<unsigned>(b) - 1u) / static_cast<unsigned>(b));
 }
 
-// Runs in the first warp (one lane per sequence, eight rounds for the largest batch); the block
-// meets once at the end.  This sits at the head of the kernel's critical path (nothing can be
-// fetched before the CTA knows its item), hence the care for the length of the dependent chain.
-__device__ __forceinline__ void build_sched(const AttnArgs& a, Sched& sc, int tid) {
-    if (tid < 32) {
-        const int G = a.Hq / a.Hkv;
-        const int nblk = (a.batch + 31) >> 5;
-        const int mt = max(a.min_tiles, 1);
-        // ---- pass 1: sizes, and the cost in row-tile x key-tile units (the same for both groupings:
-        // a row-mode pair costs two units per key tile, a single tile one) ----------------------------
-        unsigned cost = 0;   // saturates: it only seeds the search below
-        unsigned cost2 = 0;  // largest (row tiles)^2 x key tiles of a sequence: decides the grouping
-#pragma unroll 1
-        for (int i = 0; i < nblk; ++i) {
-            const int b = i * 32 + tid;
-            if (b < a.batch) {
-                int n = min(max(a.n_nodes[b], 0), a.max_tt);
-                const int L = max(a.steps[b].prefix_len, 0);
-                if (static_cast<int64_t>(L) + n > a.capacity) {
-                    atomicOr(a.status, RESPS_STATUS_KV_OVERFLOW);
-                    n = 0;
-                }
-                const int tiles = (n * G + kBM - 1) / kBM;
-                const int kt = (n > 0) ? (L + n + kBN - 1) / kBN : 0;
-                sc.n[b] = n, sc.L[b] = L, sc.kt[b] = kt;
-                cost += min(static_cast<unsigned>(a.Hkv * tiles) * static_cast<unsigned>(kt), 1u << 23);
-                cost2 = max(cost2, min(static_cast<unsigned>(tiles * tiles) * static_cast<unsigned>(kt), 1u << 26));
-            }
-        }
-        cost = __reduce_add_sync(0xFFFFFFFFu, min(cost, 1u << 26));
-        cost2 = __reduce_max_sync(0xFFFFFFFFu, cost2);
-        // a small call is cut into single row tiles (see above)
-        const bool single = cost2 <= static_cast<unsigned>(a.single_units);
-        const int group_rows = single ? kBM : kRowTiles * kBM;
-        if (tid == 0) sc.group_rows = group_rows;
-#pragma unroll 1
-        for (int i = 0; i < nblk; ++i) {
-            const int b = i * 32 + tid;
-            if (b < a.batch) {
-                const int M = sc.n[b] * G;
-                const int mp = (M + group_rows - 1) / group_rows;
-                sc.mp[b] = mp;
-                sc.nfull[b] = single ? 0 : ((mp > 0 && M - (mp - 1) * group_rows <= kBM) ? mp - 1 : mp);
-            }
-        }
-        // the lane's first sequence stays in registers (its only one up to 32 sequences)
-        int kt0 = 0, nfull0 = 0, nkey0 = 0;
-        if (tid < a.batch) kt0 = sc.kt[tid], nfull0 = sc.nfull[tid], nkey0 = sc.mp[tid] - nfull0;
-        // Smallest T (in steps of T/16) for which the items fit `rounds` rounds of the grid.  One round
-        // is the rule.  With long sequences and few groups it can leave CTAs idle (40 groups of 3 splits
-        // are 120 items for 148 CTAs); two to four rounds of shorter items then fill the grid better.
-        // An item more costs a CTA about kItemUnits units (its epilogue and the start of the next), so
-        // more rounds are only looked at when items are long, where the time of this search does not
-        // matter either.
-        constexpr int kItemUnits = 8;
-        const int forced = min(a.rounds, kMaxRounds);
-        int T = 1, best = 0x7FFFFFFF;
-#pragma unroll 1
-        for (int rounds = max(forced, 1); rounds <= (forced > 0 ? forced : kMaxRounds); ++rounds) {
-            int Tr = max(ceil_div(static_cast<int>(cost), rounds * a.sched_grid), 1);
-#pragma unroll 1
-            for (int tries = 0; tries < 24; ++tries) {
-                const int t_row = max((Tr + 1) >> 1, mt), t_key = max(Tr, mt);
-                unsigned cnt = a.Hkv * (nfull0 * ceil_div(kt0, t_row) + nkey0 * ceil_div(kt0, t_key));
-#pragma unroll 1
-                for (int i = 1; i < nblk; ++i) {
-                    const int b = i * 32 + tid;
-                    if (b < a.batch)
-                        cnt += a.Hkv * (sc.nfull[b] * ceil_div(sc.kt[b], t_row) +
-                                        (sc.mp[b] - sc.nfull[b]) * ceil_div(sc.kt[b], t_key));
-                }
-                cnt = __reduce_add_sync(0xFFFFFFFFu, min(cnt, 1u << 20));
-                if (cnt <= static_cast<unsigned>(rounds * a.sched_grid)) break;
-                Tr += max(1, Tr >> 4);
-            }
-            if (rounds * (Tr + kItemUnits) < best) best = rounds * (Tr + kItemUnits), T = Tr;
-            if (forced == 0 && Tr < 8 * kItemUnits) break;  // short items: no further rounds
-        }
-        const int s_row0 = ceil_div(kt0, max((T + 1) >> 1, mt)), s_key0 = ceil_div(kt0, max(T, mt));
-        const int t_row = max((T + 1) >> 1, mt), t_key = max(T, mt);
-        int base = 0;
-#pragma unroll 1
-        for (int i = 0; i < nblk; ++i) {
-            const int b = i * 32 + tid;
-            int mine = 0, s_row = s_row0, s_key = s_key0;
-            if (i > 0 && b < a.batch) s_row = ceil_div(sc.kt[b], t_row), s_key = ceil_div(sc.kt[b], t_key);
-            if (b < a.batch) mine = a.Hkv * (sc.nfull[b] * s_row + (sc.mp[b] - sc.nfull[b]) * s_key);
-            int incl = mine;  // inclusive prefix sum over the lanes
-            if (a.batch > 1) {
-#pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    const int v = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-                    if (tid >= d) incl += v;
-                }
-            }
-            if (b < a.batch) sc.s_row[b] = s_row, sc.s_key[b] = s_key, sc.item0[b] = base + incl - mine;
-            base += __shfl_sync(0xFFFFFFFFu, incl, a.batch > 1 ? 31 : 0);
-        }
-        if (tid == 0) sc.item0[a.batch] = base;
-    }
-    __syncthreads();
+// CTAs of a cluster that get key tiles of an item with `tiles` of them.  A lane that takes one tile more
+// costs about 1 us, the exchange between the CTAs about 2.5 us: up to five tiles stay in one CTA, beyond
+// that a CTA gets at least one tile per lane (min_tiles).
+__device__ __forceinline__ int active_ctas(int tiles, int cluster, int min_tiles) {
+    if (tiles <= 2 * min_tiles + 1) return 1;
+    return min(cluster, ceil_div(tiles, min_tiles));
 }
 
-struct Item {
-    int b, g, pair, sp, splits, first_item;
-    int n, L, M, row_base, nmt, t_begin, t_end;
-    int tok0;  // first token of the group's rows
+// ---------------------------------------------------------------------------- work list
+// Bound by latency (one CTA, once per step): a scan over the sequences, a search, then a thread per CTA or
+// item.  Positions are in key tiles of the sequence of groups (b, KV head, row tile).
+struct PlanShared {
+    unsigned long long start[kMaxBatch + 1];  // first position of a sequence
+    int group0[kMaxBatch + 1];                // first group of a sequence
+    int item0[kMaxBatch + 1];                 // mode even: first item of a sequence
+    int n[kMaxBatch], L[kMaxBatch], tiles[kMaxBatch], kt[kMaxBatch], splits[kMaxBatch];
+    unsigned long long cut[kMaxGrid + 1];
+    int n_items[kMaxGrid];
+    int mode;
 };
 
-__device__ __forceinline__ PlanItem plan_entry(const Sched& sc, int item) {
-    PlanItem p;
-    int b = 0;
-    while (item >= sc.item0[b + 1]) ++b;
-    const int nfull = sc.nfull[b], s_row = sc.s_row[b], s_key = sc.s_key[b];
-    const int row_items = nfull * s_row;
-    const int per_head = row_items + (sc.mp[b] - nfull) * s_key;
-    const int local = item - sc.item0[b];
-    const int g = static_cast<int>(static_cast<unsigned>(local) / static_cast<unsigned>(per_head));
-    const int rem = local - g * per_head;
-    int pair, splits;
-    if (rem < row_items) {
-        pair = static_cast<int>(static_cast<unsigned>(rem) / static_cast<unsigned>(s_row));
-        p.sp = rem - pair * s_row;
-        splits = s_row;
-    } else {
-        pair = nfull + static_cast<int>(static_cast<unsigned>(rem - row_items) / static_cast<unsigned>(s_key));
-        p.sp = rem - row_items - (pair - nfull) * s_key;
-        splits = s_key;
-    }
-    p.b_g = static_cast<int>(static_cast<unsigned>(b) | (static_cast<unsigned>(g) << 16));
-    p.pair_splits = static_cast<int>(static_cast<unsigned>(pair) | (static_cast<unsigned>(splits) << 16));
-    p.first_item = item - p.sp;
-    // kt <= 2^15 (cache capacity is checked on the host), so the products fit 32 bits
-    const unsigned kt = static_cast<unsigned>(sc.kt[b]), sp = static_cast<unsigned>(p.sp);
-    p.t_begin = static_cast<int>(kt * sp / static_cast<unsigned>(splits));
-    p.t_end = static_cast<int>(kt * (sp + 1u) / static_cast<unsigned>(splits));
-    p.n = sc.n[b], p.L = sc.L[b];
-    return p;
-}
-
-// The work list of one call: the per-sequence figures and one descriptor per item, written to the
-// workspace.  One CTA; it runs once per step (the list is the same for every layer).
-__global__ void __launch_bounds__(256) attention_plan_kernel(const AttnArgs a) {
-    __shared__ Sched sc;
+__global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs a) {
+    __shared__ PlanShared sh;
+    const int tid = threadIdx.x, lane = tid & 31, G = a.Hq / a.Hkv;
     pdl_wait();  // the step parameters and node counts are complete
     pdl_launch_dependents();
-    build_sched(a, sc, threadIdx.x);  // ends with __syncthreads()
-    const int total = min(sc.item0[a.batch], a.max_items);
-    if (threadIdx.x == 0) *a.plan_head = make_int4(total, sc.group_rows, 0, 0);
-    for (int b = threadIdx.x; b <= a.batch; b += blockDim.x) {
-        PlanSeq q = {};
-        q.item0 = sc.item0[b];
-        if (b < a.batch)
-            q.n = sc.n[b], q.L = sc.L[b], q.mp = sc.mp[b], q.nfull = sc.nfull[b], q.kt = sc.kt[b],
-            q.s_row = sc.s_row[b], q.s_key = sc.s_key[b];
-        a.plan_seq[b] = q;
+    if (tid < a.batch) {
+        int n = min(max(a.n_nodes[tid], 0), a.max_tt);
+        const int L = max(a.steps[tid].prefix_len, 0);
+        if (static_cast<int64_t>(L) + n > a.capacity) {
+            atomicOr(a.status, RESPS_STATUS_KV_OVERFLOW);
+            n = 0;
+        }
+        sh.n[tid] = n, sh.L[tid] = L;
+        sh.tiles[tid] = ceil_div(n * G, kBM);
+        sh.kt[tid] = (n > 0) ? ceil_div(L + n, kBN) : 0;
     }
-    for (int item = threadIdx.x; item < total; item += blockDim.x) a.plan_item[item] = plan_entry(sc, item);
+    __syncthreads();
+    if (tid < 32) {
+        unsigned long long pos = 0;
+        int group = 0;
+#pragma unroll 1
+        for (int b0 = 0; b0 < a.batch; b0 += 32) {
+            const int b = b0 + lane;
+            int groups = (b < a.batch) ? a.Hkv * sh.tiles[b] : 0;
+            unsigned long long work = (b < a.batch) ? static_cast<unsigned long long>(groups) * sh.kt[b] : 0ull;
+            const int own_groups = groups;
+            const unsigned long long own_work = work;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int g = __shfl_up_sync(kFull, groups, d);
+                const unsigned long long w = __shfl_up_sync(kFull, work, d);
+                if (lane >= d) groups += g, work += w;
+            }
+            if (b < a.batch) sh.start[b] = pos + work - own_work, sh.group0[b] = group + groups - own_groups;
+            pos += __shfl_sync(kFull, work, 31);
+            group += __shfl_sync(kFull, groups, 31);
+        }
+        if (lane == 0) sh.start[a.batch] = pos, sh.group0[a.batch] = group;
+        int mode = kModeWhole;
+        if (a.cluster == 1) {
+            // the smallest T (in steps of T/16) for which the splits fit one round of the grid
+            const int even = static_cast<int>(min((pos + a.clusters - 1) / a.clusters, 1ull << 24));  // tiles per CTA when cut evenly
+            int T = max(even, 1);
+            bool fits = false;
+#pragma unroll 1
+            for (int tries = 0; tries < 40 && !fits; ++tries) {
+                unsigned count = 0;
+#pragma unroll 1
+                for (int b = lane; b < a.batch; b += 32)
+                    count += static_cast<unsigned>(a.Hkv * sh.tiles[b] * ceil_div(sh.kt[b], max(T, a.min_tiles)));
+                count = __reduce_add_sync(kFull, min(count, 1u << 20));
+                fits = count <= static_cast<unsigned>(a.clusters);
+                if (!fits) T += max(1, T >> 4);
+            }
+            T = max(T, a.min_tiles);
+            mode = (fits && T - even <= a.stream_gain) ? kModeEven : kModeStream;
+            int base = 0;
+#pragma unroll 1
+            for (int b0 = 0; b0 < a.batch; b0 += 32) {
+                const int b = b0 + lane, splits = (b < a.batch) ? ceil_div(sh.kt[b], T) : 0;
+                int incl = (b < a.batch && mode == kModeEven) ? a.Hkv * sh.tiles[b] * splits : 0;
+                const int own = incl;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const int v = __shfl_up_sync(kFull, incl, d);
+                    if (lane >= d) incl += v;
+                }
+                if (b < a.batch) sh.splits[b] = splits, sh.item0[b] = base + incl - own;
+                base += __shfl_sync(kFull, incl, 31);
+            }
+            if (lane == 0) sh.item0[a.batch] = base;
+        }
+        if (lane == 0) {
+            sh.mode = mode;
+            PlanHead h = {};
+            h.mode = mode, h.n_groups = group;
+            *a.plan_head = h;
+        }
+    }
+    __syncthreads();
+    const int mode = sh.mode, n_groups = sh.group0[a.batch];
+    auto last_at_or_before = [&](const int* first, int x) {  // the last sequence whose entry is <= x
+        int lo = 0, hi = a.batch;
+#pragma unroll 1
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (first[mid] <= x) lo = mid; else hi = mid;
+        }
+        return lo;
+    };
+    auto item_of = [&](int b, int local) {  // what all pieces of a group share
+        PlanItem p = {};
+        const int head = static_cast<int>(static_cast<unsigned>(local) / static_cast<unsigned>(sh.tiles[b]));
+        p.b_g = static_cast<int>(static_cast<unsigned>(b) | (static_cast<unsigned>(head) << 16));
+        p.tile_active = static_cast<int>(static_cast<unsigned>(local - head * sh.tiles[b]) | (1u << 16));
+        p.n = sh.n[b], p.L = sh.L[b], p.pieces = 1;
+        return p;
+    };
+    auto write_group = [&](int group, const PlanItem& p, int first_item) {
+        PlanGroup q = {};
+        q.b_g = p.b_g, q.tile = p.tile_active & 0xFFFF, q.n = p.n, q.first_item = first_item, q.pieces = p.pieces;
+        a.plan_group[group] = q;
+    };
+    if (mode != kModeStream) {
+        // ---- an item per cluster or CTA ---------------------------------------------------------------
+        const int n = (mode == kModeWhole) ? n_groups : sh.item0[a.batch];
+        if (tid < a.clusters) {
+            PlanCluster c;
+            c.first_item = tid, c.n_items = (tid < n) ? 1 : 0;
+            a.plan_cluster[tid] = c;
+            if (tid < n && mode == kModeWhole) {
+                const int b = last_at_or_before(sh.group0, tid);
+                PlanItem p = item_of(b, tid - sh.group0[b]);
+                const int kt = sh.kt[b], act = active_ctas(kt, a.cluster, a.min_tiles);
+                p.tile_active = (p.tile_active & 0xFFFF) | (act << 16);
+#pragma unroll 1
+                for (int r = 0; r < a.cluster; ++r) {
+                    p.t_begin = p.t_end;
+                    if (r < act) p.t_end = kt * (r + 1) / act;
+                    a.plan_first[tid * a.cluster + r] = p;
+                }
+            } else if (tid < n) {
+                const int b = last_at_or_before(sh.item0, tid), splits = sh.splits[b], kt = sh.kt[b];
+                const int at = tid - sh.item0[b], local = static_cast<int>(static_cast<unsigned>(at) / static_cast<unsigned>(splits));
+                const int sp = at - local * splits;
+                PlanItem p = item_of(b, local);
+                p.t_begin = kt * sp / splits, p.t_end = kt * (sp + 1) / splits, p.pieces = splits;  // (kt <= 2^15, splits <= 2^8)
+                a.plan_first[tid] = p;
+                if (sp == 0) write_group(sh.group0[b] + local, p, tid);
+            }
+        }
+        return;
+    }
+    // ---- even cuts ------------------------------------------------------------------------------------
+    const unsigned long long total = sh.start[a.batch];
+    auto locate = [&](unsigned long long pos, int& b, int& local, int& t) {  // of a position before the end
+        int lo = 0, hi = a.batch;  // last sequence that starts at or before pos (and is not empty there)
+#pragma unroll 1
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (sh.start[mid] <= pos) lo = mid; else hi = mid;
+        }
+        b = lo;
+        const unsigned off = static_cast<unsigned>(pos - sh.start[b]);  // < groups x tiles of a sequence: fits 32 bits
+        local = static_cast<int>(off / static_cast<unsigned>(sh.kt[b]));
+        t = static_cast<int>(off - static_cast<unsigned>(local) * static_cast<unsigned>(sh.kt[b]));
+    };
+    int b = 0, local = 0, t = 0;
+    if (tid <= a.clusters) {
+        unsigned long long cut = total * static_cast<unsigned long long>(tid) / static_cast<unsigned long long>(a.clusters);
+        if (cut < total) {  // a piece shorter than its own epilogue is not worth a cut
+            locate(cut, b, local, t);
+            const int behind = sh.kt[b] - t;
+            if (t <= behind && t <= kSnap)
+                cut -= t;
+            else if (behind < t && behind <= kSnap)
+                cut += behind;
+        }
+        sh.cut[tid] = cut;
+    }
+    __syncthreads();
+    if (tid < a.clusters) {
+        int count = 0;
+        if (sh.cut[tid] < sh.cut[tid + 1]) {
+            int b1, local1, t1;
+            locate(sh.cut[tid + 1] - 1, b1, local1, t1);
+            locate(sh.cut[tid], b, local, t);
+            count = sh.group0[b1] + local1 - sh.group0[b] - local + 1;
+        }
+        sh.n_items[tid] = count;
+    }
+    __syncthreads();
+    if (tid < a.clusters) {
+        int first = 0;
+#pragma unroll 4
+        for (int i = 0; i < tid; ++i) first += sh.n_items[i];
+        const int count = min(sh.n_items[tid], max(a.max_items - first, 0));
+        const unsigned long long begin = sh.cut[tid], end = sh.cut[tid + 1];
+        auto cluster_of = [&](unsigned long long pos) {  // the last CTA that begins at or before pos
+            int lo = 0, hi = a.clusters;
+#pragma unroll 1
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (sh.cut[mid] <= pos) lo = mid; else hi = mid;
+            }
+            return lo;
+        };
+        unsigned long long pos = begin;
+#pragma unroll 1
+        for (int i = 0; i < count; ++i) {
+            const unsigned long long g0 = pos - static_cast<unsigned>(t), g1 = g0 + static_cast<unsigned>(sh.kt[b]);  // the group
+            const unsigned long long stop = g1 < end ? g1 : end;
+            const int c0 = (g0 >= begin) ? tid : cluster_of(g0), c1 = (g1 <= end) ? tid : cluster_of(g1 - 1);
+            PlanItem p = item_of(b, local);
+            p.t_begin = t, p.t_end = static_cast<int>(stop - g0), p.pieces = c1 - c0 + 1;
+            if (i == 0) a.plan_first[tid] = p;
+            a.plan_item[first + i] = p;
+            if (t == 0) write_group(sh.group0[b] + local, p, first + i);
+            // on to the next group
+            pos = stop, t = 0;
+            if (++local == a.Hkv * sh.tiles[b]) {
+                local = 0;
+                do ++b; while (b < a.batch && sh.kt[b] == 0);
+            }
+        }
+        PlanCluster c;
+        c.first_item = first, c.n_items = count;
+        a.plan_cluster[tid] = c;
+    }
 }
 
-// A CTA's view of one entry of the work list.
-__device__ __forceinline__ Item load_item(const AttnArgs& a, int item, int group_rows, int G) {
-    const int4* src = reinterpret_cast<const int4*>(a.plan_item + item);
+// A CTA's view of one item.
+struct Item {
+    int b, g, n, L, M, row_base;
+    int t_begin, t_end;  // this CTA's key tiles (none: t_begin == t_end)
+    int active;          // CTAs of the cluster that have tiles of the item
+    int pieces;
+};
+
+__device__ __forceinline__ Item load_item(const PlanItem* entry, int G) {
+    const int4* src = reinterpret_cast<const int4*>(entry);
     const int4 lo = __ldcg(src), hi = __ldcg(src + 1);
     Item it;
     it.b = lo.x & 0xFFFF, it.g = static_cast<int>(static_cast<unsigned>(lo.x) >> 16);
-    it.pair = lo.y & 0xFFFF, it.splits = static_cast<int>(static_cast<unsigned>(lo.y) >> 16);
-    it.sp = lo.z, it.first_item = lo.w;
-    it.t_begin = hi.x, it.t_end = hi.y, it.n = hi.z, it.L = hi.w;
+    it.row_base = (lo.y & 0xFFFF) * kBM, it.active = static_cast<int>(static_cast<unsigned>(lo.y) >> 16);
+    it.t_begin = lo.z, it.t_end = lo.w;
+    it.n = hi.x, it.L = hi.y, it.pieces = hi.z;
     it.M = it.n * G;
-    it.row_base = it.pair * group_rows;
-    it.nmt = (group_rows > kBM && it.M - it.row_base > kBM) ? 2 : 1;
-    it.tok0 = (it.row_base == 0) ? 0 : it.row_base / G;
     return it;
 }
 
@@ -352,19 +415,58 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
+// Never suspends the thread (a try_wait may): for looking ahead.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// Behind arrivals from other CTAs of the cluster.
+__device__ __forceinline__ bool mbar_try_cluster(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// Arrives on the barrier at the same place in the shared memory of CTA `rank` of the cluster.
+__device__ __forceinline__ void mbar_arrive_remote(uint32_t bar, int rank) {
+    asm volatile(
+        "{\n\t.reg .b32 remote;\n\t"
+        "mapa.shared::cluster.u32 remote, %0, %1;\n\t"
+        "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [remote];\n\t}" ::"r"(bar), "r"(rank)
+        : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 // Bounded wait: false when this wait ran out (about a second of SM clocks) or another thread of
-// the CTA has given up.  Kept to a few instructions, because it is inlined at every wait and the
-// kernel's code has to stay small (see the note on code size at the kernel); the caller records
-// the failure in its `alive` flag, and the status word is written once, at the end of the kernel.
+// the CTA has given up.  Kept to a few instructions, because it is inlined at every wait: a role runs
+// through its code once per launch, most of it cold, and what it costs to fetch is about a cycle per 4
+// bytes.  The caller records the failure in its `alive` flag, and the status word is written once, at
+// the end of the kernel.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
     if (mbar_try(bar, parity)) return true;  // the common case does not even read the clock
     const uint32_t t0 = static_cast<uint32_t>(clock());
-    uint32_t spins = 0;
-    while (!mbar_try(bar, parity)) {
-        // the 32-bit cycle counter wraps after two seconds; it is read far more often than that
-        if ((++spins & 255u) == 0u && (*abort_flag || static_cast<uint32_t>(clock()) - t0 > kWaitLimitCycles))
-            return false;
-    }
+#pragma unroll 1
+    while (!mbar_try(bar, parity))  // the 32-bit cycle counter wraps after two seconds; it is read far more often than that
+        if (static_cast<uint32_t>(clock()) - t0 > kWaitLimitCycles || *abort_flag) return false;
+    return true;
+}
+__device__ __forceinline__ bool cluster_bar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    const uint32_t t0 = static_cast<uint32_t>(clock());
+#pragma unroll 1
+    while (!mbar_try_cluster(bar, parity))
+        if (static_cast<uint32_t>(clock()) - t0 > kWaitLimitCycles || *abort_flag) return false;
     return true;
 }
 // For the tear-down: a copy this thread issued must have landed before the CTA gives up its shared
@@ -460,6 +562,15 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         : "memory");
 }
 #undef RESPS_R8
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+}
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
@@ -513,6 +624,7 @@ __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
+
 // ---------------------------------------------------------------------------- shared memory map
 template <int D>
 struct Smem {
@@ -522,17 +634,17 @@ struct Smem {
     static constexpr int kKVPanel = kBN * 128;
     static constexpr int kKVTile = kPanels * kKVPanel;
     static constexpr int kOffQ = 0;
-    static constexpr int kOffK = kOffQ + kRowTiles * kQTile;
+    static constexpr int kOffK = kOffQ + kQTile;
     static constexpr int kOffV = kOffK + kStagesK * kKVTile;
     static constexpr int kOffBar = kOffV + kStagesV * kKVTile;
-    static constexpr int kNumBars = 2 * (kStagesK + kStagesV) + 1 + kRowTiles * 5 + 3;
-    static constexpr int kOffMisc = kOffBar + 8 * 32;
+    static constexpr int kNumBars = 2 * (kStagesK + kStagesV) + 2 + kLanes * 6 + 3;
+    static constexpr int kOffMisc = kOffBar + 8 * 40;
     static constexpr int kOffMerge = kOffMisc + 64;          // (max, sum) of every row of both lanes
-    static constexpr int kUsed = kOffMerge + kRowTiles * kBM * 8 + 1024;  // + slack to align the base to 1024
+    static constexpr int kUsed = kOffMerge + kLanes * kBM * 8 + 1024;  // + slack to align the base to 1024
     // Never less than 120 KB, more than half of an SM's shared memory: one CTA per SM, so the
     // 512-column TMEM allocation can never wait for a neighbour.
     static constexpr int kBytes = kUsed > 120 * 1024 ? kUsed : 120 * 1024;
-    static_assert(kNumBars <= 32, "barrier area");
+    static_assert(kNumBars <= 40, "barrier area");
     static_assert(2 * kBytes > 228 * 1024, "two CTAs must not fit on one SM");
 };
 
@@ -545,18 +657,85 @@ __device__ __forceinline__ constexpr int bar_kempty(int s) { return kStagesK + k
 __device__ __forceinline__ constexpr int bar_vempty(int s) { return 2 * kStagesK + kStagesV + s; }
 constexpr int kBar0 = 2 * (kStagesK + kStagesV);  // first barrier after the ring's
 __device__ __forceinline__ constexpr int bar_qfull() { return kBar0; }
-// Lane m's S and P share a TMEM buffer (its j-th tile uses buffer j & 1) and each buffer has its own pair of
+__device__ __forceinline__ constexpr int bar_qempty() { return kBar0 + 1; }
+// Lane m's S and P share a TMEM buffer (its j-th tile uses buffer j & 1) and each buffer has its own
 // barriers: a buffer's next phase cannot complete before the other side has observed the
 // current one (QK(j+2) is issued after PV(j), which is issued after pfull(j) was seen), so a
 // parity wait never falls two phases behind.  One pfull barrier for both buffers would: the
 // softmax warps can finish tile j+1 while the MMA thread still waits for V(j).
-__device__ __forceinline__ constexpr int bar_sfull(int m, int buf) { return kBar0 + 1 + m * 5 + buf; }
-__device__ __forceinline__ constexpr int bar_pfull(int m, int buf) { return kBar0 + 1 + m * 5 + 2 + buf; }
-__device__ __forceinline__ constexpr int bar_pvdone(int m) { return kBar0 + 1 + m * 5 + 4; }
-__device__ __forceinline__ constexpr int bar_item() { return kBar0 + 1 + kRowTiles * 5; }
-__device__ __forceinline__ constexpr int bar_qempty() { return kBar0 + 2 + kRowTiles * 5; }
-// key mode: both softmax warpgroups have their partial result (and its PV completions) behind them
-__device__ __forceinline__ constexpr int bar_merge() { return kBar0 + 3 + kRowTiles * 5; }
+// pvdone likewise: whoever has seen S(j) knows that PV(j-2) has completed (QK(j) was issued behind it),
+// so PV(j) and PV(j-1) may be waited for without having looked at every tile's.
+__device__ __forceinline__ constexpr int bar_sfull(int m, int buf) { return kBar0 + 2 + m * 6 + buf; }
+__device__ __forceinline__ constexpr int bar_pfull(int m, int buf) { return kBar0 + 2 + m * 6 + 2 + buf; }
+__device__ __forceinline__ constexpr int bar_pvdone(int m, int buf) { return kBar0 + 2 + m * 6 + 4 + buf; }
+constexpr int kBar1 = kBar0 + 2 + kLanes * 6;
+__device__ __forceinline__ constexpr int bar_item() { return kBar1; }
+// both softmax warpgroups have their partial result (and its PV completions) behind them
+__device__ __forceinline__ constexpr int bar_merge() { return kBar1 + 1; }
+// every softmax warp of every CTA of the cluster has written its share of the CTA's partial
+__device__ __forceinline__ constexpr int bar_meet() { return kBar1 + 2; }
+
+// Merges the partials of an item: this CTA's share of the (16 columns, row) units, O = sum_p w_p O_p /
+// sum_p w_p l_p with w_p = 2^(m_p - max m).  Bound by the latency of L2 (one round trip for six partials,
+// whose loads are in flight together) and by its own code, which is kept short.
+template <int D>
+__device__ __forceinline__ void merge_partials(const AttnArgs& a, const Item& it, unsigned place0, int n_parts,
+                                               int rank, int tid, int G) {
+    constexpr unsigned kBatch = 6;
+    const unsigned nv = static_cast<unsigned>(min(kBM, it.M - it.row_base));  // valid rows
+    const unsigned units = nv * (D / 16);
+    const unsigned u1 = units * static_cast<unsigned>(rank + 1) / static_cast<unsigned>(a.cluster);
+#pragma unroll 1
+    for (unsigned u = units * static_cast<unsigned>(rank) / static_cast<unsigned>(a.cluster) + tid; u < u1; u += kSoftmaxThreads) {
+        const unsigned c16 = u / nv, r = u - c16 * nv;
+        float Mx = -INFINITY, den = 0.f;
+        float acc[16] = {};
+#pragma unroll 1
+        for (unsigned p0 = 0; p0 < static_cast<unsigned>(n_parts); p0 += kBatch) {
+            float4 ml[kBatch];
+            uint4 v[kBatch][2];
+#pragma unroll
+            for (unsigned i = 0; i < kBatch; ++i) {
+                const unsigned place = place0 + min(p0 + i, static_cast<unsigned>(n_parts) - 1u);
+                ml[i] = __ldcg(a.part_ml + place * kBM + r);
+                const uint4* src = a.part_o + ((place * (D / 8) + 2 * c16) * kBM + r);
+                v[i][0] = __ldcg(src), v[i][1] = __ldcg(src + kBM);
+            }
+            float mx = Mx;
+#pragma unroll
+            for (unsigned i = 0; i < kBatch; ++i) mx = fmaxf(mx, ml[i].x);
+            if (mx == -INFINITY) continue;
+            const float corr = ex2_approx(Mx - mx);  // 0 on the first batch
+            den *= corr;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) acc[e] *= corr;
+            Mx = mx;
+#pragma unroll
+            for (unsigned i = 0; i < kBatch; ++i) {
+                // 0 for an empty partial, which stores zeros, and past the end
+                const float w = p0 + i < static_cast<unsigned>(n_parts) ? ex2_approx(ml[i].x - Mx) : 0.f;
+                den += ml[i].y * w;
+                const float wo = (c16 < D / 32 ? ml[i].z : ml[i].w) * w;  // O_p = Ohat * l * scale of this half of the row
+                const uint32_t hw[8] = {v[i][0].x, v[i][0].y, v[i][0].z, v[i][0].w, v[i][1].x, v[i][1].y, v[i][1].z, v[i][1].w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hw[e]));
+                    acc[2 * e] += f.x * wo, acc[2 * e + 1] += f.y * wo;
+                }
+            }
+        }
+        const float inv = 1.f / den;
+        const unsigned R = it.row_base + r, t = R / static_cast<unsigned>(G), h = it.g * G + (R - t * G);
+        const int64_t row = (static_cast<int64_t>(it.b) * a.max_tt + t) * a.Hq + h;
+        uint32_t o[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) o[e] = pack_bf16(acc[2 * e] * inv, acc[2 * e + 1] * inv);
+        uint4* dst = reinterpret_cast<uint4*>(a.o + row * D + c16 * 16);
+        dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
+        dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+        if (a.lse && c16 == 0) a.lse[row] = (Mx + log2f(den)) * 0.6931471805599453f;
+    }
+}
 
 template <int D>
 __global__ void __launch_bounds__(kAttnThreads, 1)
@@ -568,6 +747,8 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
     unsigned char* base_ptr = smem_raw + (base - smem_u32(smem_raw));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int G = a.Hq / a.Hkv;
+    const int cluster_id = static_cast<int>(static_cast<unsigned>(blockIdx.x) / static_cast<unsigned>(a.cluster));
+    const int rank = static_cast<int>(blockIdx.x) - cluster_id * a.cluster;
     const uint32_t bars = base + S::kOffBar;
     auto bar = [&](int i) { return bars + 8u * i; };
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + S::kOffMisc);
@@ -581,36 +762,47 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
     // list is read before the wait, under the tail of the preceding kernel; only when the list was
     // written by the kernel immediately before this one does the read have to follow the wait.
     // Every thread reads the CTA's first item for itself: no role waits for another.
-    int4 head = make_int4(0, 0, 0, 0);
+    int first_item = 0, n_items = 0;
     Item first_it = {};
     auto read_plan = [&]() {
-        head = __ldcg(a.plan_head);
-        if (static_cast<int>(blockIdx.x) < head.x) first_it = load_item(a, blockIdx.x, head.y, G);
+        if (cluster_id < a.clusters) {
+            const int2 c = __ldcg(reinterpret_cast<const int2*>(a.plan_cluster + cluster_id));
+            first_it = load_item(a.plan_first + blockIdx.x, G);
+            first_item = c.x, n_items = c.y;
+        }
     };
     if (!a.plan_after_wait) read_plan();
 
     // ---- one-time set-up ---------------------------------------------------------------
+    // (the producers' barriers by the producers themselves: their first copies go out before the CTA meets)
+    if (warp >= kProducerWarp && lane == 0 && (warp == kProducerWarp || warp == kVProducerWarp)) {
+        const bool is_v = warp == kVProducerWarp;
+#pragma unroll 1
+        for (int s = 0; s < kStagesK; ++s) {  // a tile belongs to one lane
+            mbar_init(bar(is_v ? bar_vfull(s) : bar_kfull(s)), 1);
+            mbar_init(bar(is_v ? bar_vempty(s) : bar_kempty(s)), 1);
+        }
+        if (!is_v) {
+            mbar_init(bar(bar_qfull()), a.q_by_tma ? 1 : kSoftmaxThreads);
+            mbar_init(bar(bar_qempty()), kLanes);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_proxy_async();
+    }
     if (tid == 0) {
         *abort_flag = 0;
-        for (int s = 0; s < kStagesK; ++s) {
-            mbar_init(bar(bar_kfull(s)), 1);
-            mbar_init(bar(bar_kempty(s)), 2);  // one arrival per lane (two from the owner in key mode)
-        }
-        for (int s = 0; s < kStagesV; ++s) {
-            mbar_init(bar(bar_vfull(s)), 1);
-            mbar_init(bar(bar_vempty(s)), 2);
-        }
-        mbar_init(bar(bar_qfull()), a.q_by_tma ? 1 : kSoftmaxThreads);
-        mbar_init(bar(bar_qempty()), 2);
-        for (int m = 0; m < kRowTiles; ++m) {
+#pragma unroll 1
+        for (int m = 0; m < kLanes; ++m) {
+#pragma unroll 1
             for (int bf = 0; bf < 2; ++bf) {
                 mbar_init(bar(bar_sfull(m, bf)), 1);
-                mbar_init(bar(bar_pfull(m, bf)), kBM);
+                mbar_init(bar(bar_pfull(m, bf)), kBM / 32);  // one arrival per warp
+                mbar_init(bar(bar_pvdone(m, bf)), 1);
             }
-            mbar_init(bar(bar_pvdone(m)), 1);
         }
         mbar_init(bar(bar_item()), kSyncThreads);
         mbar_init(bar(bar_merge()), kSoftmaxThreads);
+        mbar_init(bar(bar_meet()), a.cluster * (kSoftmaxThreads / 32));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kMmaWarp0) {
@@ -625,128 +817,102 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_v) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_q) : "memory");
     }
-    // Everything above touches no global memory, so under programmatic dependent launch it
-    // overlaps the tail of the preceding kernel.
+    // Barriers and the TMEM address are visible to the whole cluster behind this pair (other CTAs
+    // arrive on this one's barriers).  Everything so far touches no global memory but the work list, so
+    // under programmatic dependent launch it overlaps the tail of the preceding kernel.
+    tc_fence_before();
+    __syncwarp();
+    cluster_arrive();
     pdl_wait();
     pdl_launch_dependents();
     if (a.plan_after_wait) read_plan();
-    tc_fence_before();
-    __syncthreads();  // barriers and the TMEM address are visible
+    auto load_q = [&](const Item& it) {
+        mbar_expect_tx(bar(bar_qfull()), S::kQTile);
+        tma_load_5d(base + S::kOffQ, &map_q, bar(bar_qfull()), 0, 0, it.g, it.b * a.max_tt + it.row_base / G, 0);
+    };
+    auto load_tile = [&](const Item& it, int t, uint32_t use, bool v) {
+        const int s = use % kStagesK;
+        const uint32_t full = bar(v ? bar_vfull(s) : bar_kfull(s));
+        mbar_expect_tx(full, S::kKVTile);
+        tma_load_5d(base + (v ? S::kOffV : S::kOffK) + s * S::kKVTile, v ? &map_v : &map_k, full, 0, t * kBN, it.g, it.b, 0);
+    };
+    static_assert(kStagesK == kStagesV, "load_tile");
+    // The producers issue the first copies of the CTA's first item at once.
+    const bool early = n_items > 0 && first_it.t_begin < first_it.t_end;
+    if (early && lane == 0 && (warp == kProducerWarp || warp == kVProducerWarp)) {
+        const bool is_v = warp == kVProducerWarp;
+        // (in the wait test's build the CTA's first V copy may be left out)
+        if (!(kWaitTest && is_v && (a.test_drop & 1))) load_tile(first_it, first_it.t_begin, 0, is_v);
+        if (!is_v && a.q_by_tma) load_q(first_it);
+    }
+    __syncwarp();
+    cluster_wait();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const int total_items = head.x, group_rows = head.y;
     // The list must still describe the step parameters it is used with (the caller changes them only
     // through the library, or asks for a new list): one thread compares its item's sequence.
     bool stale = false;
-    if (tid == 0 && static_cast<int>(blockIdx.x) < total_items) {
+    if (tid == 0 && n_items > 0) {
         const int n_live = min(max(a.n_nodes[first_it.b], 0), a.max_tt), L_live = max(a.steps[first_it.b].prefix_len, 0);
         stale = (n_live != first_it.n) || (L_live != first_it.L);
     }
-    // The producers issue the first copies of the CTA's first item at once.
-    const bool early = (warp == kProducerWarp || warp == kVProducerWarp) && lane == 0 &&
-                       static_cast<int>(blockIdx.x) < total_items;
-    if (early) {
-        const Item& it = first_it;
-        if (warp == kProducerWarp) {
-            mbar_expect_tx(bar(bar_kfull(0)), S::kKVTile);
-            tma_load_5d(base + S::kOffK, &map_k, bar(bar_kfull(0)), 0, it.t_begin * kBN, it.g, it.b, 0);
-            if (a.q_by_tma) {
-                mbar_expect_tx(bar(bar_qfull()), it.nmt * S::kQTile);
-                for (int m = 0; m < it.nmt; ++m)
-                    tma_load_5d(base + S::kOffQ + m * S::kQTile, &map_q, bar(bar_qfull()), 0, 0, it.g,
-                                it.b * a.max_tt + it.tok0 + m * (kBM / G), 0);
-            }
-        } else if (!(kWaitTest && (a.test_drop & 1))) {
-            mbar_expect_tx(bar(bar_vfull(0)), S::kKVTile);
-            tma_load_5d(base + S::kOffV, &map_v, bar(bar_vfull(0)), 0, it.t_begin * kBN, it.g, it.b, 0);
-        }
-    }
-    auto get_item = [&](int item, int local) {  // local = how many items this CTA has started before
-        return local == 0 ? first_it : load_item(a, item, group_rows, G);
-    };
+    auto get_item = [&](int i) { return i == 0 ? first_it : load_item(a.plan_item + first_item + i, G); };
 
     // Running use counts of the barrier families.  Every role walks the same items and tiles in
     // the same order, so each keeps its own copy.
     uint32_t kt_run = 0;     // K/V ring uses (all tiles of all items)
     uint32_t jx = 0;         // tiles this lane has taken (S/P buffers, PV completions)
-    uint32_t items_run = 0;
-    uint32_t merges_run = 0;  // key-mode items (uses of the merge barrier)
+    uint32_t items_run = 0;  // items with tiles for this CTA
     bool alive = true;
 
     // Registers follow the roles: the softmax warpgroups hold a tile of S, a tile of P and a row of
     // O; the warpgroup of the producers and MMA issuers needs few (384 x 168 at launch).
     if (warp >= kProducerWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIssue));
-    if (warp == kProducerWarp) {
-        // ================================ TMA producer: K tiles and Q =======================
+    if (warp == kProducerWarp || warp == kVProducerWarp) {
+        // ================================ TMA producers: K tiles and Q; V tiles ==============
         if (lane == 0) {
-            int li = 0;
-            for (int item = blockIdx.x; item < total_items && alive; item += gridDim.x, ++li) {
-                const Item it = get_item(item, li);
+            const bool is_v = warp == kVProducerWarp;
+#pragma unroll 1
+            for (int i = 0; i < n_items && alive; ++i) {
+                const Item it = get_item(i);
+#pragma unroll 1
                 for (int t = it.t_begin; t < it.t_end; ++t, ++kt_run) {
                     const int s = kt_run % kStagesK;
-                    if (kt_run > 0) {  // the CTA's very first tile went out during the set-up
-                        // the first use of a stage finds it free
-                        if (kt_run >= kStagesK &&
-                            !mbar_wait(bar(bar_kempty(s)), ((kt_run / kStagesK) & 1u) ^ 1u, abort_flag)) {
+                    if (kt_run == 0) {  // went out during the set-up, and the item's Q with it
+                        ++items_run;
+                        continue;
+                    }
+                    // the first use of a stage finds it free
+                    if (kt_run >= kStagesK && !mbar_wait(bar(is_v ? bar_vempty(s) : bar_kempty(s)),
+                                                         ((kt_run / kStagesK) & 1u) ^ 1u, abort_flag)) {
+                        alive = false;
+                        break;
+                    }
+                    load_tile(it, t, kt_run, is_v);
+                    if (t == it.t_begin && !is_v && a.q_by_tma) {
+                        // Q follows the first K tile: K and Q are what the first MMA needs.  The Q
+                        // tile of the previous item is free once its last QK^T has completed.
+                        if (!mbar_wait(bar(bar_qempty()), (items_run & 1u) ^ 1u, abort_flag)) {
                             alive = false;
+                            ++kt_run;
                             break;
                         }
-                        mbar_expect_tx(bar(bar_kfull(s)), S::kKVTile);
-                        tma_load_5d(base + S::kOffK + s * S::kKVTile, &map_k, bar(bar_kfull(s)), 0, t * kBN, it.g,
-                                    it.b, 0);
-                    }
-                    if (t == it.t_begin && a.q_by_tma) {
-                        // Q follows the first K tile: K and Q are what the first MMA needs.  The Q
-                        // tiles of the previous item are free once its last QK^T has completed.
-                        if (items_run > 0) {
-                            if (!mbar_wait(bar(bar_qempty()), (items_run & 1u) ^ 1u, abort_flag)) {
-                                alive = false;
-                                break;
-                            }
-                            mbar_expect_tx(bar(bar_qfull()), it.nmt * S::kQTile);
-                            for (int m = 0; m < it.nmt; ++m)
-                                tma_load_5d(base + S::kOffQ + m * S::kQTile, &map_q, bar(bar_qfull()), 0, 0, it.g,
-                                            it.b * a.max_tt + it.tok0 + m * (kBM / G), 0);
-                        }
+                        load_q(it);
                         ++items_run;
                     }
                 }
             }
             // Drain: every copy this thread issued has landed before the CTA may exit (each one is
             // waited for, also after an earlier wait has run out).
-            bool landed = !(a.q_by_tma && items_run > 0) || drain_wait(bar(bar_qfull()), (items_run - 1u) & 1u);
+            bool landed = is_v || !(a.q_by_tma && items_run > 0) || drain_wait(bar(bar_qfull()), (items_run - 1u) & 1u);
             const uint32_t issued = kt_run;
+#pragma unroll 1
             for (uint32_t u = (issued > kStagesK ? issued - kStagesK : 0u); u < issued; ++u)
-                landed = drain_wait(bar(bar_kfull(u % kStagesK)), (u / kStagesK) & 1u) && landed;
+                landed = drain_wait(bar(is_v ? bar_vfull(u % kStagesK) : bar_kfull(u % kStagesK)), (u / kStagesK) & 1u) && landed;
             alive = alive && landed;
         }
-    } else if (warp == kVProducerWarp) {
-        // ================================ TMA producer: V tiles =============================
-        if (lane == 0) {
-            int li = 0;
-            for (int item = blockIdx.x; item < total_items && alive; item += gridDim.x, ++li) {
-                const Item it = get_item(item, li);
-                for (int t = it.t_begin; t < it.t_end; ++t, ++kt_run) {
-                    const int s = kt_run % kStagesV;
-                    if (kt_run == 0) continue;  // went out during the set-up
-                    if (kt_run >= kStagesV &&
-                        !mbar_wait(bar(bar_vempty(s)), ((kt_run / kStagesV) & 1u) ^ 1u, abort_flag)) {
-                        alive = false;
-                        break;
-                    }
-                    mbar_expect_tx(bar(bar_vfull(s)), S::kKVTile);
-                    tma_load_5d(base + S::kOffV + s * S::kKVTile, &map_v, bar(bar_vfull(s)), 0, t * kBN, it.g, it.b,
-                                0);
-                }
-            }
-            const uint32_t issued = kt_run;
-            bool landed = true;
-            for (uint32_t u = (issued > kStagesV ? issued - kStagesV : 0u); u < issued; ++u)
-                landed = drain_wait(bar(bar_vfull(u % kStagesV)), (u / kStagesV) & 1u) && landed;
-            alive = alive && landed;
-        }
-    } else if (warp == kMmaWarp0 || warp == kMmaWarp0 + 1) {
+    } else {
         // ================================ MMA issuer of lane x ============================
         // The whole warp walks the loop and waits (so that every value stays warp-uniform);
         // one elected lane issues.  The MMAs of one thread execute in issue order: QK of this
@@ -757,91 +923,89 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
         constexpr uint32_t kIdescQK = instr_desc(kBN, false);
         constexpr uint32_t kIdescPV = instr_desc(D, true);
         // Descriptors differ only in the (16-byte granular) start address, the low 14 bits.
-        const uint64_t qdesc0 = smem_desc(base + S::kOffQ, 16, 1024);
+        const uint64_t qdesc = smem_desc(base + S::kOffQ, 16, 1024);
         const uint64_t kdesc0 = smem_desc(base + S::kOffK, 16, 1024);
         const uint64_t vdesc0 = smem_desc(base + S::kOffV, S::kKVPanel, 1024);
         const uint32_t o_t = tmem + x * 256 + 128;
         uint32_t k_seen = 0xFFFFFFFFu;  // ring use whose K tile this warp has already seen arrive
-        for (int item = blockIdx.x; item < total_items && alive; item += gridDim.x, ++items_run) {
-            const Item it = get_item(item, static_cast<int>(items_run));
-            const bool row_mode = it.nmt == 2;
-            const uint64_t qdesc = qdesc0 + static_cast<uint64_t>((row_mode ? x : 0) * (S::kQTile >> 4));
+#pragma unroll 1
+        for (int i = 0; i < n_items && alive; ++i) {
+            const Item it = get_item(i);
+            if (it.t_begin == it.t_end) continue;
             alive = warp_wait(bar(bar_qfull()), items_run & 1u, abort_flag);
             tc_fence_after();
-            if (row_mode && x == 1) {
-                // Lane 1 starts half a tile period behind lane 0: the lanes' bursts of MMAs (P V of one
-                // tile, Q K^T of the tile after next) then take turns on the tensor pipe instead of
-                // queueing behind each other, which is what decides when a lane gets its next S.
-                const long long t_go = clock64() + a.stagger;
-                while (clock64() < t_go) {}
-            }
-            bool have_prev = false, first_pv = true;
-            uint32_t prev_kt = 0, prev_j = 0;
-            // In key mode a tile belongs to one lane alone: its owner releases the stage for both.
-            const int releases = row_mode ? 1 : 2;
-            // P V of this lane's previous tile.  While it waits for P it looks (without blocking) at
-            // the K tile of the lane's next Q K^T, whose wait would otherwise sit between P V and the
-            // next Q K^T: the chain that decides when the softmax warps get their next S.
-            auto issue_pv = [&](uint32_t next_use) {
-                const int s = prev_kt % kStagesV;
-                if (!warp_wait(bar(bar_vfull(s)), (prev_kt / kStagesV) & 1u, abort_flag)) return false;
-                if (next_use != 0xFFFFFFFFu &&
-                    __all_sync(kFull, mbar_try(bar(bar_kfull(next_use % kStagesK)), (next_use / kStagesK) & 1u)))
-                    k_seen = next_use;
-                if (!warp_wait(bar(bar_pfull(x, prev_j & 1u)), (prev_j >> 1) & 1u, abort_flag)) return false;
-                tc_fence_after();
-                if (elect_one()) {
-                    const uint64_t vdesc = vdesc0 + static_cast<uint64_t>(s * (S::kKVTile >> 4));
-                    // P of keys 32h .. 32h+31: hi in columns 32h .. 32h+15, lo in 32h+16 .. 32h+31
-                    const uint32_t p_t = tmem + x * 256 + (prev_j & 1u) * kBN;
-#pragma unroll
-                    for (int kk = 0; kk < kBN / 16; ++kk) {
-                        const uint32_t a_t = p_t + (kk >> 1) * 32 + (kk & 1) * 8;
-                        umma_ts(o_t, a_t, vdesc + kk * (2048 >> 4), kIdescPV, (first_pv && kk == 0) ? 0u : 1u);
-                        umma_ts(o_t, a_t + 16, vdesc + kk * (2048 >> 4), kIdescPV, 1u);
+            bool first_pv = true;
+            // The lane's tiles are t_begin + x, + 2, ...; one round issues Q K^T of a tile and P V of the one
+            // before (the last round P V only).
+            const int mine = (it.t_end - it.t_begin - x + 1) >> 1;
+            const uint32_t use0 = kt_run + static_cast<uint32_t>(x);
+#pragma unroll 1
+            for (int j = 0; j <= mine && mine > 0 && alive; ++j) {
+                if (j < mine) {
+                    const uint32_t use = use0 + 2u * j;
+                    const int s = use % kStagesK;
+                    if (k_seen != use && !warp_wait(bar(bar_kfull(s)), (use / kStagesK) & 1u, abort_flag)) {
+                        alive = false;
+                        break;
                     }
-                    umma_commit(bar(bar_pvdone(x)));
-                    for (int rls = 0; rls < releases; ++rls) umma_commit(bar(bar_vempty(s)));
-                }
-                __syncwarp();
-                first_pv = false;
-                return true;
-            };
-            const int t_step = row_mode ? 1 : 2;  // distance to this lane's next tile
-            for (int t = it.t_begin; t < it.t_end && alive; ++t, ++kt_run) {
-                const int s = kt_run % kStagesK;
-                const bool own = row_mode || (((t - it.t_begin) & 1) == x);
-                if (own) {
-                    if (k_seen != kt_run)
-                        alive = warp_wait(bar(bar_kfull(s)), (kt_run / kStagesK) & 1u, abort_flag);
-                    if (!alive) break;
                     tc_fence_after();
                     if (elect_one()) {
                         const uint64_t kdesc = kdesc0 + static_cast<uint64_t>(s * (S::kKVTile >> 4));
                         const uint32_t s_t = tmem + x * 256 + (jx & 1u) * kBN;
-#pragma unroll
+#pragma unroll 2
                         for (int ks = 0; ks < D / 16; ++ks)
                             umma(s_t, qdesc + ((ks >> 2) * (S::kQPanel >> 4) + (ks & 3) * 2),
                                  kdesc + ((ks >> 2) * (S::kKVPanel >> 4) + (ks & 3) * 2), kIdescQK, ks > 0 ? 1u : 0u);
                         umma_commit(bar(bar_sfull(x, jx & 1u)));
-                        for (int rls = 0; rls < releases; ++rls) umma_commit(bar(bar_kempty(s)));
+                        umma_commit(bar(bar_kempty(s)));
                     }
                     __syncwarp();
-                    if (have_prev)
-                        alive = issue_pv(t + t_step < it.t_end ? kt_run + static_cast<uint32_t>(t_step) : 0xFFFFFFFFu);
-                    have_prev = true, prev_kt = kt_run, prev_j = jx;
                     ++jx;
                 }
+                if (j > 0) {
+                    // P V of the lane's previous tile.  While it waits for P it looks (without blocking) at
+                    // the K tile of the lane's next Q K^T, whose wait would otherwise sit between P V and
+                    // the next Q K^T: the chain that decides when the softmax warps get their next S.
+                    const uint32_t prev_use = use0 + 2u * (j - 1), prev_j = jx - (j < mine ? 2u : 1u);
+                    const uint32_t next_use = use0 + 2u * (j + 1);
+                    const int s = prev_use % kStagesV;
+                    alive = warp_wait(bar(bar_vfull(s)), (prev_use / kStagesV) & 1u, abort_flag);
+                    if (!alive) break;
+                    if (j + 1 < mine &&
+                        __all_sync(kFull, mbar_test(bar(bar_kfull(next_use % kStagesK)), (next_use / kStagesK) & 1u)))
+                        k_seen = next_use;
+                    alive = warp_wait(bar(bar_pfull(x, prev_j & 1u)), (prev_j >> 1) & 1u, abort_flag);
+                    if (!alive) break;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        const uint64_t vdesc = vdesc0 + static_cast<uint64_t>(s * (S::kKVTile >> 4));
+                        // P of keys 32h .. 32h+31: hi in columns 32h .. 32h+15, lo in 32h+16 .. 32h+31
+                        const uint32_t p_t = tmem + x * 256 + (prev_j & 1u) * kBN;
+#pragma unroll 1
+                        for (int kk = 0; kk < kBN / 16; ++kk) {
+                            const uint32_t a_t = p_t + (kk >> 1) * 32 + (kk & 1) * 8;
+                            umma_ts(o_t, a_t, vdesc + kk * (2048 >> 4), kIdescPV, (first_pv && kk == 0) ? 0u : 1u);
+                            umma_ts(o_t, a_t + 16, vdesc + kk * (2048 >> 4), kIdescPV, 1u);
+                        }
+                        umma_commit(bar(bar_pvdone(x, prev_j & 1u)));
+                        umma_commit(bar(bar_vempty(s)));
+                    }
+                    __syncwarp();
+                    first_pv = false;
+                }
                 // Q is free for the next item once the last QK^T of both lanes has completed
-                if (t + 1 == it.t_end && elect_one()) umma_commit(bar(bar_qempty()));
+                if (j + 1 == mine && elect_one()) umma_commit(bar(bar_qempty()));
                 __syncwarp();
             }
-            if (alive && have_prev) alive = issue_pv(0xFFFFFFFFu);
+            if (alive && mine == 0 && elect_one()) umma_commit(bar(bar_qempty()));
+            __syncwarp();
+            kt_run += static_cast<uint32_t>(it.t_end - it.t_begin);
             tc_fence_before();
             if (!alive) break;
             // end of item: the softmax warps have read O and S, Q and P may be overwritten
             mbar_arrive(bar(bar_item()));
             alive = warp_wait(bar(bar_item()), items_run & 1u, abort_flag);
+            ++items_run;
         }
     }
     } else {
@@ -850,346 +1014,272 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
         const int x = warp >> 2;
         const int r = (warp & 3) * 32 + lane;          // row inside the tile = TMEM lane
         const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
-        const uint32_t o_t = tmem + lane_sel + x * 256 + 128;
-        constexpr int kChunks = D / 8;                 // 16-byte pieces of a row
-        for (int item = blockIdx.x; item < total_items && alive; item += gridDim.x, ++items_run) {
-            const Item it = get_item(item, static_cast<int>(items_run));
-            const bool row_mode = it.nmt == 2;
-            // ---- Q tiles -> shared memory in the swizzled K-major layout (only when the group
-            // size does not allow the TMA view) ---------------------------------------------
-            if (!a.q_by_tma) {
-                // (a plain loop: this path serves group sizes that do not divide 128 and is not
-                // worth its unrolled form's code size)
-                const int total = it.nmt * kBM * kChunks;
+        const uint32_t s_t = tmem + lane_sel + x * 256, o_t = s_t + 128;
+        uint32_t merges = 0, meets = 0;                // uses of the end-of-item barriers
 #pragma unroll 1
-                for (int i = tid; i < total; i += kSoftmaxThreads) {
-                    const int row = i / kChunks, c = i % kChunks;
-                    const int Rq = it.row_base + row;
-                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                    if (Rq < it.M) {
-                        const int t = Rq / G, h = it.g * G + Rq % G;
-                        v = __ldg(reinterpret_cast<const uint4*>(
-                            a.q + ((static_cast<int64_t>(it.b) * a.max_tt + t) * a.Hq + h) * D + c * 8));
-                    }
-                    const int m = row / kBM, rr = row % kBM;
-                    unsigned char* dst = base_ptr + S::kOffQ + m * S::kQTile + (c >> 3) * S::kQPanel + rr * 128 +
-                                         (((c & 7) ^ (rr & 7)) << 4);
-                    *reinterpret_cast<uint4*>(dst) = v;
-                }
-                fence_proxy_async();
-                mbar_arrive(bar(bar_qfull()));
-            }
-
-            const int R = it.row_base + (row_mode ? x * kBM : 0) + r;
-            const bool row_ok = R < it.M;
-            unsigned long long mlo = 0ull, mhi = 0ull;
-            if (row_ok) {
-                const int t = R / G;
-                mlo = a.mask[(static_cast<int64_t>(it.b) * a.max_tt + t) * 2 + 0];
-                mhi = a.mask[(static_cast<int64_t>(it.b) * a.max_tt + t) * 2 + 1];
-                // only nodes of this tree can be visible
-                if (it.n < 64) {
-                    mlo &= (1ull << it.n) - 1ull;
-                    mhi = 0ull;
-                } else if (it.n < 128) {
-                    mhi &= (1ull << (it.n - 64)) - 1ull;
-                }
-            }
-            float m_ref = -INFINITY, l_run = 0.f;
-            const int kv_len = it.L + it.n;
-            // PV completions of this lane seen so far.  pvdone completes once per tile and a parity
-            // wait must never fall two phases behind, so PV(j-1) is observed before P(j) is handed
-            // over (PV(j) cannot be issued earlier): by then it has usually completed.
-            uint32_t pv_seen = jx;
-            bool first = true;
-            // A wait on a barrier costs a few hundred cycles even when its phase completed long ago,
-            // and this loop is the longest dependent chain of the kernel.  So the two things a tile
-            // has to wait for are looked at early, without blocking, and the answers are used later:
-            // PV(j-1) before the exponentials, S(j+1) between their halves.  When S(j+1) is there its
-            // load is issued before P(j) is handed over, and the next round starts with the data.
-            uint32_t sr[2][32];
-            bool s_loaded = false;
-            const int t_step = row_mode ? 1 : 2;  // distance to this lane's next tile
-
-            for (int t = it.t_begin; t < it.t_end; ++t, ++kt_run) {
-                if (!(row_mode || (((t - it.t_begin) & 1) == x))) continue;
-                const uint32_t buf = jx & 1u;
-                if (!s_loaded) {
-                    if (!warp_wait(bar(bar_sfull(x, buf)), (jx >> 1) & 1u, abort_flag)) {
-                        alive = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    tmem_ld32(tmem + lane_sel + x * 256 + buf * kBN, sr[0]);
-                    tmem_ld32(tmem + lane_sel + x * 256 + buf * kBN + 32, sr[1]);
-                }
-                tmem_wait_ld();
-
-                // ---- ancestor mask (tiles that reach past the prefix only), row maximum -------
-                const int j0 = t * kBN;
-                float tmax = -INFINITY;
-                if (j0 + kBN > it.L) {
-                    const int off = j0 - it.L;  // tile start relative to the first tree slot
-                    unsigned long long allowed;
-                    if (off >= 64)
-                        allowed = mhi >> (off - 64);
-                    else if (off > 0)
-                        allowed = (mlo >> off) | (mhi << (64 - off));
-                    else if (off == 0)
-                        allowed = mlo;
-                    else  // -64 < off < 0: the first -off keys are prefix
-                        allowed = (mlo << (-off)) | ((1ull << (-off)) - 1ull);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-#pragma unroll
-                        for (int c = 0; c < 32; ++c) {
-                            float s = __uint_as_float(sr[h][c]);
-                            if (!((allowed >> (h * 32 + c)) & 1ull)) s = -INFINITY;
-                            sr[h][c] = __float_as_uint(s);
-                            tmax = fmaxf(tmax, s);
+        for (int i = 0; i < n_items && alive; ++i) {
+            const Item it = get_item(i);
+            const int n_tiles = it.t_end - it.t_begin;
+            const bool direct = it.pieces == 1 && it.active == 1;  // one CTA has the whole group
+            if (n_tiles > 0) {
+                // ---- Q tile -> shared memory in the swizzled K-major layout (only when the group
+                // size does not allow the TMA view; a plain loop, not worth unrolled code) --------
+                if (!a.q_by_tma) {
+                    constexpr int kChunks = D / 8;  // 16-byte pieces of a row
+#pragma unroll 1
+                    for (int e = tid; e < kBM * kChunks; e += kSoftmaxThreads) {
+                        const int row = e / kChunks, c = e % kChunks;
+                        const int Rq = it.row_base + row;
+                        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                        if (Rq < it.M) {
+                            const int t = Rq / G, h = it.g * G + Rq % G;
+                            v = __ldg(reinterpret_cast<const uint4*>(
+                                a.q + ((static_cast<int64_t>(it.b) * a.max_tt + t) * a.Hq + h) * D + c * 8));
                         }
-                } else {
+                        *reinterpret_cast<uint4*>(base_ptr + S::kOffQ + (c >> 3) * S::kQPanel + row * 128 +
+                                                  (((c & 7) ^ (row & 7)) << 4)) = v;
+                    }
+                    fence_proxy_async();
+                    mbar_arrive(bar(bar_qfull()));
+                }
+
+                const int R = it.row_base + r;
+                const bool row_ok = R < it.M;
+                unsigned long long mlo = 0ull, mhi = 0ull;
+                if (row_ok) {
+                    const int t = R / G;
+                    mlo = a.mask[(static_cast<int64_t>(it.b) * a.max_tt + t) * 2 + 0];
+                    mhi = a.mask[(static_cast<int64_t>(it.b) * a.max_tt + t) * 2 + 1];
+                    // only nodes of this tree can be visible
+                    if (it.n < 64) {
+                        mlo &= (1ull << it.n) - 1ull;
+                        mhi = 0ull;
+                    } else if (it.n < 128) {
+                        mhi &= (1ull << (it.n - 64)) - 1ull;
+                    }
+                }
+                float m_ref = -INFINITY, l_run = 0.f;
+                const int kv_len = it.L + it.n;
+                bool first = true, s_loaded = false;
+                uint32_t sr[2][32];
+                auto load_s = [&](uint32_t buf) {
+                    tc_fence_after();
+                    tmem_ld32(s_t + buf * kBN, sr[0]);
+                    tmem_ld32(s_t + buf * kBN + 32, sr[1]);
+                };
+#pragma unroll 1
+                for (int t = it.t_begin + x; t < it.t_end; t += kLanes) {
+                    const uint32_t buf = jx & 1u;
+                    if (!s_loaded) {
+                        alive = warp_wait(bar(bar_sfull(x, buf)), (jx >> 1) & 1u, abort_flag);
+                        if (!alive) break;
+                        load_s(buf);
+                    }
+                    tmem_wait_ld();
+
+                    // ---- ancestor mask (tiles that reach past the prefix only), row maximum -------
+                    const int j0 = t * kBN;
+                    if (j0 + kBN > it.L) {
+                        const int off = j0 - it.L;  // tile start relative to the first tree slot
+                        unsigned long long allowed;
+                        if (off >= 64)
+                            allowed = mhi >> (off - 64);
+                        else if (off > 0)
+                            allowed = (mlo >> off) | (mhi << (64 - off));
+                        else if (off == 0)
+                            allowed = mlo;
+                        else  // -64 < off < 0: the first -off keys are prefix
+                            allowed = (mlo << (-off)) | ((1ull << (-off)) - 1ull);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const uint32_t bits = static_cast<uint32_t>(allowed >> (32 * h));
+#pragma unroll
+                            for (int c = 0; c < 32; ++c)
+                                if (!((bits >> c) & 1u)) sr[h][c] = 0xFF800000u;  // -inf
+                        }
+                    }
                     float t4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};  // four independent chains
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
 #pragma unroll
                         for (int c = 0; c < 32; c += 2)
                             t4[(c >> 1) & 3] = max3(t4[(c >> 1) & 3], __uint_as_float(sr[h][c]), __uint_as_float(sr[h][c + 1]));
-                    tmax = fmaxf(fmaxf(t4[0], t4[1]), fmaxf(t4[2], t4[3]));
-                }
-                tmax *= a.scale_log2;  // the scale is positive: max(scale * s) = scale * max(s)
-                const float m_new = fmaxf(m_ref, tmax);
-                // Lazy rescale: O and l keep the old reference maximum while the true one
-                // grew by less than 2^kRescaleSlack (fp32 accumulators have the head-room).
-                const bool need = !first && (m_new > m_ref + kRescaleSlack);
-                if (first) m_ref = m_new;
-                if (__any_sync(kFull, need)) {
-                    // O may only be touched once PV of the previous tile has completed
-                    while (pv_seen < jx) {
-                        if (!warp_wait(bar(bar_pvdone(x)), pv_seen & 1u, abort_flag)) alive = false;
-                        ++pv_seen;
-                    }
-                    if (!alive) break;
-                    const float corr = need ? ex2_approx(m_ref - m_new) : 1.f;
-                    if (need) m_ref = m_new;
-                    l_run *= corr;
-                    tc_fence_after();
-#pragma unroll 1
-                    for (int c0 = 0; c0 < D; c0 += 32) {
-                        uint32_t orr[32];
-                        tmem_ld32(o_t + c0, orr);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int c = 0; c < 32; ++c) orr[c] = __float_as_uint(__uint_as_float(orr[c]) * corr);
-                        tmem_st32(o_t + c0, orr);
-                    }
-                    tmem_wait_st();
-                }
-                const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
-                // PV(j-1): asked now, answered after the exponentials (pv_seen is jx or jx - 1 here)
-                const bool pv_probe = (pv_seen == jx) || mbar_try(bar(bar_pvdone(x)), pv_seen & 1u);
-                const bool has_next = t + t_step < it.t_end;
-                bool s_probe = false;
-
-                // ---- stale V rows of the sequence's last tile must not reach the MMA (in row mode
-                // both lanes clear them: each lane's PV is ordered behind its own warpgroup only) ----
-                const bool clear_v = j0 + kBN > kv_len;
-                if (clear_v) {
-                    const int s = kt_run % kStagesV;
-                    if (!warp_wait(bar(bar_vfull(s)), (kt_run / kStagesV) & 1u, abort_flag)) {
-                        alive = false;
-                        break;
-                    }
-                    const int valid = kv_len - j0;
-                    unsigned char* vt = base_ptr + S::kOffV + s * S::kKVTile;
-                    for (int i = r; i < (kBN - valid) * 8 * S::kPanels; i += kBM) {
-                        const int row = valid + i / (8 * S::kPanels), cc = i % (8 * S::kPanels);
-                        *reinterpret_cast<uint4*>(vt + (cc >> 3) * S::kKVPanel + row * 128 + ((cc & 7) << 4)) =
-                            make_uint4(0u, 0u, 0u, 0u);
-                    }
-                }
-
-                // ---- P = exp2(scale * S - m) as bf16 hi + lo, back into the columns S came from.
-                // hi is p truncated to bf16, so p - hi is exact and lo = bf16(p - hi) leaves an
-                // error of 2^-16 p.  Packed fp32 pairs halve the instruction count.  Each half of the
-                // tile (32 keys) becomes 16 columns of hi and 16 of lo in place of its own 32 columns
-                // of S, stored as soon as it is ready so that the store overlaps the other half.
-                {
-                    const unsigned long long sc2 = pack2(a.scale_log2, a.scale_log2);
-                    const unsigned long long nm2 = pack2(-m_use, -m_use);
-                    unsigned long long psum2 = pack2(0.f, 0.f);
-                    const uint32_t p_t = tmem + lane_sel + x * 256 + buf * kBN;
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        if (h == 1 && has_next)
-                            s_probe = mbar_try(bar(bar_sfull(x, buf ^ 1u)), ((jx + 1u) >> 1) & 1u);
-                        uint32_t w[32];
-#pragma unroll
-                        for (int c = 0; c < 16; ++c) {
-                            float x0, x1;
-                            unpack2(fma2(pack2(__uint_as_float(sr[h][2 * c]), __uint_as_float(sr[h][2 * c + 1])), sc2, nm2),
-                                    x0, x1);
-                            const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
-                            const unsigned long long p2 = pack2(p0, p1);
-                            psum2 = add2(psum2, p2);
-                            const uint32_t b0 = __float_as_uint(p0), b1 = __float_as_uint(p1);
-                            w[c] = __byte_perm(b0, b1, 0x7632);
-                            float l0, l1;
-                            unpack2(sub2(p2, pack2(__uint_as_float(b0 & 0xFFFF0000u), __uint_as_float(b1 & 0xFFFF0000u))),
-                                    l0, l1);
-                            w[16 + c] = pack_bf16(l0, l1);
-                        }
-                        tmem_st32(p_t + h * 32, w);
-                    }
-                    float ps0, ps1;
-                    unpack2(psum2, ps0, ps1);
-                    l_run += ps0 + ps1;
-                }
-                // S of this lane's next tile, if it has arrived (sr is free now)
-                s_loaded = false;
-                if (has_next) {
-                    if (!__all_sync(kFull, s_probe))
-                        s_probe = mbar_try(bar(bar_sfull(x, buf ^ 1u)), ((jx + 1u) >> 1) & 1u);
-                    if (__all_sync(kFull, s_probe)) {
+                    // the scale is positive: max(scale * s) = scale * max(s)
+                    const float tmax = fmaxf(fmaxf(t4[0], t4[1]), fmaxf(t4[2], t4[3])) * a.scale_log2;
+                    const float m_new = fmaxf(m_ref, tmax);
+                    // Lazy rescale: O and l keep the old reference maximum while the true one
+                    // grew by less than 2^kRescaleSlack (fp32 accumulators have the head-room).
+                    const bool need = !first && (m_new > m_ref + kRescaleSlack);
+                    if (first) m_ref = m_new;
+                    if (__any_sync(kFull, need)) {
+                        // O may only be touched once PV of the previous tile has completed
+                        alive = warp_wait(bar(bar_pvdone(x, buf ^ 1u)), ((jx - 1u) >> 1) & 1u, abort_flag);
+                        if (!alive) break;
+                        const float corr = need ? ex2_approx(m_ref - m_new) : 1.f;
+                        if (need) m_ref = m_new;
+                        l_run *= corr;
                         tc_fence_after();
-                        tmem_ld32(tmem + lane_sel + x * 256 + (buf ^ 1u) * kBN, sr[0]);
-                        tmem_ld32(tmem + lane_sel + x * 256 + (buf ^ 1u) * kBN + 32, sr[1]);
-                        s_loaded = true;
+#pragma unroll 1
+                        for (int c0 = 0; c0 < D; c0 += 32) {
+                            uint32_t orr[32];
+                            tmem_ld32(o_t + c0, orr);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int c = 0; c < 32; ++c) orr[c] = __float_as_uint(__uint_as_float(orr[c]) * corr);
+                            tmem_st32(o_t + c0, orr);
+                        }
+                        tmem_wait_st();
                     }
-                }
-                tmem_wait_st();
-                if (clear_v) fence_proxy_async();
-                if (pv_seen < jx) {
-                    if (!__all_sync(kFull, pv_probe) &&
-                        !warp_wait(bar(bar_pvdone(x)), pv_seen & 1u, abort_flag))
-                        alive = false;
-                    ++pv_seen;
+                    const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
+
+                    // ---- stale V rows of the sequence's last tile must not reach the MMA ----------
+                    const bool clear_v = j0 + kBN > kv_len;
+                    if (clear_v) {
+                        const uint32_t use = kt_run + static_cast<uint32_t>(t - it.t_begin);
+                        const int s = use % kStagesV;
+                        alive = warp_wait(bar(bar_vfull(s)), (use / kStagesV) & 1u, abort_flag);
+                        if (!alive) break;
+                        const int valid = kv_len - j0;
+                        unsigned char* vt = base_ptr + S::kOffV + s * S::kKVTile;
+#pragma unroll 1
+                        for (int e = r; e < (kBN - valid) * 8 * S::kPanels; e += kBM) {
+                            const int row = valid + e / (8 * S::kPanels), cc = e % (8 * S::kPanels);
+                            *reinterpret_cast<uint4*>(vt + (cc >> 3) * S::kKVPanel + row * 128 + ((cc & 7) << 4)) =
+                                make_uint4(0u, 0u, 0u, 0u);
+                        }
+                        fence_proxy_async();
+                    }
+
+                    // ---- P = exp2(scale * S - m) as bf16 hi + lo, back into the columns S came from.
+                    // hi is p truncated to bf16, so p - hi is exact and lo = bf16(p - hi) leaves an
+                    // error of 2^-16 p.  Packed fp32 pairs halve the instruction count.  Each half of the
+                    // tile (32 keys) becomes 16 columns of hi and 16 of lo in place of its own 32 columns
+                    // of S, stored as soon as it is ready so that the store overlaps the other half.
+                    {
+                        const unsigned long long sc2 = pack2(a.scale_log2, a.scale_log2);
+                        const unsigned long long nm2 = pack2(-m_use, -m_use);
+                        unsigned long long psum2 = pack2(0.f, 0.f);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            uint32_t w[32];
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) {
+                                float x0, x1;
+                                unpack2(fma2(pack2(__uint_as_float(sr[h][2 * c]), __uint_as_float(sr[h][2 * c + 1])), sc2, nm2),
+                                        x0, x1);
+                                const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
+                                const unsigned long long p2 = pack2(p0, p1);
+                                psum2 = add2(psum2, p2);
+                                const uint32_t b0 = __float_as_uint(p0), b1 = __float_as_uint(p1);
+                                w[c] = __byte_perm(b0, b1, 0x7632);
+                                float l0, l1;
+                                unpack2(sub2(p2, pack2(__uint_as_float(b0 & 0xFFFF0000u), __uint_as_float(b1 & 0xFFFF0000u))),
+                                        l0, l1);
+                                w[16 + c] = pack_bf16(l0, l1);
+                            }
+                            tmem_st32(s_t + buf * kBN + h * 32, w);
+                        }
+                        float ps0, ps1;
+                        unpack2(psum2, ps0, ps1);
+                        l_run += ps0 + ps1;
+                    }
+                    // P is handed over at once (the tensor pipe waits for it); then S of the lane's next
+                    // tile is fetched, if it has arrived (sr is free now).
+                    tmem_wait_st();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(bar_pfull(x, buf)));
+                    ++jx;
+                    first = false;
+                    s_loaded = t + kLanes < it.t_end &&
+                               __all_sync(kFull, mbar_test(bar(bar_sfull(x, buf ^ 1u)), (jx >> 1) & 1u));
+                    if (s_loaded) load_s(buf ^ 1u);
                 }
                 if (!alive) break;
-                tc_fence_before();
-                mbar_arrive(bar(bar_pfull(x, buf)));
-                ++jx;
-                first = false;
-            }
-            if (!alive) break;
+                kt_run += static_cast<uint32_t>(n_tiles);
 
-            // ---- epilogue --------------------------------------------------------------
-            // Row mode: the lane owns its rows and all their columns.  Key mode: the two lanes hold
-            // partial results over different keys for the same rows; they exchange (max, sum) through
-            // shared memory and each merges one half of the columns, reading the other lane's
-            // accumulator straight from tensor memory (same TMEM lanes, other columns).
-            const bool direct = it.splits == 1;  // the group's only item: the result is final
-            const int nt_oth = row_mode ? 0 : ((it.t_end - it.t_begin + (x ? 1 : 0)) >> 1);  // the other lane's tiles
-            while (pv_seen < jx) {
-                if (!warp_wait(bar(bar_pvdone(x)), pv_seen & 1u, abort_flag)) alive = false;
-                ++pv_seen;
-            }
-            if (!alive) break;
-            const bool use_self = !first, use_oth = nt_oth > 0;
-            float m_tot = (l_run > 0.f) ? m_ref : -INFINITY, l_tot = l_run, w_self = 1.f, w_oth = 0.f;
-            int c_begin = 0, c_end = D / 32;  // 32-column pieces of the row this thread writes
-            if (!row_mode) {
+                // ---- end of the CTA's share.  The two lanes hold partial results over different keys for the
+                // same rows; they exchange (max, sum) through shared memory and each merges one half of
+                // the columns, reading the other lane's accumulator straight from tensor memory.
+                const bool use_self = !first, use_oth = x == 1 || n_tiles > 1;
+                if (use_self) alive = warp_wait(bar(bar_pvdone(x, (jx - 1u) & 1u)), ((jx - 1u) >> 1) & 1u, abort_flag);
+                if (!alive) break;
+                const float m_self = (l_run > 0.f) ? m_ref : -INFINITY;
                 float2* xch = reinterpret_cast<float2*>(base_ptr + S::kOffMerge);
-                xch[x * kBM + r] = make_float2(m_tot, l_run);
+                xch[x * kBM + r] = make_float2(m_self, l_run);
                 tc_fence_before();
                 mbar_arrive(bar(bar_merge()));
-                alive = warp_wait(bar(bar_merge()), merges_run & 1u, abort_flag);
-                ++merges_run;
+                alive = warp_wait(bar(bar_merge()), merges & 1u, abort_flag);
+                ++merges;
                 if (!alive) break;
+                tc_fence_after();
                 const float2 oth = xch[(x ^ 1) * kBM + r];
-                const float m_self = m_tot;
-                m_tot = fmaxf(m_self, oth.x);
-                w_self = (m_self == -INFINITY) ? 0.f : ex2_approx(m_self - m_tot);
-                w_oth = (oth.x == -INFINITY) ? 0.f : ex2_approx(oth.x - m_tot);
-                l_tot = l_run * w_self + oth.y * w_oth;
-                c_begin = x * (D / 64), c_end = c_begin + D / 64;
-            }
-            tc_fence_after();
-            {
-                const int t = R / G, h = it.g * G + R % G;
+                const float m_tot = fmaxf(m_self, oth.x);
+                const float w_self = (m_self == -INFINITY) ? 0.f : ex2_approx(m_self - m_tot);
+                const float w_oth = (oth.x == -INFINITY) ? 0.f : ex2_approx(oth.x - m_tot);
+                const float l_tot = l_run * w_self + oth.y * w_oth;
                 const float inv = (l_tot > 0.f) ? 1.f / l_tot : 0.f;
-                __nv_bfloat16* dst = a.o + ((static_cast<int64_t>(it.b) * a.max_tt + t) * a.Hq + h) * D;
-                const int64_t slot = static_cast<int64_t>(item) * kRowTiles + (row_mode ? x : 0);
-                uint4* po = a.part_o + slot * (D / 8) * kBM + r;
-                const uint32_t oth_t = tmem + lane_sel + (x ^ 1) * 256 + 128;
-                if (row_ok && direct && a.lse && (row_mode || x == 0))
-                    a.lse[(static_cast<int64_t>(it.b) * a.max_tt + t) * a.Hq + h] =
-                        (m_tot + log2f(l_tot)) * 0.6931471805599453f;
-                // The row leaves tensor memory in 32-column pieces (plain loops: the stores, not
-                // the loads, bound this part, and it runs once per item, so small code wins).
-                // Partials assume a scale of 1 and keep the largest magnitude; when a row of the
-                // warp would leave the fp16 range, a second pass writes such rows again with
-                // their scale (a scale per half of the columns: the halves may come from
-                // different lanes).
-                float am[4] = {0.f, 0.f, 0.f, 0.f};
-                float scale = 1.f;  // O = Ohat * l * scale
-                uint32_t r0[32], r1[32];
+                const int tok = R / G, h = it.g * G + R % G;
+                const int64_t out_row = (static_cast<int64_t>(it.b) * a.max_tt + tok) * a.Hq + h;
+                const int64_t place = a.cluster > 1 ? static_cast<int>(blockIdx.x) : first_item + i;
+                __nv_bfloat16* dst = a.o + out_row * D;
+                uint4* po = a.part_o + place * (D / 8) * kBM + r;
+                // (a lane without tiles has nothing in tensor memory: the other's is read in its place, with weight 0)
+                const uint32_t both_t = tmem + lane_sel + 128;
+                const uint32_t self_t = both_t + (use_self ? x : x ^ 1) * 256, oth_t = both_t + (use_oth ? x ^ 1 : x) * 256;
+                if (row_ok && direct && a.lse && x == 0)
+                    a.lse[out_row] = (m_tot + log2f(l_tot)) * 0.6931471805599453f;
+                // The half row leaves tensor memory in 16-column pieces, in a loop of few instructions: it runs
+                // once per item, and unrolled over the row its 14 KB of code took 3600 cycles to fetch.
+                // Partials assume a scale of 1 and keep the largest magnitude; when a row of the warp would
+                // leave the fp16 range, a second pass writes such rows again with their scale (a scale per
+                // half of the columns: the halves come from different lanes).
+                float amax = 0.f, scale = 1.f;  // O = Ohat * l * scale
 #pragma unroll 1
                 for (int pass = 0; pass < 2; ++pass) {
                     const float mul = (pass == 0) ? inv : inv / scale;
+                    const unsigned long long ws2 = pack2(w_self * mul, w_self * mul), wo2 = pack2(w_oth * mul, w_oth * mul);
                     const bool store = row_ok && (pass == 0 || scale != 1.f);
-                    // Two loads from tensor memory are in flight together: in key mode a piece of this
-                    // lane's O and the same piece of the other lane's, in row mode two pieces of its own.
-                    // (The loads are warp-wide and their conditions warp-uniform.)
-                    const int c_step = row_mode ? 2 : 1;
 #pragma unroll 1
-                    for (int c0 = c_begin; c0 < c_end; c0 += c_step) {
-                        const bool second = row_mode && c0 + 1 < c_end;
-                        if (use_self) tmem_ld32(o_t + c0 * 32, r0);
-                        if (use_oth) tmem_ld32(oth_t + c0 * 32, r1);
-                        if (second) tmem_ld32(o_t + (c0 + 1) * 32, r1);
+                    for (int c = x * (D / 2); c < (x + 1) * (D / 2); c += 16) {
+                        uint32_t r0[16], r1[16];
+                        tmem_ld16(self_t + c, r0);
+                        tmem_ld16(oth_t + c, r1);
                         tmem_wait_ld();
+                        float g[16];
 #pragma unroll
-                        for (int h2 = 0; h2 < 2; ++h2) {
-                            if (h2 == 1 && !second) break;
-                            const int c = c0 + h2;
-                            if (store) {
+                        for (int e = 0; e < 16; e += 2) {
+                            const unsigned long long s2 = pack2(__uint_as_float(r0[e]), __uint_as_float(r0[e + 1]));
+                            const unsigned long long o2 = pack2(__uint_as_float(r1[e]), __uint_as_float(r1[e + 1]));
+                            unpack2(fma2(o2, wo2, fma2(s2, ws2, pack2(0.f, 0.f))), g[e], g[e + 1]);
+                            amax = max3(amax, fabsf(g[e]), fabsf(g[e + 1]));
+                        }
+                        uint32_t v[8];
+                        if (direct) {
 #pragma unroll
-                                for (int q4 = 0; q4 < 4; ++q4) {
-                                    float g8[8];
+                            for (int e = 0; e < 8; ++e) v[e] = pack_bf16(g[2 * e], g[2 * e + 1]);
+                        } else {
 #pragma unroll
-                                    for (int e = 0; e < 8; ++e) {
-                                        float v;
-                                        if (h2 == 1) {
-                                            v = __uint_as_float(r1[q4 * 8 + e]);
-                                        } else {
-                                            v = use_self ? __uint_as_float(r0[q4 * 8 + e]) * w_self : 0.f;
-                                            if (use_oth) v = fmaf(__uint_as_float(r1[q4 * 8 + e]), w_oth, v);
-                                        }
-                                        g8[e] = v;
-                                    }
-                                    uint4 v;
-                                    if (direct) {
-                                        v.x = pack_bf16(g8[0] * mul, g8[1] * mul), v.y = pack_bf16(g8[2] * mul, g8[3] * mul);
-                                        v.z = pack_bf16(g8[4] * mul, g8[5] * mul), v.w = pack_bf16(g8[6] * mul, g8[7] * mul);
-                                        *reinterpret_cast<uint4*>(dst + (c * 4 + q4) * 8) = v;
-                                    } else {
-                                        am[q4] = max3(am[q4], fabsf(g8[0]), fabsf(g8[1]));
-                                        am[q4] = max3(am[q4], fabsf(g8[2]), fabsf(g8[3]));
-                                        am[q4] = max3(am[q4], fabsf(g8[4]), fabsf(g8[5]));
-                                        am[q4] = max3(am[q4], fabsf(g8[6]), fabsf(g8[7]));
-                                        v.x = pack_half2(g8[0] * mul, g8[1] * mul), v.y = pack_half2(g8[2] * mul, g8[3] * mul);
-                                        v.z = pack_half2(g8[4] * mul, g8[5] * mul), v.w = pack_half2(g8[6] * mul, g8[7] * mul);
-                                        __stcg(po + (c * 4 + q4) * kBM, v);
-                                    }
-                                }
-                            }
+                            for (int e = 0; e < 8; ++e) v[e] = pack_half2(g[2 * e], g[2 * e + 1]);
+                        }
+                        uint4* to = direct ? reinterpret_cast<uint4*>(dst + c) : po + (c / 8) * kBM;
+                        if (store) {
+                            __stcg(to, make_uint4(v[0], v[1], v[2], v[3]));
+                            __stcg(to + (direct ? 1 : kBM), make_uint4(v[4], v[5], v[6], v[7]));
                         }
                     }
                     if (direct || pass == 1) break;
                     // scale: 1 unless |O / l| would exceed 2^14 (fp16 holds up to 65504)
-                    if (row_ok) {
-                        const float nmax = fmaxf(fmaxf(am[0], am[1]), fmaxf(am[2], am[3])) * inv;
-                        if (nmax > 16384.f) scale = exp2f(ceilf(log2f(nmax)) - 14.f);
-                    }
+                    if (row_ok && amax > 16384.f) scale = exp2f(ceilf(log2f(amax)) - 14.f);
                     // (the loads from tensor memory are warp-wide: the whole warp goes round again)
                     if (!__any_sync(kFull, scale != 1.f)) break;
                 }
+                // O and S have been read: the next item's MMAs may overwrite them
+                tc_fence_before();
+                mbar_arrive(bar(bar_item()));
                 if (row_ok && !direct) {
-                    float* ml = reinterpret_cast<float*>(a.part_ml + slot * kBM + r);
-                    if (row_mode) {
-                        __stcg(a.part_ml + slot * kBM + r, make_float4(m_tot, l_tot, l_tot * scale, l_tot * scale));
-                    } else if (x == 0) {
+                    float* ml = reinterpret_cast<float*>(a.part_ml + place * kBM + r);
+                    if (x == 0) {
                         __stcg(reinterpret_cast<float2*>(ml), make_float2(m_tot, l_tot));
                         __stcg(ml + 2, l_tot * scale);
                     } else {
@@ -1197,9 +1287,22 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                     }
                 }
             }
-            tc_fence_before();
-            mbar_arrive(bar(bar_item()));
-            alive = warp_wait(bar(bar_item()), items_run & 1u, abort_flag);
+
+            if (a.cluster > 1 && !direct) {
+                // ---- every CTA of the cluster says that its partial is written (a warp at a time), and merges
+                // a share of all of them ------------------------------------------------------------------
+                __syncwarp();
+                if (lane < a.cluster) mbar_arrive_remote(bar(bar_meet()), lane);
+                alive = __all_sync(kFull, cluster_bar_wait(bar(bar_meet()), meets & 1u, abort_flag));
+                ++meets;
+                if (!alive) break;
+                merge_partials<D>(a, it, static_cast<unsigned>(cluster_id * a.cluster), it.active, rank, tid, G);
+            }
+            if (n_tiles > 0) {
+                // (long complete: only keeps a thread from running an item ahead of the others)
+                alive = warp_wait(bar(bar_item()), items_run & 1u, abort_flag);
+                ++items_run;
+            }
         }
     }
 
@@ -1216,34 +1319,24 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
     }
-}
-
-// The per-sequence part of the work list, from the workspace into shared memory (the list is at
-// least two kernels old when a combine kernel starts: see the note at the attention kernel).
-__device__ __forceinline__ void load_sched(const AttnArgs& a, Sched& sc, int tid, int nthreads) {
-    for (int b = tid; b <= a.batch; b += nthreads) {
-        const int4* src = reinterpret_cast<const int4*>(a.plan_seq + b);
-        const int4 lo = __ldcg(src), hi = __ldcg(src + 1);
-        sc.item0[b] = hi.w;
-        if (b < a.batch)
-            sc.n[b] = lo.x, sc.L[b] = lo.y, sc.mp[b] = lo.z, sc.nfull[b] = lo.w, sc.kt[b] = hi.x, sc.s_row[b] = hi.y,
-            sc.s_key[b] = hi.z;
+    // A CTA that has met the others has received their last arrival and may leave.  Where a wait has run
+    // out, nobody leaves while another CTA of the cluster may still arrive on its barriers.
+    if (a.cluster > 1 && !alive) {
+        cluster_arrive();
+        cluster_wait();
     }
-    if (tid == 0) sc.group_rows = __ldcg(a.plan_head).y;
-    __syncthreads();
 }
 
-// Combines the partials of every (sequence, KV head, group of row tiles) that did not write O
-// directly: O = sum_p w_p O_p / sum_p w_p l_p with w_p = 2^(m_p - max m).  A group has one partial
-// per split and row tile (in key mode the two lanes of a CTA have merged theirs already).
+// Combines the partials of every group that is cut into several items (modes even and stream):
+// O = sum_p w_p O_p / sum_p w_p l_p with w_p = 2^(m_p - max m).
 //
 // The kernel is two dependent round trips to L2 (partials in, O out) behind a dependency wait, so
 // what counts is how many memory requests an SM has to issue: with plain loads a warp-load is four
-// 128-byte requests, an SM can only keep so many in flight, and 100 requests per warp made the
-// kernel several round trips long.  Here a CTA takes one row tile x two 8-column pieces and lets
-// the copy engine fetch its share of every partial (one bulk copy per partial and column piece,
-// one for the (max, sum, scales) of the rows) into shared memory: a few dozen requests per CTA, all
-// in flight at once.
+// 128-byte requests and an SM can only keep so many in flight.  Here a CTA takes one group x two 8-column
+// pieces and lets the copy engine fetch its share of every partial (one bulk copy per partial and column
+// piece, one for the (max, sum, scales) of the rows) into shared memory: a few dozen requests per CTA, all
+// in flight at once.  What a CTA has to do is one entry of the work list, fetched before the wait.
+constexpr int kCombineThreads = 256;
 constexpr int kCombChunk = 8;   // partials fetched together
 constexpr int kCombPieces = 2;  // 8-column pieces per CTA
 constexpr int kCombSlotBytes = (kCombPieces + 1) * kBM * 16;  // per partial: the pieces, then (max, sum, scales)
@@ -1251,429 +1344,107 @@ constexpr int kCombSlotBytes = (kCombPieces + 1) * kBM * 16;  // per partial: th
 template <int D>
 __global__ void __launch_bounds__(kCombineThreads) attention_combine_kernel(const AttnArgs a) {
     constexpr int kPieces = D / 8;                    // 16-byte pieces of a row
-    constexpr int kCtasPerTile = kPieces / kCombPieces;
+    constexpr int kShares = kPieces / kCombPieces;    // units of work per group
     static_assert(kCombineThreads == kCombPieces * kBM, "thread = (row, piece)");
     extern __shared__ __align__(128) unsigned char comb_smem[];  // [kCombChunk][kCombSlotBytes]
-    __shared__ Sched sc;
     __shared__ __align__(8) unsigned long long s_bar;
     pdl_launch_dependents();
-    // The work list is fetched and the CTA's share located before the wait for the attention
-    // kernel: all of this runs while that kernel drains.  A CTA without work leaves at once.
-    load_sched(a, sc, threadIdx.x, kCombineThreads);  // ends with __syncthreads()
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, r = tid % kBM, cc = tid / kBM;
     const int G = a.Hq / a.Hkv;
-    const int group_rows = sc.group_rows;
-    int blk = blockIdx.x, b = 0, tiles = 0;
-    for (; b < a.batch; ++b) {
-        tiles = ceil_div(sc.n[b] * G, kBM);
-        if (blk < a.Hkv * tiles * kCtasPerTile) break;
-        blk -= a.Hkv * tiles * kCtasPerTile;
-    }
-    if (b == a.batch) return;
-    const int M = sc.n[b] * G;
-    const int g = blk / (tiles * kCtasPerTile);
-    const int tile = (blk - g * tiles * kCtasPerTile) / kCtasPerTile;
-    const int c8_0 = (blk % kCtasPerTile) * kCombPieces;
-    const int R0 = tile * kBM;
-    const int nfull = sc.nfull[b], s_row = sc.s_row[b], s_key = sc.s_key[b];
-    const int pair = R0 / group_rows;
-    const bool key_mode = pair >= nfull;
-    const int splits = key_mode ? s_key : s_row;
-    if (splits <= 1) return;  // the group wrote O directly
-    const int row_items = nfull * s_row;
-    const int64_t item_first = sc.item0[b] + static_cast<int64_t>(g) * (row_items + (sc.mp[b] - nfull) * s_key) +
-                               (key_mode ? row_items + (pair - nfull) * s_key : pair * s_row);
-    const int mt = (R0 % group_rows) / kBM;  // row tile inside the group (a key-mode group is one tile)
-    const int nv = min(kBM, M - R0);         // valid rows of the tile
     const uint32_t bar = smem_u32(&s_bar);
+    // (the list is at least two kernels old when this kernel starts: see the note at the attention kernel)
+    const int units = __ldcg(&a.plan_head->n_groups) * kShares;
+    auto entry = [&](int unit, int4& lo, int& pieces) {
+        const int* p = reinterpret_cast<const int*>(a.plan_group + static_cast<unsigned>(unit) / kShares);
+        lo = __ldcg(reinterpret_cast<const int4*>(p)), pieces = __ldcg(p + 4);
+    };
+    if (static_cast<int>(blockIdx.x) >= units) return;
+    int4 lo;
+    int pieces;
+    entry(blockIdx.x, lo, pieces);
     if (tid == 0) {
         mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    const int r = tid % kBM, cc = tid / kBM;
     pdl_wait();  // the attention kernel has finished and its partials are visible
-
-    float Mx = -INFINITY, den = 0.f;
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    bool ok = true;
     uint32_t phase = 0;
 #pragma unroll 1
-    for (int p0 = 0; p0 < splits; p0 += kCombChunk, phase ^= 1u) {
-        const int np = min(kCombChunk, splits - p0);
-        // one copy per thread, so that they are issued side by side: a partial's column pieces and
-        // its (max, sum, scales), each nv x 16 contiguous bytes
-        if (tid == 0) mbar_expect_tx(bar, static_cast<uint32_t>(np * (kCombPieces + 1) * nv * 16));
-        if (tid < np * (kCombPieces + 1)) {
-            const int u = tid / (kCombPieces + 1), c = tid % (kCombPieces + 1);
-            const int64_t slot = (item_first + p0 + u) * kRowTiles + mt;
-            const uint32_t dst = smem_u32(comb_smem + u * kCombSlotBytes + c * kBM * 16);
-            const void* src = (c < kCombPieces) ? static_cast<const void*>(a.part_o + (slot * kPieces + c8_0 + c) * kBM)
-                                                : static_cast<const void*>(a.part_ml + slot * kBM);
-            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                         "l"(src), "r"(nv * 16), "r"(bar)
-                         : "memory");
-        }
-        {
+    for (int unit = blockIdx.x; unit < units; unit += gridDim.x) {
+        if (unit != static_cast<int>(blockIdx.x)) entry(unit, lo, pieces);
+        if (pieces <= 1) continue;  // the group wrote O directly
+        const int b = lo.x & 0xFFFF, g = static_cast<int>(static_cast<unsigned>(lo.x) >> 16);
+        const int R0 = lo.y * kBM, nv = min(kBM, lo.z * G - R0);  // valid rows
+        const int c8_0 = static_cast<int>(static_cast<unsigned>(unit) % kShares) * kCombPieces;
+        float Mx = -INFINITY, den = 0.f;
+        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+        for (int p0 = 0; p0 < pieces; p0 += kCombChunk) {
+            const int np = min(kCombChunk, pieces - p0);
+            // one copy per thread, so that they are issued side by side: a partial's column pieces and
+            // its (max, sum, scales), each nv x 16 contiguous bytes
+            if (tid == 0) mbar_expect_tx(bar, static_cast<uint32_t>(np * (kCombPieces + 1) * nv * 16));
+            if (tid < np * (kCombPieces + 1)) {
+                const int u = tid / (kCombPieces + 1), c = tid % (kCombPieces + 1);
+                const int64_t place = lo.w + p0 + u;
+                const uint32_t dst = smem_u32(comb_smem + u * kCombSlotBytes + c * kBM * 16);
+                const void* src = (c < kCombPieces) ? static_cast<const void*>(a.part_o + (place * kPieces + c8_0 + c) * kBM)
+                                                    : static_cast<const void*>(a.part_ml + place * kBM);
+                asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                             "l"(src), "r"(nv * 16), "r"(bar)
+                             : "memory");
+            }
             // bounded: on expiry the status word is flagged and the CTA leaves without a result
+            bool ok = mbar_try(bar, phase);
             const uint32_t t0 = static_cast<uint32_t>(clock());
-            uint32_t spins = 0;
-            while (ok && !mbar_try(bar, phase))
-                if ((++spins & 255u) == 0u && static_cast<uint32_t>(clock()) - t0 > kWaitLimitCycles) ok = false;
-        }
-        if (!__syncthreads_and(ok)) {
-            if (tid == 0) atomicOr(a.status, RESPS_STATUS_WAIT_TIMEOUT);
-            return;
+#pragma unroll 1
+            while (!ok && static_cast<uint32_t>(clock()) - t0 <= kWaitLimitCycles) ok = mbar_try(bar, phase);
+            phase ^= 1u;
+            if (!__syncthreads_and(ok)) {
+                if (tid == 0) atomicOr(a.status, RESPS_STATUS_WAIT_TIMEOUT);
+                return;
+            }
+            if (r < nv) {
+                float mx = Mx;
+#pragma unroll 1
+                for (int u = 0; u < np; ++u)
+                    mx = fmaxf(mx, reinterpret_cast<const float4*>(comb_smem + u * kCombSlotBytes + kCombPieces * kBM * 16)[r].x);
+                if (mx != -INFINITY) {
+                    const float corr = ex2_approx(Mx - mx);  // 0 on the first chunk
+                    den *= corr;
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) acc[e] *= corr;
+                    Mx = mx;
+#pragma unroll 1
+                    for (int u = 0; u < np; ++u) {
+                        const unsigned char* sl = comb_smem + u * kCombSlotBytes;
+                        const float4 ml = reinterpret_cast<const float4*>(sl + kCombPieces * kBM * 16)[r];
+                        const float w = ex2_approx(ml.x - Mx);  // 0 for an empty partial, which stores zeros
+                        den += ml.y * w;
+                        const float wo = (c8_0 + cc < kPieces / 2 ? ml.z : ml.w) * w;  // O_p = Ohat * l * scale of this half
+                        const uint4 v = reinterpret_cast<const uint4*>(sl + cc * kBM * 16)[r];
+                        const uint32_t hw[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hw[e]));
+                            acc[2 * e] += f.x * wo, acc[2 * e + 1] += f.y * wo;
+                        }
+                    }
+                }
+            }
+            __syncthreads();  // the next copies overwrite the staging area
         }
         if (r < nv) {
-            float mx = Mx;
-            for (int u = 0; u < np; ++u)
-                mx = fmaxf(mx, reinterpret_cast<const float4*>(comb_smem + u * kCombSlotBytes + kCombPieces * kBM * 16)[r].x);
-            if (mx != -INFINITY) {
-                const float corr = ex2_approx(Mx - mx);  // 0 on the first chunk
-                den *= corr;
-#pragma unroll
-                for (int e = 0; e < 8; ++e) acc[e] *= corr;
-                Mx = mx;
-#pragma unroll 2
-                for (int u = 0; u < np; ++u) {
-                    const unsigned char* sl = comb_smem + u * kCombSlotBytes;
-                    const float4 ml = reinterpret_cast<const float4*>(sl + kCombPieces * kBM * 16)[r];
-                    if (ml.x == -INFINITY) continue;  // an empty partial holds no O
-                    const float w = ex2_approx(ml.x - Mx);
-                    den += ml.y * w;
-                    const float wo = (c8_0 + cc < kPieces / 2 ? ml.z : ml.w) * w;  // O_p = Ohat * l * scale of this half
-                    const uint4 v = reinterpret_cast<const uint4*>(sl + cc * kBM * 16)[r];
-                    const uint32_t hw[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hw[e]));
-                        acc[2 * e] += f.x * wo, acc[2 * e + 1] += f.y * wo;
-                    }
-                }
-            }
-        }
-        if (p0 + kCombChunk < splits) __syncthreads();  // the next chunk overwrites the staging area
-    }
-    if (r >= nv) return;
-    const float inv = 1.f / den;
-    const int R = R0 + r;
-    const int t = R / G, h = g * G + (R - t * G);
-    __nv_bfloat16* dst = a.o + ((static_cast<int64_t>(b) * a.max_tt + t) * a.Hq + h) * D + (c8_0 + cc) * 8;
-    uint4 out;
-    out.x = pack_bf16(acc[0] * inv, acc[1] * inv);
-    out.y = pack_bf16(acc[2] * inv, acc[3] * inv);
-    out.z = pack_bf16(acc[4] * inv, acc[5] * inv);
-    out.w = pack_bf16(acc[6] * inv, acc[7] * inv);
-    *reinterpret_cast<uint4*>(dst) = out;
-    if (a.lse && c8_0 + cc == 0)
-        a.lse[(static_cast<int64_t>(b) * a.max_tt + t) * a.Hq + h] = (Mx + log2f(den)) * 0.6931471805599453f;
-}
-
-// The same with plain loads, one thread per (row, 8 columns) over a flat index space: its first
-// data arrives sooner than through the copy engine, which wins when there is little to combine (a
-// single sequence with at most two row tiles per KV head: 12.0 against 13.3 us per call on the
-// 8B-shaped workload); with more rows the copy-engine form is ahead (26.4 against 28.1 us on the
-// 70B-shaped one).
-template <int D>
-__global__ void __launch_bounds__(kCombineThreads) attention_combine_small_kernel(const AttnArgs a) {
-    __shared__ Sched sc;
-    pdl_launch_dependents();
-    // The work list is fetched, and the thread's first piece of work located, before the wait
-    // for the attention kernel: all of this runs while that kernel drains, in one round trip to
-    // memory (the list carries the tree sizes it was planned for, which the attention kernel has
-    // checked against the live ones).
-    load_sched(a, sc, threadIdx.x, kCombineThreads);  // ends with __syncthreads()
-    // A CTA past the last row of the largest tree has nothing to do and leaves: it may have started
-    // only after the attention kernel ended, and whatever it does until it exits delays the next
-    // kernel in the stream.
-    {
-        bool mine = false;
-        for (int b = 0; b < a.batch; ++b)
-            mine = mine || static_cast<long long>(blockIdx.x) * kCombineThreads < 1ll * sc.n[b] * a.Hq * (D / 8);
-        if (!mine) return;
-    }
-    const unsigned G = static_cast<unsigned>(a.Hq / a.Hkv);
-    const unsigned stride = gridDim.x * kCombineThreads;
-    const unsigned group_rows = static_cast<unsigned>(sc.group_rows);
-    // Work: (sequence, KV head, 8 columns, row) over the valid rows of groups that wrote partials;
-    // consecutive threads take consecutive rows.  Every count fits 32 bits (at most 2^11 rows per
-    // KV head, 2^4 column pieces, 2^7 heads).
-    int b = 0;
-    unsigned idx = blockIdx.x * kCombineThreads + threadIdx.x;
-    bool waited = false;
-    for (;;) {
-        // ---- the next piece of work of this thread ------------------------------------------
-        bool have = false;
-        unsigned g = 0, c8 = 0, R = 0, M = 0;
-        int splits = 0, n_parts = 0;
-        bool key_mode = false;
-        int64_t item_first = 0;
-        for (; b < a.batch; ++b, idx = blockIdx.x * kCombineThreads + threadIdx.x) {
-            const int nfull = sc.nfull[b], mp_b = sc.mp[b], s_row = sc.s_row[b], s_key_b = sc.s_key[b];
-            if (sc.n[b] == 0 || ((s_row <= 1 || nfull == 0) && (s_key_b <= 1 || nfull == mp_b)))
-                continue;  // every group wrote O directly
-            M = static_cast<unsigned>(sc.n[b]) * G;
-            const unsigned per_head = M * (D / 8);
-            for (; idx < a.Hkv * per_head; idx += stride) {
-                g = idx / per_head;
-                const unsigned rem = idx - g * per_head;
-                c8 = rem / M;
-                R = rem - c8 * M;
-                const int pair = static_cast<int>(R / group_rows);
-                key_mode = pair >= nfull;
-                splits = key_mode ? s_key_b : s_row;
-                if (splits <= 1) continue;
-                const int row_items = nfull * s_row;
-                item_first = sc.item0[b] + static_cast<int64_t>(g) * (row_items + (mp_b - nfull) * s_key_b) +
-                             (key_mode ? row_items + (pair - nfull) * s_key_b : pair * s_row);
-                n_parts = splits;
-                have = true;
-                break;
-            }
-            if (have) break;
-        }
-        if (!waited) {
-            pdl_wait();  // the attention kernel has finished and its partials are visible
-            waited = true;
-        }
-        if (!have) break;
-
-        // ---- O = sum_p w_p O_p / sum_p w_p l_p, w_p = 2^(m_p - max m): one pass over the partials,
-        // ten at a time so that their loads are in flight together ---------------------------------
-        const unsigned row2 = R % group_rows;
-        const unsigned mt = row2 / kBM, r = row2 % kBM;  // (a key-mode group is one row tile: mt = 0)
-        constexpr int kBatch = 10;
-        float Mx = -INFINITY, den = 0.f;
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 1
-        for (int p0 = 0; p0 < n_parts; p0 += kBatch) {
-            float4 ml[kBatch];
-            uint4 v[kBatch];
-#pragma unroll
-            for (int u = 0; u < kBatch; ++u) {
-                const int p = min(p0 + u, n_parts - 1);
-                const int64_t slot = (item_first + p) * kRowTiles + mt;
-                ml[u] = a.part_ml[slot * kBM + r];  // shared by the 16 column pieces of a row: through L1
-                v[u] = __ldcg(a.part_o + (slot * (D / 8) + c8) * kBM + r);
-            }
-            float mx = Mx;
-#pragma unroll
-            for (int u = 0; u < kBatch; ++u)
-                if (p0 + u < n_parts) mx = fmaxf(mx, ml[u].x);
-            if (mx == -INFINITY) continue;
-            const float corr = ex2_approx(Mx - mx);  // 0 on the first batch
-            den *= corr;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] *= corr;
-            Mx = mx;
-#pragma unroll
-            for (int u = 0; u < kBatch; ++u) {
-                if (p0 + u >= n_parts || ml[u].x == -INFINITY) continue;  // an empty partial holds no O
-                const float w = ex2_approx(ml[u].x - Mx);
-                den += ml[u].y * w;
-                const float wo = (c8 < D / 16 ? ml[u].z : ml[u].w) * w;  // O_p = Ohat * l * scale of this half of the row
-                const uint32_t hw[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hw[e]));
-                    acc[2 * e] += f.x * wo, acc[2 * e + 1] += f.y * wo;
-                }
-            }
-        }
-        const float inv = 1.f / den;
-        const unsigned t = R / G, h = g * G + (R - t * G);
-        __nv_bfloat16* dst = a.o + ((static_cast<int64_t>(b) * a.max_tt + t) * a.Hq + h) * D + c8 * 8;
-        uint4 out;
-        out.x = pack_bf16(acc[0] * inv, acc[1] * inv);
-        out.y = pack_bf16(acc[2] * inv, acc[3] * inv);
-        out.z = pack_bf16(acc[4] * inv, acc[5] * inv);
-        out.w = pack_bf16(acc[6] * inv, acc[7] * inv);
-        *reinterpret_cast<uint4*>(dst) = out;
-        if (a.lse && c8 == 0)
-            a.lse[(static_cast<int64_t>(b) * a.max_tt + t) * a.Hq + h] = (Mx + log2f(den)) * 0.6931471805599453f;
-        idx += stride;
-    }
-}
-
-// The same for batches of several sequences.  The kernel is a chain of two dependent memory round
-// trips (partials in, O out) behind a
-// dependency wait, so it is laid out for latency: one flat index space over all sequences (no
-// pass per sequence), a piece of work = (row, 8 columns, one of 1, 2 or 4 shares of the partials)
-// so that a thread has at most four partials (eight loads) to fetch and they are all in flight
-// at once, the shares merged by shuffles, and few enough registers for four CTAs per SM, so
-// that even the largest trees are one resident round.
-constexpr int kCombineBatch = 4;  // partials a thread fetches at once
-
-template <int D>
-__global__ void __launch_bounds__(kCombineThreads, 4) attention_combine_flat_kernel(const AttnArgs a) {
-    __shared__ Sched sc;
-    __shared__ unsigned s_work0[kMaxBatchSmem + 1];  // first flat index of a sequence
-    __shared__ unsigned char s_shares[kMaxBatchSmem];
-    pdl_launch_dependents();
-    // The work list is fetched, and the thread's first piece of work located, before the wait
-    // for the attention kernel: all of this runs while that kernel drains, in one round trip to
-    // memory (the list carries the tree sizes it was planned for, which the attention kernel has
-    // checked against the live ones).
-    load_sched(a, sc, threadIdx.x, kCombineThreads);  // ends with __syncthreads()
-    // A CTA past the last piece of work that the trees at hand could need (four shares each) has
-    // nothing to do and leaves: it may have started only after the attention kernel ended, and
-    // whatever it does until it exits delays the next kernel in the stream.
-    {
-        unsigned long long bound = 0;
-        for (int b = 0; b < a.batch; ++b) bound += 4ull * sc.n[b] * a.Hq * (D / 8) + 4;
-        if (static_cast<unsigned long long>(blockIdx.x) * kCombineThreads >= bound) return;
-    }
-    const unsigned G = static_cast<unsigned>(a.Hq / a.Hkv);
-    const unsigned group_rows = static_cast<unsigned>(sc.group_rows);
-    if (threadIdx.x < 32) {
-        // shares per piece of work and flat offsets (every sequence's range is a multiple of 4,
-        // so that the shares of a piece sit in adjacent, aligned lanes)
-        unsigned base = 0;
-        for (int b0 = 0; b0 < a.batch; b0 += 32) {
-            const int b = b0 + threadIdx.x;
-            unsigned mine = 0;
-            if (b < a.batch && sc.n[b] > 0) {
-                const int nfull = sc.nfull[b], nkey = sc.mp[b] - nfull;
-                const int parts = max(nfull > 0 && sc.s_row[b] > 1 ? sc.s_row[b] : 0, nkey > 0 && sc.s_key[b] > 1 ? sc.s_key[b] : 0);
-                const unsigned shares = parts <= kCombineBatch ? 1u : parts <= 2 * kCombineBatch ? 2u : 4u;
-                s_shares[b] = static_cast<unsigned char>(shares);
-                if (parts > 0) mine = (static_cast<unsigned>(sc.n[b]) * a.Hq * (D / 8) * shares + 3u) & ~3u;
-            }
-            unsigned incl = mine;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const unsigned v = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-                if (threadIdx.x >= d) incl += v;
-            }
-            if (b < a.batch) s_work0[b] = base + incl - mine;
-            base += __shfl_sync(0xFFFFFFFFu, incl, 31);
-        }
-        if (threadIdx.x == 0) s_work0[a.batch] = base;
-    }
-    __syncthreads();
-    const unsigned total = s_work0[a.batch];
-    const unsigned stride = gridDim.x * kCombineThreads;
-    bool waited = false;
-    // every lane of a warp goes round the same number of times (the merge is by shuffles)
-    for (unsigned w0 = blockIdx.x * kCombineThreads + (threadIdx.x & ~31u); w0 < total || !waited; w0 += stride) {
-        const unsigned w = w0 + (threadIdx.x & 31u);
-        // ---- this thread's piece of work ------------------------------------------------------
-        bool have = false;
-        int b = 0, n_parts = 0, splits = 0;
-        unsigned g = 0, c8 = 0, R = 0, share = 0, shares = 1;
-        bool key_mode = false;
-        int64_t item_first = 0;
-        if (w < total) {
-            int lo = 0, hi = a.batch;  // last sequence whose range starts at or before w
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (s_work0[mid] <= w) lo = mid; else hi = mid;
-            }
-            b = lo;
-            shares = s_shares[b];
-            const unsigned local = w - s_work0[b];
-            const unsigned piece = local / shares;
-            share = local - piece * shares;
-            const unsigned M = static_cast<unsigned>(sc.n[b]) * G;
-            const unsigned per_head = M * (D / 8);
-            if (piece < a.Hkv * per_head) {  // (the range is padded to a multiple of 4)
-                g = piece / per_head;
-                const unsigned rem = piece - g * per_head;
-                c8 = rem / M;
-                R = rem - c8 * M;
-                const int nfull = sc.nfull[b], s_row = sc.s_row[b], s_key_b = sc.s_key[b];
-                const int pair = static_cast<int>(R / group_rows);
-                key_mode = pair >= nfull;
-                splits = key_mode ? s_key_b : s_row;
-                if (splits > 1) {  // otherwise the group wrote O directly
-                    const int row_items = nfull * s_row;
-                    item_first = sc.item0[b] + static_cast<int64_t>(g) * (row_items + (sc.mp[b] - nfull) * s_key_b) +
-                                 (key_mode ? row_items + (pair - nfull) * s_key_b : pair * s_row);
-                    n_parts = splits;
-                    have = true;
-                }
-            }
-        }
-        if (!waited) {
-            pdl_wait();  // the attention kernel has finished and its partials are visible
-            waited = true;
-        }
-        if (!__any_sync(0xFFFFFFFFu, have)) continue;
-
-        // ---- this share's partials: p = share, share + shares, ... ------------------------------
-        const unsigned row2 = R % group_rows;
-        const unsigned mt = row2 / kBM, r = row2 % kBM;
-        float Mx = -INFINITY, den = 0.f;
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if (have) {
-#pragma unroll 1
-            for (int p0 = static_cast<int>(share); p0 < n_parts; p0 += kCombineBatch * static_cast<int>(shares)) {
-                float4 ml[kCombineBatch];
-                uint4 v[kCombineBatch];
-#pragma unroll
-                for (int u = 0; u < kCombineBatch; ++u) {
-                    const int p = min(p0 + u * static_cast<int>(shares), n_parts - 1);
-                    const int64_t slot = (item_first + p) * kRowTiles + mt;
-                    ml[u] = a.part_ml[slot * kBM + r];  // shared by the 16 column pieces of a row: through L1
-                    v[u] = __ldcg(a.part_o + (slot * (D / 8) + c8) * kBM + r);
-                }
-                float mx = Mx;
-#pragma unroll
-                for (int u = 0; u < kCombineBatch; ++u)
-                    if (p0 + u * static_cast<int>(shares) < n_parts) mx = fmaxf(mx, ml[u].x);
-                if (mx == -INFINITY) continue;
-                const float corr = ex2_approx(Mx - mx);  // 0 on the first batch
-                den *= corr;
-#pragma unroll
-                for (int e = 0; e < 8; ++e) acc[e] *= corr;
-                Mx = mx;
-#pragma unroll
-                for (int u = 0; u < kCombineBatch; ++u) {
-                    if (p0 + u * static_cast<int>(shares) >= n_parts || ml[u].x == -INFINITY) continue;  // an empty partial holds no O
-                    const float wgt = ex2_approx(ml[u].x - Mx);
-                    den += ml[u].y * wgt;
-                    const float wo = (c8 < D / 16 ? ml[u].z : ml[u].w) * wgt;  // O_p = Ohat * l * scale of this half of the row
-                    const uint32_t hw[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hw[e]));
-                        acc[2 * e] += f.x * wo, acc[2 * e + 1] += f.y * wo;
-                    }
-                }
-            }
-        }
-        // ---- the shares of a piece sit in adjacent lanes: merge them (every lane takes part) ----
-#pragma unroll
-        for (unsigned d = 1; d < 4; d <<= 1) {
-            const float Mo = __shfl_xor_sync(0xFFFFFFFFu, Mx, d);
-            const float Mn = fmaxf(Mx, Mo);
-            const float sc_self = (Mx == -INFINITY) ? 0.f : ex2_approx(Mx - Mn);
-            const bool on = d < shares;
-            float dn = den * sc_self;
-            float ac[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) ac[e] = acc[e] * sc_self;
-            const float dno = __shfl_xor_sync(0xFFFFFFFFu, dn, d);
-            if (on) den = dn + dno, Mx = Mn;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float o = __shfl_xor_sync(0xFFFFFFFFu, ac[e], d);
-                if (on) acc[e] = ac[e] + o;
-            }
-        }
-        if (have && share == 0) {
             const float inv = 1.f / den;
-            const unsigned t = R / G, h = g * G + (R - t * G);
-            __nv_bfloat16* dst = a.o + ((static_cast<int64_t>(b) * a.max_tt + t) * a.Hq + h) * D + c8 * 8;
+            const int R = R0 + r, t = R / G, h = g * G + (R - t * G);
+            const int64_t row = (static_cast<int64_t>(b) * a.max_tt + t) * a.Hq + h;
             uint4 out;
             out.x = pack_bf16(acc[0] * inv, acc[1] * inv);
             out.y = pack_bf16(acc[2] * inv, acc[3] * inv);
             out.z = pack_bf16(acc[4] * inv, acc[5] * inv);
             out.w = pack_bf16(acc[6] * inv, acc[7] * inv);
-            *reinterpret_cast<uint4*>(dst) = out;
-            if (a.lse && c8 == 0)
-                a.lse[(static_cast<int64_t>(b) * a.max_tt + t) * a.Hq + h] = (Mx + log2f(den)) * 0.6931471805599453f;
+            *reinterpret_cast<uint4*>(a.o + row * D + (c8_0 + cc) * 8) = out;
+            if (a.lse && c8_0 + cc == 0) a.lse[row] = (Mx + log2f(den)) * 0.6931471805599453f;
         }
     }
 }
@@ -1767,6 +1538,7 @@ struct HostState {
     cudaStream_t plan_stream = nullptr;
     // ... and this many kernels of the library have been enqueued behind the one that wrote it.
     int plan_age = 0;
+    int resident[kMaxCluster + 1] = {};  // clusters of each size that are resident at once
 };
 constexpr size_t kMaxCachedMaps = 4096;
 
@@ -1784,56 +1556,92 @@ const CUtensorMap* cached_map(HostState* hs, const MapKey& key, int D) {
     return &hs->maps.emplace(key, m).first->second;
 }
 
+// CTAs per cluster for mode whole, or 1 for the two-kernel modes.  Mode whole saves the second kernel and the
+// boundary between the two (about 3 us of a call), and pays with CTAs that stay without work: `groups` (of the
+// largest trees) clusters of C CTAs instead of the whole GPU.  With 0.6 us per key tile and CTA that is
+// 0.6 groups kt (1 / (C groups) - 1 / SMs) us for kt key tiles, so it is taken while the longest prefix the
+// cache can hold costs no more than it saves.  Cluster sizes that do not leave SMs of a GPC unused only.
+constexpr double kWholeGainTiles = 5.0;  // 3 us / 0.6 us
+int choose_cluster(const int* resident, int sm_count, int64_t groups, int kt_most) {
+    for (int c : {8, 6, 4, 3, 2}) {
+        if (resident[c] < groups) continue;
+        const double lost = 1.0 / c - static_cast<double>(groups) / sm_count;
+        if (lost * kt_most <= kWholeGainTiles) return c;
+    }
+    return kt_most <= 5 && groups <= resident[1] ? 2 : 1;
+}
+int forced_cluster(const int* resident, int cluster, int groups) {
+    while (cluster > 1 && resident[cluster] < groups) --cluster;
+    return cluster;
+}
+constexpr int kStreamGain = 6;  // key tiles a CTA must be spared before groups are cut at odd places
+
+// Clusters of C CTAs that are resident at once with this kernel's shared memory (index C; the GPCs are not
+// multiples of every size), asked for once per device.
+struct Residency {
+    int clusters[kMaxCluster + 1] = {};
+    bool known = false;
+};
+std::mutex g_residency_mu;
+Residency g_residency[2][64];  // [head dim 64, 128][device]
+
 template <int D>
-cudaError_t launch_for_dim(const resps_ctx* ctx, const AttnArgs& a, const CUtensorMap& mk, const CUtensorMap& mv,
+cudaError_t launch_for_dim(const resps_ctx* ctx, const AttnArgs& a, int grid, const CUtensorMap& mk, const CUtensorMap& mv,
                            const CUtensorMap& mq, cudaStream_t st) {
-    cudaError_t e = launch_pdl(tree_attention_kernel<D>, dim3(ctx->ws.attn_grid), dim3(kAttnThreads), Smem<D>::kBytes, st, a, mk,
-                               mv, mq);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid), cfg.blockDim = dim3(kAttnThreads), cfg.dynamicSmemBytes = Smem<D>::kBytes, cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = static_cast<unsigned>(a.cluster), attr[1].val.clusterDim.y = 1, attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr, cfg.numAttrs = a.cluster > 1 ? 2 : 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, tree_attention_kernel<D>, a, mk, mv, mq);
+    if (e != cudaSuccess || a.cluster > 1) return e;
+    // the units of work of the largest trees, at most one resident round of CTAs
+    const int64_t units = static_cast<int64_t>(a.batch) * a.Hkv * ((a.max_tt * (a.Hq / a.Hkv) + kBM - 1) / kBM) * (D / 8 / kCombPieces);
+    const int combine_grid = static_cast<int>(std::min<int64_t>(units, 4 * ctx->sm_count));
+    return launch_pdl(attention_combine_kernel<D>, dim3(combine_grid), dim3(kCombineThreads), kCombChunk * kCombSlotBytes, st, a);
+}
+
+template <int D>
+cudaError_t setup_for_dim(int device, int sm_count, int* clusters) {
+    cudaError_t e = cudaFuncSetAttribute(tree_attention_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<D>::kBytes);
     if (e != cudaSuccess) return e;
-    // One resident round of CTAs at most, and no more than the largest trees could use.  A single
-    // sequence (or two) is served best by few, register-heavy threads that all start under the
-    // attention kernel's tail; a batch by the flat index space and four CTAs per SM.
-    const long long pieces = 1ll * a.max_tt * a.Hq * (D / 8);
-    if (a.batch > 2) {
-        const long long most = (4ll * a.batch * (pieces + 1) + kCombineThreads - 1) / kCombineThreads;
-        const int grid = static_cast<int>(std::min<long long>(ctx->ws.attn_combine_flat_grid, std::max<long long>(most, 1)));
-        return launch_pdl(attention_combine_flat_kernel<D>, dim3(grid), dim3(kCombineThreads), 0, st, a);
+    e = cudaFuncSetAttribute(attention_combine_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombChunk * kCombSlotBytes);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(g_residency_mu);
+    Residency local;
+    Residency& r = (device >= 0 && device < 64) ? g_residency[D == 128][device] : local;
+    if (!r.known) {
+        r.clusters[1] = std::min(sm_count, kMaxGrid);
+        for (int c = 2; c <= kMaxCluster; ++c) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(static_cast<unsigned>(sm_count / c * c)), cfg.blockDim = dim3(kAttnThreads);
+            cfg.dynamicSmemBytes = Smem<D>::kBytes;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = static_cast<unsigned>(c), attr[0].val.clusterDim.y = 1, attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr, cfg.numAttrs = 1;
+            int n = 0;
+            e = cudaOccupancyMaxActiveClusters(&n, tree_attention_kernel<D>, &cfg);
+            if (e != cudaSuccess) return e;
+            r.clusters[c] = std::min(n, kMaxGrid / c);
+        }
+        r.known = true;
     }
-    const int G = a.Hq / a.Hkv;
-    if (a.max_tt * G <= kRowTiles * kBM) {
-        const long long few = (a.batch * pieces + kCombineThreads - 1) / kCombineThreads;
-        return launch_pdl(attention_combine_small_kernel<D>, dim3(static_cast<unsigned>(std::max<long long>(few, 1))),
-                          dim3(kCombineThreads), 0, st, a);
-    }
-    // one CTA per (row tile, pair of column pieces) of the largest trees (CTAs past the trees at hand leave at once)
-    const long long most = 1ll * a.batch * a.Hkv * ((a.max_tt * G + kBM - 1) / kBM) * (D / 8 / kCombPieces);
-    return launch_pdl(attention_combine_kernel<D>, dim3(static_cast<unsigned>(std::max<long long>(most, 1))),
-                      dim3(kCombineThreads), kCombChunk * kCombSlotBytes, st, a);
+    for (int c = 1; c <= kMaxCluster; ++c) clusters[c] = r.clusters[c];
+    return cudaSuccess;
 }
 
 }  // namespace
 
 cudaError_t attention_setup(resps_ctx* ctx) {
-    ctx->attn_host = new (std::nothrow) HostState();
-    if (!ctx->attn_host) return cudaErrorMemoryAllocation;
-    cudaError_t e = cudaFuncSetAttribute(tree_attention_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         Smem<128>::kBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(tree_attention_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<64>::kBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attention_combine_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kCombChunk * kCombSlotBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attention_combine_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kCombChunk * kCombSlotBytes);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = (ctx->shape.head_dim == 128)
-            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, attention_combine_flat_kernel<128>, kCombineThreads, 0)
-            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, attention_combine_flat_kernel<64>, kCombineThreads, 0);
-    if (e != cudaSuccess) return e;
-    ctx->ws.attn_combine_flat_grid = ctx->sm_count * std::max(per_sm, 1);
-    return cudaSuccess;
+    HostState* hs = new (std::nothrow) HostState();
+    if (!hs) return cudaErrorMemoryAllocation;
+    ctx->attn_host = hs;
+    return ctx->shape.head_dim == 128 ? setup_for_dim<128>(ctx->device, ctx->sm_count, hs->resident)
+                                      : setup_for_dim<64>(ctx->device, ctx->sm_count, hs->resident);
 }
 
 void attention_teardown(resps_ctx* ctx) {
@@ -1857,6 +1665,7 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
                                   const __nv_bfloat16* v_cache, int64_t stride_seq,
                                   int64_t stride_head, int64_t stride_tok, int64_t capacity,
                                   const uint64_t* mask, float scale, cudaStream_t st) {
+    const Workspace& w = ctx->ws;
     AttnArgs a;
     a.steps = d_steps, a.n_nodes = d_n_nodes, a.batch = batch;
     a.q = q, a.o = o, a.lse = lse;
@@ -1864,20 +1673,28 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
     a.mask = mask;
     a.scale_log2 = scale * 1.4426950408889634f;
     a.Hq = ctx->shape.n_q_heads, a.Hkv = ctx->shape.n_kv_heads, a.max_tt = ctx->shape.max_tt;
-    a.part_o = reinterpret_cast<uint4*>(ctx->ws.attn_part_o), a.part_ml = ctx->ws.attn_part_ml;
-    a.max_items = ctx->ws.attn_max_items, a.sched_grid = ctx->ws.attn_grid;
-    a.min_tiles = ctx->ws.attn_min_tiles, a.status = ctx->ws.status;
-    a.single_units = ctx->ws.attn_single;
-    a.rounds = ctx->ws.attn_rounds;
-    a.stagger = ctx->ws.attn_stagger;
-    a.plan_head = reinterpret_cast<int4*>(ctx->ws.attn_plan);
-    a.plan_seq = reinterpret_cast<PlanSeq*>(ctx->ws.attn_plan + 16);
-    a.plan_item = reinterpret_cast<PlanItem*>(ctx->ws.attn_plan + 16 + sizeof(PlanSeq) * (ctx->shape.max_batch + 1));
+    a.part_o = reinterpret_cast<uint4*>(w.attn_part_o), a.part_ml = w.attn_part_ml;
+    a.max_items = w.attn_max_items;
+    a.min_tiles = w.attn_min_tiles, a.status = w.status;
+    unsigned char* plan = w.attn_plan;
+    a.plan_head = reinterpret_cast<PlanHead*>(plan), plan += sizeof(PlanHead);
+    a.plan_cluster = reinterpret_cast<PlanCluster*>(plan), plan += sizeof(PlanCluster) * kMaxGrid;
+    a.plan_first = reinterpret_cast<PlanItem*>(plan), plan += sizeof(PlanItem) * kMaxGrid;
+    a.plan_item = reinterpret_cast<PlanItem*>(plan), plan += sizeof(PlanItem) * w.attn_max_items;
+    a.plan_group = reinterpret_cast<PlanGroup*>(plan);
+    a.test_drop = w.test_drop;
     const int D = ctx->shape.head_dim;
     const int G = a.Hq / a.Hkv;
     a.q_by_tma = (G <= kBM && kBM % G == 0) ? 1 : 0;
     HostState* hs = host_state(ctx);
     std::lock_guard<std::mutex> lock(hs->mu);
+    a.cluster = choose_cluster(hs->resident, ctx->sm_count, static_cast<int64_t>(batch) * a.Hkv * ((a.max_tt * G + kBM - 1) / kBM),
+                               static_cast<int>((capacity + kBN - 1) / kBN));
+    if (w.attn_cluster > 0) a.cluster = forced_cluster(hs->resident, std::min(w.attn_cluster, kMaxCluster), batch * a.Hkv * ((a.max_tt * G + kBM - 1) / kBM));
+    a.clusters = a.cluster > 1 ? batch * a.Hkv * ((a.max_tt * G + kBM - 1) / kBM) : hs->resident[1];
+    const int grid = a.clusters * a.cluster;
+    if (w.attn_rounds > 0 && a.cluster == 1) a.clusters = std::max(1, a.clusters / w.attn_rounds);
+    a.stream_gain = w.attn_stream >= 0 ? w.attn_stream : kStreamGain;
     MapKey kk = {k_cache, stride_tok, stride_head, stride_seq, capacity, a.Hkv, batch, 0};
     MapKey kv = kk;
     kv.base = v_cache;
@@ -1895,23 +1712,26 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
     const bool reuse = hs->plan_valid && hs->plan_steps == d_steps && hs->plan_n_nodes == d_n_nodes &&
                        hs->plan_batch == batch && hs->plan_capacity == capacity && hs->plan_stream == st;
     if (!reuse) {
-        cudaError_t e = launch_pdl(attention_plan_kernel, dim3(1), dim3(256), 0, st, a);
+        cudaError_t e = launch_pdl(attention_plan_kernel, dim3(1), dim3(kMaxGrid), 0, st, a);
         if (e != cudaSuccess) return e;
         hs->plan_valid = true, hs->plan_steps = d_steps, hs->plan_n_nodes = d_n_nodes, hs->plan_batch = batch;
         hs->plan_capacity = capacity, hs->plan_stream = st, hs->plan_age = 0;
     }
     a.plan_after_wait = hs->plan_age == 0 ? 1 : 0;
-    a.test_drop = ctx->ws.test_drop;
-    cudaError_t e = D == 128 ? launch_for_dim<128>(ctx, a, *mk, *mv, *mq, st) : launch_for_dim<64>(ctx, a, *mk, *mv, *mq, st);
-    hs->plan_age += 2;
+    cudaError_t e = D == 128 ? launch_for_dim<128>(ctx, a, grid, *mk, *mv, *mq, st) : launch_for_dim<64>(ctx, a, grid, *mk, *mv, *mq, st);
+    hs->plan_age += a.cluster > 1 ? 1 : 2;
     return e;
 }
 
-int attention_item_rows() { return kRowTiles * kBM; }
-int attention_max_rounds() { return kMaxRounds; }
-int attention_max_batch() { return kMaxBatchSmem; }
-size_t attention_plan_bytes(int max_batch, int max_items) {
-    return 16 + sizeof(PlanSeq) * (max_batch + 1) + sizeof(PlanItem) * static_cast<size_t>(max_items);
+int attention_max_batch() { return kMaxBatch; }
+int attention_place_rows() { return kBM; }
+int attention_max_groups(int batch, int n_kv_heads, int max_tt, int group) {
+    return batch * n_kv_heads * ((max_tt * group + kBM - 1) / kBM);
+}
+int attention_max_items(int groups, int sm_count) { return groups + std::min(sm_count, kMaxGrid); }  // (also the most partials)
+size_t attention_plan_bytes(int max_items, int max_groups) {
+    return sizeof(PlanHead) + sizeof(PlanCluster) * kMaxGrid + sizeof(PlanItem) * (kMaxGrid + static_cast<size_t>(max_items)) +
+           sizeof(PlanGroup) * static_cast<size_t>(max_groups);
 }
 
 }  // namespace resps

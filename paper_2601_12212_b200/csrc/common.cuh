@@ -46,17 +46,15 @@ struct Workspace {
     double* samp_scratch = nullptr;          // acceptance under sampling: partial sums, then (p, q) of every token and sequence
     unsigned int* amax_seq_counter = nullptr;  // [max_batch] arg-max CTAs of a sequence that have delivered (self-resetting)
     // attention
-    int attn_grid = 0;          // persistent CTAs (one per SM)
-    int attn_combine_flat_grid = 0;  // ... of its variant for batches
-    int attn_min_tiles = 0;     // smallest key-tile count a split is given
-    int attn_single = 2000;     // single row tiles while no sequence has more than this many row tiles^2 x key tiles
-    int attn_stagger = 1000;    // cycles lane 1 starts behind lane 0 (RESPS_ATTN_STAGGER)
-    int attn_rounds = 0;        // 0: chosen by the work list; else forced (RESPS_ATTN_ROUNDS, for tests)
-    int attn_max_items = 0;     // partial slots
-    unsigned char* attn_plan = nullptr;  // the attention work list: header, per-sequence and per-item entries
-    __half* attn_part_o = nullptr;  // [items][item rows][D] fp16
-    float4* attn_part_ml = nullptr; // [items][item rows]
+    int attn_min_tiles = 2;     // fewest key tiles a CTA of a cluster is given
+    int attn_stream = -1;       // >= 0: key tiles a CTA must be spared for mode stream (tests)
+    int attn_cluster = 0;       // > 0: CTAs per cluster (tests)
+    int attn_rounds = 0;        // > 0: the work list is cut for 1/n of the clusters (tests)
+    int attn_max_items = 0;
     int attn_max_groups = 0;
+    unsigned char* attn_plan = nullptr;  // the attention work list: per-cluster and per-item entries
+    __half* attn_part_o = nullptr;       // [places][rows][D] fp16
+    float4* attn_part_ml = nullptr;      // [places][rows]
     // Only read by the test build (RESPS_WAIT_TEST): bit 0 = the attention kernel's first V copy is
     // never issued, bit 1 = the streaming scan's second chunk copy is never issued.
     int test_drop = 0;
@@ -141,7 +139,7 @@ cudaError_t attention_setup(resps_ctx* ctx);  // one-time function attributes, h
 void attention_teardown(resps_ctx* ctx);
 // The arrays behind `steps_or_null` (step parameters or node counts; null = any) are about to change.
 void attention_plan_invalidate(resps_ctx* ctx, const void* steps_or_null = nullptr);
-size_t attention_plan_bytes(int max_batch, int max_items);
+size_t attention_plan_bytes(int max_items, int max_groups);
 
 // Launch with programmatic stream serialization (see pdl_wait above).
 template <typename Kernel, typename... Args>
