@@ -63,7 +63,8 @@ constexpr int kSyncThreads = 320;  // softmax warps + the MMA warps meet at the 
 constexpr int kMaxBatch = 256;
 constexpr int kMaxCluster = 8;     // CTAs of a cluster (the portable limit)
 constexpr int kMaxGrid = 256;      // clusters x CTAs (one per SM)
-constexpr int kSnap = 2;           // mode stream: a cut this close to a group's edge (key tiles) is moved onto it
+constexpr int kSnap = 4;           // mode stream: a cut this close to a group's edge (key tiles) is moved onto it
+constexpr int kItemTiles = 4;      // ... and what an item costs a CTA besides its tiles (its start, epilogue and partial)
 constexpr int kTmemCols = 512;
 constexpr uint32_t kWaitLimitCycles = kWaitTest ? 2000000u : 0x70000000u;  // bounded waits give up after ~1 s of SM clocks
 constexpr float kRescaleSlack = 8.0f;  // O is rescaled only when the running max grows by > 2^8
@@ -121,6 +122,7 @@ struct AttnArgs {
     int cluster;      // CTAs per cluster (1: modes even and stream)
     int clusters;     // clusters the work list is cut for (at most gridDim / cluster)
     int max_items;
+    int comb_chunk;   // partials the combine kernel fetches together
     int stream_gain;  // mode stream when it saves a CTA more than this many key tiles
     int min_tiles;    // fewest key tiles a CTA is given
     int q_by_tma;     // 1: Q tiles come by TMA (128 % (Hq/Hkv) == 0), 0: by plain loads
@@ -131,7 +133,7 @@ struct AttnArgs {
     PlanHead* plan_head;
     PlanCluster* plan_cluster;  // [kMaxGrid]
     PlanItem* plan_first;       // [kMaxGrid] every CTA's first item once more (one load instead of two in a row)
-    PlanItem* plan_item;        // [max_items x cluster]
+    PlanItem* plan_item;        // [max_items x cluster] (mode even has one item per CTA and does without)
     PlanGroup* plan_group;      // [groups]
 };
 
@@ -151,7 +153,8 @@ __device__ __forceinline__ int active_ctas(int tiles, int cluster, int min_tiles
 // Bound by latency (one CTA, once per step): a scan over the sequences, a search, then a thread per CTA or
 // item.  Positions are in key tiles of the sequence of groups (b, KV head, row tile).
 struct PlanShared {
-    unsigned long long start[kMaxBatch + 1];  // first position of a sequence
+    unsigned long long start[kMaxBatch + 1];  // first position of a sequence, in key tiles ...
+    unsigned long long cost0[kMaxBatch + 1];  // ... and with every group's kItemTiles
     int group0[kMaxBatch + 1];                // first group of a sequence
     int item0[kMaxBatch + 1];                 // mode even: first item of a sequence
     int n[kMaxBatch], L[kMaxBatch], tiles[kMaxBatch], kt[kMaxBatch], splits[kMaxBatch];
@@ -193,16 +196,24 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
                 const unsigned long long w = __shfl_up_sync(kFull, work, d);
                 if (lane >= d) groups += g, work += w;
             }
-            if (b < a.batch) sh.start[b] = pos + work - own_work, sh.group0[b] = group + groups - own_groups;
+            if (b < a.batch) {
+                sh.start[b] = pos + work - own_work, sh.group0[b] = group + groups - own_groups;
+                sh.cost0[b] = sh.start[b] + static_cast<unsigned long long>(sh.group0[b]) * kItemTiles;
+            }
             pos += __shfl_sync(kFull, work, 31);
             group += __shfl_sync(kFull, groups, 31);
         }
-        if (lane == 0) sh.start[a.batch] = pos, sh.group0[a.batch] = group;
+        if (lane == 0) {
+            sh.start[a.batch] = pos, sh.group0[a.batch] = group;
+            sh.cost0[a.batch] = pos + static_cast<unsigned long long>(group) * kItemTiles;
+        }
         int mode = kModeWhole;
         if (a.cluster == 1) {
             // the smallest T (in steps of T/16) for which the splits fit one round of the grid
-            const int even = static_cast<int>(min((pos + a.clusters - 1) / a.clusters, 1ull << 24));  // tiles per CTA when cut evenly
-            int T = max(even, 1);
+            const unsigned long long cost = pos + static_cast<unsigned long long>(group) * kItemTiles;
+            const int even = static_cast<int>(min((cost + a.clusters - 1) / a.clusters, 1ull << 24));  // per CTA when cut evenly
+            int T = static_cast<int>(min((pos + a.clusters - 1) / a.clusters, 1ull << 24));
+            T = max(T, 1);
             bool fits = false;
 #pragma unroll 1
             for (int tries = 0; tries < 40 && !fits; ++tries) {
@@ -267,19 +278,26 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
         // ---- an item per cluster or CTA ---------------------------------------------------------------
         const int n = (mode == kModeWhole) ? n_groups : sh.item0[a.batch];
         if (tid < a.clusters) {
+            // (mode whole has more groups than clusters only if a tree is larger than the context's limits allow)
             PlanCluster c;
-            c.first_item = tid, c.n_items = (tid < n) ? 1 : 0;
+            c.first_item = static_cast<int>(static_cast<unsigned>(n) * tid / a.clusters);
+            c.n_items = static_cast<int>(static_cast<unsigned>(n) * (tid + 1) / a.clusters) - c.first_item;
+            if (n <= a.clusters) c.first_item = tid, c.n_items = (tid < n) ? 1 : 0;
             a.plan_cluster[tid] = c;
-            if (tid < n && mode == kModeWhole) {
-                const int b = last_at_or_before(sh.group0, tid);
-                PlanItem p = item_of(b, tid - sh.group0[b]);
-                const int kt = sh.kt[b], act = active_ctas(kt, a.cluster, a.min_tiles);
-                p.tile_active = (p.tile_active & 0xFFFF) | (act << 16);
+            if (mode == kModeWhole) {
 #pragma unroll 1
-                for (int r = 0; r < a.cluster; ++r) {
-                    p.t_begin = p.t_end;
-                    if (r < act) p.t_end = kt * (r + 1) / act;
-                    a.plan_first[tid * a.cluster + r] = p;
+                for (int i = 0; i < c.n_items; ++i) {
+                    const int group = c.first_item + i, b = last_at_or_before(sh.group0, group);
+                    PlanItem p = item_of(b, group - sh.group0[b]);
+                    const int kt = sh.kt[b], act = active_ctas(kt, a.cluster, a.min_tiles);
+                    p.tile_active = (p.tile_active & 0xFFFF) | (act << 16);
+#pragma unroll 1
+                    for (int r = 0; r < a.cluster; ++r) {
+                        p.t_begin = p.t_end;
+                        if (r < act) p.t_end = kt * (r + 1) / act;
+                        if (i == 0) a.plan_first[tid * a.cluster + r] = p;
+                        a.plan_item[group * a.cluster + r] = p;
+                    }
                 }
             } else if (tid < n) {
                 const int b = last_at_or_before(sh.item0, tid), splits = sh.splits[b], kt = sh.kt[b];
@@ -294,29 +312,33 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
         return;
     }
     // ---- even cuts ------------------------------------------------------------------------------------
-    const unsigned long long total = sh.start[a.batch];
-    auto locate = [&](unsigned long long pos, int& b, int& local, int& t) {  // of a position before the end
+    // (of a position before the end; `extra` units of every group come before its tiles)
+    auto locate = [&](const unsigned long long* first, unsigned long long pos, int extra, int& b, int& local, int& t) {
         int lo = 0, hi = a.batch;  // last sequence that starts at or before pos (and is not empty there)
 #pragma unroll 1
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
-            if (sh.start[mid] <= pos) lo = mid; else hi = mid;
+            if (first[mid] <= pos) lo = mid; else hi = mid;
         }
         b = lo;
-        const unsigned off = static_cast<unsigned>(pos - sh.start[b]);  // < groups x tiles of a sequence: fits 32 bits
-        local = static_cast<int>(off / static_cast<unsigned>(sh.kt[b]));
-        t = static_cast<int>(off - static_cast<unsigned>(local) * static_cast<unsigned>(sh.kt[b]));
+        const unsigned off = static_cast<unsigned>(pos - first[b]);  // < groups x length of a group: fits 32 bits
+        const unsigned len = static_cast<unsigned>(sh.kt[b] + extra);
+        local = static_cast<int>(off / len);
+        t = max(static_cast<int>(off - static_cast<unsigned>(local) * len) - extra, 0);
     };
     int b = 0, local = 0, t = 0;
     if (tid <= a.clusters) {
-        unsigned long long cut = total * static_cast<unsigned long long>(tid) / static_cast<unsigned long long>(a.clusters);
-        if (cut < total) {  // a piece shorter than its own epilogue is not worth a cut
-            locate(cut, b, local, t);
+        const unsigned long long cost = sh.cost0[a.batch];
+        const unsigned long long at = cost * static_cast<unsigned long long>(tid) / static_cast<unsigned long long>(a.clusters);
+        unsigned long long cut = sh.start[a.batch];
+        if (at < cost) {  // a piece shorter than its own epilogue is not worth a cut
+            locate(sh.cost0, at, kItemTiles, b, local, t);
             const int behind = sh.kt[b] - t;
             if (t <= behind && t <= kSnap)
-                cut -= t;
+                t = 0;
             else if (behind < t && behind <= kSnap)
-                cut += behind;
+                t = sh.kt[b];
+            cut = sh.start[b] + static_cast<unsigned long long>(local) * sh.kt[b] + t;
         }
         sh.cut[tid] = cut;
     }
@@ -325,8 +347,8 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
         int count = 0;
         if (sh.cut[tid] < sh.cut[tid + 1]) {
             int b1, local1, t1;
-            locate(sh.cut[tid + 1] - 1, b1, local1, t1);
-            locate(sh.cut[tid], b, local, t);
+            locate(sh.start, sh.cut[tid + 1] - 1, 0, b1, local1, t1);
+            locate(sh.start, sh.cut[tid], 0, b, local, t);
             count = sh.group0[b1] + local1 - sh.group0[b] - local + 1;
         }
         sh.n_items[tid] = count;
@@ -856,7 +878,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
         const int n_live = min(max(a.n_nodes[first_it.b], 0), a.max_tt), L_live = max(a.steps[first_it.b].prefix_len, 0);
         stale = (n_live != first_it.n) || (L_live != first_it.L);
     }
-    auto get_item = [&](int i) { return i == 0 ? first_it : load_item(a.plan_item + first_item + i, G); };
+    auto get_item = [&](int i) { return i == 0 ? first_it : load_item(a.plan_item + (first_item + i) * a.cluster + rank, G); };
 
     // Running use counts of the barrier families.  Every role walks the same items and tiles in
     // the same order, so each keeps its own copy.
@@ -935,6 +957,9 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
             alive = warp_wait(bar(bar_qfull()), items_run & 1u, abort_flag);
             tc_fence_after();
             bool first_pv = true;
+#ifdef STAG
+            if (x == 1 && it.t_end - it.t_begin >= 8) { const uint32_t c0 = clock(); while (static_cast<uint32_t>(clock()) - c0 < STAG) {} }
+#endif
             // The lane's tiles are t_begin + x, + 2, ...; one round issues Q K^T of a tile and P V of the one
             // before (the last round P V only).
             const int mine = (it.t_end - it.t_begin - x + 1) >> 1;
@@ -1022,22 +1047,27 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
             const int n_tiles = it.t_end - it.t_begin;
             const bool direct = it.pieces == 1 && it.active == 1;  // one CTA has the whole group
             if (n_tiles > 0) {
-                // ---- Q tile -> shared memory in the swizzled K-major layout (only when the group
-                // size does not allow the TMA view; a plain loop, not worth unrolled code) --------
+                // ---- Q tile -> shared memory in the swizzled K-major layout (only when the group size does not
+                // allow the TMA view): every thread's pieces are in flight together (one at a time they
+                // took 8 us) --------------------------------------------------------------------------
                 if (!a.q_by_tma) {
-                    constexpr int kChunks = D / 8;  // 16-byte pieces of a row
-#pragma unroll 1
-                    for (int e = tid; e < kBM * kChunks; e += kSoftmaxThreads) {
-                        const int row = e / kChunks, c = e % kChunks;
-                        const int Rq = it.row_base + row;
-                        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                        if (Rq < it.M) {
-                            const int t = Rq / G, h = it.g * G + Rq % G;
-                            v = __ldg(reinterpret_cast<const uint4*>(
+                    constexpr int kChunks = D / 8, kPer = kBM * kChunks / kSoftmaxThreads;  // 16-byte pieces of a row, of a thread
+                    uint4 v[kPer];
+                    const int c = tid % kChunks;
+#pragma unroll
+                    for (int e = 0; e < kPer; ++e) {
+                        const unsigned Rq = it.row_base + tid / kChunks + e * (kSoftmaxThreads / kChunks);
+                        const unsigned t = Rq / static_cast<unsigned>(G), h = it.g * G + (Rq - t * G);
+                        v[e] = make_uint4(0u, 0u, 0u, 0u);
+                        if (Rq < static_cast<unsigned>(it.M))
+                            v[e] = __ldg(reinterpret_cast<const uint4*>(
                                 a.q + ((static_cast<int64_t>(it.b) * a.max_tt + t) * a.Hq + h) * D + c * 8));
-                        }
+                    }
+#pragma unroll
+                    for (int e = 0; e < kPer; ++e) {
+                        const int row = tid / kChunks + e * (kSoftmaxThreads / kChunks);
                         *reinterpret_cast<uint4*>(base_ptr + S::kOffQ + (c >> 3) * S::kQPanel + row * 128 +
-                                                  (((c & 7) ^ (row & 7)) << 4)) = v;
+                                                  (((c & 7) ^ (row & 7)) << 4)) = v[e];
                     }
                     fence_proxy_async();
                     mbar_arrive(bar(bar_qfull()));
@@ -1221,7 +1251,9 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 const float inv = (l_tot > 0.f) ? 1.f / l_tot : 0.f;
                 const int tok = R / G, h = it.g * G + R % G;
                 const int64_t out_row = (static_cast<int64_t>(it.b) * a.max_tt + tok) * a.Hq + h;
-                const int64_t place = a.cluster > 1 ? static_cast<int>(blockIdx.x) : first_item + i;
+                // (two places per CTA of a cluster, in turn: an item's partials are read behind the meeting of the
+                // CTAs, and the next but one item's are written behind the next meeting)
+                const int64_t place = a.cluster > 1 ? static_cast<int>(blockIdx.x + (meets & 1u) * gridDim.x) : first_item + i;
                 __nv_bfloat16* dst = a.o + out_row * D;
                 uint4* po = a.part_o + place * (D / 8) * kBM + r;
                 // (a lane without tiles has nothing in tensor memory: the other's is read in its place, with weight 0)
@@ -1294,9 +1326,9 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 __syncwarp();
                 if (lane < a.cluster) mbar_arrive_remote(bar(bar_meet()), lane);
                 alive = __all_sync(kFull, cluster_bar_wait(bar(bar_meet()), meets & 1u, abort_flag));
-                ++meets;
                 if (!alive) break;
-                merge_partials<D>(a, it, static_cast<unsigned>(cluster_id * a.cluster), it.active, rank, tid, G);
+                merge_partials<D>(a, it, static_cast<unsigned>(cluster_id * a.cluster) + (meets & 1u) * gridDim.x, it.active, rank, tid, G);
+                ++meets;
             }
             if (n_tiles > 0) {
                 // (long complete: only keeps a thread from running an item ahead of the others)
@@ -1337,7 +1369,8 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
 // piece, one for the (max, sum, scales) of the rows) into shared memory: a few dozen requests per CTA, all
 // in flight at once.  What a CTA has to do is one entry of the work list, fetched before the wait.
 constexpr int kCombineThreads = 256;
-constexpr int kCombChunk = 8;   // partials fetched together
+constexpr int kCombChunk = 8;       // partials fetched together; with few groups, when a CTA has an SM to itself,
+constexpr int kCombChunkMost = 32;  // all of a group's up to this many
 constexpr int kCombPieces = 2;  // 8-column pieces per CTA
 constexpr int kCombSlotBytes = (kCombPieces + 1) * kBM * 16;  // per partial: the pieces, then (max, sum, scales)
 
@@ -1346,7 +1379,7 @@ __global__ void __launch_bounds__(kCombineThreads) attention_combine_kernel(cons
     constexpr int kPieces = D / 8;                    // 16-byte pieces of a row
     constexpr int kShares = kPieces / kCombPieces;    // units of work per group
     static_assert(kCombineThreads == kCombPieces * kBM, "thread = (row, piece)");
-    extern __shared__ __align__(128) unsigned char comb_smem[];  // [kCombChunk][kCombSlotBytes]
+    extern __shared__ __align__(128) unsigned char comb_smem[];  // [comb_chunk][kCombSlotBytes]
     __shared__ __align__(8) unsigned long long s_bar;
     pdl_launch_dependents();
     const int tid = threadIdx.x, r = tid % kBM, cc = tid / kBM;
@@ -1379,8 +1412,8 @@ __global__ void __launch_bounds__(kCombineThreads) attention_combine_kernel(cons
         float Mx = -INFINITY, den = 0.f;
         float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
-        for (int p0 = 0; p0 < pieces; p0 += kCombChunk) {
-            const int np = min(kCombChunk, pieces - p0);
+        for (int p0 = 0; p0 < pieces; p0 += a.comb_chunk) {
+            const int np = min(a.comb_chunk, pieces - p0);
             // one copy per thread, so that they are issued side by side: a partial's column pieces and
             // its (max, sum, scales), each nv x 16 contiguous bytes
             if (tid == 0) mbar_expect_tx(bar, static_cast<uint32_t>(np * (kCombPieces + 1) * nv * 16));
@@ -1562,19 +1595,25 @@ const CUtensorMap* cached_map(HostState* hs, const MapKey& key, int D) {
 // 0.6 groups kt (1 / (C groups) - 1 / SMs) us for kt key tiles, so it is taken while the longest prefix the
 // cache can hold costs no more than it saves.  Cluster sizes that do not leave SMs of a GPC unused only.
 constexpr double kWholeGainTiles = 5.0;  // 3 us / 0.6 us
-int choose_cluster(const int* resident, int sm_count, int64_t groups, int kt_most) {
+// In a batch the cache may hold one long sequence among short ones, which only its own clusters work on.
+int choose_cluster(const int* resident, int sm_count, int groups, int batch, int kt_most) {
     for (int c : {8, 6, 4, 3, 2}) {
         if (resident[c] < groups) continue;
-        const double lost = 1.0 / c - static_cast<double>(groups) / sm_count;
+        const double lost = 1.0 / c - static_cast<double>(groups / batch) / sm_count;
         if (lost * kt_most <= kWholeGainTiles) return c;
     }
-    return kt_most <= 5 && groups <= resident[1] ? 2 : 1;
+    return 1;
 }
 int forced_cluster(const int* resident, int cluster, int groups) {
     while (cluster > 1 && resident[cluster] < groups) --cluster;
     return cluster;
 }
-constexpr int kStreamGain = 6;  // key tiles a CTA must be spared before groups are cut at odd places
+constexpr int kStreamGain = 3;  // key tiles a CTA must be spared before groups are cut at odd places
+
+// Nodes of the largest tree a context builds: min(max_tt, 1 + n_cand).
+int most_nodes(const resps_shape& s) {
+    return static_cast<int>(std::min<int64_t>(s.max_tt, 1 + s.max_k + static_cast<int64_t>(s.max_depth - 1) * s.max_k * s.max_k));
+}
 
 // Clusters of C CTAs that are resident at once with this kernel's shared memory (index C; the GPCs are not
 // multiples of every size), asked for once per device.
@@ -1601,14 +1640,14 @@ cudaError_t launch_for_dim(const resps_ctx* ctx, const AttnArgs& a, int grid, co
     // the units of work of the largest trees, at most one resident round of CTAs
     const int64_t units = static_cast<int64_t>(a.batch) * a.Hkv * ((a.max_tt * (a.Hq / a.Hkv) + kBM - 1) / kBM) * (D / 8 / kCombPieces);
     const int combine_grid = static_cast<int>(std::min<int64_t>(units, 4 * ctx->sm_count));
-    return launch_pdl(attention_combine_kernel<D>, dim3(combine_grid), dim3(kCombineThreads), kCombChunk * kCombSlotBytes, st, a);
+    return launch_pdl(attention_combine_kernel<D>, dim3(combine_grid), dim3(kCombineThreads), a.comb_chunk * kCombSlotBytes, st, a);
 }
 
 template <int D>
 cudaError_t setup_for_dim(int device, int sm_count, int* clusters) {
     cudaError_t e = cudaFuncSetAttribute(tree_attention_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<D>::kBytes);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attention_combine_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombChunk * kCombSlotBytes);
+    e = cudaFuncSetAttribute(attention_combine_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombChunkMost * kCombSlotBytes);
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lock(g_residency_mu);
     Residency local;
@@ -1680,7 +1719,7 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
     a.plan_head = reinterpret_cast<PlanHead*>(plan), plan += sizeof(PlanHead);
     a.plan_cluster = reinterpret_cast<PlanCluster*>(plan), plan += sizeof(PlanCluster) * kMaxGrid;
     a.plan_first = reinterpret_cast<PlanItem*>(plan), plan += sizeof(PlanItem) * kMaxGrid;
-    a.plan_item = reinterpret_cast<PlanItem*>(plan), plan += sizeof(PlanItem) * w.attn_max_items;
+    a.plan_item = reinterpret_cast<PlanItem*>(plan), plan += sizeof(PlanItem) * w.attn_max_items * kMaxCluster;
     a.plan_group = reinterpret_cast<PlanGroup*>(plan);
     a.test_drop = w.test_drop;
     const int D = ctx->shape.head_dim;
@@ -1688,12 +1727,14 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
     a.q_by_tma = (G <= kBM && kBM % G == 0) ? 1 : 0;
     HostState* hs = host_state(ctx);
     std::lock_guard<std::mutex> lock(hs->mu);
-    a.cluster = choose_cluster(hs->resident, ctx->sm_count, static_cast<int64_t>(batch) * a.Hkv * ((a.max_tt * G + kBM - 1) / kBM),
-                               static_cast<int>((capacity + kBN - 1) / kBN));
-    if (w.attn_cluster > 0) a.cluster = forced_cluster(hs->resident, std::min(w.attn_cluster, kMaxCluster), batch * a.Hkv * ((a.max_tt * G + kBM - 1) / kBM));
-    a.clusters = a.cluster > 1 ? batch * a.Hkv * ((a.max_tt * G + kBM - 1) / kBM) : hs->resident[1];
+    // the most groups of a tree this context builds (attention over larger ones is correct, and slower)
+    const int groups = batch * a.Hkv * ceil_div(most_nodes(ctx->shape) * G, kBM);
+    a.cluster = choose_cluster(hs->resident, ctx->sm_count, groups, batch, static_cast<int>((capacity + kBN - 1) / kBN));
+    if (w.attn_cluster > 0) a.cluster = forced_cluster(hs->resident, std::min(w.attn_cluster, kMaxCluster), groups);
+    a.clusters = a.cluster > 1 ? groups : hs->resident[1];
     const int grid = a.clusters * a.cluster;
     if (w.attn_rounds > 0 && a.cluster == 1) a.clusters = std::max(1, a.clusters / w.attn_rounds);
+    a.comb_chunk = groups * (D / 8 / kCombPieces) <= ctx->sm_count ? kCombChunkMost : kCombChunk;
     a.stream_gain = w.attn_stream >= 0 ? w.attn_stream : kStreamGain;
     MapKey kk = {k_cache, stride_tok, stride_head, stride_seq, capacity, a.Hkv, batch, 0};
     MapKey kv = kk;
@@ -1728,9 +1769,10 @@ int attention_place_rows() { return kBM; }
 int attention_max_groups(int batch, int n_kv_heads, int max_tt, int group) {
     return batch * n_kv_heads * ((max_tt * group + kBM - 1) / kBM);
 }
-int attention_max_items(int groups, int sm_count) { return groups + std::min(sm_count, kMaxGrid); }  // (also the most partials)
+// (also the most partials)
+int attention_max_items(int groups, int sm_count) { return std::max(groups, std::min(sm_count, kMaxGrid)) + std::min(sm_count, kMaxGrid); }
 size_t attention_plan_bytes(int max_items, int max_groups) {
-    return sizeof(PlanHead) + sizeof(PlanCluster) * kMaxGrid + sizeof(PlanItem) * (kMaxGrid + static_cast<size_t>(max_items)) +
+    return sizeof(PlanHead) + sizeof(PlanCluster) * kMaxGrid + sizeof(PlanItem) * (kMaxGrid + static_cast<size_t>(max_items) * kMaxCluster) +
            sizeof(PlanGroup) * static_cast<size_t>(max_groups);
 }
 
