@@ -59,12 +59,12 @@ constexpr int kVProducerWarp = 11; // V tiles
 constexpr int kAttnThreads = 384;
 constexpr int kRegsSoftmax = 216;  // setmaxnreg: 256 x 216 + 128 x 72 = 384 x 168 <= 64 K registers
 constexpr int kRegsIssue = 72;
-constexpr int kSyncThreads = 320;  // softmax warps + the MMA warps meet at the end of an item
 constexpr int kMaxBatch = 256;
 constexpr int kMaxCluster = 8;     // CTAs of a cluster (the portable limit)
 constexpr int kMaxGrid = 256;      // clusters x CTAs (one per SM)
 constexpr int kSnap = 4;           // mode stream: a cut this close to a group's edge (key tiles) is moved onto it
-constexpr int kItemTiles = 4;      // ... and what an item costs a CTA besides its tiles (its start, epilogue and partial)
+constexpr int kItemTiles = 4;      // what an item costs a CTA besides its tiles (its start and epilogue), in key tiles
+constexpr int kCutTiles = 6;       // what cut groups cost a call (partials, the combine kernel's round trips)
 constexpr int kTmemCols = 512;
 constexpr uint32_t kWaitLimitCycles = kWaitTest ? 2000000u : 0x70000000u;  // bounded waits give up after ~1 s of SM clocks
 constexpr float kRescaleSlack = 8.0f;  // O is rescaled only when the running max grows by > 2^8
@@ -77,11 +77,13 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 //  even    single CTAs; every group is cut into splits of at most T key tiles with the smallest T for which
 //          the splits fit one round of the grid; a second, small kernel combines the partials.
 //  stream  the same two kernels; the key tiles of all groups, one group after the other, are cut into equal
-//          contiguous ranges, one per CTA (a CTA may end one group and begin another).
+//          contiguous ranges, one per CTA (a CTA may end one group and begin another), or into ranges of whole
+//          groups.
+// Of even and stream the one with the smallest largest share is taken (tiles, items, cut groups).
 constexpr int kModeWhole = 0, kModeEven = 1, kModeStream = 2;
 
 struct PlanHead {
-    int mode, n_groups, pad[2];
+    int n_groups, pad[3];
 };
 // A cluster's (or CTA's) first item and its number of items.
 struct PlanCluster {
@@ -123,7 +125,7 @@ struct AttnArgs {
     int clusters;     // clusters the work list is cut for (at most gridDim / cluster)
     int max_items;
     int comb_chunk;   // partials the combine kernel fetches together
-    int stream_gain;  // mode stream when it saves a CTA more than this many key tiles
+    int stream_gain;  // -1: own choice; 0: never mode even; else always where it fits (tests)
     int min_tiles;    // fewest key tiles a CTA is given
     int q_by_tma;     // 1: Q tiles come by TMA (128 % (Hq/Hkv) == 0), 0: by plain loads
     int plan_after_wait;  // 1: the work list was written by the kernel just before this one
@@ -158,9 +160,9 @@ struct PlanShared {
     int group0[kMaxBatch + 1];                // first group of a sequence
     int item0[kMaxBatch + 1];                 // mode even: first item of a sequence
     int n[kMaxBatch], L[kMaxBatch], tiles[kMaxBatch], kt[kMaxBatch], splits[kMaxBatch];
-    unsigned long long cut[kMaxGrid + 1];
+    unsigned long long cut[2][kMaxGrid + 1];
     int n_items[kMaxGrid];
-    int mode;
+    int even_cost, range_cost[2];  // largest share of a CTA: mode even; ranges of whole groups, equal ranges
 };
 
 __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs a) {
@@ -207,11 +209,8 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
             sh.start[a.batch] = pos, sh.group0[a.batch] = group;
             sh.cost0[a.batch] = pos + static_cast<unsigned long long>(group) * kItemTiles;
         }
-        int mode = kModeWhole;
         if (a.cluster == 1) {
             // the smallest T (in steps of T/16) for which the splits fit one round of the grid
-            const unsigned long long cost = pos + static_cast<unsigned long long>(group) * kItemTiles;
-            const int even = static_cast<int>(min((cost + a.clusters - 1) / a.clusters, 1ull << 24));  // per CTA when cut evenly
             int T = static_cast<int>(min((pos + a.clusters - 1) / a.clusters, 1ull << 24));
             T = max(T, 1);
             bool fits = false;
@@ -226,12 +225,13 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
                 if (!fits) T += max(1, T >> 4);
             }
             T = max(T, a.min_tiles);
-            mode = (fits && T - even <= a.stream_gain) ? kModeEven : kModeStream;
-            int base = 0;
+            // (its cost is compared with the ranges' below)
+            int base = 0, most = 0;
 #pragma unroll 1
             for (int b0 = 0; b0 < a.batch; b0 += 32) {
                 const int b = b0 + lane, splits = (b < a.batch) ? ceil_div(sh.kt[b], T) : 0;
-                int incl = (b < a.batch && mode == kModeEven) ? a.Hkv * sh.tiles[b] * splits : 0;
+                int incl = (b < a.batch && fits) ? a.Hkv * sh.tiles[b] * splits : 0;
+                most = max(most, splits > 0 ? ceil_div(sh.kt[b], splits) + kItemTiles + (splits > 1 ? kCutTiles : 0) : 0);
                 const int own = incl;
 #pragma unroll
                 for (int d = 1; d < 32; d <<= 1) {
@@ -241,17 +241,21 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
                 if (b < a.batch) sh.splits[b] = splits, sh.item0[b] = base + incl - own;
                 base += __shfl_sync(kFull, incl, 31);
             }
-            if (lane == 0) sh.item0[a.batch] = base;
+            most = __reduce_max_sync(kFull, most);
+            if (lane == 0) {
+                sh.item0[a.batch] = base;
+                sh.even_cost = fits ? most + (a.stream_gain < 0 ? 0 : a.stream_gain ? -(1 << 28) : 1 << 28) : 1 << 30;
+            }
         }
         if (lane == 0) {
-            sh.mode = mode;
+            sh.range_cost[0] = sh.range_cost[1] = 0;
             PlanHead h = {};
-            h.mode = mode, h.n_groups = group;
+            h.n_groups = group;
             *a.plan_head = h;
         }
     }
     __syncthreads();
-    const int mode = sh.mode, n_groups = sh.group0[a.batch];
+    const int n_groups = sh.group0[a.batch];
     auto last_at_or_before = [&](const int* first, int x) {  // the last sequence whose entry is <= x
         int lo = 0, hi = a.batch;
 #pragma unroll 1
@@ -274,6 +278,54 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
         q.b_g = p.b_g, q.tile = p.tile_active & 0xFFFF, q.n = p.n, q.first_item = first_item, q.pieces = p.pieces;
         a.plan_group[group] = q;
     };
+    // ---- ranges ---------------------------------------------------------------------------------------
+    // (of a position before the end; `extra` units of every group come before its tiles)
+    auto locate = [&](const unsigned long long* first, unsigned long long pos, int extra, int& b, int& local, int& t) {
+        int lo = 0, hi = a.batch;  // last sequence that starts at or before pos (and is not empty there)
+#pragma unroll 1
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (first[mid] <= pos) lo = mid; else hi = mid;
+        }
+        b = lo;
+        const unsigned off = static_cast<unsigned>(pos - first[b]);  // < groups x length of a group: fits 32 bits
+        const unsigned len = static_cast<unsigned>(sh.kt[b] + extra);
+        local = static_cast<int>(off / len);
+        t = max(static_cast<int>(off - static_cast<unsigned>(local) * len) - extra, 0);
+    };
+    int b = 0, local = 0, t = 0;
+    if (a.cluster == 1) {
+        if (tid <= a.clusters) {
+            const unsigned long long cost = sh.cost0[a.batch];
+            const unsigned long long at = cost * static_cast<unsigned long long>(tid) / static_cast<unsigned long long>(a.clusters);
+            unsigned long long whole = sh.start[a.batch], equal = whole;
+            if (at < cost) {
+                locate(sh.cost0, at, kItemTiles, b, local, t);
+                const int behind = sh.kt[b] - t;
+                const unsigned long long g0 = sh.start[b] + static_cast<unsigned long long>(local) * sh.kt[b];
+                whole = g0 + (t <= behind ? 0 : sh.kt[b]);
+                // a piece shorter than its own epilogue is not worth a cut
+                equal = (min(t, behind) <= kSnap) ? whole : g0 + t;
+            }
+            sh.cut[0][tid] = whole, sh.cut[1][tid] = equal;
+        }
+        __syncthreads();
+        if (tid < a.clusters) {
+#pragma unroll 1
+            for (int w = 0; w < 2; ++w) {
+                const unsigned long long begin = sh.cut[w][tid], end = sh.cut[w][tid + 1];
+                if (begin == end) continue;
+                int b1, local1, t1;
+                locate(sh.start, end - 1, 0, b1, local1, t1);
+                locate(sh.start, begin, 0, b, local, t);
+                const int items = sh.group0[b1] + local1 - sh.group0[b] - local + 1;
+                atomicMax(&sh.range_cost[w], static_cast<int>(end - begin) + items * kItemTiles + (w ? kCutTiles : 0));
+            }
+        }
+        __syncthreads();
+    }
+    const int ranges = sh.range_cost[1] < sh.range_cost[0] ? 1 : 0;
+    const int mode = a.cluster > 1 ? kModeWhole : sh.even_cost <= sh.range_cost[ranges] ? kModeEven : kModeStream;
     if (mode != kModeStream) {
         // ---- an item per cluster or CTA ---------------------------------------------------------------
         const int n = (mode == kModeWhole) ? n_groups : sh.item0[a.batch];
@@ -311,44 +363,13 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
         }
         return;
     }
-    // ---- even cuts ------------------------------------------------------------------------------------
-    // (of a position before the end; `extra` units of every group come before its tiles)
-    auto locate = [&](const unsigned long long* first, unsigned long long pos, int extra, int& b, int& local, int& t) {
-        int lo = 0, hi = a.batch;  // last sequence that starts at or before pos (and is not empty there)
-#pragma unroll 1
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (first[mid] <= pos) lo = mid; else hi = mid;
-        }
-        b = lo;
-        const unsigned off = static_cast<unsigned>(pos - first[b]);  // < groups x length of a group: fits 32 bits
-        const unsigned len = static_cast<unsigned>(sh.kt[b] + extra);
-        local = static_cast<int>(off / len);
-        t = max(static_cast<int>(off - static_cast<unsigned>(local) * len) - extra, 0);
-    };
-    int b = 0, local = 0, t = 0;
-    if (tid <= a.clusters) {
-        const unsigned long long cost = sh.cost0[a.batch];
-        const unsigned long long at = cost * static_cast<unsigned long long>(tid) / static_cast<unsigned long long>(a.clusters);
-        unsigned long long cut = sh.start[a.batch];
-        if (at < cost) {  // a piece shorter than its own epilogue is not worth a cut
-            locate(sh.cost0, at, kItemTiles, b, local, t);
-            const int behind = sh.kt[b] - t;
-            if (t <= behind && t <= kSnap)
-                t = 0;
-            else if (behind < t && behind <= kSnap)
-                t = sh.kt[b];
-            cut = sh.start[b] + static_cast<unsigned long long>(local) * sh.kt[b] + t;
-        }
-        sh.cut[tid] = cut;
-    }
-    __syncthreads();
+    const unsigned long long* const cuts = sh.cut[ranges];
     if (tid < a.clusters) {
         int count = 0;
-        if (sh.cut[tid] < sh.cut[tid + 1]) {
+        if (cuts[tid] < cuts[tid + 1]) {
             int b1, local1, t1;
-            locate(sh.start, sh.cut[tid + 1] - 1, 0, b1, local1, t1);
-            locate(sh.start, sh.cut[tid], 0, b, local, t);
+            locate(sh.start, cuts[tid + 1] - 1, 0, b1, local1, t1);
+            locate(sh.start, cuts[tid], 0, b, local, t);
             count = sh.group0[b1] + local1 - sh.group0[b] - local + 1;
         }
         sh.n_items[tid] = count;
@@ -359,13 +380,13 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
 #pragma unroll 4
         for (int i = 0; i < tid; ++i) first += sh.n_items[i];
         const int count = min(sh.n_items[tid], max(a.max_items - first, 0));
-        const unsigned long long begin = sh.cut[tid], end = sh.cut[tid + 1];
+        const unsigned long long begin = cuts[tid], end = cuts[tid + 1];
         auto cluster_of = [&](unsigned long long pos) {  // the last CTA that begins at or before pos
             int lo = 0, hi = a.clusters;
 #pragma unroll 1
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
-                if (sh.cut[mid] <= pos) lo = mid; else hi = mid;
+                if (cuts[mid] <= pos) lo = mid; else hi = mid;
             }
             return lo;
         };
@@ -691,6 +712,7 @@ __device__ __forceinline__ constexpr int bar_sfull(int m, int buf) { return kBar
 __device__ __forceinline__ constexpr int bar_pfull(int m, int buf) { return kBar0 + 2 + m * 6 + 2 + buf; }
 __device__ __forceinline__ constexpr int bar_pvdone(int m, int buf) { return kBar0 + 2 + m * 6 + 4 + buf; }
 constexpr int kBar1 = kBar0 + 2 + kLanes * 6;
+// the softmax warpgroups have read an item's O: the next item's P V may overwrite it (its Q K^T need not wait)
 __device__ __forceinline__ constexpr int bar_item() { return kBar1; }
 // both softmax warpgroups have their partial result (and its PV completions) behind them
 __device__ __forceinline__ constexpr int bar_merge() { return kBar1 + 1; }
@@ -822,7 +844,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 mbar_init(bar(bar_pvdone(m, bf)), 1);
             }
         }
-        mbar_init(bar(bar_item()), kSyncThreads);
+        mbar_init(bar(bar_item()), kSoftmaxThreads);
         mbar_init(bar(bar_merge()), kSoftmaxThreads);
         mbar_init(bar(bar_meet()), a.cluster * (kSoftmaxThreads / 32));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -957,9 +979,6 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
             alive = warp_wait(bar(bar_qfull()), items_run & 1u, abort_flag);
             tc_fence_after();
             bool first_pv = true;
-#ifdef STAG
-            if (x == 1 && it.t_end - it.t_begin >= 8) { const uint32_t c0 = clock(); while (static_cast<uint32_t>(clock()) - c0 < STAG) {} }
-#endif
             // The lane's tiles are t_begin + x, + 2, ...; one round issues Q K^T of a tile and P V of the one
             // before (the last round P V only).
             const int mine = (it.t_end - it.t_begin - x + 1) >> 1;
@@ -1000,6 +1019,8 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                         __all_sync(kFull, mbar_test(bar(bar_kfull(next_use % kStagesK)), (next_use / kStagesK) & 1u)))
                         k_seen = next_use;
                     alive = warp_wait(bar(bar_pfull(x, prev_j & 1u)), (prev_j >> 1) & 1u, abort_flag);
+                    if (alive && first_pv && items_run > 0)
+                        alive = warp_wait(bar(bar_item()), (items_run - 1u) & 1u, abort_flag);
                     if (!alive) break;
                     tc_fence_after();
                     if (elect_one()) {
@@ -1025,11 +1046,6 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
             if (alive && mine == 0 && elect_one()) umma_commit(bar(bar_qempty()));
             __syncwarp();
             kt_run += static_cast<uint32_t>(it.t_end - it.t_begin);
-            tc_fence_before();
-            if (!alive) break;
-            // end of item: the softmax warps have read O and S, Q and P may be overwritten
-            mbar_arrive(bar(bar_item()));
-            alive = warp_wait(bar(bar_item()), items_run & 1u, abort_flag);
             ++items_run;
         }
     }
@@ -1306,7 +1322,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                     // (the loads from tensor memory are warp-wide: the whole warp goes round again)
                     if (!__any_sync(kFull, scale != 1.f)) break;
                 }
-                // O and S have been read: the next item's MMAs may overwrite them
+                // O has been read: the next item's P V may overwrite it
                 tc_fence_before();
                 mbar_arrive(bar(bar_item()));
                 if (row_ok && !direct) {
@@ -1608,8 +1624,6 @@ int forced_cluster(const int* resident, int cluster, int groups) {
     while (cluster > 1 && resident[cluster] < groups) --cluster;
     return cluster;
 }
-constexpr int kStreamGain = 3;  // key tiles a CTA must be spared before groups are cut at odd places
-
 // Nodes of the largest tree a context builds: min(max_tt, 1 + n_cand).
 int most_nodes(const resps_shape& s) {
     return static_cast<int>(std::min<int64_t>(s.max_tt, 1 + s.max_k + static_cast<int64_t>(s.max_depth - 1) * s.max_k * s.max_k));
@@ -1734,8 +1748,9 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
     a.clusters = a.cluster > 1 ? groups : hs->resident[1];
     const int grid = a.clusters * a.cluster;
     if (w.attn_rounds > 0 && a.cluster == 1) a.clusters = std::max(1, a.clusters / w.attn_rounds);
+    // one resident round of units with room for all of a group's partials, else more CTAs per SM
     a.comb_chunk = groups * (D / 8 / kCombPieces) <= ctx->sm_count ? kCombChunkMost : kCombChunk;
-    a.stream_gain = w.attn_stream >= 0 ? w.attn_stream : kStreamGain;
+    a.stream_gain = w.attn_stream;
     MapKey kk = {k_cache, stride_tok, stride_head, stride_seq, capacity, a.Hkv, batch, 0};
     MapKey kv = kk;
     kv.base = v_cache;

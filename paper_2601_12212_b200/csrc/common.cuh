@@ -47,7 +47,7 @@ struct Workspace {
     unsigned int* amax_seq_counter = nullptr;  // [max_batch] arg-max CTAs of a sequence that have delivered (self-resetting)
     // attention
     int attn_min_tiles = 2;     // fewest key tiles a CTA of a cluster is given
-    int attn_stream = -1;       // >= 0: key tiles a CTA must be spared for mode stream (tests)
+    int attn_stream = -1;       // 0: never equal splits per group, > 0: always where they fit (tests)
     int attn_cluster = 0;       // > 0: CTAs per cluster (tests)
     int attn_rounds = 0;        // > 0: the work list is cut for 1/n of the clusters (tests)
     int attn_max_items = 0;
