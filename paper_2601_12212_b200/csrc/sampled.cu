@@ -11,22 +11,26 @@
 //
 // All of it is a walk of at most max_depth + 1 nodes, but each step of the walk needs sums over the
 // whole vocabulary (normalisers of softmax and of residuals, the cumulative sum the token is drawn
-// from).  A thread-block cluster of 8 CTAs serves one sequence: every CTA takes an eighth of the
+// from).  A thread-block cluster of 16 CTAs serves one sequence: every CTA takes a sixteenth of the
 // vocabulary, every CTA writes its partial sums into every peer's shared memory behind the hardware
-// cluster barrier (no spinning anywhere), and every CTA then takes the same decision from the same
+// cluster barrier (no spinning anywhere), and every thread then takes the same decision from the same
 // numbers.  Arithmetic is fp64 throughout: a decision (accept or not, which token) is a comparison of
 // sums over 10^5 terms, and only at fp64 is the order of summation immaterial to it.
 //
-// The exponentials dominate, so each is taken once per visited node.  The target-side value P of
-// every token of the CTA's slice lives in shared memory (in an L2-resident scratch when the slice is
-// too large) and is brought up to date in place by the pass that needs it next -- first the division
-// by the softmax sum, then one rejection round per pass.  The draft side is the raw exponentials Q in
-// the scratch times one scalar (softmax sum and renormalisations are the same factor for every
-// token; a removed token's entry is set to zero), so a pass reads 8 bytes per token from L2 and
-// multiplies.  Only the thread that owns a token touches its values; (P, Q) of the current node's
-// children, which every CTA needs for the decisions, are copied by their owners into a small table
-// behind the same barrier that carries the sums (two tables in turn, so that a pass never writes the
-// one being read).
+// The exponentials are taken once per visited node.  The target-side value P and the raw draft-side
+// exponential Q of every token of the CTA's slice live in shared memory (what does not fit, in an
+// L2-resident scratch); token e belongs to thread e % 512, so rows are read once and coalesced and only the
+// owner touches a token's values.  The draft side is Q times one scalar (softmax sum and renormalisations
+// are the same factor for every token; a removed token's entry is set to zero).
+//
+// Bound by a chain of small steps: per node two row slices from HBM, 2 x 16 fp64 exponentials a thread and
+// three exchanges over the cluster (0.7 us each), per rejection one pass over shared memory and one exchange.
+// What is kept short: the children are found by ballots, their (P, Q) are pushed into every CTA's shared
+// memory behind the exchange's barrier, every thread takes the decision for itself, the rows of the child
+// that is tried first are asked into L2 while its parent is worked on, and the loops are short (the kernel
+// runs once per step: unrolled over the tokens it was 70 KB of code).  With clusters of 8 CTAs of 1024 threads,
+// the draft side in L2, one thread looking up children and deciding, the calls of TT=60 d=7 k=10 V=128256 took
+// 100 us.
 #include <cmath>
 
 #include "common.cuh"
@@ -34,8 +38,9 @@
 namespace resps {
 namespace {
 
-constexpr int kClu = 8;             // CTAs per sequence
-constexpr int kSampThreads = 1024;
+constexpr int kClu = 16;            // CTAs per sequence (more than 8: not portable, sm_100 has it)
+constexpr int kSampThreads = 512;
+constexpr int kWarps = kSampThreads / 32;
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
 struct SampledArgs {
@@ -53,14 +58,10 @@ struct SampledArgs {
     int vocab, max_tt, max_depth, max_k;
     int32_t *accept_path, *accept_len, *out_tokens;
     resps_step* steps_next;
-    double* scratch;  // [batch][kScratchPerSeq] small words, then [batch][kClu][2][per_thr * kSampThreads] (P, Q)
-    int64_t state_per_cta;  // doubles of one CTA's p (or q) array
-    int staged;             // 1: a row's slice fits the staging area in shared memory
-    int p_in_smem;          // 1: the target-side values live in shared memory (else in the scratch)
+    double* scratch;        // [batch][kClu][2][state] (P, Q) of tokens that do not fit shared memory
+    int64_t state;          // doubles of one CTA's P (or Q) array, padding included
+    int p_in_smem, q_in_smem;
 };
-constexpr int kTableAt = 4 * kClu + 8;
-constexpr int kScratchPerSeq = kTableAt + 2 * 2 * RESPS_MAX_K;  // two alternating sets of pairs of partials, the
-                                                                // drawn token, two alternating tables of the children's (p, q)
 
 __device__ __forceinline__ unsigned cluster_rank() {
     unsigned r;
@@ -74,57 +75,6 @@ __device__ __forceinline__ void cluster_barrier() {
 struct Pair {
     double x, y;
 };
-
-// Two sums (or two maxima) over the CTA at once, result in every thread.
-template <bool MAX>
-__device__ __forceinline__ Pair block_reduce2(Pair v, double* s_red) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double wx = __shfl_xor_sync(kFull, v.x, o), wy = __shfl_xor_sync(kFull, v.y, o);
-        v.x = MAX ? fmax(v.x, wx) : v.x + wx;
-        v.y = MAX ? fmax(v.y, wy) : v.y + wy;
-    }
-    __syncthreads();  // s_red is free again
-    if (lane == 0) s_red[2 * warp] = v.x, s_red[2 * warp + 1] = v.y;
-    __syncthreads();
-    Pair r = {s_red[0], s_red[1]};
-    for (int w = 1; w < kSampThreads / 32; ++w) {
-        r.x = MAX ? fmax(r.x, s_red[2 * w]) : r.x + s_red[2 * w];
-        r.y = MAX ? fmax(r.y, s_red[2 * w + 1]) : r.y + s_red[2 * w + 1];
-    }
-    return r;
-}
-
-// Store one double into the shared memory of CTA `peer` of the cluster, at the address `local` has here.
-__device__ __forceinline__ void store_to_peer(double* local, unsigned peer, double v) {
-    const uint32_t mine = static_cast<uint32_t>(__cvta_generic_to_shared(local));
-    uint32_t remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(mine), "r"(peer));
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(v) : "memory");
-}
-
-// The same over the cluster: every CTA writes its result into every peer's shared memory (slot
-// `rank` of `s_peer[set]`), the hardware cluster barrier orders the writes, and every thread adds the
-// eight up in rank order, so all CTAs hold the same bits.  `set` alternates between consecutive
-// reductions (a set is written again only after everyone has read it: the barrier of the reduction
-// in between).  The barrier also makes the children's table a pass has written visible to the cluster.
-template <bool MAX>
-__device__ __forceinline__ Pair cluster_reduce2(Pair v, double* s_red, double (*s_peer)[kClu][2], int& set, unsigned rank) {
-    const Pair mine = block_reduce2<MAX>(v, s_red);
-    if (threadIdx.x < kClu) {
-        store_to_peer(&s_peer[set][rank][0], threadIdx.x, mine.x);
-        store_to_peer(&s_peer[set][rank][1], threadIdx.x, mine.y);
-    }
-    cluster_barrier();
-    Pair r = {s_peer[set][0][0], s_peer[set][0][1]};
-    for (int c = 1; c < kClu; ++c) {
-        r.x = MAX ? fmax(r.x, s_peer[set][c][0]) : r.x + s_peer[set][c][0];
-        r.y = MAX ? fmax(r.y, s_peer[set][c][1]) : r.y + s_peer[set][c][1];
-    }
-    set ^= 1;
-    return r;
-}
 
 // What the stored target-side value of a token still lacks: the division by the softmax sum, or one
 // rejection round (Section 3.2, "Acceptance Criterion": target side -> normalised max(0, p - q)).  The
@@ -146,198 +96,214 @@ __device__ __forceinline__ double apply(const Pending& pd, double p, double q_ra
     return p;
 }
 
+struct SampledShared {
+    double red[kWarps][2];
+    double peer[2][kClu][2];      // the cluster's partial results, written by the peers (two sets in turn)
+    unsigned peer_max[kClu][2];
+    double tab[2][RESPS_MAX_K][2];   // (P, Q) of the children's tokens, written by their owners
+    double scan[kWarps];
+    double u[RESPS_MAX_K];
+    unsigned red_max[kWarps][2];
+    int tok[RESPS_MAX_TT], par[RESPS_MAX_TT], row[RESPS_MAX_TT], children[RESPS_MAX_TT];
+    int count[4];
+    int pick;
+};
+
+__device__ __forceinline__ uint32_t peer_address(const void* local, unsigned peer) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                 : "=r"(remote)
+                 : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(local))), "r"(peer));
+    return remote;
+}
+__device__ __forceinline__ void store_pair_to_peer(double* local, unsigned peer, double x, double y) {
+    asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(peer_address(local, peer)), "d"(x), "d"(y) : "memory");
+}
+// The part of [from, from + count) floats that the bulk prefetch can take (16-byte granular).
+__device__ __forceinline__ void prefetch_l2(const float* from, int count) {
+    const uintptr_t lo = (reinterpret_cast<uintptr_t>(from) + 15) & ~static_cast<uintptr_t>(15);
+    const uintptr_t hi = reinterpret_cast<uintptr_t>(from + count) & ~static_cast<uintptr_t>(15);
+    if (hi > lo)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(lo), "r"(static_cast<uint32_t>(hi - lo)) : "memory");
+}
+
 __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const SampledArgs a) {
     pdl_wait();  // the kernel before this one in the stream has completed
     pdl_launch_dependents();
-    __shared__ double s_red[2 * (kSampThreads / 32)];
-    __shared__ double s_scan[kSampThreads / 32];
-    __shared__ double s_peer[2][kClu][2];  // the cluster's partial results, written by the peers
-    __shared__ int s_tok[RESPS_MAX_TT], s_par[RESPS_MAX_TT];
-    __shared__ int s_children[RESPS_MAX_TT];
-    __shared__ int s_decision;                  // accepted child, or -1
-    __shared__ int s_nchild;
+    __shared__ SampledShared sh;
+    extern __shared__ __align__(16) unsigned char s_dyn[];
     const unsigned rank = cluster_rank();
-    const int b = blockIdx.x / kClu, tid = threadIdx.x;
+    const int b = blockIdx.x / kClu, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = min(max(a.n_nodes[b], 1), a.max_tt);
     const int64_t ob = static_cast<int64_t>(b) * a.max_tt;
     const int cap = a.max_depth + 1;
-    double* scratch = a.scratch + static_cast<int64_t>(b) * kScratchPerSeq;
-    int set = 0;
-    if (tid < n) s_tok[tid] = a.tokens[ob + tid], s_par[tid] = a.parent[ob + tid];
+    if (tid < RESPS_MAX_TT) {
+        sh.tok[tid] = (tid < n) ? a.tokens[ob + tid] : -1;
+        sh.par[tid] = (tid < n) ? a.parent[ob + tid] : -2;
+        sh.row[tid] = (tid < n) ? a.node_row[ob + tid] : -1;
+    }
     if (rank == 0 && tid < cap) {
         a.accept_path[b * cap + tid] = (tid == 0) ? 0 : -1;
         a.out_tokens[b * cap + tid] = -1;
     }
+    if (tid == 0) sh.pick = -1;
     __syncthreads();
-    // this CTA's share of the vocabulary, and inside it this thread's contiguous run
-    const int V = a.vocab;
-    const int per_cta = (V + kClu - 1) / kClu;
-    const int c_lo = min(V, static_cast<int>(rank) * per_cta), c_hi = min(V, c_lo + per_cta);
-    const int per_thr = (per_cta + kSampThreads - 1) / kSampThreads;
-    const int t_lo = min(c_hi, c_lo + tid * per_thr), t_hi = min(c_hi, t_lo + per_thr);
-    // Target-side value P and raw draft-side weight Q of the token at place i of thread t's run: element
-    // i * threads + t of the owning CTA's arrays, so that a warp's accesses of one pass are contiguous.
-    // Q lives in the L2-resident scratch; P in shared memory when the slice fits, else in the scratch too.
-    extern __shared__ __align__(16) unsigned char s_dyn[];
-    double* state0 = a.scratch + static_cast<int64_t>(gridDim.x / kClu) * kScratchPerSeq +
-                     (static_cast<int64_t>(b) * kClu + rank) * 2 * a.state_per_cta;
-    double* P = a.p_in_smem ? reinterpret_cast<double*>(s_dyn) : state0;
-    double* Q = state0 + a.state_per_cta;
-    float* s_stage = reinterpret_cast<float*>(s_dyn + (a.p_in_smem ? sizeof(double) * a.state_per_cta : 0));  // [threads][per_thr + 1]
-    double* table = scratch + kTableAt;  // [2][RESPS_MAX_K][2]
-    // After a pass (and a CTA barrier): the owners copy (P, Q) of the children's tokens into table `par`.
-    auto publish_children = [&](int par, int n_child) {
+    // this CTA's share of the vocabulary; token e of it belongs to thread e % 512, place e / 512
+    const int V = a.vocab, per_cta = (V + kClu - 1) / kClu;
+    const int c_lo = min(V, static_cast<int>(rank) * per_cta), n_cta = min(V, c_lo + per_cta) - c_lo;
+    const int per = (n_cta + kSampThreads - 1) / kSampThreads;  // places
+    // (a padded place per 16: the runs of the draw would otherwise meet on the same banks)
+    auto at = [](int e) { return e + (e >> 4); };
+    double* const own = a.scratch + (static_cast<int64_t>(b) * kClu + rank) * 2 * a.state;
+    double* const P = a.p_in_smem ? reinterpret_cast<double*>(s_dyn) : own;
+    double* const Q = a.q_in_smem ? reinterpret_cast<double*>(s_dyn) + a.state : own + a.state;
+    int set = 0;
+    // two sums over the cluster, the same bits in every thread of every CTA
+    auto cluster_sum = [&](double x, double y) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o), y += __shfl_xor_sync(kFull, y, o);
+        if (lane == 0) sh.red[warp][0] = x, sh.red[warp][1] = y;
         __syncthreads();
-        if (tid < n_child && tid < RESPS_MAX_K) {
-            const int x = s_tok[s_children[tid]];
-            if (x >= c_lo && x < c_hi) {
-                const int in_cta = x - c_lo, t = in_cta / per_thr, i = in_cta - t * per_thr;
-                double* dst = table + (par * RESPS_MAX_K + tid) * 2;
-                __stcg(dst, P[static_cast<int64_t>(i) * kSampThreads + t]);
-                __stcg(dst + 1, __ldcg(Q + static_cast<int64_t>(i) * kSampThreads + t));
-            }
+        if (warp == 0) {
+            x = (lane < kWarps) ? sh.red[lane][0] : 0.0, y = (lane < kWarps) ? sh.red[lane][1] : 0.0;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o), y += __shfl_xor_sync(kFull, y, o);
+            if (lane < kClu) store_pair_to_peer(sh.peer[set][rank], lane, x, y);
         }
+        cluster_barrier();
+        Pair r = {0.0, 0.0};
+#pragma unroll 4
+        for (int c = 0; c < kClu; ++c) r.x += sh.peer[set][c][0], r.y += sh.peer[set][c][1];
+        set ^= 1;
+        return r;
     };
-    // The CTA's slice of a row through the staging area: coalesced loads (consecutive threads, consecutive
-    // tokens), token e of the slice parked at [e / per_thr][e % per_thr] with a padded row, from where
-    // every thread reads its own run without bank conflicts.  Returns the maximum this thread saw.
-    auto stage_row = [&](const float* row, bool store) {
-        constexpr int kGroup = 8;  // loads in flight per thread
-        const int n_cta = c_hi - c_lo;
-        float fm = -INFINITY;
-        for (int e0 = tid; e0 < n_cta; e0 += kGroup * kSampThreads) {
-            float x[kGroup];
-#pragma unroll
-            for (int u = 0; u < kGroup; ++u) {
-                const int e = e0 + u * kSampThreads;
-                x[u] = (e < n_cta) ? __ldg(row + c_lo + e) : -INFINITY;
-            }
-#pragma unroll
-            for (int u = 0; u < kGroup; ++u) {
-                const int e = e0 + u * kSampThreads;
-                if (e >= n_cta) break;
-                if (store) {
-                    const int t = e / per_thr, i = e - t * per_thr;
-                    s_stage[t * (per_thr + 1) + i] = x[u];
-                }
-                fm = fmaxf(fm, x[u]);
-            }
-        }
-        return fm;
+    auto drow_of = [&](int node) {
+        const int row = sh.row[node];
+        return a.draft + b * a.dld_b + (row / RESPS_MAX_K) * a.dld_level + (row % RESPS_MAX_K) * a.dld_row;
     };
 
     int cur = 0, acc = 0;
     for (;;) {
-        const float* trow = a.target + b * a.ld_b + cur * a.ld_row;
-        // ---- the children of the current node, in node order --------------------------------------
-        if (tid == 0) {
-            int m = 0;
-            if (acc < a.max_depth)  // (the path array holds max_depth + 1 nodes; a tree is never deeper)
-                for (int c = 1; c < n; ++c)
-                    if (s_par[c] == cur) s_children[m++] = c;
-            s_nchild = m;
-        }
-        __syncthreads();  // (also: the previous node's readers are done with the staging area)
-        const int n_child = s_nchild;
-        const float* drow = nullptr;
-        if (n_child > 0) {
-            const int row = a.node_row[ob + cur];  // >= 0 for a node with children
-            drow = a.draft + b * a.dld_b + (row / RESPS_MAX_K) * a.dld_level + (row % RESPS_MAX_K) * a.dld_row;
-        }
-        // ---- P_T(. | cur) = softmax(row / T) and the draft's P_d: maxima, then the exponentials (stored)
-        // and their sums.  The staging area holds one row at a time: the target's while the maxima are
-        // taken (the draft row is only looked at), then the draft's (read again, from L2) -------------
-        float fm_t = -INFINITY, fm_d = -INFINITY;
-        if (a.staged) {
-            fm_t = stage_row(trow, true);
-            if (drow) fm_d = stage_row(drow, false);
-        } else {
-            for (int v = t_lo; v < t_hi; ++v) {
-                fm_t = fmaxf(fm_t, __ldg(trow + v));
-                if (drow) fm_d = fmaxf(fm_d, __ldg(drow + v));
-            }
-        }
-        // (the reduction's barriers also order the staging area)
-        const Pair mx = cluster_reduce2<true>(Pair{static_cast<double>(fm_t), static_cast<double>(fm_d)}, s_red, s_peer,
-                                              set, rank);
-        const double mx_t = mx.x * a.inv_t, mx_d = mx.y * a.inv_t;
-        Pair sum = {0.0, 0.0};
-        for (int v = t_lo, i = 0; v < t_hi; ++v, ++i) {
-            const float xt = a.staged ? s_stage[tid * (per_thr + 1) + i] : __ldg(trow + v);
-            const double wt = exp(static_cast<double>(xt) * a.inv_t - mx_t);
-            P[static_cast<int64_t>(i) * kSampThreads + tid] = wt;
-            sum.x += wt;
-        }
-        if (drow) {
-            if (a.staged) {
-                __syncthreads();  // everyone has read the target row
-                stage_row(drow, true);
-                __syncthreads();
-            }
-            for (int v = t_lo, i = 0; v < t_hi; ++v, ++i) {
-                const float xd = a.staged ? s_stage[tid * (per_thr + 1) + i] : __ldg(drow + v);
-                const double wd = exp(static_cast<double>(xd) * a.inv_t - mx_d);
-                __stcg(Q + static_cast<int64_t>(i) * kSampThreads + tid, wd);
-                sum.y += wd;
-            }
-        }
-        publish_children(0, n_child);
-        sum = cluster_reduce2<false>(sum, s_red, s_peer, set, rank);
-        Pending pend = {1, recip_or_zero(sum.x), 0.0, -1};
-        double sq = drow ? recip_or_zero(sum.y) : 0.0;  // draft side: q = Q * sq
-        // One pass over this thread's tokens: bring P up to date in place (and retire the token the pending
-        // round removed), hand the current (p, q) of each token to `f`.  The draft side is only read at
-        // nodes that have children (`with_q`); a leaf has no draft row.
-        auto pass = [&](bool with_q, auto&& f) {
-            constexpr int kGroup = 4;  // draft-side values fetched together: their loads are in flight at once
-            for (int v0 = t_lo, i0 = 0; v0 < t_hi; v0 += kGroup, i0 += kGroup) {
-                double q_raw[kGroup];
+        // ---- the rows of the current node: loads in flight while its children are looked up --------------
+        const float* trow = a.target + b * a.ld_b + cur * a.ld_row + c_lo;
+        const bool maybe_d = sh.row[cur] >= 0;  // a node with children was expanded
+        const float* drow = drow_of(maybe_d ? cur : 0) + c_lo;
+        float ft = -INFINITY, fd = -INFINITY;
+        constexpr int kGroup = 8;  // of each row, in flight together
+#pragma unroll 1
+        for (int e0 = tid; e0 < n_cta; e0 += kGroup * kSampThreads) {
+            float xt[kGroup], xd[kGroup];
 #pragma unroll
-                for (int u = 0; u < kGroup; ++u)
-                    q_raw[u] = (with_q && v0 + u < t_hi) ? __ldcg(Q + static_cast<int64_t>(i0 + u) * kSampThreads + tid) : 0.0;
+            for (int u = 0; u < kGroup; ++u) {
+                const int e = e0 + u * kSampThreads;
+                xt[u] = (e < n_cta) ? __ldg(trow + e) : -INFINITY;
+                xd[u] = (e < n_cta && maybe_d) ? __ldg(drow + e) : -INFINITY;
+            }
 #pragma unroll
-                for (int u = 0; u < kGroup; ++u) {
-                    const int v = v0 + u;
-                    if (v >= t_hi) break;
-                    double* pp = P + static_cast<int64_t>(i0 + u) * kSampThreads + tid;
-                    double p = *pp;
-                    if (pend.kind) {
-                        p = apply(pend, p, q_raw[u]);
-                        *pp = p;
-                        if (pend.kind == 2 && v == pend.x) {
-                            __stcg(Q + static_cast<int64_t>(i0 + u) * kSampThreads + tid, 0.0);
-                            q_raw[u] = 0.0;
-                        }
-                    }
-                    f(v, p, q_raw[u] * sq);
-                }
+            for (int u = 0; u < kGroup; ++u) {
+                const int e = e0 + u * kSampThreads;
+                ft = fmaxf(ft, xt[u]), fd = fmaxf(fd, xd[u]);
+                if (e < n_cta) P[at(e)] = static_cast<double>(xt[u]), Q[at(e)] = static_cast<double>(xd[u]);
+            }
+        }
+        // ---- the children of the current node, in node order ----------------------------------------------
+        // (the path array holds max_depth + 1 nodes; a tree is never deeper)
+        const bool is_child = tid > 0 && tid < n && sh.par[tid & (RESPS_MAX_TT - 1)] == cur && acc < a.max_depth;
+        const unsigned bal = __ballot_sync(kFull, is_child);
+        if (warp < 4 && lane == 0) sh.count[warp] = __popc(bal);
+        __syncthreads();  // (everyone is done with the previous node's children)
+        int n_child = 0;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            if (is_child && w == warp) sh.children[n_child + __popc(bal & ((1u << lane) - 1u))] = tid;
+            n_child += sh.count[w];
+        }
+        if (tid < n_child && tid < a.max_k && tid < RESPS_MAX_K)
+            sh.u[tid] = a.u_accept[(static_cast<int64_t>(b) * cap + acc) * a.max_k + tid];
+        const bool with_q = n_child > 0;
+        // ---- P_T(. | cur) = softmax(row / T) and the draft's P_d: maxima, exponentials, sums ------------------
+        const unsigned mt = __reduce_max_sync(kFull, float_to_ordered(ft)), md = __reduce_max_sync(kFull, float_to_ordered(fd));
+        if (lane == 0) sh.red_max[warp][0] = mt, sh.red_max[warp][1] = md;
+        __syncthreads();
+        if (warp == 0) {
+            const unsigned wt = __reduce_max_sync(kFull, lane < kWarps ? sh.red_max[lane][0] : 0u);
+            const unsigned wd = __reduce_max_sync(kFull, lane < kWarps ? sh.red_max[lane][1] : 0u);
+            if (lane < kClu)
+                asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(peer_address(sh.peer_max[rank], lane)), "r"(wt), "r"(wd)
+                             : "memory");
+            // the rows of the child that is tried first
+            if (lane == 0 && with_q) {
+                const int child = sh.children[0];
+                prefetch_l2(a.target + b * a.ld_b + child * a.ld_row + c_lo, n_cta);
+                if (sh.row[child] >= 0) prefetch_l2(drow_of(child) + c_lo, n_cta);
+            }
+        }
+        cluster_barrier();
+        unsigned top_t = 0u, top_d = 0u;
+#pragma unroll 4
+        for (int c = 0; c < kClu; ++c) top_t = max(top_t, sh.peer_max[c][0]), top_d = max(top_d, sh.peer_max[c][1]);
+        const double mx_t = static_cast<double>(ordered_to_float(top_t)) * a.inv_t;
+        const double mx_d = static_cast<double>(ordered_to_float(top_d)) * a.inv_t;
+        double sum_t = 0.0, sum_d = 0.0;
+#pragma unroll 2
+        for (int e = tid; e < n_cta; e += kSampThreads) {
+            const double w = exp(P[at(e)] * a.inv_t - mx_t);
+            P[at(e)] = w;
+            sum_t += w;
+        }
+        if (with_q) {
+#pragma unroll 2
+            for (int e = tid; e < n_cta; e += kSampThreads) {
+                const double w = exp(Q[at(e)] * a.inv_t - mx_d);
+                Q[at(e)] = w;
+                sum_d += w;
+            }
+        }
+        // The owners of the children's tokens push (P, Q) into table `par` of every CTA, behind the barrier of
+        // the reduction that follows.
+        auto publish_children = [&](int par, int from) {
+#pragma unroll 1
+            for (int j = from; j < n_child && j < RESPS_MAX_K; ++j) {
+                const int e = sh.tok[sh.children[j]] - c_lo;
+                if (e < 0 || e >= n_cta || e % kSampThreads != tid) continue;
+                const double p = P[at(e)], q = Q[at(e)];
+#pragma unroll 1
+                for (int c = 0; c < kClu; ++c) store_pair_to_peer(sh.tab[par][j], c, p, q);
             }
         };
-        // ---- try the children ---------------------------------------------------------------------
+        publish_children(0, 0);
+        const Pair sum = cluster_sum(sum_t, sum_d);
+        // What P (and the table's entries) still lack; a pass brings P up to date.
+        Pending pend = {1, recip_or_zero(sum.x), 0.0, -1};
+        double sq = with_q ? recip_or_zero(sum.y) : 0.0;     // draft side: q = Q * sq
+        // ---- try the children -----------------------------------------------------------------------------
         int next = -1;
+#pragma unroll 1
         for (int j = 0; j < n_child && j < a.max_k; ++j) {
-            const int child = s_children[j];
-            const int x = s_tok[child];
-            if (tid == 0) {
-                // (P, Q) of child j's token as the last pass left them, brought up to date here
-                const double* at = table + ((j & 1) * RESPS_MAX_K + j) * 2;
-                const double q_raw = __ldcg(at + 1);
-                const double p = apply(pend, __ldcg(at), q_raw), q = q_raw * sq;
+            const int child = sh.children[j];
+            {
+                const double q_raw = sh.tab[j & 1][j][1];
+                const double p = apply(pend, sh.tab[j & 1][j][0], q_raw), q = q_raw * sq;
                 const double alpha = q > 0.0 ? fmin(1.0, p / q) : (p > 0.0 ? 1.0 : 0.0);
-                const double u = a.u_accept[(static_cast<int64_t>(b) * cap + acc) * a.max_k + j];
-                s_decision = (u < alpha) ? child : -1;
+                if (sh.u[j] < alpha) next = child;
             }
-            __syncthreads();
-            next = s_decision;
             if (next >= 0) break;
             // rejected: the residual's normaliser and the draft mass that is left without x
-            Pair zr = {0.0, 0.0};
-            pass(true, [&](int v, double p, double q) {
-                zr.x += fmax(p - q, 0.0);
-                if (v != x) zr.y += q;
-            });
-            publish_children((j + 1) & 1, n_child);
-            zr = cluster_reduce2<false>(zr, s_red, s_peer, set, rank);
+            const int x = sh.tok[child], at_x = x - c_lo;
+            double zx = 0.0, zy = 0.0;
+            // (the pass applies what is pending, and retires the token the round before removed)
+#pragma unroll 4
+            for (int e = tid; e < n_cta; e += kSampThreads) {
+                double q_raw = Q[at(e)];
+                const double p = apply(pend, P[at(e)], q_raw);
+                P[at(e)] = p;
+                if (pend.kind == 2 && e == pend.x - c_lo) Q[at(e)] = q_raw = 0.0;
+                const double q = q_raw * sq;
+                zx += fmax(p - q, 0.0);
+                zy += (e != at_x) ? q : 0.0;
+            }
+            publish_children((j + 1) & 1, j + 1);
+            const Pair zr = cluster_sum(zx, zy);
             pend = Pending{2, recip_or_zero(zr.x), sq, x};
             if (zr.y > 0.0) sq = sq * (1.0 / zr.y);
         }
@@ -346,61 +312,63 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
             ++acc;
             if (rank == 0 && tid == 0) {
                 a.accept_path[b * cap + acc] = cur;
-                a.out_tokens[b * cap + acc - 1] = s_tok[cur];
+                a.out_tokens[b * cap + acc - 1] = sh.tok[cur];
             }
-            continue;  // (the next node's first reduction is a cluster barrier before anything is overwritten)
+            continue;
         }
-        // ---- nobody accepted (or a leaf): draw from the current target-side distribution --------------
-        // inverse CDF in token order: this thread's run, the runs before it in the CTA, the CTAs before it
+        // ---- nobody accepted (or a leaf): draw from the current target-side distribution by inverse CDF in
+        // token order: the tokens change hands so that a thread holds a contiguous run --------------------------
+#pragma unroll 4
+        for (int e = tid; e < n_cta; e += kSampThreads) P[at(e)] = apply(pend, P[at(e)], with_q ? Q[at(e)] : 0.0);
+        __syncthreads();
+        const int t_lo = min(n_cta, tid * per), t_hi = min(n_cta, t_lo + per);
         double run = 0.0;
-        pass(drow != nullptr, [&](int, double p, double) { run += p; });
-        pend.kind = 0;
-        // exclusive prefix of the runs over the CTA's threads
-        const int lane = tid & 31, warp = tid >> 5;
-        double inc = run;
+#pragma unroll 4
+        for (int e = t_lo; e < t_hi; ++e) run += P[at(e)];
+        double inc = run;  // exclusive prefix of the runs over the CTA's threads
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const double w = __shfl_up_sync(kFull, inc, o);
             if (lane >= o) inc += w;
         }
-        __syncthreads();
-        if (lane == 31) s_scan[warp] = inc;
+        if (lane == 31) sh.scan[warp] = inc;
         __syncthreads();
         double before = 0.0, cta_total = 0.0;
-        for (int w = 0; w < kSampThreads / 32; ++w) {
-            if (w < warp) before += s_scan[w];
-            cta_total += s_scan[w];
+#pragma unroll 4
+        for (int w = 0; w < kWarps; ++w) {
+            if (w < warp) before += sh.scan[w];
+            cta_total += sh.scan[w];
         }
         const double excl = before + inc - run;
-        if (tid < kClu) store_to_peer(&s_peer[set][rank][0], tid, cta_total);
-        if (rank == 0 && tid == 0) __stcg(scratch + 4 * kClu, -1.0);
+        if (tid < kClu) store_pair_to_peer(sh.peer[set][rank], tid, cta_total, 0.0);
         cluster_barrier();
         double offset = 0.0, total = 0.0;
+#pragma unroll 4
         for (int c = 0; c < kClu; ++c) {
-            const double t = s_peer[set][c][0];
+            const double t = sh.peer[set][c][0];
             if (c < static_cast<int>(rank)) offset += t;
             total += t;
         }
-        set ^= 1;
         const double target = a.u_sample[static_cast<int64_t>(b) * cap + acc] * total;
         // the owner of the target: the last non-empty run that starts at or before it
         const double start = offset + excl;
-        const bool last_run = (t_hi == V) && (t_lo < t_hi);
+        const bool last_run = t_lo < t_hi && c_lo + t_hi == V;
         if (t_lo < t_hi && start <= target && (start + run > target || last_run)) {
             double cum = start;
             int pick = t_hi - 1;
-            for (int v = t_lo, i = 0; v < t_hi; ++v, ++i) {
-                cum += P[static_cast<int64_t>(i) * kSampThreads + tid];  // (up to date since the pass above)
+#pragma unroll 1
+            for (int e = t_lo; e < t_hi; ++e) {
+                cum += P[at(e)];
                 if (cum > target) {
-                    pick = v;
+                    pick = e;
                     break;
                 }
             }
-            __stcg(scratch + 4 * kClu, static_cast<double>(pick));
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_address(&sh.pick, 0u)), "r"(c_lo + pick) : "memory");
         }
         cluster_barrier();
         if (rank == 0 && tid == 0) {
-            int tok = static_cast<int>(__ldcg(scratch + 4 * kClu));
+            int tok = sh.pick;
             if (tok < 0) tok = V - 1;  // rounding left the target past every run: the last token
             a.out_tokens[b * cap + acc] = tok;
             a.accept_len[b] = acc;
@@ -412,34 +380,26 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
         }
         break;
     }
-    cluster_barrier();  // nobody leaves while a peer may still be at the barrier before
+    // (the barrier before is the last access to a peer's shared memory)
 }
 
 }  // namespace
 
-constexpr size_t kDynSmemCap = 220 * 1024;
-static int sampled_per_thr(int vocab) {
-    const int per_cta = (vocab + kClu - 1) / kClu;
-    return (per_cta + kSampThreads - 1) / kSampThreads;
-}
-static size_t sampled_stage_bytes(int vocab) {  // one row's slice, padded rows
-    return sizeof(float) * kSampThreads * static_cast<size_t>(sampled_per_thr(vocab) + 1);
-}
-static size_t sampled_p_bytes(int vocab) { return sizeof(double) * kSampThreads * static_cast<size_t>(sampled_per_thr(vocab)); }
+constexpr size_t kDynSmemCap = 216 * 1024;
 
-cudaError_t sampled_setup(resps_ctx*) {
-    return cudaFuncSetAttribute(accept_sampled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(kDynSmemCap));
-}
-
-static int64_t sampled_state_per_cta(int vocab) {
+static int64_t sampled_state(int vocab) {  // padded doubles of one CTA's slice
     const int per_cta = (vocab + kClu - 1) / kClu;
-    const int per_thr = (per_cta + kSampThreads - 1) / kSampThreads;
-    return static_cast<int64_t>(per_thr) * kSampThreads;
+    return per_cta + per_cta / 16 + 2;
 }
 
 size_t sampled_scratch_doubles(int max_batch, int vocab) {
-    return static_cast<size_t>(max_batch) * (kScratchPerSeq + kClu * 2 * sampled_state_per_cta(vocab));
+    return static_cast<size_t>(max_batch) * kClu * 2 * sampled_state(vocab);
+}
+
+cudaError_t sampled_setup(resps_ctx*) {
+    cudaError_t e = cudaFuncSetAttribute(accept_sampled_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(accept_sampled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kDynSmemCap));
 }
 
 cudaError_t launch_accept_sampled(const resps_ctx* ctx, const resps_step* d_steps, const int32_t* d_n_nodes, int batch,
@@ -459,11 +419,11 @@ cudaError_t launch_accept_sampled(const resps_ctx* ctx, const resps_step* d_step
     a.max_k = ctx->shape.max_k;
     a.accept_path = accept_path, a.accept_len = accept_len, a.out_tokens = out_tokens, a.steps_next = steps_next;
     a.scratch = ctx->ws.samp_scratch;
-    a.state_per_cta = sampled_state_per_cta(ctx->shape.vocab);
-    const size_t stage_bytes = sampled_stage_bytes(ctx->shape.vocab), p_bytes = sampled_p_bytes(ctx->shape.vocab);
-    a.p_in_smem = (p_bytes + stage_bytes <= kDynSmemCap) ? 1 : 0;
-    a.staged = ((a.p_in_smem ? p_bytes : 0) + stage_bytes <= kDynSmemCap) ? 1 : 0;
-    const size_t dyn_bytes = (a.p_in_smem ? p_bytes : 0) + (a.staged ? stage_bytes : 0);
+    a.state = sampled_state(ctx->shape.vocab);
+    const size_t side = sizeof(double) * static_cast<size_t>(a.state);  // both sides fit up to a vocabulary of 208 000
+    a.p_in_smem = side <= kDynSmemCap ? 1 : 0;
+    a.q_in_smem = 2 * side <= kDynSmemCap ? 1 : 0;
+    const size_t dyn_bytes = a.q_in_smem ? 2 * side : a.p_in_smem ? side : 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(batch * kClu), cfg.blockDim = dim3(kSampThreads), cfg.dynamicSmemBytes = dyn_bytes, cfg.stream = st;
     cudaLaunchAttribute attr[2];
