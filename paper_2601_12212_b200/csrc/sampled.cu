@@ -24,11 +24,12 @@
 // are the same factor for every token; a removed token's entry is set to zero).
 //
 // Bound by a chain of small steps: per node two row slices from HBM, 2 x 16 fp64 exponentials a thread and
-// three exchanges over the cluster (0.7 us each), per rejection one pass over shared memory and one exchange.
+// one exchange over the cluster (1.3 us), per rejection one pass over shared memory and one exchange.
 // What is kept short: the children are found by ballots, their (P, Q) are pushed into every CTA's shared
 // memory behind the exchange's barrier, every thread takes the decision for itself, the rows of the child
 // that is tried first are asked into L2 while its parent is worked on, and the loops are short (the kernel
-// runs once per step: unrolled over the tokens it was 70 KB of code).  With clusters of 8 CTAs of 1024 threads,
+// runs once per step: unrolled over the tokens it was 70 KB of code).  The exponentials are relative to the CTA's
+// own maximum, so that maxima and sums cross the cluster together.  With clusters of 8 CTAs of 1024 threads,
 // the draft side in L2, one thread looking up children and deciding, the calls of TT=60 d=7 k=10 V=128256 took
 // 100 us.
 #include <cmath>
@@ -76,35 +77,60 @@ struct Pair {
     double x, y;
 };
 
+// e^t for t <= 0 (below -700: 0), to about one unit in the last place: table-driven (P. Tang, "Table-driven
+// implementation of the exponential function in IEEE floating-point arithmetic", 1989).  t = k ln2/64 + r,
+// |r| <= ln2/128, e^t = 2^(k/64) e^r with 2^(i/64) from a table in shared memory and five terms of the series
+// for e^r - 1 (the next one is below 4e-17).  11 fp64 operations, half of what exp() takes for its full range.
+constexpr int kExpTable = 64;
+__device__ __forceinline__ double exp_le0(double t, const double* table) {
+    constexpr double kMagic = 6755399441055744.0;  // 1.5 * 2^52: the sum's low word is the rounded integer
+    const double biased = fma(t, 92.33248261689366, kMagic);  // 64 / ln 2
+    const int k = __double2loint(biased);
+    const double kd = biased - kMagic;
+    double r = fma(kd, -0.010830424696249145, t);  // ln 2 / 64, rounded,
+    r = fma(kd, -3.623510646634843e-19, r);        // and the rest of it
+    double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+    q = fma(q, r, 1.0 / 6.0);
+    q = fma(q, r, 0.5);
+    q = fma(q, r, 1.0) * r;
+    const double head = table[k & (kExpTable - 1)];
+    const double y = fma(head, q, head);  // about 2^(k/64 mod 1) e^r: 2^(k >> 6) goes into its exponent
+    const double v = __hiloint2double(__double2hiint(y) + ((k >> 6) << 20), __double2loint(y));
+    return t > -700.0 ? v : 0.0;
+}
+
 // What the stored target-side value of a token still lacks: the division by the softmax sum, or one
 // rejection round (Section 3.2, "Acceptance Criterion": target side -> normalised max(0, p - q)).  The
 // draft side is kept as the raw exponentials times one scalar for the whole row (the softmax sum and
 // the renormalisations after every removal are the same factor for every token), with the entry of
 // a removed token set to zero.
 struct Pending {
-    int kind;      // 0 nothing, 1 softmax sum, 2 a rejection round
+    int kind;      // 1 the softmax sum, 2 a rejection round
     double a;      // reciprocal of the target's sum (kind 1) / of the residual's normaliser (kind 2; 0: residual empty, p is kept)
     double sq_old; // kind 2: the draft side's scalar as it was when the round's child was tried
-    int x;         // kind 2: the rejected token
 };
 // A division by a normaliser is a multiplication by its fp64 reciprocal (one rounding more than the
 // quotient; the decisions compare sums of 10^5 such terms and are taken with a margin far above that).
 __device__ __forceinline__ double recip_or_zero(double s) { return s > 0.0 ? 1.0 / s : 0.0; }
-__device__ __forceinline__ double apply(const Pending& pd, double p, double q_raw) {
-    if (pd.kind == 1) return p * pd.a;
-    if (pd.kind == 2 && pd.a > 0.0) return fmax(p - q_raw * pd.sq_old, 0.0) * pd.a;
-    return p;
+// `factor` puts a softmax weight on the row's scale (kind 1); q_raw is on it already.
+__device__ __forceinline__ double apply(const Pending& pd, double p, double factor, double q_raw) {
+    if (pd.kind == 1) return p * (factor * pd.a);
+    return pd.a > 0.0 ? fmax(p - q_raw * pd.sq_old, 0.0) * pd.a : p;
 }
 
 struct SampledShared {
+    double exp2_64[kExpTable];       // 2^(i/64)
     double red[kWarps][2];
-    double peer[2][kClu][2];      // the cluster's partial results, written by the peers (two sets in turn)
-    unsigned peer_max[kClu][2];
+    double peer[2][kClu][2];         // the cluster's partial results, written by the peers (two sets in turn)
+    double peer_max[kClu][2];        // ... and the maxima they are relative to, times 1 / T
+    double factor[kClu][2];          // e^(a CTA's maximum - the row's)
     double tab[2][RESPS_MAX_K][2];   // (P, Q) of the children's tokens, written by their owners
     double scan[kWarps];
     double u[RESPS_MAX_K];
     unsigned red_max[kWarps][2];
     int tok[RESPS_MAX_TT], par[RESPS_MAX_TT], row[RESPS_MAX_TT], children[RESPS_MAX_TT];
+    int child_at[RESPS_MAX_K];       // a child's token in this CTA's slice, -1: not here
+    int child_clu[RESPS_MAX_K];      // the CTA that has it
     int count[4];
     int pick;
 };
@@ -147,6 +173,7 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
         a.out_tokens[b * cap + tid] = -1;
     }
     if (tid == 0) sh.pick = -1;
+    if (tid < kExpTable) sh.exp2_64[tid] = exp2(static_cast<double>(tid) / kExpTable);
     __syncthreads();
     // this CTA's share of the vocabulary; token e of it belongs to thread e % 512, place e / 512
     const int V = a.vocab, per_cta = (V + kClu - 1) / kClu;
@@ -158,8 +185,11 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
     double* const P = a.p_in_smem ? reinterpret_cast<double*>(s_dyn) : own;
     double* const Q = a.q_in_smem ? reinterpret_cast<double*>(s_dyn) + a.state : own + a.state;
     int set = 0;
-    // two sums over the cluster, the same bits in every thread of every CTA
-    auto cluster_sum = [&](double x, double y) {
+    int cur = 0, acc = 0, n_child = 0;
+    // Two sums over the cluster, the same bits in every thread of every CTA.  Meanwhile (P, Q) of the children's
+    // tokens from `from` on, as the pass before left them, go into table `par` of every CTA.  At the start of a
+    // node the maxima travel along, and the sums are put on the row's common scale.
+    auto cluster_sum = [&](double x, double y, int par, int from, bool at_start, double max_t, double max_d) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o), y += __shfl_xor_sync(kFull, y, o);
         if (lane == 0) sh.red[warp][0] = x, sh.red[warp][1] = y;
@@ -168,12 +198,38 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
             x = (lane < kWarps) ? sh.red[lane][0] : 0.0, y = (lane < kWarps) ? sh.red[lane][1] : 0.0;
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o), y += __shfl_xor_sync(kFull, y, o);
-            if (lane < kClu) store_pair_to_peer(sh.peer[set][rank], lane, x, y);
+            if (lane < kClu) {
+                store_pair_to_peer(sh.peer[set][rank], lane, x, y);
+                if (at_start) store_pair_to_peer(sh.peer_max[rank], lane, max_t, max_d);
+            }
+        } else if (warp == 1 && lane >= from && lane < n_child) {
+            const int e = sh.child_at[lane];
+            if (e >= 0) {
+                const double p = P[at(e)], q = Q[at(e)];
+#pragma unroll 1
+                for (int c = 0; c < kClu; ++c) store_pair_to_peer(sh.tab[par][lane], c, p, q);
+            }
         }
+        __syncwarp();
         cluster_barrier();
         Pair r = {0.0, 0.0};
+        if (at_start) {
+            if (tid < 2 * kClu) {
+                const int side = tid & 1;
+                double top = -INFINITY;
 #pragma unroll 4
-        for (int c = 0; c < kClu; ++c) r.x += sh.peer[set][c][0], r.y += sh.peer[set][c][1];
+                for (int c = 0; c < kClu; ++c) top = fmax(top, sh.peer_max[c][side]);
+                // (a CTA without tokens, or no draft row: nothing to scale)
+                const double m = sh.peer_max[tid >> 1][side];
+                sh.factor[tid >> 1][side] = m > -INFINITY ? exp_le0(m - top, sh.exp2_64) : 0.0;
+            }
+            __syncthreads();
+#pragma unroll 4
+            for (int c = 0; c < kClu; ++c) r.x += sh.peer[set][c][0] * sh.factor[c][0], r.y += sh.peer[set][c][1] * sh.factor[c][1];
+        } else {
+#pragma unroll 4
+            for (int c = 0; c < kClu; ++c) r.x += sh.peer[set][c][0], r.y += sh.peer[set][c][1];
+        }
         set ^= 1;
         return r;
     };
@@ -182,14 +238,13 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
         return a.draft + b * a.dld_b + (row / RESPS_MAX_K) * a.dld_level + (row % RESPS_MAX_K) * a.dld_row;
     };
 
-    int cur = 0, acc = 0;
     for (;;) {
         // ---- the rows of the current node: loads in flight while its children are looked up --------------
         const float* trow = a.target + b * a.ld_b + cur * a.ld_row + c_lo;
         const bool maybe_d = sh.row[cur] >= 0;  // a node with children was expanded
         const float* drow = drow_of(maybe_d ? cur : 0) + c_lo;
         float ft = -INFINITY, fd = -INFINITY;
-        constexpr int kGroup = 8;  // of each row, in flight together
+        constexpr int kGroup = 16;  // of each row, in flight together
 #pragma unroll 1
         for (int e0 = tid; e0 < n_cta; e0 += kGroup * kSampThreads) {
             float xt[kGroup], xd[kGroup];
@@ -212,7 +267,7 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
         const unsigned bal = __ballot_sync(kFull, is_child);
         if (warp < 4 && lane == 0) sh.count[warp] = __popc(bal);
         __syncthreads();  // (everyone is done with the previous node's children)
-        int n_child = 0;
+        n_child = 0;
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
             if (is_child && w == warp) sh.children[n_child + __popc(bal & ((1u << lane) - 1u))] = tid;
@@ -221,90 +276,89 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
         if (tid < n_child && tid < a.max_k && tid < RESPS_MAX_K)
             sh.u[tid] = a.u_accept[(static_cast<int64_t>(b) * cap + acc) * a.max_k + tid];
         const bool with_q = n_child > 0;
-        // ---- P_T(. | cur) = softmax(row / T) and the draft's P_d: maxima, exponentials, sums ------------------
+        // ---- P_T(. | cur) = softmax(row / T) and the draft's P_d: the CTA's maxima, exponentials, sums ----------
         const unsigned mt = __reduce_max_sync(kFull, float_to_ordered(ft)), md = __reduce_max_sync(kFull, float_to_ordered(fd));
         if (lane == 0) sh.red_max[warp][0] = mt, sh.red_max[warp][1] = md;
-        __syncthreads();
-        if (warp == 0) {
-            const unsigned wt = __reduce_max_sync(kFull, lane < kWarps ? sh.red_max[lane][0] : 0u);
-            const unsigned wd = __reduce_max_sync(kFull, lane < kWarps ? sh.red_max[lane][1] : 0u);
-            if (lane < kClu)
-                asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(peer_address(sh.peer_max[rank], lane)), "r"(wt), "r"(wd)
-                             : "memory");
-            // the rows of the child that is tried first
-            if (lane == 0 && with_q) {
-                const int child = sh.children[0];
-                prefetch_l2(a.target + b * a.ld_b + child * a.ld_row + c_lo, n_cta);
-                if (sh.row[child] >= 0) prefetch_l2(drow_of(child) + c_lo, n_cta);
-            }
-        }
-        cluster_barrier();
+        __syncthreads();  // (also: the children)
         unsigned top_t = 0u, top_d = 0u;
 #pragma unroll 4
-        for (int c = 0; c < kClu; ++c) top_t = max(top_t, sh.peer_max[c][0]), top_d = max(top_d, sh.peer_max[c][1]);
+        for (int w = 0; w < kWarps; ++w) top_t = max(top_t, sh.red_max[w][0]), top_d = max(top_d, sh.red_max[w][1]);
         const double mx_t = static_cast<double>(ordered_to_float(top_t)) * a.inv_t;
         const double mx_d = static_cast<double>(ordered_to_float(top_d)) * a.inv_t;
+        if (tid < n_child && tid < RESPS_MAX_K) {
+            const int x = sh.tok[sh.children[tid]], owner = static_cast<int>(static_cast<unsigned>(x) / static_cast<unsigned>(per_cta));
+            sh.child_clu[tid] = min(owner, kClu - 1), sh.child_at[tid] = (owner == static_cast<int>(rank)) ? x - c_lo : -1;
+        }
+        // the rows of the child that is tried first
+        if (tid == kSampThreads - 1 && with_q) {
+            const int child = sh.children[0];
+            prefetch_l2(a.target + b * a.ld_b + child * a.ld_row + c_lo, n_cta);
+            if (sh.row[child] >= 0) prefetch_l2(drow_of(child) + c_lo, n_cta);
+        }
         double sum_t = 0.0, sum_d = 0.0;
-#pragma unroll 2
+#pragma unroll 4
         for (int e = tid; e < n_cta; e += kSampThreads) {
-            const double w = exp(P[at(e)] * a.inv_t - mx_t);
+            const double w = exp_le0(fma(P[at(e)], a.inv_t, -mx_t), sh.exp2_64);
             P[at(e)] = w;
             sum_t += w;
         }
         if (with_q) {
-#pragma unroll 2
+#pragma unroll 4
             for (int e = tid; e < n_cta; e += kSampThreads) {
-                const double w = exp(Q[at(e)] * a.inv_t - mx_d);
+                const double w = exp_le0(fma(Q[at(e)], a.inv_t, -mx_d), sh.exp2_64);
                 Q[at(e)] = w;
                 sum_d += w;
             }
         }
-        // The owners of the children's tokens push (P, Q) into table `par` of every CTA, behind the barrier of
-        // the reduction that follows.
-        auto publish_children = [&](int par, int from) {
-#pragma unroll 1
-            for (int j = from; j < n_child && j < RESPS_MAX_K; ++j) {
-                const int e = sh.tok[sh.children[j]] - c_lo;
-                if (e < 0 || e >= n_cta || e % kSampThreads != tid) continue;
-                const double p = P[at(e)], q = Q[at(e)];
-#pragma unroll 1
-                for (int c = 0; c < kClu; ++c) store_pair_to_peer(sh.tab[par][j], c, p, q);
-            }
-        };
-        publish_children(0, 0);
-        const Pair sum = cluster_sum(sum_t, sum_d);
+        const Pair sum = cluster_sum(sum_t, sum_d, 0, 0, true, n_cta > 0 ? mx_t : -INFINITY, n_cta > 0 && with_q ? mx_d : -INFINITY);
         // What P (and the table's entries) still lack; a pass brings P up to date.
-        Pending pend = {1, recip_or_zero(sum.x), 0.0, -1};
-        double sq = with_q ? recip_or_zero(sum.y) : 0.0;     // draft side: q = Q * sq
+        Pending pend = {1, recip_or_zero(sum.x), 0.0};
+        double sq = with_q ? recip_or_zero(sum.y) : 0.0;  // draft side: q = Q * factor * sq
+        const double own_t = sh.factor[rank][0], own_d = sh.factor[rank][1];
         // ---- try the children -----------------------------------------------------------------------------
         int next = -1;
 #pragma unroll 1
         for (int j = 0; j < n_child && j < a.max_k; ++j) {
             const int child = sh.children[j];
             {
-                const double q_raw = sh.tab[j & 1][j][1];
-                const double p = apply(pend, sh.tab[j & 1][j][0], q_raw), q = q_raw * sq;
-                const double alpha = q > 0.0 ? fmin(1.0, p / q) : (p > 0.0 ? 1.0 : 0.0);
-                if (sh.u[j] < alpha) next = child;
+                const double q_raw = sh.tab[j & 1][j][1] * sh.factor[sh.child_clu[j]][1];
+                const double p = apply(pend, sh.tab[j & 1][j][0], sh.factor[sh.child_clu[j]][0], q_raw);
+                const double q = q_raw * sq;
+                // u < min(1, p / q), without the quotient
+                if (q > 0.0 ? sh.u[j] * q < p : p > 0.0) next = child;
             }
             if (next >= 0) break;
             // rejected: the residual's normaliser and the draft mass that is left without x
-            const int x = sh.tok[child], at_x = x - c_lo;
+            const int x_at = sh.child_at[j];
             double zx = 0.0, zy = 0.0;
-            // (the pass applies what is pending, and retires the token the round before removed)
+            const double scale = own_d * sq;
+            if (pend.kind == 1) {
+                const double mul = own_t * pend.a;
 #pragma unroll 4
-            for (int e = tid; e < n_cta; e += kSampThreads) {
-                double q_raw = Q[at(e)];
-                const double p = apply(pend, P[at(e)], q_raw);
-                P[at(e)] = p;
-                if (pend.kind == 2 && e == pend.x - c_lo) Q[at(e)] = q_raw = 0.0;
-                const double q = q_raw * sq;
-                zx += fmax(p - q, 0.0);
-                zy += (e != at_x) ? q : 0.0;
+                for (int e = tid; e < n_cta; e += kSampThreads) {
+                    const double p = P[at(e)] * mul, q = Q[at(e)] * scale;
+                    P[at(e)] = p;
+                    zx += fmax(p - q, 0.0);
+                    zy += (e != x_at) ? q : 0.0;
+                }
+            } else {
+                const double scale_old = own_d * pend.sq_old;
+                const bool keep = !(pend.a > 0.0);  // the residual was empty: p stays
+#pragma unroll 4
+                for (int e = tid; e < n_cta; e += kSampThreads) {
+                    const double q_raw = Q[at(e)], q = q_raw * scale, old = P[at(e)];
+                    const double p = keep ? old : fmax(old - q_raw * scale_old, 0.0) * pend.a;
+                    P[at(e)] = p;
+                    zx += fmax(p - q, 0.0);
+                    zy += (e != x_at) ? q : 0.0;
+                }
             }
-            publish_children((j + 1) & 1, j + 1);
-            const Pair zr = cluster_sum(zx, zy);
-            pend = Pending{2, recip_or_zero(zr.x), sq, x};
+            const Pair zr = cluster_sum(zx, zy, (j + 1) & 1, j + 1, false, 0.0, 0.0);
+            pend = Pending{2, recip_or_zero(zr.x), sq};
+            if (x_at >= 0 && x_at % kSampThreads == tid) {  // x leaves the draft side; its own round is applied here
+                if (pend.a > 0.0) P[at(x_at)] -= Q[at(x_at)] * scale;
+                Q[at(x_at)] = 0.0;
+            }
             if (zr.y > 0.0) sq = sq * (1.0 / zr.y);
         }
         if (next >= 0) {
@@ -319,7 +373,8 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
         // ---- nobody accepted (or a leaf): draw from the current target-side distribution by inverse CDF in
         // token order: the tokens change hands so that a thread holds a contiguous run --------------------------
 #pragma unroll 4
-        for (int e = tid; e < n_cta; e += kSampThreads) P[at(e)] = apply(pend, P[at(e)], with_q ? Q[at(e)] : 0.0);
+        for (int e = tid; e < n_cta; e += kSampThreads)
+            P[at(e)] = apply(pend, P[at(e)], own_t, with_q ? Q[at(e)] * own_d : 0.0);
         __syncthreads();
         const int t_lo = min(n_cta, tid * per), t_hi = min(n_cta, t_lo + per);
         double run = 0.0;
