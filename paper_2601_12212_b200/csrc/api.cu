@@ -273,14 +273,9 @@ int resps_row_scan_shard(resps_ctx* ctx, const resps_step* d_steps, int batch, c
     if (ctx->shape.vocab < ctx->shape.max_k) return RESPS_ERR_UNSUPPORTED_SHAPE;  // a shard holds at least max_k columns
     if (n_levels > ctx->shape.max_depth) n_levels = ctx->shape.max_depth;
     if (n_slots > ctx->shape.max_k) n_slots = ctx->shape.max_k;
+    const resps::ScanRows out = {d_part_val, d_part_id, d_part_lse};
     if (resps::launch_row_scan(ctx, d_steps, batch, d_draft_logits, ld_b, ld_level, ld_row, n_levels, n_slots, -1,
-                               stream) != cudaSuccess)
-        return RESPS_ERR_CUDA;
-    const resps::Workspace& w = ctx->ws;
-    const size_t rows = static_cast<size_t>(batch) * w.max_rows;
-    if (cudaMemcpyAsync(d_part_val, w.row_val, rows * ctx->shape.max_k * sizeof(float), cudaMemcpyDeviceToDevice, stream) != cudaSuccess ||
-        cudaMemcpyAsync(d_part_id, w.row_id, rows * ctx->shape.max_k * sizeof(int32_t), cudaMemcpyDeviceToDevice, stream) != cudaSuccess ||
-        cudaMemcpyAsync(d_part_lse, w.row_lse, rows * sizeof(double), cudaMemcpyDeviceToDevice, stream) != cudaSuccess)
+                               stream, &out) != cudaSuccess)
         return RESPS_ERR_CUDA;
     return RESPS_OK;
 }

@@ -88,9 +88,14 @@ struct AcceptArgs {
 };
 
 // ---- launchers (one per translation unit) ---------------------------------
+struct ScanRows {  // scanned rows somewhere else than in the workspace
+    float* val;      // [batch][max_rows][max_k]
+    int32_t* id;
+    double* lse;     // [batch][max_rows]
+};
 cudaError_t launch_row_scan(const resps_ctx* ctx, const resps_step* d_steps, int batch,
                             const float* logits, int64_t ld_b, int64_t ld_level, int64_t ld_row,
-                            int n_levels, int n_slots, int only_level, cudaStream_t st);
+                            int n_levels, int n_slots, int only_level, cudaStream_t st, const ScanRows* out = nullptr);
 // What the level form of the tree expansion hands back per level: the members of the new frontier.
 struct FrontierOut {
     int32_t *tokens, *parent_slot, *position_ids, *node_index;  // [batch][max_k]

@@ -25,7 +25,8 @@ struct ScanArgs {
     int n_levels, n_slots;
     int vocab, max_tt, max_k, max_rows;
     int chunk, splits;
-    int slices, cps;  // streaming kernel: slices per row, chunks per slice (partials keep the stride `splits`)
+    int batch;
+    int slices;       // streaming kernel: > 0: about as many slices per row at most (partials keep the stride `splits`)
     int test_drop;    // test build only: 2 = the second chunk copy of every slice is left out
     int only_level;   // -1: the rows of all levels; j >= 0: only level j's rows (blockIdx.y = slot)
     unsigned long long* part_key;
@@ -52,9 +53,11 @@ struct LseAcc {
 // rank-by-counting selection: the `k` largest of n keys in shared memory, written in order.
 template <typename Out>
 __device__ __forceinline__ void select_top_by_rank(const unsigned long long* keys, int n, int k, Out out) {
+#pragma unroll 1
     for (int c = threadIdx.x; c < n; c += kScanThreads) {  // callers run it with kScanThreads threads
         const unsigned long long mine = keys[c];
         int rank = 0;
+#pragma unroll 2
         for (int j = 0; j < n; ++j) rank += (keys[j] > mine) || (keys[j] == mine && j < c);
         if (rank < k) out(rank, mine);
     }
@@ -185,10 +188,15 @@ __global__ void __launch_bounds__(kScanThreads, 4) row_scan_kernel(const ScanArg
     // ---- candidates: every logit at or before tau ------------------------------------------------
     if (quad_key >= tau && has_any) {  // only the k quads whose maximum qualifies can hold any
         const float tau_v = (tau == 0ull) ? -INFINITY : key_val(tau);
+        uint32_t hits = 0u;
 #pragma unroll
-        for (int i = 0; i < kScanPerThread; ++i) {
-            if (v[i] >= tau_v && elem_id(i) < end) {
-                const unsigned long long key = pack_val_id(v[i], elem_id(i));
+        for (int i = 0; i < kScanPerThread; ++i) hits |= (v[i] >= tau_v) ? (1u << i) : 0u;
+#pragma unroll 1
+        while (hits) {  // (a few; re-read by index: the registers cannot be indexed)
+            const int e = elem_id(__ffs(hits) - 1);
+            hits &= hits - 1u;
+            if (e < end) {
+                const unsigned long long key = pack_val_id(__ldg(row + e), e);
                 if (key >= tau) s_keys[atomicAdd(&s_count, 1)] = key;
             }
         }
@@ -201,6 +209,7 @@ __global__ void __launch_bounds__(kScanThreads, 4) row_scan_kernel(const ScanArg
     if (tid >= n_cand && tid < k) part[tid] = 0ull;  // fewer than k logits in the chunk
     if (tid == 0) {
         LseAcc t;
+#pragma unroll 1
         for (int w = 0; w < kScanThreads / 32; ++w) t.merge(s_ms[w].x, s_ms[w].y);
         a.part_ms[prow * a.splits + sp] = make_float2(t.m2, t.s);
     }
@@ -213,6 +222,7 @@ __global__ void __launch_bounds__(kScanThreads, 4) row_scan_kernel(const ScanArg
     // ---- last CTA of the row: merge the partial lists and the partial sums ----
     __threadfence();
     const unsigned long long* parts = a.part_key + prow * a.splits * a.max_k;
+#pragma unroll 1
     for (int i = tid; i < a.splits * k; i += kScanThreads)
         s_keys[i] = __ldcg(parts + (i / k) * a.max_k + (i % k));
     float2 my_ms = make_float2(-INFINITY, 0.f);
@@ -249,16 +259,27 @@ __global__ void __launch_bounds__(kScanThreads, 4) row_scan_kernel(const ScanArg
 }
 
 // ---------------------------------------------------------------------------------------
-// Streaming variant (16-byte aligned rows): a CTA walks a slice of several chunks of one row.
-// One thread issues bulk copies (cp.async.bulk, global -> shared, completion on an mbarrier)
-// three chunks ahead, so the loads of the next chunks run under the arithmetic of the current
-// one.  The first chunk establishes the threshold tau as above; afterwards tau is the k-th best
-// logit seen so far, a chunk contributes only the (few) logits at or above it, and the list is
-// cut back to its k best when it has grown.  The log-sum-exp state stays in registers across
-// chunks.  A chunk whose hits would not fit the list (adversarial order) re-derives a threshold
-// of its own from its quad maxima, which bounds its candidates by 128 k.
+// Streaming variant (16-byte aligned rows).  The 8192-logit chunks of all rows of all sequences stand in one
+// line; two CTAs per SM take equal ranges of it, so that all of them finish together whatever the number of rows.
+// The part of a row inside a CTA's range is a slice.  One thread issues bulk copies (cp.async.bulk, global ->
+// shared, completion on an mbarrier) three chunks ahead, across slices, so that the copies run under the
+// arithmetic and under a slice's tail.
+//
+// A chunk costs its eight consumer warps one wait, a maximum and the exponentials: no barrier, no selection.
+// At the end of a slice the k-th best of the 64 quad maxima (quad = 4 threads, 128 logits of every chunk) is
+// a lower bound tau of the slice's k-th best; the threads whose own maximum reaches tau (about k of 256) are
+// the only ones that can hold a candidate, and their logits are read once more, from L2, by all threads
+// together.  About 2 k candidates are ranked by counting.  Should they not fit the list (many equal logits,
+// adversarial order), tau is raised until the strictly better ones do, and the lowest ids among its equals
+// fill up.
+//
+// Bound by HBM where there are many rows; where a CTA has two or three chunks by its start, the slice's tail
+// and the merge of the row.  With selection chunk by chunk (two to six barriers a chunk) and a fixed grid of slices
+// the tree build of d=8 k=32 (225 rows of 128256 logits) took 98 us (now 69), a shard's scan 14.2 us (now 10.1).
 // ---------------------------------------------------------------------------------------
 constexpr int kStreamStages = 3;
+constexpr int kStreamMaxBatch = 256; // sequences of one launch
+constexpr int kStreamList = 1024;    // candidates of a slice
 constexpr long long kScanWaitLimitCycles = kWaitTest ? 2000000ll : 4000000000ll;
 
 __device__ __forceinline__ uint32_t scan_smem_u32(const void* p) {
@@ -280,9 +301,9 @@ __device__ __forceinline__ bool scan_mbar_try(uint32_t bar, uint32_t parity) {
 __device__ __forceinline__ void scan_mbar_wait(uint32_t bar, uint32_t parity, int32_t* status) {
     if (scan_mbar_try(bar, parity)) return;
     const long long t0 = clock64();
-    unsigned spins = 0;
+#pragma unroll 1
     while (!scan_mbar_try(bar, parity)) {
-        if ((++spins & 63u) == 0u && clock64() - t0 > kScanWaitLimitCycles) {
+        if (clock64() - t0 > kScanWaitLimitCycles) {
             if (status) atomicOr(status, RESPS_STATUS_WAIT_TIMEOUT);
             return;
         }
@@ -292,299 +313,379 @@ __device__ __forceinline__ void scan_mbar_wait(uint32_t bar, uint32_t parity, in
 constexpr int kStreamThreads = kScanThreads + 32;  // eight consumer warps + the copy-issuing warp
 
 __device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-__device__ __forceinline__ bool consumer_any(bool pred) {  // barrier over the consumers, OR of pred
-    uint32_t out;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 q, %1, 0;\n\t"
-        "bar.red.or.pred p, 1, 256, q;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(out)
-        : "r"(pred ? 1u : 0u)
-        : "memory");
-    return out != 0;
+
+struct StreamShared {
+    unsigned long long bar[2 * kStreamStages];  // full[3], empty[3]
+    unsigned long long list[kStreamList];
+    unsigned long long top[RESPS_MAX_K];
+    float quad[kQuads];
+    float2 ms[kScanThreads / 32];
+    float2 total;
+    int row0[kStreamMaxBatch + 1];  // first row of a sequence
+    int k[kStreamMaxBatch];
+    int warp_count[kScanThreads / 32];
+    unsigned char thr[kScanThreads];  // threads that may hold candidates
+    float tau;
+    int count, last;
+};
+
+// k-th best value (by value alone) of `n` >= k keys, to `*out`; the `k` best in order to `top` when given.
+__device__ __forceinline__ void rank_list(const unsigned long long* keys, int n, int k, unsigned long long* top, float* kth) {
+#pragma unroll 1
+    for (int c = threadIdx.x; c < n; c += kScanThreads) {
+        const unsigned long long mine = keys[c];
+        int rank = 0;
+#pragma unroll 4
+        for (int j = 0; j < n; ++j) rank += (keys[j] > mine) ? 1 : 0;
+        if (top && rank < k) top[rank] = mine;
+        if (kth && rank == k - 1) *kth = key_val(mine);
+    }
 }
+
+__device__ __forceinline__ float warp_maximum(float x) {
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(kFull, x, o));
+    return x;
+}
+__device__ __forceinline__ float warp_total(float x) {
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+    return x;
+}
+// a sum relative to the maximum m, relative to M >= m instead (0 where there is none yet)
+__device__ __forceinline__ float weighted(float s, float m, float M) { return m > -INFINITY ? s * ex2_approx(m - M) : 0.f; }
 
 __global__ void __launch_bounds__(kStreamThreads, 2) row_scan_stream_kernel(const ScanArgs a) {
     extern __shared__ __align__(128) unsigned char s_raw[];
-    float* s_stage = reinterpret_cast<float*>(s_raw);                                    // [3][8192]
-    unsigned long long* s_keys =
-        reinterpret_cast<unsigned long long*>(s_raw + kStreamStages * kScanChunkMax * sizeof(float));  // list
-    __shared__ __align__(8) unsigned long long s_bar[2 * kStreamStages];  // full[3], empty[3]
-    __shared__ unsigned long long s_quad[kQuads];
-    __shared__ unsigned long long s_top[RESPS_MAX_K];
-    __shared__ unsigned long long s_tau;
-    __shared__ int s_count;
-    __shared__ float2 s_ms[kScanThreads / 32];
-    __shared__ bool s_last;
-    const int b = blockIdx.z, ry = blockIdx.y, sl = blockIdx.x;
+    float* s_stage = reinterpret_cast<float*>(s_raw);  // [3][8192]
+    __shared__ __align__(16) StreamShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t bar0 = scan_smem_u32(s_bar);
+    const uint32_t bar0 = scan_smem_u32(sh.bar);
     auto full_bar = [&](int st) { return bar0 + 8u * st; };
     auto empty_bar = [&](int st) { return bar0 + 8u * (kStreamStages + st); };
     // the barriers are set up under the tail of the preceding kernel: nothing here touches global memory
     if (tid == 0) {
+#pragma unroll 1
         for (int st = 0; st < kStreamStages; ++st) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full_bar(st)) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(empty_bar(st)), "r"(kScanThreads) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(empty_bar(st)), "r"(kScanThreads / 32) : "memory");
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        s_count = 0;
-        s_tau = 0ull;
+        sh.count = 0;
     }
-    __syncthreads();
     pdl_wait();  // the kernel before this one in the stream has completed
     pdl_launch_dependents();
-    const StepDims sd = clamp_step(a.steps[b], a.n_levels, a.n_slots, a.max_tt, a.max_k, a.vocab);
-    const int k = sd.k;
-    const int rows = 1 + (sd.d - 1) * k;
-    if (a.only_level >= 0 && ry >= (a.only_level == 0 ? 1 : k)) return;
-    const int r = (a.only_level < 0) ? ry : (a.only_level == 0 ? 0 : 1 + (a.only_level - 1) * k + ry);
-    if (r >= rows) return;
-    if (sd.clamped && r == 0 && sl == 0 && tid == 0) atomicOr(a.status, RESPS_STATUS_STEP_CLAMPED);
-    const int level = (r == 0) ? 0 : 1 + (r - 1) / k;
-    const int slot = (r == 0) ? 0 : (r - 1) % k;
-    const float* row = a.logits + b * a.ld_b + level * a.ld_level + slot * a.ld_row;
-    const int c_begin = sl * a.cps;
-    const int c_end = min(a.splits, c_begin + a.cps);  // chunks [c_begin, c_end) of this row
-    const int list_cap = (kQuadElems + 1) * a.max_k;
+    // ---- the rows of every sequence -------------------------------------------------------------------
+    if (warp == 0) {
+        int base = 0;
+#pragma unroll 1
+        for (int b0 = 0; b0 < a.batch; b0 += 32) {
+            const int b = b0 + lane;
+            int rows = 0;
+            if (b < a.batch) {
+                const StepDims sd = clamp_step(a.steps[b], a.n_levels, a.n_slots, a.max_tt, a.max_k, a.vocab);
+                sh.k[b] = sd.k;
+                rows = (a.only_level < 0) ? 1 + (sd.d - 1) * sd.k : a.only_level >= sd.d ? 0 : a.only_level == 0 ? 1 : sd.k;
+                if (sd.clamped && blockIdx.x == 0) atomicOr(a.status, RESPS_STATUS_STEP_CLAMPED);
+            }
+            int incl = rows;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int v = __shfl_up_sync(kFull, incl, d);
+                if (lane >= d) incl += v;
+            }
+            if (b < a.batch) sh.row0[b] = base + incl - rows;
+            base += __shfl_sync(kFull, incl, 31);
+        }
+        if (lane == 0) sh.row0[a.batch] = base;
+    }
+    __syncthreads();
+    // the ranges: never so short that a row's merge (slices x k entries) would not fit the list
+    const int total = sh.row0[a.batch] * a.splits;
+    const int most_slices = max(1, min(a.slices > 0 ? a.slices : a.splits, kStreamList / a.max_k - 2));
+    const int least = (a.splits + most_slices - 1) / most_slices;
+    const int ctas = max(1, min(static_cast<int>(gridDim.x), total / least));
+    if (static_cast<int>(blockIdx.x) >= ctas) return;
+    const int base = total / ctas, longer = total - base * ctas;  // the first `longer` ranges have one chunk more
+    const int me = blockIdx.x;
+    const int x_begin = me * base + min(me, longer), x_end = x_begin + base + (me < longer ? 1 : 0);
+    auto owner = [&](int x) {
+        const int cut = longer * (base + 1);
+        return x < cut ? x / (base + 1) : longer + (x - cut) / base;
+    };
+    const int only = min(max(a.only_level, 0), 1);  // (arithmetic: a condition would double the loops' code)
+    struct Work {
+        int b, r, k, c_begin, c_end;
+        const float* row;
+    };
+    auto work_at = [&](int x) {  // the slice that starts at chunk x
+        Work w;
+        const int row = x / a.splits;
+        w.c_begin = x - row * a.splits, w.c_end = min(a.splits, w.c_begin + x_end - x);
+        int lo = 0, hi = a.batch;  // last sequence that starts at or before the row (and is not empty)
+#pragma unroll 1
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (sh.row0[mid] <= row) lo = mid; else hi = mid;
+        }
+        w.b = lo, w.k = sh.k[lo];
+        const int local = row - sh.row0[lo];
+        w.r = local + only * (1 + (a.only_level - 1) * w.k);
+        const int level = (w.r == 0) ? 0 : 1 + (w.r - 1) / w.k;
+        const int slot = (w.r == 0) ? 0 : (w.r - 1) - (level - 1) * w.k;
+        w.row = a.logits + w.b * a.ld_b + level * a.ld_level + slot * a.ld_row;
+        return w;
+    };
 
     if (warp == kScanThreads / 32) {
-        // ---- copy-issuing warp: a stage is refilled as soon as every consumer has read it ----------
+        // ---- copy-issuing warp: a stage is refilled as soon as every consumer warp has read it ----------
         if (lane == 0) {
-            for (int c = c_begin; c < c_end; ++c) {
-                const int u = c - c_begin, st = u % kStreamStages;
-                scan_mbar_wait(empty_bar(st), ((u / kStreamStages) & 1u) ^ 1u, a.status);
-                const int e0 = c * kScanChunkMax;
-                const uint32_t bytes = static_cast<uint32_t>(min(a.vocab - e0, kScanChunkMax)) * 4u;
-                if (kWaitTest && (a.test_drop & 2) && u == 1) continue;
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full_bar(st)), "r"(bytes)
-                             : "memory");
-                asm volatile(
-                    "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                        scan_smem_u32(s_stage + st * kScanChunkMax)),
-                    "l"(row + e0), "r"(bytes), "r"(full_bar(st))
-                    : "memory");
+            uint32_t u = 0;
+#pragma unroll 1
+            for (int x = x_begin; x < x_end;) {
+                const Work w = work_at(x);
+                x += w.c_end - w.c_begin;
+#pragma unroll 1
+                for (int c = w.c_begin; c < w.c_end; ++c, ++u) {
+                    const uint32_t st = u % kStreamStages;
+                    scan_mbar_wait(empty_bar(st), ((u / kStreamStages) & 1u) ^ 1u, a.status);
+                    const int e0 = c * kScanChunkMax;
+                    const uint32_t bytes = static_cast<uint32_t>(min(a.vocab - e0, kScanChunkMax)) * 4u;
+                    if (kWaitTest && (a.test_drop & 2) && u == 1) continue;
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full_bar(st)), "r"(bytes)
+                                 : "memory");
+                    asm volatile(
+                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                            scan_smem_u32(s_stage + st * kScanChunkMax)),
+                        "l"(w.row + e0), "r"(bytes), "r"(full_bar(st))
+                        : "memory");
+                }
             }
         }
         return;  // the consumers wait for every copy that was issued
     }
 
-    int list_n = 0;                // entries of the candidate list (same in every thread)
-    LseAcc acc;                    // this thread's running (max, sum) over all its logits
-    unsigned long long tau = 0ull; // k-th best so far (0 = none yet: everything qualifies)
-    float tau_v = -INFINITY;
-
-    for (int c = c_begin; c < c_end; ++c) {
-        const int u0 = c - c_begin, st = u0 % kStreamStages;
-        const int begin = c * kScanChunkMax;
-        const int end = min(a.vocab, begin + kScanChunkMax);
-        scan_mbar_wait(full_bar(st), (u0 / kStreamStages) & 1u, a.status);
-        float v[kScanPerThread];
+    uint32_t u0 = 0;
+#pragma unroll 1
+    for (int x = x_begin; x < x_end;) {
+        const Work w = work_at(x);
+        const int k = w.k, row0 = x - w.c_begin;  // first chunk of the row
+        const int first = owner(row0), slices = owner(row0 + a.splits - 1) - first + 1, sl = me - first;
+        x += w.c_end - w.c_begin;
+        LseAcc acc;                // this thread's running (max, sum) over all its logits of the slice
+        float best = -INFINITY;    // its best logit
+#pragma unroll 1
+        for (int c = w.c_begin; c < w.c_end; ++c, ++u0) {
+            const uint32_t st = u0 % kStreamStages;
+            const int begin = c * kScanChunkMax, end = min(a.vocab, begin + kScanChunkMax);
+            scan_mbar_wait(full_bar(st), (u0 / kStreamStages) & 1u, a.status);
+            float v[kScanPerThread];
+            if (end - begin == kScanChunkMax) {
 #pragma unroll
-        for (int u = 0; u < kScanPerThread / 4; ++u) {
-            const int off = (u * kScanThreads + tid) * 4;
-            v[4 * u] = v[4 * u + 1] = v[4 * u + 2] = v[4 * u + 3] = -INFINITY;
-            if (begin + off < end) {  // the vocabulary is a multiple of 4 on this path
-                const float4 x = *reinterpret_cast<const float4*>(s_stage + st * kScanChunkMax + off);
-                v[4 * u] = x.x, v[4 * u + 1] = x.y, v[4 * u + 2] = x.z, v[4 * u + 3] = x.w;
+                for (int u = 0; u < kScanPerThread / 4; ++u) {
+                    const float4 x = *reinterpret_cast<const float4*>(s_stage + st * kScanChunkMax + (u * kScanThreads + tid) * 4);
+                    v[4 * u] = x.x, v[4 * u + 1] = x.y, v[4 * u + 2] = x.z, v[4 * u + 3] = x.w;
+                }
+            } else {
+#pragma unroll
+                for (int u = 0; u < kScanPerThread / 4; ++u) {
+                    const int off = (u * kScanThreads + tid) * 4;
+                    float4 x = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+                    if (begin + off < end) x = *reinterpret_cast<const float4*>(s_stage + st * kScanChunkMax + off);  // (the vocabulary is a multiple of 4)
+                    v[4 * u] = x.x, v[4 * u + 1] = x.y, v[4 * u + 2] = x.z, v[4 * u + 3] = x.w;
+                }
             }
-        }
-        auto release_stage = [&]() {
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty_bar(st)) : "memory");
-        };
-        auto elem_id = [&](int i) { return begin + ((i >> 2) * kScanThreads + tid) * 4 + (i & 3); };
-        const bool has_any = elem_id(0) < end;
-
-        // ---- thread maximum, log-sum-exp update ---------------------------------------------------
-        float tmax = v[0];
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty_bar(st)) : "memory");
+            float tmax = v[0];
 #pragma unroll
-        for (int i = 1; i + 1 < kScanPerThread; i += 2) tmax = max3f(tmax, v[i], v[i + 1]);
-        tmax = fmaxf(tmax, v[kScanPerThread - 1]);
-        if (has_any) {
+            for (int i = 1; i + 1 < kScanPerThread; i += 2) tmax = max3f(tmax, v[i], v[i + 1]);
+            tmax = fmaxf(tmax, v[kScanPerThread - 1]);
+            best = fmaxf(best, tmax);
             const float m_new = fmaxf(acc.m2, tmax * kLog2e);
-            float s0 = acc.s * ex2_approx(acc.m2 - m_new), s1 = 0.f;  // 0 * 2^-inf = 0 on the first chunk
+            if (m_new > -INFINITY) {
+                float s0 = acc.s * ex2_approx(acc.m2 - m_new), s1 = 0.f;  // 0 * 2^-inf = 0 on the first chunk
 #pragma unroll
-            for (int i = 0; i < kScanPerThread; i += 2) {
-                s0 += ex2_approx(fmaf(v[i], kLog2e, -m_new));
-                s1 += ex2_approx(fmaf(v[i + 1], kLog2e, -m_new));
-            }
-            acc.m2 = m_new, acc.s = s0 + s1;
-        }
-        const bool first = (c == c_begin);
-        // One barrier per chunk in the common case: does any thread hold a logit at or above tau?
-        // (branch-free bit mask; the few hits are then re-read from the stage by index)
-        uint32_t hits = 0u;
-        if (!first) {
-            if (tmax >= tau_v) {  // only a thread whose best logit qualifies has anything to mark
-#pragma unroll
-                for (int i = 0; i < kScanPerThread; ++i) hits |= (v[i] >= tau_v) ? (1u << i) : 0u;
-            }
-            if (!consumer_any(hits != 0u)) {
-                release_stage();
-                continue;
+                for (int i = 0; i < kScanPerThread; i += 2) {
+                    s0 += ex2_approx(fmaf(v[i], kLog2e, -m_new));
+                    s1 += ex2_approx(fmaf(v[i + 1], kLog2e, -m_new));
+                }
+                acc.m2 = m_new, acc.s = s0 + s1;
             }
         }
 
-        // Threads that hold such logits append them to the list.  Should the list overflow
-        // (adversarial order: every logit beats the threshold), the appended entries are dropped
-        // and the chunk takes the bounded path below.
-        bool slow = first;
-        if (!first) {
-            const float* stage = s_stage + st * kScanChunkMax;
-            while (hits) {
-                const int i = __ffs(hits) - 1;
-                hits &= hits - 1u;
-                const int e = elem_id(i);
-                if (e < end) {
-                    const unsigned long long key = pack_val_id(stage[e - begin], e);
-                    if (key >= tau) {
-                        const int at = atomicAdd(&s_count, 1);
-                        if (at < list_cap) s_keys[at] = key;
-                    }
-                }
-            }
-            consumer_sync();
-            slow = s_count > list_cap;  // fixed until the next barrier
+        // ---- tau: the k-th best of the quad maxima (-inf: fewer than k quads hold anything) -----------------
+        {
+            float q = fmaxf(best, __shfl_xor_sync(kFull, best, 1));
+            q = fmaxf(q, __shfl_xor_sync(kFull, q, 2));
+            if ((lane & 3) == 0) sh.quad[tid >> 2] = q;
+            if (tid == 0) sh.count = 0;
         }
-        release_stage();
-        if (slow) {
-            // the chunk's own threshold from its quad maxima (see row_scan_kernel); the list is cut
-            // to its k best first so that the chunk's at most 128 k candidates fit behind them
-            if (!first) {  // the first list_n entries are the list as it was before this chunk
-                for (int cidx = tid; cidx < list_n; cidx += kScanThreads) {
-                    const unsigned long long mine = s_keys[cidx];
-                    int rank = 0;
-                    for (int j = 0; j < list_n; ++j) rank += (s_keys[j] > mine) ? 1 : 0;
-                    if (rank < k) s_top[rank] = mine;
-                }
-                consumer_sync();
-                const int nk = min(list_n, k);
-                if (tid < nk) s_keys[tid] = s_top[tid];
-                if (tid == 0) s_count = nk;
-                consumer_sync();
+        const float warp_max = warp_maximum(acc.m2);  // log-sum-exp partial of the warp, merged below
+        const float warp_sum = warp_total(weighted(acc.s, acc.m2, warp_max));
+        if (lane == 0) sh.ms[warp] = make_float2(warp_max, warp_sum);
+        consumer_sync();
+        if (tid < kQuads) {
+            const float mine = sh.quad[tid];
+            int rank = 0;
+#pragma unroll 4
+            for (int j = 0; j < kQuads; j += 4) {
+                const float4 o = *reinterpret_cast<const float4*>(sh.quad + j);
+                rank += (o.x > mine || (o.x == mine && j < tid)) + (o.y > mine || (o.y == mine && j + 1 < tid)) +
+                        (o.z > mine || (o.z == mine && j + 2 < tid)) + (o.w > mine || (o.w == mine && j + 3 < tid));
             }
-            int tpos = 0;
-#pragma unroll
-            for (int i = kScanPerThread - 1; i >= 0; --i)
-                if (v[i] == tmax) tpos = i;
-            const unsigned long long my_key = has_any ? pack_val_id(tmax, elem_id(tpos)) : 0ull;
-            unsigned long long quad_key = my_key;
-            {
-                unsigned long long o = __shfl_xor_sync(kFull, quad_key, 1);
-                quad_key = o > quad_key ? o : quad_key;
-                o = __shfl_xor_sync(kFull, quad_key, 2);
-                quad_key = o > quad_key ? o : quad_key;
-            }
-            if ((lane & 3) == 0) s_quad[tid >> 2] = quad_key;
-            consumer_sync();
-            if (tid < kQuads) {
-                const unsigned long long mine = s_quad[tid];
-                int rank = 0;
-#pragma unroll 8
-                for (int j = 0; j < kQuads; ++j) {
-                    const unsigned long long o = s_quad[j];
-                    rank += (o > mine) || (o == mine && j < tid);
-                }
-                if (rank == min(k, kQuads) - 1) s_tau = mine;
-            }
-            consumer_sync();
-            const unsigned long long tau_c = s_tau > tau ? s_tau : tau;  // never below the running one
-            if (quad_key >= tau_c && has_any) {
-                const float tv = (tau_c == 0ull) ? -INFINITY : key_val(tau_c);
-#pragma unroll
-                for (int i = 0; i < kScanPerThread; ++i)
-                    if (v[i] >= tv && elem_id(i) < end) {
-                        const unsigned long long key = pack_val_id(v[i], elem_id(i));
-                        if (key >= tau_c) s_keys[atomicAdd(&s_count, 1)] = key;
-                    }
-            }
+            if (rank == k - 1) sh.tau = mine;
         }
         consumer_sync();
-        // ---- tighten: tau = k-th best of the list; cut the list back when it has grown ----------
-        const int n_list = s_count;
-        list_n = n_list;
-        if (slow || n_list > 8 * k) {
-            for (int cidx = tid; cidx < n_list; cidx += kScanThreads) {
-                const unsigned long long mine = s_keys[cidx];
-                int rank = 0;
-                for (int j = 0; j < n_list; ++j) rank += (s_keys[j] > mine) ? 1 : 0;
-                if (rank < k) s_top[rank] = mine;
-            }
-            consumer_sync();
-            const int nk = min(n_list, k);
-            if (tid < nk) s_keys[tid] = s_top[tid];
-            if (tid == 0) {
-                s_count = nk;
-                s_tau = (n_list >= k) ? s_top[k - 1] : 0ull;
-            }
-            consumer_sync();
-            tau = s_tau;
-            tau_v = (tau == 0ull) ? -INFINITY : key_val(tau);
-            list_n = nk;
+        float tau = sh.tau;
+        // ---- the threads that may hold candidates; their logits once more, by everybody ----------------------
+        const bool mine = best >= tau && best > -INFINITY;
+        const unsigned bal = __ballot_sync(kFull, mine);
+        if (lane == 0) sh.warp_count[warp] = __popc(bal);
+        consumer_sync();
+        int n_thr = 0, at = __popc(bal & ((1u << lane) - 1u));
+#pragma unroll
+        for (int q = 0; q < kScanThreads / 32; ++q) {
+            if (q < warp) at += sh.warp_count[q];
+            n_thr += sh.warp_count[q];
         }
-    }
-
-    // ---- the slice's k best and its log-sum-exp partial ------------------------------------------
-    consumer_sync();
-    const int n_cand = s_count;
-    const int64_t prow = static_cast<int64_t>(b) * a.max_rows + r;
-    unsigned long long* part = a.part_key + (prow * a.splits + sl) * a.max_k;
-    select_top_by_rank(s_keys, n_cand, k, [&](int rank, unsigned long long key) { part[rank] = key; });
-    if (tid >= n_cand && tid < k) part[tid] = 0ull;
+        if (mine) sh.thr[at] = static_cast<unsigned char>(tid);
+        consumer_sync();
+        const int per_thr = (w.c_end - w.c_begin) * (kScanPerThread / 4), n_vec = n_thr * per_thr;
+        // Every logit at or above tau is appended while the list has room (-inf only by the filling below).  If
+        // there were too many, tau becomes the k-th best found so far, and only the better ones are taken.
+        const uint32_t ord_max = float_to_ordered(INFINITY);  // (NaNs of positive sign lie above)
+        uint32_t least_ord = max(float_to_ordered(tau == 0.f ? -0.f : tau), float_to_ordered(-INFINITY) + 1u);
+        int n_cand;
+#pragma unroll 1
+        for (;;) {
+            constexpr int kAhead = 4;  // loads in flight per thread
+#pragma unroll 1
+            for (int i0 = tid; i0 < n_vec; i0 += kAhead * kScanThreads) {
+                float4 x[kAhead];
+                int e[kAhead];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float om = __shfl_xor_sync(kFull, acc.m2, o);
-        const float os = __shfl_xor_sync(kFull, acc.s, o);
-        acc.merge(om, os);
-    }
-    if (lane == 0) s_ms[warp] = make_float2(acc.m2, acc.s);
-    consumer_sync();
-    if (tid == 0) {
-        LseAcc t;
-        for (int w = 0; w < kScanThreads / 32; ++w) t.merge(s_ms[w].x, s_ms[w].y);
-        a.part_ms[prow * a.splits + sl] = make_float2(t.m2, t.s);
-    }
-    __threadfence();
-    consumer_sync();
-    if (tid == 0) s_last = (atomicAdd(a.counter + prow, 1u) == static_cast<unsigned>(a.slices - 1));
-    consumer_sync();
-    if (!s_last) return;
-
-    // ---- last CTA of the row: merge the slices ---------------------------------------------------
-    __threadfence();
-    const unsigned long long* parts = a.part_key + prow * a.splits * a.max_k;
-    for (int i = tid; i < a.slices * k; i += kScanThreads) s_keys[i] = __ldcg(parts + (i / k) * a.max_k + (i % k));
-    float2 my_ms = make_float2(-INFINITY, 0.f);
-    if (tid < a.slices) my_ms = __ldcg(a.part_ms + prow * a.splits + tid);
-    consumer_sync();
-    float* oval = a.row_val + prow * a.max_k;
-    int32_t* oid = a.row_id + prow * a.max_k;
-    select_top_by_rank(s_keys, a.slices * k, k, [&](int rank, unsigned long long key) {
-        oval[rank] = key_val(key);
-        oid[rank] = key_id(key);
-    });
-    if (warp < 4) {
-        float M = my_ms.x;
+                for (int q = 0; q < kAhead; ++q) {
+                    const int i = min(i0 + q * kScanThreads, n_vec - 1), t = i / per_thr, rest = i - t * per_thr;
+                    e[q] = w.c_begin * kScanChunkMax + (rest * kScanThreads + sh.thr[t]) * 4;
+                    x[q] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+                    if (e[q] < a.vocab && i0 + q * kScanThreads < n_vec) x[q] = __ldg(reinterpret_cast<const float4*>(w.row + e[q]));
+                }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(kFull, M, o));
-        if (lane == 0) s_ms[warp] = make_float2(M, 0.f);
-    }
-    consumer_sync();
-    if (warp < 4) {
-        const float M = fmaxf(fmaxf(s_ms[0].x, s_ms[1].x), fmaxf(s_ms[2].x, s_ms[3].x));
-        double sum = (my_ms.y > 0.f) ? static_cast<double>(my_ms.y) * static_cast<double>(ex2_approx(my_ms.x - M)) : 0.0;
+                for (int q = 0; q < kAhead; ++q) {
+                    const float y[4] = {x[q].x, x[q].y, x[q].z, x[q].w};
+                    unsigned hits = 0u;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
-        if (lane == 0) s_quad[warp] = __double_as_longlong(sum);
-    }
-    consumer_sync();
-    if (tid == 0) {
-        const float M = fmaxf(fmaxf(s_ms[0].x, s_ms[1].x), fmaxf(s_ms[2].x, s_ms[3].x));
-        const double sum = __longlong_as_double(s_quad[0]) + __longlong_as_double(s_quad[1]) +
-                           __longlong_as_double(s_quad[2]) + __longlong_as_double(s_quad[3]);
-        a.row_lse[prow] = (static_cast<double>(M) + log2(sum)) * 0.6931471805599453094;
-        a.counter[prow] = 0u;
+                    for (int z = 0; z < 4; ++z)
+                        hits |= (float_to_ordered(y[z]) - least_ord <= ord_max - least_ord) ? (1u << z) : 0u;
+                    if (!hits) continue;
+                    int to = atomicAdd(&sh.count, __popc(hits));
+#pragma unroll
+                    for (int z = 0; z < 4; ++z)
+                        if ((hits >> z) & 1u) {
+                            if (to < kStreamList) sh.list[to] = pack_val_id(y[z], e[q] + z);
+                            ++to;
+                        }
+                }
+            }
+            consumer_sync();
+            n_cand = sh.count;
+            if (n_cand <= kStreamList) break;
+            rank_list(sh.list, kStreamList, k, nullptr, &sh.tau);
+            consumer_sync();
+            tau = sh.tau, least_ord = float_to_ordered(tau) + 1u;
+            if (tid == 0) sh.count = 0;
+            consumer_sync();
+        }
+        // fewer than k: the lowest ids among tau's equals fill up (tau = -inf: fewer than k finite logits)
+        const int e_end = min(a.vocab, w.c_end * kScanChunkMax);
+#pragma unroll 1
+        for (int e0 = w.c_begin * kScanChunkMax; e0 < e_end && n_cand < k; e0 += 4 * kScanThreads) {
+            const int e = e0 + tid * 4;
+            unsigned hits = 0u;
+            if (e < e_end) {
+                const float4 x = __ldg(reinterpret_cast<const float4*>(w.row + e));
+                const uint32_t t = float_to_ordered(tau);
+                hits = (float_to_ordered(x.x) == t) | (float_to_ordered(x.y) == t) << 1 | (float_to_ordered(x.z) == t) << 2 |
+                       (float_to_ordered(x.w) == t) << 3;
+            }
+            int incl = __popc(hits);
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int v = __shfl_up_sync(kFull, incl, d);
+                if (lane >= d) incl += v;
+            }
+            if (lane == 31) sh.warp_count[warp] = incl;
+            consumer_sync();
+            int to = n_cand + incl - __popc(hits), all = 0;
+#pragma unroll
+            for (int q = 0; q < kScanThreads / 32; ++q) {
+                if (q < warp) to += sh.warp_count[q];
+                all += sh.warp_count[q];
+            }
+#pragma unroll 1
+            for (; hits && to < k; hits &= hits - 1u) sh.list[to++] = pack_val_id(tau, e + __ffs(hits) - 1);
+            n_cand = min(k, n_cand + all);
+            consumer_sync();
+        }
+        // ---- the slice's k best and its log-sum-exp partial ------------------------------------------------
+        const int64_t prow = static_cast<int64_t>(w.b) * a.max_rows + w.r;
+        unsigned long long* part = a.part_key + (prow * a.splits + sl) * a.max_k;
+        rank_list(sh.list, n_cand, k, slices > 1 ? part : sh.top, nullptr);
+        if (tid >= n_cand && tid < k) (slices > 1 ? part : sh.top)[tid] = 0ull;  // fewer than k logits in the slice
+        if (warp == kScanThreads / 32 - 1) {
+            const float2 ms = lane < kScanThreads / 32 ? sh.ms[lane] : make_float2(-INFINITY, 0.f);
+            const float M = warp_maximum(ms.x), S = warp_total(weighted(ms.y, ms.x, M));
+            if (lane == 0) (slices > 1 ? a.part_ms[prow * a.splits + sl] : sh.total) = make_float2(M, S);
+        }
+        bool last = true;
+        if (slices > 1) {
+            __threadfence();
+            consumer_sync();
+            if (tid == 0) sh.last = (atomicAdd(a.counter + prow, 1u) == static_cast<unsigned>(slices - 1));
+            consumer_sync();
+            last = sh.last != 0;
+        }
+        if (last) {
+            // ---- last CTA of the row: merge the slices --------------------------------------------------
+            if (slices > 1) {
+                __threadfence();
+                const unsigned long long* parts = a.part_key + prow * a.splits * a.max_k;
+#pragma unroll 1
+                for (int i = tid; i < slices * k; i += kScanThreads) {
+                    const int from = i / k;
+                    sh.list[i] = __ldcg(parts + from * a.max_k + (i - from * k));
+                }
+                consumer_sync();
+                rank_list(sh.list, slices * k, k, sh.top, nullptr);
+            }
+            if (warp == kScanThreads / 32 - 1) {  // weights in fp32 (relative error 2^-22), accumulation in fp64
+                float M = -INFINITY;
+                double sum = 0.0;
+                __syncwarp();
+#pragma unroll 1
+                for (int i = lane; i < slices; i += 32) {
+                    const float2 ms = slices > 1 ? __ldcg(a.part_ms + prow * a.splits + i) : sh.total;
+                    const float m = fmaxf(M, ms.x);
+                    sum = sum * weighted(1.f, M, m) + weighted(ms.y, ms.x, m);
+                    M = m;
+                }
+                const float all = warp_maximum(M);
+                sum *= weighted(1.f, M, all);
+#pragma unroll 1
+                for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+                if (lane == 0) {
+                    a.row_lse[prow] = (static_cast<double>(all) + log2(sum)) * 0.6931471805599453094;
+                    if (slices > 1) a.counter[prow] = 0u;
+                }
+            }
+            consumer_sync();
+            if (tid < k) {
+                a.row_val[prow * a.max_k + tid] = key_val(sh.top[tid]);
+                a.row_id[prow * a.max_k + tid] = max(key_id(sh.top[tid]), 0);  // (< 0 only after an expired wait)
+            }
+        }
+        consumer_sync();  // the next slice writes what this one has read
     }
 }
 
@@ -854,15 +955,18 @@ __global__ void __launch_bounds__(128) shard_merge_rows_kernel(const ShardMergeA
     if (r >= 1 + (sd.d - 1) * k) return;
     const int64_t prow = static_cast<int64_t>(b) * a.max_rows + r;
     const int n = a.n_shards * k;
+#pragma unroll 1
     for (int i = tid; i < n; i += blockDim.x) {
         const int p = i / k, q = i - p * k;
         const int64_t src = (static_cast<int64_t>(p) * a.batch * a.max_rows + prow) * a.max_k + q;
         s_keys[i] = pack_val_id(a.all_val[src], a.all_id[src] + a.shard_offset[p]);
     }
     __syncthreads();
+#pragma unroll 1
     for (int c = tid; c < n; c += blockDim.x) {
         const unsigned long long mine = s_keys[c];
         int rank = 0;
+#pragma unroll 4
         for (int j = 0; j < n; ++j) rank += (s_keys[j] > mine) || (s_keys[j] == mine && j < c);
         if (rank < k) {
             a.row_val[prow * a.max_k + rank] = key_val(mine);
@@ -871,8 +975,10 @@ __global__ void __launch_bounds__(128) shard_merge_rows_kernel(const ShardMergeA
     }
     if (tid == 0) {  // log of the sum over the shards of exp(shard's log-sum-exp), fp64
         double m = -INFINITY;
+#pragma unroll 1
         for (int p = 0; p < a.n_shards; ++p) m = fmax(m, a.all_lse[static_cast<int64_t>(p) * a.batch * a.max_rows + prow]);
         double sum = 0.0;
+#pragma unroll 1
         for (int p = 0; p < a.n_shards; ++p) sum += exp(a.all_lse[static_cast<int64_t>(p) * a.batch * a.max_rows + prow] - m);
         a.row_lse[prow] = m + log(sum);
     }
@@ -910,22 +1016,17 @@ inline bool vec_ok(const void* p, int64_t s0, int64_t s1, int64_t s2, int vocab,
 
 int scan_chunk_max() { return kScanChunkMax; }
 
-static size_t stream_smem_bytes(int max_k, int slices) {
-    return kStreamStages * kScanChunkMax * sizeof(float) +
-           sizeof(unsigned long long) * max((kQuadElems + 1) * max_k, slices * max_k);
-}
+constexpr size_t kStreamSmem = kStreamStages * kScanChunkMax * sizeof(float);
 
-cudaError_t scan_setup(resps_ctx* ctx) {
-    cudaError_t e = cudaFuncSetAttribute(row_argmax_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kStreamStages * kScanChunkMax * sizeof(float)));
+cudaError_t scan_setup(resps_ctx*) {
+    cudaError_t e = cudaFuncSetAttribute(row_argmax_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamSmem));
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(row_scan_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(stream_smem_bytes(ctx->shape.max_k, 128)));
+    return cudaFuncSetAttribute(row_scan_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamSmem));
 }
 
 cudaError_t launch_row_scan(const resps_ctx* ctx, const resps_step* d_steps, int batch,
                             const float* logits, int64_t ld_b, int64_t ld_level, int64_t ld_row,
-                            int n_levels, int n_slots, int only_level, cudaStream_t st) {
+                            int n_levels, int n_slots, int only_level, cudaStream_t st, const ScanRows* out) {
     const Workspace& w = ctx->ws;
     ScanArgs a;
     a.steps = d_steps;
@@ -935,29 +1036,30 @@ cudaError_t launch_row_scan(const resps_ctx* ctx, const resps_step* d_steps, int
     a.vocab = ctx->shape.vocab, a.max_tt = ctx->shape.max_tt, a.max_k = ctx->shape.max_k;
     a.max_rows = w.max_rows, a.chunk = w.scan_chunk, a.splits = w.scan_splits;
     a.part_key = w.part_key, a.part_ms = w.part_ms, a.counter = w.row_counter;
-    a.row_val = w.row_val, a.row_id = w.row_id, a.row_lse = w.row_lse, a.status = w.status;
+    a.row_val = out ? out->val : w.row_val, a.row_id = out ? out->id : w.row_id, a.row_lse = out ? out->lse : w.row_lse;
+    a.status = w.status;
     const int k_ext = min(n_slots, ctx->shape.max_k);
     a.only_level = only_level;
     const int rows = (only_level >= 0) ? (only_level == 0 ? 1 : k_ext) : ((n_levels > 1) ? 1 + (n_levels - 1) * k_ext : 1);
-    a.slices = w.scan_splits, a.cps = 1;
+    a.slices = w.scan_slices_hint;
     a.test_drop = w.test_drop;
-    const size_t smem = sizeof(unsigned long long) * ctx->shape.max_k * max(kQuadElems, w.scan_splits);
-    if (vec_ok(logits, ld_b, ld_level, ld_row, a.vocab, a.chunk) && w.scan_chunk == kScanChunkMax) {
-        // Slices per row: two CTAs fit an SM, and a slice's first chunk costs about three later ones (the
-        // threshold has to be found), so a row is cut only as far as all CTAs still run at once; with
-        // more rows than that, one slice per row (measured at 712 rows: 108 us in one slice, 119 in two).
-        int want = max(1, 2 * ctx->sm_count / max(rows * batch, 1));
-        if (w.scan_slices_hint > 0) want = w.scan_slices_hint;
-        const int slices0 = max(1, min(w.scan_splits, want));
-        a.cps = (w.scan_splits + slices0 - 1) / slices0;
-        a.slices = (w.scan_splits + a.cps - 1) / a.cps;
-        dim3 grid(a.slices, rows, batch);
-        return launch_pdl(row_scan_stream_kernel, grid, dim3(kStreamThreads), stream_smem_bytes(ctx->shape.max_k, a.slices), st, a);
-    } else {
-        dim3 grid(w.scan_splits, rows, batch);
-        return launch_pdl(row_scan_kernel<false>, grid, dim3(kScanThreads), smem, st, a);
+    if (!(vec_ok(logits, ld_b, ld_level, ld_row, a.vocab, a.chunk) && w.scan_chunk == kScanChunkMax)) {
+        const size_t smem = sizeof(unsigned long long) * ctx->shape.max_k * max(kQuadElems, w.scan_splits);
+        return launch_pdl(row_scan_kernel<false>, dim3(w.scan_splits, rows, batch), dim3(kScanThreads), smem, st, a);
     }
-    return cudaGetLastError();
+    for (int b0 = 0; b0 < batch; b0 += kStreamMaxBatch) {
+        a.batch = min(kStreamMaxBatch, batch - b0);
+        // two resident CTAs per SM, no more than there are chunks
+        const int64_t most = static_cast<int64_t>(rows) * a.batch * w.scan_splits;
+        const int grid = static_cast<int>(min(static_cast<int64_t>(2 * ctx->sm_count), most));
+        const cudaError_t e = launch_pdl(row_scan_stream_kernel, dim3(grid), dim3(kStreamThreads), kStreamSmem, st, a);
+        if (e != cudaSuccess) return e;
+        const int64_t rows_on = static_cast<int64_t>(a.batch) * w.max_rows;
+        a.steps += a.batch, a.logits += a.batch * ld_b;
+        a.part_key += rows_on * a.splits * a.max_k, a.part_ms += rows_on * a.splits, a.counter += rows_on;
+        a.row_val += rows_on * a.max_k, a.row_id += rows_on * a.max_k, a.row_lse += rows_on;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_row_argmax(const resps_ctx* ctx, const int32_t* d_n_nodes, int batch,
@@ -985,8 +1087,7 @@ cudaError_t launch_row_argmax(const resps_ctx* ctx, const int32_t* d_n_nodes, in
         if (walk) wa = *walk;
         if (walked) *walked = walk != nullptr;
         dim3 grid(a.slices, ctx->shape.max_tt, batch);
-        return launch_pdl(row_argmax_stream_kernel, grid, dim3(kStreamThreads),
-                          kStreamStages * kScanChunkMax * sizeof(float), st, a, wa, walk ? 1 : 0);
+        return launch_pdl(row_argmax_stream_kernel, grid, dim3(kStreamThreads), kStreamSmem, st, a, wa, walk ? 1 : 0);
     }
     dim3 grid(w.scan_splits, ctx->shape.max_tt, batch);
     if (vec_ok(logits, ld_b, ld_row, 0, a.vocab, a.chunk))
