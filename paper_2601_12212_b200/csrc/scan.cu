@@ -268,14 +268,16 @@ __global__ void __launch_bounds__(kScanThreads, 4) row_scan_kernel(const ScanArg
 // A chunk costs its eight consumer warps one wait, a maximum and the exponentials: no barrier, no selection.
 // At the end of a slice the k-th best of the 64 quad maxima (quad = 4 threads, 128 logits of every chunk) is
 // a lower bound tau of the slice's k-th best; the threads whose own maximum reaches tau (about k of 256) are
-// the only ones that can hold a candidate, and their logits are read once more, from L2, by all threads
-// together.  About 2 k candidates are ranked by counting.  Should they not fit the list (many equal logits,
+// the only ones that can hold a candidate.  Those of the chunk of a thread's maximum (of all its chunks, where a
+// second one reaches tau) are read once more, from the stages if they still stand there, else from L2, by all
+// threads together.  About 2 k candidates are ranked by counting.  Should they not fit the list (many equal logits,
 // adversarial order), tau is raised until the strictly better ones do, and the lowest ids among its equals
 // fill up.
 //
 // Bound by HBM where there are many rows; where a CTA has two or three chunks by its start, the slice's tail
 // and the merge of the row.  With selection chunk by chunk (two to six barriers a chunk) and a fixed grid of slices
-// the tree build of d=8 k=32 (225 rows of 128256 logits) took 98 us (now 69), a shard's scan 14.2 us (now 10.1).
+// the tree build of d=8 k=32 (225 rows of 128256 logits) took 98 us (now 63), the scan of 680
+// rows of 128256 logits ran at 6.0 TB/s (now 7.5), a shard's scan took 14.2 us (now 9.8).
 // ---------------------------------------------------------------------------------------
 constexpr int kStreamStages = 3;
 constexpr int kStreamMaxBatch = 256; // sequences of one launch
@@ -324,9 +326,9 @@ struct StreamShared {
     int row0[kStreamMaxBatch + 1];  // first row of a sequence
     int k[kStreamMaxBatch];
     int warp_count[kScanThreads / 32];
-    unsigned char thr[kScanThreads];  // threads that may hold candidates
+    int pick[kScanThreads];  // threads that may hold candidates: from the front in one chunk, from the back in any
     float tau;
-    int count, last;
+    int count, singles, wholes, last;
 };
 
 // k-th best value (by value alone) of `n` >= k keys, to `*out`; the `k` best in order to `top` when given.
@@ -403,7 +405,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) row_scan_stream_kernel(cons
     // the ranges: never so short that a row's merge (slices x k entries) would not fit the list
     const int total = sh.row0[a.batch] * a.splits;
     const int most_slices = max(1, min(a.slices > 0 ? a.slices : a.splits, kStreamList / a.max_k - 2));
-    const int least = (a.splits + most_slices - 1) / most_slices;
+    const int least = (a.splits + most_slices - 1) / most_slices;  // chunks
     const int ctas = max(1, min(static_cast<int>(gridDim.x), total / least));
     if (static_cast<int>(blockIdx.x) >= ctas) return;
     const int base = total / ctas, longer = total - base * ctas;  // the first `longer` ranges have one chunk more
@@ -437,53 +439,52 @@ __global__ void __launch_bounds__(kStreamThreads, 2) row_scan_stream_kernel(cons
         return w;
     };
 
-    if (warp == kScanThreads / 32) {
-        // ---- copy-issuing warp: a stage is refilled as soon as every consumer warp has read it ----------
-        if (lane == 0) {
-            uint32_t u = 0;
+    // A range that fits the stages stays there, and the second look at the logits reads it from there.
+    const bool stays = x_end - x_begin <= kStreamStages;
+    uint32_t stage = 0, phase = 0;  // of the next chunk
+    auto advance = [&]() {
+        if (++stage == kStreamStages) stage = 0, phase ^= 1u;
+    };
 #pragma unroll 1
-            for (int x = x_begin; x < x_end;) {
-                const Work w = work_at(x);
-                x += w.c_end - w.c_begin;
+    for (int x = x_begin; x < x_end;) {  // one loop for both roles: the code that finds a slice is fetched once
+        const Work w = work_at(x);
+        const int row0 = x - w.c_begin;  // first chunk of the row
+        x += w.c_end - w.c_begin;
+        if (warp == kScanThreads / 32) {
+            // ---- copy-issuing warp: a stage is refilled as soon as every consumer warp has read it ------
+            if (lane == 0) {
 #pragma unroll 1
-                for (int c = w.c_begin; c < w.c_end; ++c, ++u) {
-                    const uint32_t st = u % kStreamStages;
-                    scan_mbar_wait(empty_bar(st), ((u / kStreamStages) & 1u) ^ 1u, a.status);
+                for (int c = w.c_begin; c < w.c_end; ++c, advance()) {
+                    scan_mbar_wait(empty_bar(stage), phase ^ 1u, a.status);
                     const int e0 = c * kScanChunkMax;
                     const uint32_t bytes = static_cast<uint32_t>(min(a.vocab - e0, kScanChunkMax)) * 4u;
-                    if (kWaitTest && (a.test_drop & 2) && u == 1) continue;
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full_bar(st)), "r"(bytes)
+                    if (kWaitTest && (a.test_drop & 2) && stage == 1 && phase == 0) continue;
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full_bar(stage)), "r"(bytes)
                                  : "memory");
                     asm volatile(
                         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                            scan_smem_u32(s_stage + st * kScanChunkMax)),
-                        "l"(w.row + e0), "r"(bytes), "r"(full_bar(st))
+                            scan_smem_u32(s_stage + stage * kScanChunkMax)),
+                        "l"(w.row + e0), "r"(bytes), "r"(full_bar(stage))
                         : "memory");
                 }
             }
+            continue;  // the consumers wait for every copy that was issued
         }
-        return;  // the consumers wait for every copy that was issued
-    }
-
-    uint32_t u0 = 0;
-#pragma unroll 1
-    for (int x = x_begin; x < x_end;) {
-        const Work w = work_at(x);
-        const int k = w.k, row0 = x - w.c_begin;  // first chunk of the row
+        const int k = w.k;
         const int first = owner(row0), slices = owner(row0 + a.splits - 1) - first + 1, sl = me - first;
-        x += w.c_end - w.c_begin;
-        LseAcc acc;                // this thread's running (max, sum) over all its logits of the slice
-        float best = -INFINITY;    // its best logit
+        const float* again = stays ? s_stage + stage * kScanChunkMax : w.row + w.c_begin * kScanChunkMax;
+        LseAcc acc;                                  // this thread's running (max, sum) over all its logits of the slice
+        float best = -INFINITY, second = -INFINITY;  // its best logit, the best one of its other chunks
+        int best_c = 0;                              // chunk of the best, from the slice's first
 #pragma unroll 1
-        for (int c = w.c_begin; c < w.c_end; ++c, ++u0) {
-            const uint32_t st = u0 % kStreamStages;
+        for (int c = w.c_begin; c < w.c_end; ++c, advance()) {
             const int begin = c * kScanChunkMax, end = min(a.vocab, begin + kScanChunkMax);
-            scan_mbar_wait(full_bar(st), (u0 / kStreamStages) & 1u, a.status);
+            scan_mbar_wait(full_bar(stage), phase, a.status);
             float v[kScanPerThread];
             if (end - begin == kScanChunkMax) {
 #pragma unroll
                 for (int u = 0; u < kScanPerThread / 4; ++u) {
-                    const float4 x = *reinterpret_cast<const float4*>(s_stage + st * kScanChunkMax + (u * kScanThreads + tid) * 4);
+                    const float4 x = *reinterpret_cast<const float4*>(s_stage + stage * kScanChunkMax + (u * kScanThreads + tid) * 4);
                     v[4 * u] = x.x, v[4 * u + 1] = x.y, v[4 * u + 2] = x.z, v[4 * u + 3] = x.w;
                 }
             } else {
@@ -491,16 +492,18 @@ __global__ void __launch_bounds__(kStreamThreads, 2) row_scan_stream_kernel(cons
                 for (int u = 0; u < kScanPerThread / 4; ++u) {
                     const int off = (u * kScanThreads + tid) * 4;
                     float4 x = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-                    if (begin + off < end) x = *reinterpret_cast<const float4*>(s_stage + st * kScanChunkMax + off);  // (the vocabulary is a multiple of 4)
+                    if (begin + off < end) x = *reinterpret_cast<const float4*>(s_stage + stage * kScanChunkMax + off);  // (the vocabulary is a multiple of 4)
                     v[4 * u] = x.x, v[4 * u + 1] = x.y, v[4 * u + 2] = x.z, v[4 * u + 3] = x.w;
                 }
             }
             __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty_bar(st)) : "memory");
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty_bar(stage)) : "memory");
             float tmax = v[0];
 #pragma unroll
             for (int i = 1; i + 1 < kScanPerThread; i += 2) tmax = max3f(tmax, v[i], v[i + 1]);
             tmax = fmaxf(tmax, v[kScanPerThread - 1]);
+            second = fmaxf(second, fminf(best, tmax));
+            best_c = tmax > best ? c - w.c_begin : best_c;
             best = fmaxf(best, tmax);
             const float m_new = fmaxf(acc.m2, tmax * kLog2e);
             if (m_new > -INFINITY) {
@@ -519,39 +522,36 @@ __global__ void __launch_bounds__(kStreamThreads, 2) row_scan_stream_kernel(cons
             float q = fmaxf(best, __shfl_xor_sync(kFull, best, 1));
             q = fmaxf(q, __shfl_xor_sync(kFull, q, 2));
             if ((lane & 3) == 0) sh.quad[tid >> 2] = q;
-            if (tid == 0) sh.count = 0;
+            if (tid == 0) sh.count = sh.singles = sh.wholes = 0;
         }
         const float warp_max = warp_maximum(acc.m2);  // log-sum-exp partial of the warp, merged below
         const float warp_sum = warp_total(weighted(acc.s, acc.m2, warp_max));
         if (lane == 0) sh.ms[warp] = make_float2(warp_max, warp_sum);
         consumer_sync();
-        if (tid < kQuads) {
-            const float mine = sh.quad[tid];
+        {  // four threads per quad, each against 16 others
+            const int q = tid >> 2, part = tid & 3;
+            const float mine = sh.quad[q];
             int rank = 0;
-#pragma unroll 4
-            for (int j = 0; j < kQuads; j += 4) {
+#pragma unroll
+            for (int j = part * 16; j < part * 16 + 16; j += 4) {
                 const float4 o = *reinterpret_cast<const float4*>(sh.quad + j);
-                rank += (o.x > mine || (o.x == mine && j < tid)) + (o.y > mine || (o.y == mine && j + 1 < tid)) +
-                        (o.z > mine || (o.z == mine && j + 2 < tid)) + (o.w > mine || (o.w == mine && j + 3 < tid));
+                rank += (o.x > mine || (o.x == mine && j < q)) + (o.y > mine || (o.y == mine && j + 1 < q)) +
+                        (o.z > mine || (o.z == mine && j + 2 < q)) + (o.w > mine || (o.w == mine && j + 3 < q));
             }
-            if (rank == k - 1) sh.tau = mine;
+            rank += __shfl_xor_sync(kFull, rank, 1);
+            rank += __shfl_xor_sync(kFull, rank, 2);
+            if (part == 0 && rank == k - 1) sh.tau = mine;
         }
         consumer_sync();
         float tau = sh.tau;
-        // ---- the threads that may hold candidates; their logits once more, by everybody ----------------------
-        const bool mine = best >= tau && best > -INFINITY;
-        const unsigned bal = __ballot_sync(kFull, mine);
-        if (lane == 0) sh.warp_count[warp] = __popc(bal);
-        consumer_sync();
-        int n_thr = 0, at = __popc(bal & ((1u << lane) - 1u));
-#pragma unroll
-        for (int q = 0; q < kScanThreads / 32; ++q) {
-            if (q < warp) at += sh.warp_count[q];
-            n_thr += sh.warp_count[q];
+        // ---- the threads that may hold candidates, most of them in one chunk only; their logits once more ----
+        if (best >= tau && best > -INFINITY) {
+            if (second < tau) sh.pick[atomicAdd(&sh.singles, 1)] = best_c << 8 | tid;
+            else sh.pick[kScanThreads - 1 - atomicAdd(&sh.wholes, 1)] = tid;
         }
-        if (mine) sh.thr[at] = static_cast<unsigned char>(tid);
         consumer_sync();
-        const int per_thr = (w.c_end - w.c_begin) * (kScanPerThread / 4), n_vec = n_thr * per_thr;
+        const int per_thr = (w.c_end - w.c_begin) * (kScanPerThread / 4), n_single = sh.singles * (kScanPerThread / 4);
+        const int n_vec = n_single + sh.wholes * per_thr;
         // Every logit at or above tau is appended while the list has room (-inf only by the filling below).  If
         // there were too many, tau becomes the k-th best found so far, and only the better ones are taken.
         const uint32_t ord_max = float_to_ordered(INFINITY);  // (NaNs of positive sign lie above)
@@ -566,10 +566,20 @@ __global__ void __launch_bounds__(kStreamThreads, 2) row_scan_stream_kernel(cons
                 int e[kAhead];
 #pragma unroll
                 for (int q = 0; q < kAhead; ++q) {
-                    const int i = min(i0 + q * kScanThreads, n_vec - 1), t = i / per_thr, rest = i - t * per_thr;
-                    e[q] = w.c_begin * kScanChunkMax + (rest * kScanThreads + sh.thr[t]) * 4;
+                    const int i = min(i0 + q * kScanThreads, n_vec - 1);
+                    int from, at;  // entry of the list, position among the thread's groups of 4 logits
+                    if (i < n_single) {
+                        from = sh.pick[i / (kScanPerThread / 4)];
+                        at = (from >> 8) * (kScanPerThread / 4) + i % (kScanPerThread / 4);
+                    } else {
+                        const int t = (i - n_single) / per_thr;
+                        from = sh.pick[kScanThreads - 1 - t];
+                        at = i - n_single - t * per_thr;
+                    }
+                    const int off = (at * kScanThreads + (from & (kScanThreads - 1))) * 4;
+                    e[q] = w.c_begin * kScanChunkMax + off;
                     x[q] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-                    if (e[q] < a.vocab && i0 + q * kScanThreads < n_vec) x[q] = __ldg(reinterpret_cast<const float4*>(w.row + e[q]));
+                    if (e[q] < a.vocab && i0 + q * kScanThreads < n_vec) x[q] = *reinterpret_cast<const float4*>(again + off);
                 }
 #pragma unroll
                 for (int q = 0; q < kAhead; ++q) {
