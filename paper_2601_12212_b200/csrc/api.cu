@@ -50,14 +50,12 @@ void carve(resps_ctx* c, Carver& cv) {
     cv.take(w.row_counter, rows);
     cv.take(w.amax_counter, nodes);
     cv.take(w.amax_seq_counter, s.max_batch);
-    cv.take(w.ctl_counter, s.max_batch);
     const int64_t zero_end = cv.off;  // everything above must start as zero
     (void)zero_end;
     cv.take(w.node_row, nodes);
     cv.take(w.tree_frontier, static_cast<int64_t>(s.max_batch) * RESPS_MAX_DEPTH * RESPS_MAX_K);
     cv.take(w.tree_score, static_cast<int64_t>(s.max_batch) * RESPS_MAX_DEPTH * RESPS_MAX_K);
     cv.take(w.amax_local, nodes);
-    cv.take(w.ctl_h1, static_cast<int64_t>(s.max_batch) * resps::controller_max_hidden());
     cv.take(w.samp_scratch, static_cast<int64_t>(resps::sampled_scratch_doubles(s.max_batch, s.vocab)));
     cv.take(w.part_key, rows * w.scan_splits * s.max_k);
     cv.take(w.part_ms, rows * w.scan_splits);
@@ -153,7 +151,8 @@ int resps_create(resps_ctx** out, const resps_shape* shape) {
     real.base = static_cast<char*>(c->arena);
     carve(c, real);
     if (resps::attention_setup(c) != cudaSuccess || resps::tree_setup(c) != cudaSuccess ||
-        resps::scan_setup(c) != cudaSuccess || resps::sampled_setup(c) != cudaSuccess) {
+        resps::scan_setup(c) != cudaSuccess || resps::sampled_setup(c) != cudaSuccess ||
+        resps::controller_setup(c) != cudaSuccess) {
         cudaFree(c->arena);
         resps::attention_teardown(c);
         delete c;
@@ -212,7 +211,6 @@ int resps_status(resps_ctx* ctx, resps_stream stream, int32_t* status) {
         if (cudaMemsetAsync(w.row_counter, 0, rows * sizeof(unsigned int), stream) != cudaSuccess ||
             cudaMemsetAsync(w.amax_counter, 0, nodes * sizeof(unsigned int), stream) != cudaSuccess ||
             cudaMemsetAsync(w.amax_seq_counter, 0, ctx->shape.max_batch * sizeof(unsigned int), stream) != cudaSuccess ||
-            cudaMemsetAsync(w.ctl_counter, 0, ctx->shape.max_batch * sizeof(unsigned int), stream) != cudaSuccess ||
             cudaStreamSynchronize(stream) != cudaSuccess)
             return RESPS_ERR_CUDA;
     }

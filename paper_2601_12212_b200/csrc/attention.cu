@@ -490,8 +490,6 @@ __device__ __forceinline__ void mbar_arrive_remote(uint32_t bar, int rank) {
         "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [remote];\n\t}" ::"r"(bar), "r"(rank)
         : "memory");
 }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 // Bounded wait: false when this wait ran out (about a second of SM clocks) or another thread of
 // the CTA has given up.  Kept to a few instructions, because it is inlined at every wait: a role runs
 // through its code once per launch, most of it cold, and what it costs to fetch is about a cycle per 4

@@ -41,8 +41,6 @@ struct Workspace {
     int32_t* node_row = nullptr;             // [max_batch][max_tt] draft row behind every node's children (tree build)
     int32_t* tree_frontier = nullptr;        // [max_batch][RESPS_MAX_DEPTH][RESPS_MAX_K] level form: frontiers so far
     double* tree_score = nullptr;            // ... and their path scores
-    float* ctl_h1 = nullptr;                 // controller: first hidden layer [max_batch][256]
-    unsigned int* ctl_counter = nullptr;     // controller: hidden units done per sequence (self-resetting)
     double* samp_scratch = nullptr;          // acceptance under sampling: partial sums, then (p, q) of every token and sequence
     unsigned int* amax_seq_counter = nullptr;  // [max_batch] arg-max CTAs of a sequence that have delivered (self-resetting)
     // attention
@@ -157,6 +155,19 @@ cudaError_t launch_pdl(Kernel kernel, dim3 grid, dim3 block, size_t smem, cudaSt
     cfg.attrs = attr, cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
+// The same for clusters of `cluster` CTAs along x.
+template <typename Kernel, typename... Args>
+cudaError_t launch_pdl_cluster(Kernel kernel, unsigned cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid, cfg.blockDim = block, cfg.dynamicSmemBytes = smem, cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster, attr[1].val.clusterDim.y = 1, attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr, cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 cudaError_t launch_accept_sampled(const resps_ctx* ctx, const resps_step* d_steps, const int32_t* d_n_nodes, int batch,
                                   const float* target, int64_t ld_b, int64_t ld_row, const float* draft, int64_t dld_b,
                                   int64_t dld_level, int64_t dld_row, double temperature, const int32_t* tokens,
@@ -174,6 +185,7 @@ int controller_max_actions();
 cudaError_t tree_setup(resps_ctx* ctx);
 cudaError_t scan_setup(resps_ctx* ctx);
 cudaError_t sampled_setup(resps_ctx* ctx);
+cudaError_t controller_setup(resps_ctx* ctx);
 int tree_candidate_limit();
 
 // ---- device helpers --------------------------------------------------------
@@ -263,6 +275,26 @@ __device__ __forceinline__ void accept_walk_device(const AcceptArgs& a, int b, i
 }
 
 // Step parameters clamped into the extents the caller supplied.
+// Thread-block clusters: this CTA's rank, the barrier over all threads, a peer's copy of a shared variable.
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+__device__ __forceinline__ void cluster_barrier() {
+    cluster_arrive();
+    cluster_wait();
+}
+__device__ __forceinline__ uint32_t peer_address(const void* local, unsigned peer) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                 : "=r"(remote)
+                 : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(local))), "r"(peer));
+    return remote;
+}
+
 struct StepDims {
     int tt, d, k, L;
     bool clamped;

@@ -5,11 +5,18 @@
 // just finished and, when the interval is over, asks the policy and writes the new (TT, d, k) into the
 // device-resident step parameters, where the kernels of the step read them.
 //
-// The policy's first layer is a matrix-vector product over the 3 x 4096 state (6 MB of fp32 weights):
-// a CTA per hidden unit and sequence, each thread a strided share of the features in 16-byte loads that
-// are all in flight together, fp32 accumulation.  The last CTA of a sequence to arrive runs the two
-// small layers (two threads per output, half a row each), picks the action and updates the state;
-// sequences whose cached action is still valid skip the product altogether.
+// A cluster of 16 CTAs serves one sequence, every CTA a sixteenth of each layer's outputs.  The first layer
+// is a matrix-vector product over the 3 x 4096 state (6 MB of fp32 weights): a CTA stages the state in shared
+// memory once for all of its hidden units, a few warps share a unit, and a thread keeps eight 16-byte loads in
+// flight.  The weights of the two small layers are asked into L2 before that and then wait in registers, a row to a
+// warp; the layers' outputs travel to the peers' shared memory behind the cluster's barrier, so that nothing goes
+// through global memory.  The choice is made by one CTA:
+// maximum, exponentials and running sums by all of its threads.
+//
+// Bound by the first layer's weights through L2 into 16 SMs per sequence (0.4 MB each, about 3 us), around it
+// a chain of three exchanges; a step whose cached action is still valid is bound by its launch.  With a CTA
+// per hidden unit and the last one to arrive running both small layers and, by one thread, the softmax, a step
+// that asks took 40 us at 8 sequences of the 3 x 4096 state and 180 actions (now 15), one that does not the same 2.2.
 #include <cmath>
 
 #include "common.cuh"
@@ -17,10 +24,16 @@
 namespace resps {
 namespace {
 
-constexpr int kCtlThreads = 256;
+constexpr int kCtlThreads = 512;
+constexpr int kWarps = kCtlThreads / 32;
+constexpr int kClu = 16;            // CTAs per sequence (more than 8: not portable, sm_100 has it)
 constexpr int kMaxHidden = 256;
 constexpr int kMaxActions = 1024;
+constexpr int kStage = 16384;       // features staged at once
+constexpr int kAhead = 8;           // 16-byte loads of a thread in flight
 constexpr unsigned kFull = 0xFFFFFFFFu;
+static_assert(kMaxHidden <= kClu * kWarps, "a warp per hidden unit in the second layer");
+static_assert(kMaxActions <= 2 * kCtlThreads, "two actions per thread in the choice");
 
 struct ControllerArgs {
     resps_policy pol;
@@ -36,83 +49,66 @@ struct ControllerArgs {
     float* reward_avg;           // [batch]: written when an interval closes (else left alone)
     float* logits_out;           // [batch][n_actions] or null
     int32_t* action_out;         // [batch] or null
-    float* h1;                   // workspace [batch][hidden]
-    unsigned int* counter;       // workspace [batch]
 };
 
-__device__ __forceinline__ float block_sum(float v, float* s_red) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    float r = 0.f;
-    for (int w = 0; w < kCtlThreads / 32; ++w) r += s_red[w];
-    return r;
-}
+struct ControllerShared {
+    alignas(16) __nv_bfloat16 state[kStage];
+    float h1[kMaxHidden], h2[kMaxHidden];  // written by the peers
+    float logit[kMaxActions];              // of the first CTA: written by the peers
+    float part[kWarps];
+    unsigned long long key[kWarps];
+    double sum[kWarps];
+    int action;
+};
 
 __device__ __forceinline__ bool aligned_to(const void* p, unsigned bytes) {
     return (reinterpret_cast<unsigned long long>(p) & (bytes - 1u)) == 0ull;
 }
-
-// out(o) = bias[o] + sum_i W[o][i] * s_in[i] for o < n_out, by the whole CTA: two threads per output, each
-// half a row in 16-byte loads that are all in flight together (rows of 16-byte aligned fp32, n_in a
-// multiple of 8; one thread per output and scalar loads otherwise).
-template <typename Out>
-__device__ __forceinline__ void dense_layer(const float* W, const float* bias, const float* s_in, int n_out, int n_in,
-                                            Out out) {
-    const int tid = threadIdx.x;
-    if ((n_in & 7) == 0 && aligned_to(W, 16)) {
-        const int half = tid & 1, quads = n_in >> 3;  // float4 per half row
-        for (int o0 = 0; o0 < n_out; o0 += kCtlThreads / 2) {
-            const int o = o0 + (tid >> 1);
-            float acc = 0.f;
-            if (o < n_out) {
-                const float4* w4 = reinterpret_cast<const float4*>(W + static_cast<int64_t>(o) * n_in) + half * quads;
-                const float* x = s_in + half * quads * 4;
-#pragma unroll 8
-                for (int i = 0; i < quads; ++i) {
-                    const float4 w = __ldg(w4 + i);
-                    acc = fmaf(w.x, x[4 * i], fmaf(w.y, x[4 * i + 1], fmaf(w.z, x[4 * i + 2], fmaf(w.w, x[4 * i + 3], acc))));
-                }
-            }
-            acc += __shfl_xor_sync(kFull, acc, 1);
-            if (o < n_out && half == 0) out(o, acc + bias[o]);
-        }
-    } else {
-        for (int o = tid; o < n_out; o += kCtlThreads) {
-            const float* w = W + static_cast<int64_t>(o) * n_in;
-            float acc = bias[o];
-            for (int i = 0; i < n_in; ++i) acc = fmaf(__ldg(w + i), s_in[i], acc);
-            out(o, acc);
-        }
-    }
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    return v;
 }
+// one float to the same place in the shared memory of peer `lane` (of all peers: by 16 lanes)
+__device__ __forceinline__ void store_to_peer(float* local, unsigned peer, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(peer_address(local, peer)), "f"(v) : "memory");
+}
+// row . s_x over n inputs by a warp, the row's elements already in registers (n <= kMaxHidden)
+struct Row {
+    float w[kMaxHidden / 32];
+    __device__ __forceinline__ void load(const float* row, int n, int lane, bool valid) {
+#pragma unroll
+        for (int j = 0; j < kMaxHidden / 32; ++j) w[j] = (valid && lane + 32 * j < n) ? __ldg(row + lane + 32 * j) : 0.f;
+    }
+    __device__ __forceinline__ float dot(const float* s_x, int n, int lane) const {
+        float acc = 0.f;
+#pragma unroll
+        for (int j = 0; j < kMaxHidden / 32; ++j)
+            if (lane + 32 * j < n) acc = fmaf(w[j], s_x[lane + 32 * j], acc);
+        return warp_sum(acc);
+    }
+};
 
-__global__ void __launch_bounds__(kCtlThreads) controller_kernel(const ControllerArgs a) {
+__global__ void __launch_bounds__(kCtlThreads, 2) controller_kernel(const ControllerArgs a) {
     pdl_wait();  // the kernel before this one in the stream has completed
     pdl_launch_dependents();
-    __shared__ float s_red[kCtlThreads / 32];
-    __shared__ float s_h1[kMaxHidden], s_h2[kMaxHidden];
-    __shared__ float s_logit[kMaxActions];
-    __shared__ double s_term[kMaxActions];
-    __shared__ double s_mx;
-    __shared__ unsigned long long s_key[kCtlThreads / 32];
-    __shared__ int s_last;
-    const int b = blockIdx.y, unit = blockIdx.x, tid = threadIdx.x;
+    __shared__ ControllerShared sh;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned rank = cluster_rank();
+    const int b = blockIdx.x / kClu;
     const resps_controller_state st = a.state[b];
     const bool ask = (st.cache_step == 0) || (st.action < 0);
-    const int H = a.pol.hidden, F = a.pol.n_features, A = a.pol.n_actions;
+    const bool writer = rank == 0 && tid == 0;
+    cluster_arrive();  // waited for before the state, or a peer's shared memory, is written
+    resps_controller_state n = st;
+    if (writer && a.accept_len) {  // the finished step's reward
+        n.reward_sum += static_cast<float>(a.accept_len[b] + 1) / a.elapsed_s[b];
+        n.reward_steps += 1;
+    }
     if (!ask) {
-        // ---- the cached action stays: book the finished step's reward, advance the cache step ----------
-        // (by the last CTA of the sequence to come by, when every other one has read the state)
-        if (tid == 0 && atomicAdd(a.counter + b, 1u) == static_cast<unsigned>(H - 1)) {
-            a.counter[b] = 0u;
-            resps_controller_state n = st;
-            if (a.accept_len) {
-                n.reward_sum += static_cast<float>(a.accept_len[b] + 1) / a.elapsed_s[b];
-                n.reward_steps += 1;
-            }
+        // ---- the cached action stays: advance the cache step (once every CTA has read the state) ------------
+        cluster_wait();
+        if (writer) {
             n.cache_step += 1;
             if (n.cache_step >= a.interval) n.cache_step = 0;
             a.state[b] = n;
@@ -120,112 +116,162 @@ __global__ void __launch_bounds__(kCtlThreads) controller_kernel(const Controlle
         }
         return;
     }
-    // ---- first layer: hidden unit `unit` of sequence b -------------------------------------------------
+    const int H = a.pol.hidden, F = a.pol.n_features, A = a.pol.n_actions;
+    const int units = (H + kClu - 1) / kClu, u_lo = static_cast<int>(rank) * units, n_units = max(0, min(H - u_lo, units));
+    const int rows = (A + kClu - 1) / kClu, r_lo = static_cast<int>(rank) * rows, n_rows = max(0, min(A - r_lo, rows));
+    const float* row2 = a.pol.w2 + static_cast<int64_t>(u_lo + warp) * H;
+    const float* row3 = a.pol.w3 + static_cast<int64_t>(r_lo + warp) * H;
+    if (lane * 32 < H) {
+        if (warp < n_units) asm volatile("prefetch.global.L2 [%0];" ::"l"(row2 + lane * 32));
+        if (warp < n_rows) asm volatile("prefetch.global.L2 [%0];" ::"l"(row3 + lane * 32));
+    }
+
+    // ---- first layer: `per_unit` warps share a hidden unit ----------------------------------------------
+    const int per_unit = kWarps / units, mine = warp / per_unit, share = warp - mine * per_unit;
+    float acc = 0.f;
     {
         const int per_layer = F / 3;
-        const float* w = a.pol.w1 + static_cast<int64_t>(unit) * F;
-        float acc = 0.f;
-        const bool vec = (per_layer & 3) == 0 && (a.ld_hidden & 3) == 0 && aligned_to(a.pol.w1, 16) &&
-                         aligned_to(a.hidden[0], 8) && aligned_to(a.hidden[1], 8) && aligned_to(a.hidden[2], 8);
-        if (vec) {
-            // four weights (16 bytes) and four features (8 bytes) per load, the loads of a thread independent
-            // of one another: the 6 MB of weights stream in one or two round trips
+        const bool vec_h = (per_layer & 7) == 0 && (a.ld_hidden & 7) == 0 && aligned_to(a.hidden[0], 16) &&
+                           aligned_to(a.hidden[1], 16) && aligned_to(a.hidden[2], 16);
+        const bool vec_w = (F & 3) == 0 && aligned_to(a.pol.w1, 16);
+#pragma unroll 1
+        for (int f0 = 0; f0 < F; f0 += kStage) {
+            const int nf = min(kStage, F - f0);
+            if (f0 > 0) __syncthreads();  // the last part has been read
+            const float* w = a.pol.w1 + static_cast<int64_t>(u_lo + mine) * F + f0;
+            const float4* w4 = reinterpret_cast<const float4*>(w);
+            const int quads = (vec_w && mine < n_units) ? nf >> 2 : 0, step = per_unit * 32;
+            float4 x[kAhead];
+            int i = share * 32 + lane;
 #pragma unroll
-            for (int layer = 0; layer < 3; ++layer) {
-                const float4* w4 = reinterpret_cast<const float4*>(w + layer * per_layer);
-                const uint2* h2 = reinterpret_cast<const uint2*>(a.hidden[layer] + b * a.ld_hidden);
+            for (int q = 0; q < kAhead; ++q)
+                if (i + q * step < quads) x[q] = __ldg(w4 + i + q * step);
+            if (vec_h) {
 #pragma unroll 4
-                for (int i = tid; i < (per_layer >> 2); i += kCtlThreads) {
-                    const float4 x = __ldg(w4 + i);
-                    const uint2 h = __ldg(h2 + i);
-                    acc = fmaf(x.x, __uint_as_float(h.x << 16), acc);
-                    acc = fmaf(x.y, __uint_as_float(h.x & 0xFFFF0000u), acc);
-                    acc = fmaf(x.z, __uint_as_float(h.y << 16), acc);
-                    acc = fmaf(x.w, __uint_as_float(h.y & 0xFFFF0000u), acc);
+                for (int e = tid * 8; e < nf; e += kCtlThreads * 8) {
+                    const int f = f0 + e, layer = (f >= per_layer) + (f >= 2 * per_layer);
+                    *reinterpret_cast<uint4*>(sh.state + e) =
+                        __ldg(reinterpret_cast<const uint4*>(a.hidden[layer] + b * a.ld_hidden + f - layer * per_layer));
+                }
+            } else {
+#pragma unroll 1
+                for (int e = tid; e < nf; e += kCtlThreads) {
+                    const int f = f0 + e, layer = (f >= per_layer) + (f >= 2 * per_layer);
+                    sh.state[e] = a.hidden[layer][b * a.ld_hidden + f - layer * per_layer];
                 }
             }
-        } else {
-            for (int i = tid; i < F; i += kCtlThreads) {
-                const int layer = i / per_layer, e = i - layer * per_layer;
-                acc = fmaf(__ldg(w + i), __bfloat162float(a.hidden[layer][b * a.ld_hidden + e]), acc);
-            }
-        }
-        acc = block_sum(acc, s_red);
-        if (tid == 0) {
-            a.h1[b * H + unit] = tanhf(acc + a.pol.b1[unit]);
-            __threadfence();
-            s_last = (atomicAdd(a.counter + b, 1u) == static_cast<unsigned>(H - 1));
-        }
-        __syncthreads();
-        if (!s_last) return;
-    }
-    // ---- the last CTA of the sequence: second layer, action logits, the choice ---------------------------
-    __threadfence();
-    for (int i = tid; i < H; i += kCtlThreads) s_h1[i] = __ldcg(a.h1 + b * H + i);
-    __syncthreads();
-    dense_layer(a.pol.w2, a.pol.b2, s_h1, H, H, [&](int o, float v) { s_h2[o] = tanhf(v); });
-    __syncthreads();
-    dense_layer(a.pol.w3, a.pol.b3, s_h2, A, H, [&](int o, float v) {
-        s_logit[o] = v;
-        if (a.logits_out) a.logits_out[static_cast<int64_t>(b) * A + o] = v;
-    });
-    __syncthreads();
-    const bool draw = a.temperature > 0.f;
-    if (draw) {
-        // softmax(logits / T) in fp64: the maximum by one thread, the exponentials by all, the sums below in
-        // action order by one thread again (a few hundred terms)
-        if (tid == 0) {
-            double mx = -INFINITY;
-            for (int o = 0; o < A; ++o) mx = fmax(mx, static_cast<double>(s_logit[o]) / a.temperature);
-            s_mx = mx;
-        }
-        __syncthreads();
-        for (int o = tid; o < A; o += kCtlThreads) s_term[o] = exp(static_cast<double>(s_logit[o]) / a.temperature - s_mx);
-        __syncthreads();
-    }
-    if (!draw) {
-        // arg-max over the actions, ties -> lowest index: (ordered value, ~index) keys, largest wins
-        unsigned long long best = 0ull;
-        for (int o = tid; o < A; o += kCtlThreads) {
-            const unsigned u = __float_as_uint(s_logit[o]);
-            const unsigned ord = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-            const unsigned long long key = (static_cast<unsigned long long>(ord) << 32) | (0xFFFFFFFFu - static_cast<unsigned>(o));
-            best = key > best ? key : best;
-        }
+            __syncthreads();
+#pragma unroll 1
+            for (; i < quads; i += kAhead * step) {
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const unsigned long long other = __shfl_xor_sync(kFull, best, off);
-            best = other > best ? other : best;
-        }
-        if ((tid & 31) == 0) s_key[tid >> 5] = best;
-        __syncthreads();
-    }
-    if (tid == 0) {
-        int action = 0;
-        if (!draw) {
-            unsigned long long best = s_key[0];
-            for (int wq = 1; wq < kCtlThreads / 32; ++wq) best = s_key[wq] > best ? s_key[wq] : best;
-            action = static_cast<int>(0xFFFFFFFFu - static_cast<unsigned>(best & 0xFFFFFFFFull));
-        } else {
-            // inverse CDF in action order
-            double total = 0.0;
-            for (int o = 0; o < A; ++o) total += s_term[o];
-            const double target = a.uniform[b] * total;
-            double run = 0.0;
-            action = A - 1;
-            for (int o = 0; o < A; ++o) {
-                run += s_term[o];
-                if (run > target) {
-                    action = o;
-                    break;
-                }
+                for (int q = 0; q < kAhead; ++q)
+                    if (i + q * step < quads) {
+                        const uint2 h = *reinterpret_cast<const uint2*>(sh.state + 4 * (i + q * step));
+                        acc = fmaf(x[q].x, __uint_as_float(h.x << 16), acc);
+                        acc = fmaf(x[q].y, __uint_as_float(h.x & 0xFFFF0000u), acc);
+                        acc = fmaf(x[q].z, __uint_as_float(h.y << 16), acc);
+                        acc = fmaf(x[q].w, __uint_as_float(h.y & 0xFFFF0000u), acc);
+                        if (i + (q + kAhead) * step < quads) x[q] = __ldg(w4 + i + (q + kAhead) * step);
+                    }
+            }
+            if (!vec_w && mine < n_units) {
+#pragma unroll 4
+                for (int e = share * 32 + lane; e < nf; e += step) acc = fmaf(__ldg(w + e), __bfloat162float(sh.state[e]), acc);
             }
         }
-        resps_controller_state n = st;
-        if (a.accept_len) {
-            n.reward_sum += static_cast<float>(a.accept_len[b] + 1) / a.elapsed_s[b];
-            n.reward_steps += 1;
+    }
+    Row w2, w3;
+    w2.load(row2, H, lane, warp < n_units);
+    w3.load(row3, H, lane, warp < n_rows);
+    acc = warp_sum(acc);
+    if (lane == 0) sh.part[warp] = acc;
+    __syncthreads();
+    cluster_wait();
+    if (warp < n_units) {  // unit `warp`: its warps' shares
+        float v = a.pol.b1[u_lo + warp];
+#pragma unroll 1
+        for (int q = 0; q < per_unit; ++q) v += sh.part[warp * per_unit + q];
+        v = tanhf(v);
+        if (lane < kClu) store_to_peer(&sh.h1[u_lo + warp], lane, v);
+    }
+    cluster_barrier();
+    // ---- second layer: a unit per warp ------------------------------------------------------------------
+    if (warp < n_units) {
+        const float v = tanhf(w2.dot(sh.h1, H, lane) + a.pol.b2[u_lo + warp]);
+        if (lane < kClu) store_to_peer(&sh.h2[u_lo + warp], lane, v);
+    }
+    cluster_barrier();
+    // ---- action logits, to the first CTA ------------------------------------------------------------------
+#pragma unroll 1
+    for (int r = warp; r < n_rows; r += kWarps) {
+        if (r != warp) w3.load(a.pol.w3 + static_cast<int64_t>(r_lo + r) * H, H, lane, true);
+        const float v = w3.dot(sh.h2, H, lane) + a.pol.b3[r_lo + r];
+        if (lane == 0) {
+            store_to_peer(&sh.logit[r_lo + r], 0u, v);
+            if (a.logits_out) a.logits_out[static_cast<int64_t>(b) * A + r_lo + r] = v;
         }
+    }
+    cluster_barrier();
+    if (rank != 0) return;
+
+    // ---- the choice.  Actions [per * tid, per * tid + per) belong to a thread -----------------------------
+    const int per = A > kCtlThreads ? 2 : 1;
+    // largest logit, ties -> lowest index: (ordered value, ~index) keys
+    unsigned long long best = 0ull;
+#pragma unroll 1
+    for (int o = per * tid; o < min(A, per * tid + per); ++o) {
+        const unsigned long long key = pack_val_id(sh.logit[o], o);
+        best = key > best ? key : best;
+    }
+#pragma unroll 1
+    for (int off = 16; off > 0; off >>= 1) {
+        const unsigned long long other = __shfl_xor_sync(kFull, best, off);
+        best = other > best ? other : best;
+    }
+    if (lane == 0) sh.key[warp] = best;
+    if (tid == 0) sh.action = A - 1;
+    __syncthreads();
+    best = sh.key[lane & (kWarps - 1)];
+#pragma unroll 1
+    for (int off = kWarps / 2; off > 0; off >>= 1) {
+        const unsigned long long other = __shfl_xor_sync(kFull, best, off);
+        best = other > best ? other : best;
+    }
+    int action = key_id(best);
+    if (a.temperature > 0.f) {
+        // softmax(logits / T) in fp64 (a quotient grows with its numerator: the maximum is the best logit's), the
+        // inverse of its running sum in action order
+        const double T = static_cast<double>(a.temperature), mx = static_cast<double>(key_val(best)) / T;
+        double e[2] = {0.0, 0.0}, run;
+#pragma unroll 1
+        for (int i = 0; i < per; ++i)
+            if (per * tid + i < A) {
+                const double v = exp(static_cast<double>(sh.logit[per * tid + i]) / T - mx);
+                if (i == 0) e[0] = v; else e[1] = v;
+            }
+        double incl = e[0] + e[1];
+#pragma unroll 1
+        for (int off = 1; off < 32; off <<= 1) {
+            const double before = __shfl_up_sync(kFull, incl, off);
+            if (lane >= off) incl += before;
+        }
+        if (lane == 31) sh.sum[warp] = incl;
+        __syncthreads();
+        double upto = sh.sum[lane & (kWarps - 1)];
+#pragma unroll 1
+        for (int off = 1; off < kWarps; off <<= 1) {
+            const double before = __shfl_up_sync(kFull, upto, off, kWarps);
+            if ((lane & (kWarps - 1)) >= off) upto += before;
+        }
+        const double target = a.uniform[b] * __shfl_sync(kFull, upto, kWarps - 1);
+        const double before = __shfl_sync(kFull, upto, (warp + kWarps - 1) & (kWarps - 1));
+        run = (warp > 0 ? before : 0.0) + incl - e[1];  // up to and with the thread's first action
+        if (per * tid < A && run > target) atomicMin(&sh.action, per * tid);
+        else if (per == 2 && per * tid + 1 < A && run + e[1] > target) atomicMin(&sh.action, per * tid + 1);
+        __syncthreads();
+        action = sh.action;
+    }
+    if (writer) {
         if (n.reward_steps > 0) a.reward_avg[b] = n.reward_sum / static_cast<float>(n.reward_steps);  // Eq. 5
         n.reward_sum = 0.f, n.reward_steps = 0;
         n.action = action;
@@ -236,7 +282,6 @@ __global__ void __launch_bounds__(kCtlThreads) controller_kernel(const Controlle
         s.tt = a.pol.actions[3 * action + 0], s.d = a.pol.actions[3 * action + 1], s.k = a.pol.actions[3 * action + 2];
         a.steps[b] = s;
         if (a.action_out) a.action_out[b] = action;
-        a.counter[b] = 0u;
     }
 }
 
@@ -245,7 +290,11 @@ __global__ void __launch_bounds__(kCtlThreads) controller_kernel(const Controlle
 int controller_max_hidden() { return kMaxHidden; }
 int controller_max_actions() { return kMaxActions; }
 
-cudaError_t launch_controller(const resps_ctx* ctx, const resps_policy* pol, const void* h, const void* m, const void* l,
+cudaError_t controller_setup(resps_ctx*) {
+    return cudaFuncSetAttribute(controller_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+
+cudaError_t launch_controller(const resps_ctx*, const resps_policy* pol, const void* h, const void* m, const void* l,
                               int64_t ld_hidden, int batch, int interval, float temperature, const double* uniform,
                               const int32_t* accept_len, const float* elapsed_s, resps_controller_state* state,
                               resps_step* steps, float* reward_avg, float* logits_out, int32_t* action_out,
@@ -258,8 +307,7 @@ cudaError_t launch_controller(const resps_ctx* ctx, const resps_policy* pol, con
     a.ld_hidden = ld_hidden, a.batch = batch, a.interval = interval, a.temperature = temperature;
     a.uniform = uniform, a.accept_len = accept_len, a.elapsed_s = elapsed_s;
     a.state = state, a.steps = steps, a.reward_avg = reward_avg, a.logits_out = logits_out, a.action_out = action_out;
-    a.h1 = ctx->ws.ctl_h1, a.counter = ctx->ws.ctl_counter;
-    return launch_pdl(controller_kernel, dim3(pol->hidden, batch), dim3(kCtlThreads), 0, st, a);
+    return launch_pdl_cluster(controller_kernel, kClu, dim3(batch * kClu), dim3(kCtlThreads), 0, st, a);
 }
 
 }  // namespace resps

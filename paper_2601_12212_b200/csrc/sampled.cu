@@ -64,15 +64,6 @@ struct SampledArgs {
     int p_in_smem, q_in_smem;
 };
 
-__device__ __forceinline__ unsigned cluster_rank() {
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 struct Pair {
     double x, y;
 };
@@ -135,13 +126,6 @@ struct SampledShared {
     int pick;
 };
 
-__device__ __forceinline__ uint32_t peer_address(const void* local, unsigned peer) {
-    uint32_t remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
-                 : "=r"(remote)
-                 : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(local))), "r"(peer));
-    return remote;
-}
 __device__ __forceinline__ void store_pair_to_peer(double* local, unsigned peer, double x, double y) {
     asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(peer_address(local, peer)), "d"(x), "d"(y) : "memory");
 }
@@ -158,6 +142,7 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
     pdl_launch_dependents();
     __shared__ SampledShared sh;
     extern __shared__ __align__(16) unsigned char s_dyn[];
+    cluster_arrive();  // waited for before the first store to a peer
     const unsigned rank = cluster_rank();
     const int b = blockIdx.x / kClu, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = min(max(a.n_nodes[b], 1), a.max_tt);
@@ -175,6 +160,7 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
     if (tid == 0) sh.pick = -1;
     if (tid < kExpTable) sh.exp2_64[tid] = exp2(static_cast<double>(tid) / kExpTable);
     __syncthreads();
+    cluster_wait();
     // this CTA's share of the vocabulary; token e of it belongs to thread e % 512, place e / 512
     const int V = a.vocab, per_cta = (V + kClu - 1) / kClu;
     const int c_lo = min(V, static_cast<int>(rank) * per_cta), n_cta = min(V, c_lo + per_cta) - c_lo;
@@ -479,15 +465,7 @@ cudaError_t launch_accept_sampled(const resps_ctx* ctx, const resps_step* d_step
     a.p_in_smem = side <= kDynSmemCap ? 1 : 0;
     a.q_in_smem = 2 * side <= kDynSmemCap ? 1 : 0;
     const size_t dyn_bytes = a.q_in_smem ? 2 * side : a.p_in_smem ? side : 0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(batch * kClu), cfg.blockDim = dim3(kSampThreads), cfg.dynamicSmemBytes = dyn_bytes, cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = kClu, attr[1].val.clusterDim.y = 1, attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr, cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, accept_sampled_kernel, a);
+    return launch_pdl_cluster(accept_sampled_kernel, kClu, dim3(batch * kClu), dim3(kSampThreads), dyn_bytes, st, a);
 }
 
 }  // namespace resps
