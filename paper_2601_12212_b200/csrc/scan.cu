@@ -26,7 +26,7 @@ struct ScanArgs {
     int vocab, max_tt, max_k, max_rows;
     int chunk, splits;
     int batch;
-    int slices;       // streaming kernel: > 0: about as many slices per row at most (partials keep the stride `splits`)
+    int least;        // streaming kernel: fewest chunks of a range, so that a row's merge fits its list
     int test_drop;    // test build only: 2 = the second chunk copy of every slice is left out
     int only_level;   // -1: the rows of all levels; j >= 0: only level j's rows (blockIdx.y = slot)
     unsigned long long* part_key;
@@ -275,13 +275,15 @@ __global__ void __launch_bounds__(kScanThreads, 4) row_scan_kernel(const ScanArg
 // fill up.
 //
 // Bound by HBM where there are many rows; where a CTA has two or three chunks by its start, the slice's tail
-// and the merge of the row.  With selection chunk by chunk (two to six barriers a chunk) and a fixed grid of slices
-// the tree build of d=8 k=32 (225 rows of 128256 logits) took 98 us (now 63), the scan of 680
-// rows of 128256 logits ran at 6.0 TB/s (now 7.5), a shard's scan took 14.2 us (now 9.8).
+// and the merge of the row, and these by the fetching of their code (about 4 bytes a clock), so that loops stay rolled
+// and divisions are fp32 quotients.  With selection chunk by chunk (two to six barriers a chunk) and a fixed grid of
+// slices the scan of 61 rows of 128256 logits took 15.6 us (now 13.2), 13 rows of 1024 logits 6.1 us (now 4.8),
+// 225 rows at k=32 65 us (now 30); 680 rows ran at 6.0 TB/s (now 7.8).
 // ---------------------------------------------------------------------------------------
 constexpr int kStreamStages = 3;
 constexpr int kStreamMaxBatch = 256; // sequences of one launch
 constexpr int kStreamList = 1024;    // candidates of a slice
+constexpr int kStreamPicks = 1024;   // (thread, chunk) pairs that are read once more; more of them: all
 constexpr long long kScanWaitLimitCycles = kWaitTest ? 2000000ll : 4000000000ll;
 
 __device__ __forceinline__ uint32_t scan_smem_u32(const void* p) {
@@ -326,9 +328,9 @@ struct StreamShared {
     int row0[kStreamMaxBatch + 1];  // first row of a sequence
     int k[kStreamMaxBatch];
     int warp_count[kScanThreads / 32];
-    int pick[kScanThreads];  // threads that may hold candidates: from the front in one chunk, from the back in any
+    unsigned short pick[kStreamPicks];  // (chunk << 8 | thread) that may hold candidates
     float tau;
-    int count, singles, wholes, last;
+    int count, picks, last;
 };
 
 // k-th best value (by value alone) of `n` >= k keys, to `*out`; the `k` best in order to `top` when given.
@@ -344,13 +346,17 @@ __device__ __forceinline__ void rank_list(const unsigned long long* keys, int n,
     }
 }
 
-__device__ __forceinline__ float warp_maximum(float x) {
-#pragma unroll 1
-    for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(kFull, x, o));
-    return x;
+// n / d for 0 <= n < 2^24, d > 0: the quotient in fp32 is off by one at most (half the code of the division, and
+// a kernel that has just been launched waits for its code)
+__device__ __forceinline__ int divide(int n, int d) {
+    int q = __float2int_rz(__fdividef(static_cast<float>(n), static_cast<float>(d)));
+    const int r = n - q * d;
+    q += (r >= d) - (r < 0);
+    return q;
 }
+__device__ __forceinline__ float warp_maximum(float x) { return ordered_to_float(__reduce_max_sync(kFull, float_to_ordered(x))); }
 __device__ __forceinline__ float warp_total(float x) {
-#pragma unroll 1
+#pragma unroll
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
     return x;
 }
@@ -391,29 +397,27 @@ __global__ void __launch_bounds__(kStreamThreads, 2) row_scan_stream_kernel(cons
                 if (sd.clamped && blockIdx.x == 0) atomicOr(a.status, RESPS_STATUS_STEP_CLAMPED);
             }
             int incl = rows;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
+#pragma unroll 1
+            for (int d = 1; d < min(a.batch, 32); d <<= 1) {
                 const int v = __shfl_up_sync(kFull, incl, d);
                 if (lane >= d) incl += v;
             }
             if (b < a.batch) sh.row0[b] = base + incl - rows;
-            base += __shfl_sync(kFull, incl, 31);
+            base += __shfl_sync(kFull, incl, min(31, a.batch - 1 - b0));
         }
         if (lane == 0) sh.row0[a.batch] = base;
     }
     __syncthreads();
-    // the ranges: never so short that a row's merge (slices x k entries) would not fit the list
+    // the ranges
     const int total = sh.row0[a.batch] * a.splits;
-    const int most_slices = max(1, min(a.slices > 0 ? a.slices : a.splits, kStreamList / a.max_k - 2));
-    const int least = (a.splits + most_slices - 1) / most_slices;  // chunks
-    const int ctas = max(1, min(static_cast<int>(gridDim.x), total / least));
+    const int ctas = max(1, min(static_cast<int>(gridDim.x), divide(total, a.least)));
     if (static_cast<int>(blockIdx.x) >= ctas) return;
-    const int base = total / ctas, longer = total - base * ctas;  // the first `longer` ranges have one chunk more
+    const int base = divide(total, ctas), longer = total - base * ctas;  // the first `longer` ranges have one chunk more
     const int me = blockIdx.x;
     const int x_begin = me * base + min(me, longer), x_end = x_begin + base + (me < longer ? 1 : 0);
     auto owner = [&](int x) {
         const int cut = longer * (base + 1);
-        return x < cut ? x / (base + 1) : longer + (x - cut) / base;
+        return x < cut ? divide(x, base + 1) : longer + divide(x - cut, base);
     };
     const int only = min(max(a.only_level, 0), 1);  // (arithmetic: a condition would double the loops' code)
     struct Work {
@@ -422,7 +426,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) row_scan_stream_kernel(cons
     };
     auto work_at = [&](int x) {  // the slice that starts at chunk x
         Work w;
-        const int row = x / a.splits;
+        const int row = divide(x, a.splits);
         w.c_begin = x - row * a.splits, w.c_end = min(a.splits, w.c_begin + x_end - x);
         int lo = 0, hi = a.batch;  // last sequence that starts at or before the row (and is not empty)
 #pragma unroll 1
@@ -433,7 +437,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) row_scan_stream_kernel(cons
         w.b = lo, w.k = sh.k[lo];
         const int local = row - sh.row0[lo];
         w.r = local + only * (1 + (a.only_level - 1) * w.k);
-        const int level = (w.r == 0) ? 0 : 1 + (w.r - 1) / w.k;
+        const int level = (w.r == 0) ? 0 : 1 + divide(w.r - 1, w.k);
         const int slot = (w.r == 0) ? 0 : (w.r - 1) - (level - 1) * w.k;
         w.row = a.logits + w.b * a.ld_b + level * a.ld_level + slot * a.ld_row;
         return w;
@@ -522,7 +526,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) row_scan_stream_kernel(cons
             float q = fmaxf(best, __shfl_xor_sync(kFull, best, 1));
             q = fmaxf(q, __shfl_xor_sync(kFull, q, 2));
             if ((lane & 3) == 0) sh.quad[tid >> 2] = q;
-            if (tid == 0) sh.count = sh.singles = sh.wholes = 0;
+            if (tid == 0) sh.count = sh.picks = 0;
         }
         const float warp_max = warp_maximum(acc.m2);  // log-sum-exp partial of the warp, merged below
         const float warp_sum = warp_total(weighted(acc.s, acc.m2, warp_max));
@@ -545,57 +549,49 @@ __global__ void __launch_bounds__(kStreamThreads, 2) row_scan_stream_kernel(cons
         consumer_sync();
         float tau = sh.tau;
         // ---- the threads that may hold candidates, most of them in one chunk only; their logits once more ----
+        const int n_chunks = w.c_end - w.c_begin;
         if (best >= tau && best > -INFINITY) {
-            if (second < tau) sh.pick[atomicAdd(&sh.singles, 1)] = best_c << 8 | tid;
-            else sh.pick[kScanThreads - 1 - atomicAdd(&sh.wholes, 1)] = tid;
+            const bool one = second < tau;
+            int to = atomicAdd(&sh.picks, one ? 1 : n_chunks), c = one ? best_c : 0;
+            const int c_to = one ? best_c + 1 : n_chunks;
+#pragma unroll 1
+            for (; c < c_to && to < kStreamPicks; ++c, ++to) sh.pick[to] = static_cast<unsigned short>(c << 8 | tid);
         }
         consumer_sync();
-        const int per_thr = (w.c_end - w.c_begin) * (kScanPerThread / 4), n_single = sh.singles * (kScanPerThread / 4);
-        const int n_vec = n_single + sh.wholes * per_thr;
+        const bool every = sh.picks > kStreamPicks;  // (many equal logits: all of the slice once more)
+        const int n_vec = (every ? n_chunks * kScanThreads : sh.picks) * (kScanPerThread / 4);
         // Every logit at or above tau is appended while the list has room (-inf only by the filling below).  If
         // there were too many, tau becomes the k-th best found so far, and only the better ones are taken.
         const uint32_t ord_max = float_to_ordered(INFINITY);  // (NaNs of positive sign lie above)
-        uint32_t least_ord = max(float_to_ordered(tau == 0.f ? -0.f : tau), float_to_ordered(-INFINITY) + 1u);
+        uint32_t least_ord = max(float_to_ordered(tau), float_to_ordered(-INFINITY) + 1u);
         int n_cand;
 #pragma unroll 1
         for (;;) {
             constexpr int kAhead = 4;  // loads in flight per thread
+            auto place = [&](int i) {  // of group i of 4 logits, from the slice's first
+                const int from = every ? i / (kScanPerThread / 4) : sh.pick[i / (kScanPerThread / 4)];
+                return (((from >> 8) * (kScanPerThread / 4) + i % (kScanPerThread / 4)) * kScanThreads + (from & (kScanThreads - 1))) * 4;
+            };
+            const int e_first = w.c_begin * kScanChunkMax;
 #pragma unroll 1
             for (int i0 = tid; i0 < n_vec; i0 += kAhead * kScanThreads) {
                 float4 x[kAhead];
-                int e[kAhead];
 #pragma unroll
                 for (int q = 0; q < kAhead; ++q) {
-                    const int i = min(i0 + q * kScanThreads, n_vec - 1);
-                    int from, at;  // entry of the list, position among the thread's groups of 4 logits
-                    if (i < n_single) {
-                        from = sh.pick[i / (kScanPerThread / 4)];
-                        at = (from >> 8) * (kScanPerThread / 4) + i % (kScanPerThread / 4);
-                    } else {
-                        const int t = (i - n_single) / per_thr;
-                        from = sh.pick[kScanThreads - 1 - t];
-                        at = i - n_single - t * per_thr;
-                    }
-                    const int off = (at * kScanThreads + (from & (kScanThreads - 1))) * 4;
-                    e[q] = w.c_begin * kScanChunkMax + off;
+                    const int off = place(min(i0 + q * kScanThreads, n_vec - 1));
                     x[q] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-                    if (e[q] < a.vocab && i0 + q * kScanThreads < n_vec) x[q] = *reinterpret_cast<const float4*>(again + off);
+                    if (e_first + off < a.vocab && i0 + q * kScanThreads < n_vec) x[q] = *reinterpret_cast<const float4*>(again + off);
                 }
+                unsigned hits = 0u;
+                auto hit = [&](float y, int z) { hits |= (float_to_ordered(y) - least_ord <= ord_max - least_ord) ? (1u << z) : 0u; };
 #pragma unroll
-                for (int q = 0; q < kAhead; ++q) {
-                    const float y[4] = {x[q].x, x[q].y, x[q].z, x[q].w};
-                    unsigned hits = 0u;
-#pragma unroll
-                    for (int z = 0; z < 4; ++z)
-                        hits |= (float_to_ordered(y[z]) - least_ord <= ord_max - least_ord) ? (1u << z) : 0u;
-                    if (!hits) continue;
-                    int to = atomicAdd(&sh.count, __popc(hits));
-#pragma unroll
-                    for (int z = 0; z < 4; ++z)
-                        if ((hits >> z) & 1u) {
-                            if (to < kStreamList) sh.list[to] = pack_val_id(y[z], e[q] + z);
-                            ++to;
-                        }
+                for (int q = 0; q < kAhead; ++q) hit(x[q].x, 4 * q), hit(x[q].y, 4 * q + 1), hit(x[q].z, 4 * q + 2), hit(x[q].w, 4 * q + 3);
+                if (!hits) continue;
+                int to = atomicAdd(&sh.count, __popc(hits));
+#pragma unroll 1
+                for (; hits && to < kStreamList; hits &= hits - 1u, ++to) {  // (re-read: registers have no index)
+                    const int z = __ffs(hits) - 1, off = place(i0 + (z >> 2) * kScanThreads) + (z & 3);
+                    sh.list[to] = pack_val_id(again[off], e_first + off);
                 }
             }
             consumer_sync();
@@ -658,24 +654,27 @@ __global__ void __launch_bounds__(kStreamThreads, 2) row_scan_stream_kernel(cons
         }
         if (last) {
             // ---- last CTA of the row: merge the slices --------------------------------------------------
+            float2 ms0 = make_float2(-INFINITY, 0.f);
             if (slices > 1) {
                 __threadfence();
                 const unsigned long long* parts = a.part_key + prow * a.splits * a.max_k;
+                if (warp == kScanThreads / 32 - 1 && lane < slices) ms0 = __ldcg(a.part_ms + prow * a.splits + lane);
 #pragma unroll 1
                 for (int i = tid; i < slices * k; i += kScanThreads) {
-                    const int from = i / k;
+                    const int from = divide(i, k);
                     sh.list[i] = __ldcg(parts + from * a.max_k + (i - from * k));
                 }
                 consumer_sync();
                 rank_list(sh.list, slices * k, k, sh.top, nullptr);
             }
             if (warp == kScanThreads / 32 - 1) {  // weights in fp32 (relative error 2^-22), accumulation in fp64
-                float M = -INFINITY;
-                double sum = 0.0;
                 __syncwarp();
+                if (slices == 1 && lane == 0) ms0 = sh.total;
+                float M = ms0.x;
+                double sum = ms0.y;
 #pragma unroll 1
-                for (int i = lane; i < slices; i += 32) {
-                    const float2 ms = slices > 1 ? __ldcg(a.part_ms + prow * a.splits + i) : sh.total;
+                for (int i = lane + 32; i < slices; i += 32) {
+                    const float2 ms = __ldcg(a.part_ms + prow * a.splits + i);
                     const float m = fmaxf(M, ms.x);
                     sum = sum * weighted(1.f, M, m) + weighted(ms.y, ms.x, m);
                     M = m;
@@ -1051,7 +1050,8 @@ cudaError_t launch_row_scan(const resps_ctx* ctx, const resps_step* d_steps, int
     const int k_ext = min(n_slots, ctx->shape.max_k);
     a.only_level = only_level;
     const int rows = (only_level >= 0) ? (only_level == 0 ? 1 : k_ext) : ((n_levels > 1) ? 1 + (n_levels - 1) * k_ext : 1);
-    a.slices = w.scan_slices_hint;
+    const int most_slices = max(1, min(w.scan_slices_hint > 0 ? w.scan_slices_hint : a.splits, kStreamList / a.max_k - 2));
+    a.least = (a.splits + most_slices - 1) / most_slices;
     a.test_drop = w.test_drop;
     if (!(vec_ok(logits, ld_b, ld_level, ld_row, a.vocab, a.chunk) && w.scan_chunk == kScanChunkMax)) {
         const size_t smem = sizeof(unsigned long long) * ctx->shape.max_k * max(kQuadElems, w.scan_splits);
