@@ -921,7 +921,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
 #pragma unroll 1
                 for (int t = it.t_begin; t < it.t_end; ++t, ++kt_run) {
                     const int s = kt_run % kStagesK;
-                    if (kt_run == 0) {  // went out during the set-up, and the item's Q with it
+                    if (kt_run == 0 && early) {  // went out during the set-up, and the item's Q with it
                         ++items_run;
                         continue;
                     }
