@@ -954,43 +954,54 @@ struct ShardMergeArgs {
     double* row_lse;
 };
 
-__global__ void __launch_bounds__(128) shard_merge_rows_kernel(const ShardMergeArgs a) {
+// A CTA per row: the shards' candidates ranked by counting, and beside that, by a warp of its own with a lane per shard,
+// the log of the sum over the shards of exp(shard's log-sum-exp).  Bound by its chain of round trips to L2 (step
+// parameters, candidates); the log-sum-exp by one thread, one load after another, took 1.5 us more.
+constexpr int kMergeThreads = 160;
+constexpr int kMaxShards = 16;
+
+__global__ void __launch_bounds__(kMergeThreads) shard_merge_rows_kernel(const ShardMergeArgs a) {
     pdl_wait();  // the kernel before this one in the stream has completed
     pdl_launch_dependents();
-    __shared__ unsigned long long s_keys[16 * RESPS_MAX_K];
-    const int b = blockIdx.y, r = blockIdx.x, tid = threadIdx.x;
+    __shared__ unsigned long long s_keys[kMaxShards * RESPS_MAX_K];
+    const int b = blockIdx.y, r = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+    const int64_t prow = static_cast<int64_t>(b) * a.max_rows + r, shard_rows = static_cast<int64_t>(a.batch) * a.max_rows;
+    const bool sums = tid >= kMergeThreads - 32;
+    const double lse = (sums && lane < a.n_shards) ? __ldg(a.all_lse + lane * shard_rows + prow) : -INFINITY;  // (any row may be read)
     const StepDims sd = clamp_step(a.steps[b], a.n_levels, a.n_slots, a.max_tt, a.max_k, a.vocab);
     const int k = sd.k;
     if (r >= 1 + (sd.d - 1) * k) return;
-    const int64_t prow = static_cast<int64_t>(b) * a.max_rows + r;
     const int n = a.n_shards * k;
+    if (!sums) {
 #pragma unroll 1
-    for (int i = tid; i < n; i += blockDim.x) {
-        const int p = i / k, q = i - p * k;
-        const int64_t src = (static_cast<int64_t>(p) * a.batch * a.max_rows + prow) * a.max_k + q;
-        s_keys[i] = pack_val_id(a.all_val[src], a.all_id[src] + a.shard_offset[p]);
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int c = tid; c < n; c += blockDim.x) {
-        const unsigned long long mine = s_keys[c];
-        int rank = 0;
-#pragma unroll 4
-        for (int j = 0; j < n; ++j) rank += (s_keys[j] > mine) || (s_keys[j] == mine && j < c);
-        if (rank < k) {
-            a.row_val[prow * a.max_k + rank] = key_val(mine);
-            a.row_id[prow * a.max_k + rank] = key_id(mine);
+        for (int i = tid; i < n; i += kMergeThreads - 32) {
+            const int p = divide(i, k), q = i - p * k;
+            const int64_t src = (p * shard_rows + prow) * a.max_k + q;
+            s_keys[i] = pack_val_id(a.all_val[src], a.all_id[src] + a.shard_offset[p]);
         }
     }
-    if (tid == 0) {  // log of the sum over the shards of exp(shard's log-sum-exp), fp64
-        double m = -INFINITY;
+    __syncthreads();
+    if (!sums) {
 #pragma unroll 1
-        for (int p = 0; p < a.n_shards; ++p) m = fmax(m, a.all_lse[static_cast<int64_t>(p) * a.batch * a.max_rows + prow]);
-        double sum = 0.0;
-#pragma unroll 1
-        for (int p = 0; p < a.n_shards; ++p) sum += exp(a.all_lse[static_cast<int64_t>(p) * a.batch * a.max_rows + prow] - m);
-        a.row_lse[prow] = m + log(sum);
+        for (int c = tid; c < n; c += kMergeThreads - 32) {
+            const unsigned long long mine = s_keys[c];
+            int rank = 0;
+#pragma unroll 4
+            for (int j = 0; j < n; ++j) rank += (s_keys[j] > mine) || (s_keys[j] == mine && j < c);
+            if (rank < k) {
+                a.row_val[prow * a.max_k + rank] = key_val(mine);
+                a.row_id[prow * a.max_k + rank] = key_id(mine);
+            }
+        }
+        return;
     }
+    double m = lse;
+#pragma unroll 1
+    for (int o = kMaxShards / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(kFull, m, o));
+    double sum = (lane < a.n_shards) ? exp(lse - m) : 0.0;
+#pragma unroll 1
+    for (int o = kMaxShards / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+    if (lane == 0) a.row_lse[prow] = m + log(sum);
 }
 
 struct ShardArgmaxArgs {
@@ -1119,7 +1130,7 @@ cudaError_t launch_shard_merge_rows(const resps_ctx* ctx, const resps_step* d_st
     a.row_val = w.row_val, a.row_id = w.row_id, a.row_lse = w.row_lse;
     const int k_ext = min(n_slots, ctx->shape.max_k);
     const int rows = (n_levels > 1) ? 1 + (n_levels - 1) * k_ext : 1;
-    return launch_pdl(shard_merge_rows_kernel, dim3(rows, batch), dim3(128), 0, st, a);
+    return launch_pdl(shard_merge_rows_kernel, dim3(rows, batch), dim3(kMergeThreads), 0, st, a);
 }
 
 cudaError_t launch_shard_merge_argmax(const resps_ctx* ctx, const int32_t* d_n_nodes, int batch, int n_shards,
