@@ -369,10 +369,28 @@ class DeviceWorkload:
         self.verify(i)          # prefix_len += accepted + 1, in place on the device
         self.compact()
 
+    def attention_launches(self):
+        """Kernels of one attention call behind the first of a step (one, or attention + combine): the nodes of a
+        captured graph of two calls, less the one that makes the work list."""
+        torch = self.torch
+        from cuda.bindings import runtime
+        g = torch.cuda.CUDAGraph(keep_graph=True)
+        self.ctx.attention_replan()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(g):
+            self.attention(0)
+            self.attention(0)
+        self.ctx.attention_replan()
+        handle = runtime.cudaGraph_t(init_value=g.raw_cuda_graph())
+        _, _, n = runtime.cudaGraphGetNodes(handle)
+        return (n - 1) // 2
+
     def launches_per_step(self):
-        # scan, tree build; the attention work list once; attention + combine per layer; arg-max with the walk
-        # in its tail; compaction (the launch list under profiles/ shows the same 69 per step at 32 layers)
-        return 2 + 1 + 2 * self.w.n_layers + 1 + 1
+        # scan, tree build; the attention work list once; attention per layer; arg-max with the walk in its tail;
+        # compaction
+        if not hasattr(self, "_per_layer"):
+            self._per_layer = self.attention_launches()
+        return 2 + 1 + self._per_layer * self.w.n_layers + 1 + 1
 
     # -- end to end: host buffers in, host result out ---------------------------------------
     def step_e2e(self, i):
