@@ -30,6 +30,7 @@ constexpr int kClu = 16;            // CTAs per sequence (more than 8: not porta
 constexpr int kMaxHidden = 256;
 constexpr int kMaxActions = 1024;
 constexpr int kStage = 16384;       // features staged at once
+constexpr int kPiece = 2048;        // features of a W1 row asked into L2 by one instruction
 constexpr int kAhead = 8;           // 16-byte loads of a thread in flight
 constexpr unsigned kFull = 0xFFFFFFFFu;
 static_assert(kMaxHidden <= kClu * kWarps, "a warp per hidden unit in the second layer");
@@ -126,6 +127,18 @@ __global__ void __launch_bounds__(kCtlThreads, 2) controller_kernel(const Contro
         if (warp < n_rows) asm volatile("prefetch.global.L2 [%0];" ::"l"(row3 + lane * 32));
     }
 
+    // W1 is likely to have left L2 since it was last read, and a thread's eight loads would take a round trip to HBM
+    // each: the rows are asked into L2 at once.  (By one of the sequences next to one another that ask.)
+    const bool asked_before = b > 0 && (a.state[b - 1].cache_step == 0 || a.state[b - 1].action < 0);
+    if ((F & 3) == 0 && aligned_to(a.pol.w1, 16) && !asked_before) {
+        const int pieces = (F + kPiece - 1) / kPiece;
+#pragma unroll 1
+        for (int i = tid; i < n_units * pieces; i += kCtlThreads) {
+            const int u = i / pieces, f = (i - u * pieces) * kPiece;
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.pol.w1 + static_cast<int64_t>(u_lo + u) * F + f),
+                         "r"(min(kPiece, F - f) * 4));
+        }
+    }
     // ---- first layer: `per_unit` warps share a hidden unit ----------------------------------------------
     const int per_unit = kWarps / units, mine = warp / per_unit, share = warp - mine * per_unit;
     float acc = 0.f;
