@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(kCtlThreads, 2) controller_kernel(const Contro
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned rank = cluster_rank();
     const int b = blockIdx.x / kClu;
-    const resps_controller_state st = a.state[b];
+    const resps_controller_state st = a.state[b], beside = a.state[max(b - 1, 0)];
     const bool ask = (st.cache_step == 0) || (st.action < 0);
     const bool writer = rank == 0 && tid == 0;
     cluster_arrive();  // waited for before the state, or a peer's shared memory, is written
@@ -127,18 +127,6 @@ __global__ void __launch_bounds__(kCtlThreads, 2) controller_kernel(const Contro
         if (warp < n_rows) asm volatile("prefetch.global.L2 [%0];" ::"l"(row3 + lane * 32));
     }
 
-    // W1 is likely to have left L2 since it was last read, and a thread's eight loads would take a round trip to HBM
-    // each: the rows are asked into L2 at once.  (By one of the sequences next to one another that ask.)
-    const bool asked_before = b > 0 && (a.state[b - 1].cache_step == 0 || a.state[b - 1].action < 0);
-    if ((F & 3) == 0 && aligned_to(a.pol.w1, 16) && !asked_before) {
-        const int pieces = (F + kPiece - 1) / kPiece;
-#pragma unroll 1
-        for (int i = tid; i < n_units * pieces; i += kCtlThreads) {
-            const int u = i / pieces, f = (i - u * pieces) * kPiece;
-            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.pol.w1 + static_cast<int64_t>(u_lo + u) * F + f),
-                         "r"(min(kPiece, F - f) * 4));
-        }
-    }
     // ---- first layer: `per_unit` warps share a hidden unit ----------------------------------------------
     const int per_unit = kWarps / units, mine = warp / per_unit, share = warp - mine * per_unit;
     float acc = 0.f;
@@ -159,6 +147,17 @@ __global__ void __launch_bounds__(kCtlThreads, 2) controller_kernel(const Contro
 #pragma unroll
             for (int q = 0; q < kAhead; ++q)
                 if (i + q * step < quads) x[q] = __ldg(w4 + i + q * step);
+            // W1 is likely to have left L2 since it was last read, and a thread's eight loads would take a round trip to
+            // HBM each: the rows are asked into L2 at once.  (By one of the sequences next to one another that ask.)
+            if (f0 == 0 && vec_w && !(b > 0 && (beside.cache_step == 0 || beside.action < 0))) {
+                const int u = tid >> 5, at = lane * kPiece;
+                if (u < n_units) {
+#pragma unroll 1
+                    for (int f = at; f < F; f += 32 * kPiece)
+                        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.pol.w1 + static_cast<int64_t>(u_lo + u) * F + f),
+                                     "r"(min(kPiece, F - f) * 4));
+                }
+            }
             if (vec_h) {
 #pragma unroll 4
                 for (int e = tid * 8; e < nf; e += kCtlThreads * 8) {
