@@ -109,13 +109,21 @@ __device__ __forceinline__ double apply(const Pending& pd, double p, double fact
     return pd.a > 0.0 ? fmax(p - q_raw * pd.sq_old, 0.0) * pd.a : p;
 }
 
+// What the peers write into this CTA's shared memory in one exchange over the cluster.  There are two sets, used
+// in turn by ALL exchanges of the walk, whatever they carry (the start of a node, a rejection, the draw).  Set s of
+// exchange i is written before the cluster barrier of exchange i and read between that barrier and this CTA's arrival
+// at the barrier of exchange i + 1; exchange i + 2, the next to write it, begins behind that second barrier.  So one
+// barrier per exchange orders every write of a peer behind every read of what it replaces.
+struct Exchange {
+    double sum[kClu][2];             // partial sums
+    double top[kClu][2];             // the maxima they are relative to, times 1 / T (start of a node)
+    double tab[RESPS_MAX_K][2];      // (P, Q) of the children's tokens, written by their owners
+};
 struct SampledShared {
     double exp2_64[kExpTable];       // 2^(i/64)
     double red[kWarps][2];
-    double peer[2][kClu][2];         // the cluster's partial results, written by the peers (two sets in turn)
-    double peer_max[kClu][2];        // ... and the maxima they are relative to, times 1 / T
+    Exchange ex[2];                  // written by the peers
     double factor[kClu][2];          // e^(a CTA's maximum - the row's)
-    double tab[2][RESPS_MAX_K][2];   // (P, Q) of the children's tokens, written by their owners
     double scan[kWarps];
     double u[RESPS_MAX_K];
     unsigned red_max[kWarps][2];
@@ -170,12 +178,12 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
     double* const own = a.scratch + (static_cast<int64_t>(b) * kClu + rank) * 2 * a.state;
     double* const P = a.p_in_smem ? reinterpret_cast<double*>(s_dyn) : own;
     double* const Q = a.q_in_smem ? reinterpret_cast<double*>(s_dyn) + a.state : own + a.state;
-    int set = 0;
+    int set = 0;  // the set of the next exchange
     int cur = 0, acc = 0, n_child = 0;
     // Two sums over the cluster, the same bits in every thread of every CTA.  Meanwhile (P, Q) of the children's
-    // tokens from `from` on, as the pass before left them, go into table `par` of every CTA.  At the start of a
-    // node the maxima travel along, and the sums are put on the row's common scale.
-    auto cluster_sum = [&](double x, double y, int par, int from, bool at_start, double max_t, double max_d) {
+    // tokens from `from` on, as the pass before left them, go into the table of every CTA (after the call: that of
+    // set ^ 1).  At the start of a node the maxima travel along, and the sums are put on the row's common scale.
+    auto cluster_sum = [&](double x, double y, int from, bool at_start, double max_t, double max_d) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o), y += __shfl_xor_sync(kFull, y, o);
         if (lane == 0) sh.red[warp][0] = x, sh.red[warp][1] = y;
@@ -185,36 +193,37 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o), y += __shfl_xor_sync(kFull, y, o);
             if (lane < kClu) {
-                store_pair_to_peer(sh.peer[set][rank], lane, x, y);
-                if (at_start) store_pair_to_peer(sh.peer_max[rank], lane, max_t, max_d);
+                store_pair_to_peer(sh.ex[set].sum[rank], lane, x, y);
+                if (at_start) store_pair_to_peer(sh.ex[set].top[rank], lane, max_t, max_d);
             }
         } else if (warp == 1 && lane >= from && lane < n_child) {
             const int e = sh.child_at[lane];
             if (e >= 0) {
                 const double p = P[at(e)], q = Q[at(e)];
 #pragma unroll 1
-                for (int c = 0; c < kClu; ++c) store_pair_to_peer(sh.tab[par][lane], c, p, q);
+                for (int c = 0; c < kClu; ++c) store_pair_to_peer(sh.ex[set].tab[lane], c, p, q);
             }
         }
         __syncwarp();
-        cluster_barrier();
+        cluster_barrier();  // (the other set may be written from here on: its readers have arrived)
+        const Exchange& ex = sh.ex[set];
         Pair r = {0.0, 0.0};
         if (at_start) {
             if (tid < 2 * kClu) {
                 const int side = tid & 1;
                 double top = -INFINITY;
 #pragma unroll 4
-                for (int c = 0; c < kClu; ++c) top = fmax(top, sh.peer_max[c][side]);
+                for (int c = 0; c < kClu; ++c) top = fmax(top, ex.top[c][side]);
                 // (a CTA without tokens, or no draft row: nothing to scale)
-                const double m = sh.peer_max[tid >> 1][side];
+                const double m = ex.top[tid >> 1][side];
                 sh.factor[tid >> 1][side] = m > -INFINITY ? exp_le0(m - top, sh.exp2_64) : 0.0;
             }
             __syncthreads();
 #pragma unroll 4
-            for (int c = 0; c < kClu; ++c) r.x += sh.peer[set][c][0] * sh.factor[c][0], r.y += sh.peer[set][c][1] * sh.factor[c][1];
+            for (int c = 0; c < kClu; ++c) r.x += ex.sum[c][0] * sh.factor[c][0], r.y += ex.sum[c][1] * sh.factor[c][1];
         } else {
 #pragma unroll 4
-            for (int c = 0; c < kClu; ++c) r.x += sh.peer[set][c][0], r.y += sh.peer[set][c][1];
+            for (int c = 0; c < kClu; ++c) r.x += ex.sum[c][0], r.y += ex.sum[c][1];
         }
         set ^= 1;
         return r;
@@ -296,7 +305,7 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
                 sum_d += w;
             }
         }
-        const Pair sum = cluster_sum(sum_t, sum_d, 0, 0, true, n_cta > 0 ? mx_t : -INFINITY, n_cta > 0 && with_q ? mx_d : -INFINITY);
+        const Pair sum = cluster_sum(sum_t, sum_d, 0, true, n_cta > 0 ? mx_t : -INFINITY, n_cta > 0 && with_q ? mx_d : -INFINITY);
         // What P (and the table's entries) still lack; a pass brings P up to date.
         Pending pend = {1, recip_or_zero(sum.x), 0.0};
         double sq = with_q ? recip_or_zero(sum.y) : 0.0;  // draft side: q = Q * factor * sq
@@ -307,8 +316,9 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
         for (int j = 0; j < n_child && j < a.max_k; ++j) {
             const int child = sh.children[j];
             {
-                const double q_raw = sh.tab[j & 1][j][1] * sh.factor[sh.child_clu[j]][1];
-                const double p = apply(pend, sh.tab[j & 1][j][0], sh.factor[sh.child_clu[j]][0], q_raw);
+                const double* const entry = sh.ex[set ^ 1].tab[j];  // of the exchange just behind
+                const double q_raw = entry[1] * sh.factor[sh.child_clu[j]][1];
+                const double p = apply(pend, entry[0], sh.factor[sh.child_clu[j]][0], q_raw);
                 const double q = q_raw * sq;
                 // u < min(1, p / q), without the quotient
                 if (q > 0.0 ? sh.u[j] * q < p : p > 0.0) next = child;
@@ -339,7 +349,7 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
                     zy += (e != x_at) ? q : 0.0;
                 }
             }
-            const Pair zr = cluster_sum(zx, zy, (j + 1) & 1, j + 1, false, 0.0, 0.0);
+            const Pair zr = cluster_sum(zx, zy, j + 1, false, 0.0, 0.0);
             pend = Pending{2, recip_or_zero(zr.x), sq};
             if (x_at >= 0 && x_at % kSampThreads == tid) {  // x leaves the draft side; its own round is applied here
                 if (pend.a > 0.0) P[at(x_at)] -= Q[at(x_at)] * scale;
@@ -381,12 +391,12 @@ __global__ void __launch_bounds__(kSampThreads, 1) accept_sampled_kernel(const S
             cta_total += sh.scan[w];
         }
         const double excl = before + inc - run;
-        if (tid < kClu) store_pair_to_peer(sh.peer[set][rank], tid, cta_total, 0.0);
+        if (tid < kClu) store_pair_to_peer(sh.ex[set].sum[rank], tid, cta_total, 0.0);
         cluster_barrier();
         double offset = 0.0, total = 0.0;
 #pragma unroll 4
         for (int c = 0; c < kClu; ++c) {
-            const double t = sh.peer[set][c][0];
+            const double t = sh.ex[set].sum[c][0];
             if (c < static_cast<int>(rank)) offset += t;
             total += t;
         }
