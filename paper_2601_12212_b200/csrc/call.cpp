@@ -126,6 +126,13 @@ bool tensor_address(PyObject* o, char code, int64_t* out) {
     return true;
 }
 
+// The interpreter lock is given up for the call and taken again on every way out of the scope, an exception's too
+// (Python's own pair of macros leaves it with the lock given up).
+struct WithoutLock {
+    PyThreadState* const state = PyEval_SaveThread();
+    ~WithoutLock() { PyEval_RestoreThread(state); }
+};
+
 PyObject* call_entry(PyObject* self, PyObject* const* args, Py_ssize_t n) {
     const Entry* e = static_cast<const Entry*>(PyCapsule_GetPointer(self, nullptr));
     if (!e) return nullptr;
@@ -158,9 +165,8 @@ PyObject* call_entry(PyObject* self, PyObject* const* args, Py_ssize_t n) {
             }
             if ((s.i == -1 || s.d == -1.0) && PyErr_Occurred()) return nullptr;
         }
-        Py_BEGIN_ALLOW_THREADS
+        const WithoutLock unlocked;
         rc = e->spec->call(e->fn, slots);
-        Py_END_ALLOW_THREADS
     } catch (const std::exception& ex) {
         PyErr_SetString(PyExc_RuntimeError, ex.what());
         return nullptr;
