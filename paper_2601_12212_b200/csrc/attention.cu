@@ -1591,16 +1591,25 @@ constexpr size_t kMaxCachedMaps = 4096;
 
 HostState* host_state(const resps_ctx* ctx) { return static_cast<HostState*>(ctx->attn_host); }
 
-const CUtensorMap* cached_map(HostState* hs, const MapKey& key, int D) {
-    auto it = hs->maps.find(key);
-    if (it != hs->maps.end()) return &it->second;
-    CUtensorMap m;
-    const bool ok = key.kind == 0 ? make_kv_map(&m, key.base, D, key.d, key.hkv, key.batch, key.a, key.b, key.c)
-                                  : make_q_map(&m, key.base, D, static_cast<int>(key.a), key.hkv,
+// Copies the map into `out`: a map inserted later may clear the table.  False where the map cannot be encoded or
+// there is no host memory for its entry (no exception may leave the C entry points).
+bool cached_map(HostState* hs, const MapKey& key, int D, CUtensorMap* out) {
+    const auto it = hs->maps.find(key);
+    if (it != hs->maps.end()) {
+        *out = it->second;
+        return true;
+    }
+    const bool ok = key.kind == 0 ? make_kv_map(out, key.base, D, key.d, key.hkv, key.batch, key.a, key.b, key.c)
+                                  : make_q_map(out, key.base, D, static_cast<int>(key.a), key.hkv,
                                                static_cast<int>(key.b), key.batch);
-    if (!ok) return nullptr;
+    if (!ok) return false;
     if (hs->maps.size() >= kMaxCachedMaps) hs->maps.clear();
-    return &hs->maps.emplace(key, m).first->second;
+    try {
+        hs->maps.emplace(key, *out);
+    } catch (const std::bad_alloc&) {
+        return false;
+    }
+    return true;
 }
 
 // CTAs per cluster for mode whole, or 1 for the two-kernel modes.  Mode whole saves the second kernel and the
@@ -1752,14 +1761,13 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
     MapKey kk = {k_cache, stride_tok, stride_head, stride_seq, capacity, a.Hkv, batch, 0};
     MapKey kv = kk;
     kv.base = v_cache;
-    const CUtensorMap* mk = cached_map(hs, kk, D);
-    const CUtensorMap* mv = cached_map(hs, kv, D);
-    if (!mk || !mv) return cudaErrorInvalidValue;
-    const CUtensorMap* mq = mk;  // unused by the kernel unless Q comes by TMA
+    CUtensorMap mk, mv, mq;
+    if (!cached_map(hs, kk, D, &mk) || !cached_map(hs, kv, D, &mv)) return cudaErrorInvalidValue;
     if (a.q_by_tma) {
-        MapKey kq = {q, G, a.max_tt, 0, 0, a.Hkv, batch, 1};
-        mq = cached_map(hs, kq, D);
-        if (!mq) return cudaErrorInvalidValue;
+        const MapKey kq = {q, G, a.max_tt, 0, 0, a.Hkv, batch, 1};
+        if (!cached_map(hs, kq, D, &mq)) return cudaErrorInvalidValue;
+    } else {
+        mq = mk;  // unused by the kernel
     }
     // The work list: made by the first call after anything that may have changed the step, reused
     // by the calls for the other layers.
@@ -1772,7 +1780,7 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
         hs->plan_capacity = capacity, hs->plan_stream = st, hs->plan_age = 0;
     }
     a.plan_after_wait = hs->plan_age == 0 ? 1 : 0;
-    cudaError_t e = D == 128 ? launch_for_dim<128>(ctx, a, grid, *mk, *mv, *mq, st) : launch_for_dim<64>(ctx, a, grid, *mk, *mv, *mq, st);
+    cudaError_t e = D == 128 ? launch_for_dim<128>(ctx, a, grid, mk, mv, mq, st) : launch_for_dim<64>(ctx, a, grid, mk, mv, mq, st);
     hs->plan_age += a.cluster > 1 ? 1 : 2;
     return e;
 }
