@@ -961,6 +961,10 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
         // lane's tile j+1 is issued before PV of tile j, so the tensor pipe has S(j+1) to work on
         // while the softmax warps turn S(j) into P(j), and QK(j+2) cannot overwrite the TMEM
         // buffer j & 1 before PV(j) has read P(j) from it.
+        // The MMAs of a tile are unrolled: one elected thread issues them, and what it needs per instruction is on
+        // the chain of every tile.  As loops (QK by two, PV rolled) a call took, in us: 70B shape at 4096 keys 24.6
+        // against 22.7, at 32 000 143.5 / 130.4, 8B shape with 128 nodes at 32 000 105 / 98, the 13B shape 16.0 / 15.5;
+        // calls of one or two tiles a lane, where code is fetched cold, the same (9.6 / 9.5).
         const int x = warp - kMmaWarp0;
         constexpr uint32_t kIdescQK = instr_desc(kBN, false);
         constexpr uint32_t kIdescPV = instr_desc(D, true);
@@ -994,7 +998,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                     if (elect_one()) {
                         const uint64_t kdesc = kdesc0 + static_cast<uint64_t>(s * (S::kKVTile >> 4));
                         const uint32_t s_t = tmem + x * 256 + (jx & 1u) * kBN;
-#pragma unroll 2
+#pragma unroll
                         for (int ks = 0; ks < D / 16; ++ks)
                             umma(s_t, qdesc + ((ks >> 2) * (S::kQPanel >> 4) + (ks & 3) * 2),
                                  kdesc + ((ks >> 2) * (S::kKVPanel >> 4) + (ks & 3) * 2), kIdescQK, ks > 0 ? 1u : 0u);
@@ -1025,7 +1029,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                         const uint64_t vdesc = vdesc0 + static_cast<uint64_t>(s * (S::kKVTile >> 4));
                         // P of keys 32h .. 32h+31: hi in columns 32h .. 32h+15, lo in 32h+16 .. 32h+31
                         const uint32_t p_t = tmem + x * 256 + (prev_j & 1u) * kBN;
-#pragma unroll 1
+#pragma unroll
                         for (int kk = 0; kk < kBN / 16; ++kk) {
                             const uint32_t a_t = p_t + (kk >> 1) * 32 + (kk & 1) * 8;
                             umma_ts(o_t, a_t, vdesc + kk * (2048 >> 4), kIdescPV, (first_pv && kk == 0) ? 0u : 1u);
