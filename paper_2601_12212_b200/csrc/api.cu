@@ -184,6 +184,7 @@ int resps_debug_set(resps_ctx* ctx, int key, int value) {
         case RESPS_DEBUG_ATTN_MIN_TILES: w.attn_min_tiles = std::max(1, value); break;
         case RESPS_DEBUG_ATTN_SINGLE: w.attn_stream = std::min(1 << 26, std::max(0, value)); break;
         case RESPS_DEBUG_ATTN_CLUSTER: w.attn_cluster = std::max(0, value); break;
+        case RESPS_DEBUG_ATTN_EVEN_ROUNDS: w.attn_even_rounds = std::max(0, value); break;
         case RESPS_DEBUG_SCAN_SLICES: w.scan_slices_hint = std::max(0, value); break;
 #ifdef RESPS_WAIT_TEST
         case 100: w.test_drop = value; break;  // test build only: which copy is left out (see common.cuh)

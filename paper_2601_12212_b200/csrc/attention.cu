@@ -64,6 +64,8 @@ constexpr int kMaxCluster = 8;     // CTAs of a cluster (the portable limit)
 constexpr int kMaxGrid = 256;      // clusters x CTAs (one per SM)
 constexpr int kSnap = 4;           // mode stream: a cut this close to a group's edge (key tiles) is moved onto it
 constexpr int kItemTiles = 4;      // what an item costs a CTA besides its tiles (its start and epilogue), in key tiles
+constexpr int kMaxRounds = 4;      // mode even: most rounds of splits
+constexpr int kRereadNum = 5, kRereadDen = 4;
 constexpr int kCutTiles = 6;       // what cut groups cost a call (partials, the combine kernel's round trips)
 constexpr int kTmemCols = 512;
 constexpr uint32_t kWaitLimitCycles = kWaitTest ? 2000000u : 0x70000000u;  // bounded waits give up after ~1 s of SM clocks
@@ -75,11 +77,20 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 //          the group's key tiles, leave normalised partial results in the workspace (L2), meet on an
 //          mbarrier and merge a share of the rows x columns each: one kernel does the layer.
 //  even    single CTAs; every group is cut into splits of at most T key tiles with the smallest T for which
-//          the splits fit one round of the grid; a second, small kernel combines the partials.
+//          the splits fit one round of the grid, or two to four (CTA c takes splits c, c + CTAs, ... in the order of
+//          sequence, KV head, row tile and keys); a second, small kernel combines the partials.
 //  stream  the same two kernels; the key tiles of all groups, one group after the other, are cut into equal
 //          contiguous ranges, one per CTA (a CTA may end one group and begin another), or into ranges of whole
 //          groups.
-// Of even and stream the one with the smallest largest share is taken (tiles, items, cut groups).
+// Of even (each number of rounds) and stream the one with the smallest largest share is taken (tiles, items, cut
+// groups).  In mode even the row tiles of a KV head go through the same keys at the same time, in mode stream at
+// different times: where K and V do not stay in L2 meanwhile, every row tile reads them from HBM again.  Measured per
+// unit of the largest share, several row tiles per head: K and V of a call up to 67 MB 0.75-0.80 us in all modes; from
+// 131 MB on even 0.65-0.78, stream 0.88-0.95.  So the share of mode stream counts kRereadNum / kRereadDen times as much
+// beyond `l2_tiles` key tiles (all KV heads of the sequences with several row tiles).  In us a call, stream against
+// the best of even: 8 x 24 000 keys, 80 nodes, 8B shape 464 / 408; 5 x 28 000 keys, 40-96 nodes, 56 query heads
+// 528 / 459; 4 x 8192 keys, 96 nodes, 70B shape 162 / 151; 16 x 4096 keys, 64 nodes, 8B shape 120 / 112; 12 ragged
+// sequences up to 16 000 keys, 28 query heads 126 / 107; one round against two: 32 000 keys, 128 nodes, 8B shape 108 / 98.
 constexpr int kModeWhole = 0, kModeEven = 1, kModeStream = 2;
 
 struct PlanHead {
@@ -96,11 +107,11 @@ struct PlanItem {
     int t_begin, t_end;  // this CTA's key tiles (none: t_begin == t_end)
     int n, L;            // the sequence's tree size and prefix length
     int pieces;          // items the group is cut into
-    int pad;
+    int place;           // where its partial goes (mode whole: by CTA)
 };
-// For the combine kernel: the partials of a group are those of consecutive items.
+// For the combine kernel: the partials of a group are in consecutive places.
 struct PlanGroup {
-    int b_g, tile, n, first_item, pieces, pad[3];
+    int b_g, tile, n, first_place, pieces, pad[3];
 };
 static_assert(sizeof(PlanHead) == 16 && sizeof(PlanCluster) == 8 && sizeof(PlanItem) == 32 && sizeof(PlanGroup) == 32, "vector loads");
 
@@ -126,6 +137,8 @@ struct AttnArgs {
     int max_items;
     int comb_chunk;   // partials the combine kernel fetches together
     int stream_gain;  // -1: own choice; 0: never mode even; else always where it fits (tests)
+    int rounds;       // mode even: 0: own choice; else this many rounds (tests)
+    int l2_tiles;     // K and V of more key tiles (of a KV head) than this do not stay in L2
     int min_tiles;    // fewest key tiles a CTA is given
     int q_by_tma;     // 1: Q tiles come by TMA (128 % (Hq/Hkv) == 0), 0: by plain loads
     int plan_after_wait;  // 1: the work list was written by the kernel just before this one
@@ -135,7 +148,7 @@ struct AttnArgs {
     PlanHead* plan_head;
     PlanCluster* plan_cluster;  // [kMaxGrid]
     PlanItem* plan_first;       // [kMaxGrid] every CTA's first item once more (one load instead of two in a row)
-    PlanItem* plan_item;        // [max_items x cluster] (mode even has one item per CTA and does without)
+    PlanItem* plan_item;        // [max_items x cluster]
     PlanGroup* plan_group;      // [groups]
 };
 
@@ -158,12 +171,16 @@ struct PlanShared {
     unsigned long long start[kMaxBatch + 1];  // first position of a sequence, in key tiles ...
     unsigned long long cost0[kMaxBatch + 1];  // ... and with every group's kItemTiles
     int group0[kMaxBatch + 1];                // first group of a sequence
-    int item0[kMaxBatch + 1];                 // mode even: first item of a sequence
-    int n[kMaxBatch], L[kMaxBatch], tiles[kMaxBatch], kt[kMaxBatch], splits[kMaxBatch];
+    int n[kMaxBatch], L[kMaxBatch], tiles[kMaxBatch], kt[kMaxBatch];
+    // mode even, by rounds - 1 (a warp each)
+    int item0[kMaxRounds][kMaxBatch + 1];     // first item of a sequence (also the first place of its partials)
+    int splits[kMaxRounds][kMaxBatch];        // items a group is cut into
     unsigned long long cut[2][kMaxGrid + 1];
     int n_items[kMaxGrid];
-    int even_cost, range_cost[2];  // largest share of a CTA: mode even; ranges of whole groups, equal ranges
+    int even_cost[kMaxRounds], even_share[kMaxRounds], range_cost[2];  // largest share of a CTA: mode even; ranges of whole groups, equal ranges
+    int reread;                                // K and V are read again by every row tile in mode stream
 };
+static_assert(kMaxGrid >= 32 * kMaxRounds, "a warp per number of rounds");
 
 __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs a) {
     __shared__ PlanShared sh;
@@ -209,44 +226,6 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
             sh.start[a.batch] = pos, sh.group0[a.batch] = group;
             sh.cost0[a.batch] = pos + static_cast<unsigned long long>(group) * kItemTiles;
         }
-        if (a.cluster == 1) {
-            // the smallest T (in steps of T/16) for which the splits fit one round of the grid
-            int T = static_cast<int>(min((pos + a.clusters - 1) / a.clusters, 1ull << 24));
-            T = max(T, 1);
-            bool fits = false;
-#pragma unroll 1
-            for (int tries = 0; tries < 40 && !fits; ++tries) {
-                unsigned count = 0;
-#pragma unroll 1
-                for (int b = lane; b < a.batch; b += 32)
-                    count += static_cast<unsigned>(a.Hkv * sh.tiles[b] * ceil_div(sh.kt[b], max(T, a.min_tiles)));
-                count = __reduce_add_sync(kFull, min(count, 1u << 20));
-                fits = count <= static_cast<unsigned>(a.clusters);
-                if (!fits) T += max(1, T >> 4);
-            }
-            T = max(T, a.min_tiles);
-            // (its cost is compared with the ranges' below)
-            int base = 0, most = 0;
-#pragma unroll 1
-            for (int b0 = 0; b0 < a.batch; b0 += 32) {
-                const int b = b0 + lane, splits = (b < a.batch) ? ceil_div(sh.kt[b], T) : 0;
-                int incl = (b < a.batch && fits) ? a.Hkv * sh.tiles[b] * splits : 0;
-                most = max(most, splits > 0 ? ceil_div(sh.kt[b], splits) + kItemTiles + (splits > 1 ? kCutTiles : 0) : 0);
-                const int own = incl;
-#pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    const int v = __shfl_up_sync(kFull, incl, d);
-                    if (lane >= d) incl += v;
-                }
-                if (b < a.batch) sh.splits[b] = splits, sh.item0[b] = base + incl - own;
-                base += __shfl_sync(kFull, incl, 31);
-            }
-            most = __reduce_max_sync(kFull, most);
-            if (lane == 0) {
-                sh.item0[a.batch] = base;
-                sh.even_cost = fits ? most + (a.stream_gain < 0 ? 0 : a.stream_gain ? -(1 << 28) : 1 << 28) : 1 << 30;
-            }
-        }
         if (lane == 0) {
             sh.range_cost[0] = sh.range_cost[1] = 0;
             PlanHead h = {};
@@ -256,6 +235,50 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
     }
     __syncthreads();
     const int n_groups = sh.group0[a.batch];
+    if (a.cluster == 1 && tid < 32 * kMaxRounds) {
+        // ---- mode even: the smallest T (in steps of T/16) for which the splits fit the rounds ----------------------
+        const int w = tid >> 5, rounds = w + 1, room = rounds * a.clusters;
+        const unsigned long long work = sh.start[a.batch];
+        int T = max(static_cast<int>(min((work + room - 1) / room, 1ull << 24)), 1);
+        bool fits = false;
+#pragma unroll 1
+        for (int tries = 0; tries < 40 && !fits; ++tries) {
+            unsigned count = 0;
+#pragma unroll 1
+            for (int b = lane; b < a.batch; b += 32)
+                count += static_cast<unsigned>(a.Hkv * sh.tiles[b] * ceil_div(sh.kt[b], max(T, a.min_tiles)));
+            count = __reduce_add_sync(kFull, min(count, 1u << 20));
+            fits = count <= static_cast<unsigned>(room);
+            if (!fits) T += max(1, T >> 4);
+        }
+        T = max(T, a.min_tiles);
+        int base = 0, tiles = 0;
+        bool cut = false;
+#pragma unroll 1
+        for (int b0 = 0; b0 < a.batch; b0 += 32) {
+            const int b = b0 + lane, splits = (b < a.batch) ? ceil_div(sh.kt[b], T) : 0;
+            int incl = (b < a.batch && fits) ? a.Hkv * sh.tiles[b] * splits : 0;
+            cut = cut || splits > 1;
+            if (b < a.batch && sh.tiles[b] > 1) tiles += min(a.Hkv * sh.kt[b], 1 << 22);
+            const int own = incl;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int v = __shfl_up_sync(kFull, incl, d);
+                if (lane >= d) incl += v;
+            }
+            if (b < a.batch) sh.splits[w][b] = splits, sh.item0[w][b] = base + incl - own;
+            base += __shfl_sync(kFull, incl, 31);
+        }
+        tiles = __reduce_add_sync(kFull, min(tiles, 1 << 25));
+        cut = __any_sync(kFull, cut);
+        if (lane == 0) {
+            sh.item0[w][a.batch] = base;
+            const bool allowed = fits && base <= a.max_items && a.stream_gain != 0 && (a.rounds == 0 || a.rounds == rounds);
+            sh.even_share[w] = 0;
+            sh.even_cost[w] = !allowed ? 1 << 30 : (cut ? kCutTiles : 0) - (a.stream_gain > 0 ? 1 << 28 : 0);  // besides the share
+            if (w == 0) sh.reread = tiles > a.l2_tiles;
+        }
+    }
     auto last_at_or_before = [&](const int* first, int x) {  // the last sequence whose entry is <= x
         int lo = 0, hi = a.batch;
 #pragma unroll 1
@@ -273,9 +296,9 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
         p.n = sh.n[b], p.L = sh.L[b], p.pieces = 1;
         return p;
     };
-    auto write_group = [&](int group, const PlanItem& p, int first_item) {
+    auto write_group = [&](int group, const PlanItem& p) {  // by the group's first item
         PlanGroup q = {};
-        q.b_g = p.b_g, q.tile = p.tile_active & 0xFFFF, q.n = p.n, q.first_item = first_item, q.pieces = p.pieces;
+        q.b_g = p.b_g, q.tile = p.tile_active & 0xFFFF, q.n = p.n, q.first_place = p.place, q.pieces = p.pieces;
         a.plan_group[group] = q;
     };
     // ---- ranges ---------------------------------------------------------------------------------------
@@ -321,44 +344,75 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
                 const int items = sh.group0[b1] + local1 - sh.group0[b] - local + 1;
                 atomicMax(&sh.range_cost[w], static_cast<int>(end - begin) + items * kItemTiles + (w ? kCutTiles : 0));
             }
+            // (sequences of different lengths give items of different lengths: a CTA's real sum counts.  One sequence's
+            // are the same to a tile.)
+#pragma unroll 1
+            for (int w = 0; w < kMaxRounds; ++w) {
+                if (sh.even_cost[w] == 1 << 30) continue;
+                const int n = sh.item0[w][a.batch];
+                int share = 0;
+#pragma unroll 1
+                for (int item = tid; item < n; item += a.clusters) {
+                    const int b = a.batch > 1 ? last_at_or_before(sh.item0[w], item) : 0;
+                    share += ceil_div(sh.kt[b], sh.splits[w][b]) + kItemTiles;
+                }
+                atomicMax(&sh.even_share[w], share);
+            }
         }
         __syncthreads();
     }
     const int ranges = sh.range_cost[1] < sh.range_cost[0] ? 1 : 0;
-    const int mode = a.cluster > 1 ? kModeWhole : sh.even_cost <= sh.range_cost[ranges] ? kModeEven : kModeStream;
-    if (mode != kModeStream) {
-        // ---- an item per cluster or CTA ---------------------------------------------------------------
-        const int n = (mode == kModeWhole) ? n_groups : sh.item0[a.batch];
+    int mode = kModeWhole, even = 0;
+    if (a.cluster == 1) {
+#pragma unroll 1
+        for (int w = 1; w < kMaxRounds; ++w)
+            if (sh.even_cost[w] + sh.even_share[w] < sh.even_cost[even] + sh.even_share[even]) even = w;
+        const long long range_cost = static_cast<long long>(sh.range_cost[ranges]) * (sh.reread ? kRereadNum : kRereadDen);
+        mode = static_cast<long long>(sh.even_cost[even] + sh.even_share[even]) * kRereadDen <= range_cost ? kModeEven : kModeStream;
+    }
+    if (mode == kModeEven) {
+        // ---- CTA c takes items c, c + CTAs, ... --------------------------------------------------------------------
+        const int n = sh.item0[even][a.batch];
         if (tid < a.clusters) {
-            // (mode whole has more groups than clusters only if a tree is larger than the context's limits allow)
             PlanCluster c;
-            c.first_item = static_cast<int>(static_cast<unsigned>(n) * tid / a.clusters);
-            c.n_items = static_cast<int>(static_cast<unsigned>(n) * (tid + 1) / a.clusters) - c.first_item;
-            if (n <= a.clusters) c.first_item = tid, c.n_items = (tid < n) ? 1 : 0;
-            a.plan_cluster[tid] = c;
-            if (mode == kModeWhole) {
+            c.first_item = tid * kMaxRounds, c.n_items = 0;
 #pragma unroll 1
-                for (int i = 0; i < c.n_items; ++i) {
-                    const int group = c.first_item + i, b = last_at_or_before(sh.group0, group);
-                    PlanItem p = item_of(b, group - sh.group0[b]);
-                    const int kt = sh.kt[b], act = active_ctas(kt, a.cluster, a.min_tiles);
-                    p.tile_active = (p.tile_active & 0xFFFF) | (act << 16);
-#pragma unroll 1
-                    for (int r = 0; r < a.cluster; ++r) {
-                        p.t_begin = p.t_end;
-                        if (r < act) p.t_end = kt * (r + 1) / act;
-                        if (i == 0) a.plan_first[tid * a.cluster + r] = p;
-                        a.plan_item[group * a.cluster + r] = p;
-                    }
-                }
-            } else if (tid < n) {
-                const int b = last_at_or_before(sh.item0, tid), splits = sh.splits[b], kt = sh.kt[b];
-                const int at = tid - sh.item0[b], local = static_cast<int>(static_cast<unsigned>(at) / static_cast<unsigned>(splits));
+            for (int item = tid; item < n; item += a.clusters, ++c.n_items) {
+                const int b = last_at_or_before(sh.item0[even], item), splits = sh.splits[even][b], kt = sh.kt[b];
+                const int at = item - sh.item0[even][b], local = static_cast<int>(static_cast<unsigned>(at) / static_cast<unsigned>(splits));
                 const int sp = at - local * splits;
                 PlanItem p = item_of(b, local);
-                p.t_begin = kt * sp / splits, p.t_end = kt * (sp + 1) / splits, p.pieces = splits;  // (kt <= 2^15, splits <= 2^8)
-                a.plan_first[tid] = p;
-                if (sp == 0) write_group(sh.group0[b] + local, p, tid);
+                p.t_begin = kt * sp / splits, p.t_end = kt * (sp + 1) / splits;  // (kt <= 2^15, splits <= 2^10)
+                p.pieces = splits, p.place = item;
+                if (c.n_items == 0) a.plan_first[tid] = p;
+                a.plan_item[c.first_item + c.n_items] = p;
+                if (sp == 0) write_group(sh.group0[b] + local, p);
+            }
+            a.plan_cluster[tid] = c;
+        }
+        return;
+    }
+    if (mode == kModeWhole) {
+        // ---- a group per cluster (more groups than clusters only if a tree is larger than the context's limits allow)
+        if (tid < a.clusters) {
+            PlanCluster c;
+            c.first_item = static_cast<int>(static_cast<unsigned>(n_groups) * tid / a.clusters);
+            c.n_items = static_cast<int>(static_cast<unsigned>(n_groups) * (tid + 1) / a.clusters) - c.first_item;
+            if (n_groups <= a.clusters) c.first_item = tid, c.n_items = (tid < n_groups) ? 1 : 0;
+            a.plan_cluster[tid] = c;
+#pragma unroll 1
+            for (int i = 0; i < c.n_items; ++i) {
+                const int group = c.first_item + i, b = last_at_or_before(sh.group0, group);
+                PlanItem p = item_of(b, group - sh.group0[b]);
+                const int kt = sh.kt[b], act = active_ctas(kt, a.cluster, a.min_tiles);
+                p.tile_active = (p.tile_active & 0xFFFF) | (act << 16);
+#pragma unroll 1
+                for (int r = 0; r < a.cluster; ++r) {
+                    p.t_begin = p.t_end;
+                    if (r < act) p.t_end = kt * (r + 1) / act;
+                    if (i == 0) a.plan_first[tid * a.cluster + r] = p;
+                    a.plan_item[group * a.cluster + r] = p;
+                }
             }
         }
         return;
@@ -397,10 +451,10 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
             const unsigned long long stop = g1 < end ? g1 : end;
             const int c0 = (g0 >= begin) ? tid : cluster_of(g0), c1 = (g1 <= end) ? tid : cluster_of(g1 - 1);
             PlanItem p = item_of(b, local);
-            p.t_begin = t, p.t_end = static_cast<int>(stop - g0), p.pieces = c1 - c0 + 1;
+            p.t_begin = t, p.t_end = static_cast<int>(stop - g0), p.pieces = c1 - c0 + 1, p.place = first + i;
             if (i == 0) a.plan_first[tid] = p;
             a.plan_item[first + i] = p;
-            if (t == 0) write_group(sh.group0[b] + local, p, first + i);
+            if (t == 0) write_group(sh.group0[b] + local, p);
             // on to the next group
             pos = stop, t = 0;
             if (++local == a.Hkv * sh.tiles[b]) {
@@ -419,7 +473,7 @@ struct Item {
     int b, g, n, L, M, row_base;
     int t_begin, t_end;  // this CTA's key tiles (none: t_begin == t_end)
     int active;          // CTAs of the cluster that have tiles of the item
-    int pieces;
+    int pieces, place;
 };
 
 __device__ __forceinline__ Item load_item(const PlanItem* entry, int G) {
@@ -429,7 +483,7 @@ __device__ __forceinline__ Item load_item(const PlanItem* entry, int G) {
     it.b = lo.x & 0xFFFF, it.g = static_cast<int>(static_cast<unsigned>(lo.x) >> 16);
     it.row_base = (lo.y & 0xFFFF) * kBM, it.active = static_cast<int>(static_cast<unsigned>(lo.y) >> 16);
     it.t_begin = lo.z, it.t_end = lo.w;
-    it.n = hi.x, it.L = hi.y, it.pieces = hi.z;
+    it.n = hi.x, it.L = hi.y, it.pieces = hi.z, it.place = hi.w;
     it.M = it.n * G;
     return it;
 }
@@ -1271,7 +1325,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 const int64_t out_row = (static_cast<int64_t>(it.b) * a.max_tt + tok) * a.Hq + h;
                 // (two places per CTA of a cluster, in turn: an item's partials are read behind the meeting of the
                 // CTAs, and the next but one item's are written behind the next meeting)
-                const int64_t place = a.cluster > 1 ? static_cast<int>(blockIdx.x + (meets & 1u) * gridDim.x) : first_item + i;
+                const int64_t place = a.cluster > 1 ? static_cast<int>(blockIdx.x + (meets & 1u) * gridDim.x) : it.place;
                 __nv_bfloat16* dst = a.o + out_row * D;
                 uint4* po = a.part_o + place * (D / 8) * kBM + r;
                 // (a lane without tiles has nothing in tensor memory: the other's is read in its place, with weight 0)
@@ -1631,6 +1685,8 @@ int choose_cluster(const int* resident, int sm_count, int groups, int batch, int
     }
     return 1;
 }
+// K and V of this many bytes are taken to stay in L2 between the row tiles of a head (measured between 67 and 131 MB).
+constexpr int64_t kL2Bytes = 96 << 20;
 int forced_cluster(const int* resident, int cluster, int groups) {
     while (cluster > 1 && resident[cluster] < groups) --cluster;
     return cluster;
@@ -1761,7 +1817,8 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
     if (w.attn_rounds > 0 && a.cluster == 1) a.clusters = std::max(1, a.clusters / w.attn_rounds);
     // one resident round of units with room for all of a group's partials, else more CTAs per SM
     a.comb_chunk = groups * (D / 8 / kCombPieces) <= ctx->sm_count ? kCombChunkMost : kCombChunk;
-    a.stream_gain = w.attn_stream;
+    a.stream_gain = w.attn_stream, a.rounds = w.attn_even_rounds;
+    a.l2_tiles = static_cast<int>(kL2Bytes / (2 * 2 * kBN * D));
     MapKey kk = {k_cache, stride_tok, stride_head, stride_seq, capacity, a.Hkv, batch, 0};
     MapKey kv = kk;
     kv.base = v_cache;
@@ -1795,7 +1852,10 @@ int attention_max_groups(int batch, int n_kv_heads, int max_tt, int group) {
     return batch * n_kv_heads * ((max_tt * group + kBM - 1) / kBM);
 }
 // (also the most partials)
-int attention_max_items(int groups, int sm_count) { return std::max(groups, std::min(sm_count, kMaxGrid)) + std::min(sm_count, kMaxGrid); }
+int attention_max_items(int groups, int sm_count) {
+    const int grid = std::min(sm_count, kMaxGrid);
+    return std::max(groups, (kMaxRounds - 1) * grid) + grid;
+}
 size_t attention_plan_bytes(int max_items, int max_groups) {
     return sizeof(PlanHead) + sizeof(PlanCluster) * kMaxGrid + sizeof(PlanItem) * (kMaxGrid + static_cast<size_t>(max_items) * kMaxCluster) +
            sizeof(PlanGroup) * static_cast<size_t>(max_groups);

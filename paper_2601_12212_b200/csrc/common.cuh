@@ -47,6 +47,7 @@ struct Workspace {
     int attn_min_tiles = 2;     // fewest key tiles a CTA of a cluster is given
     int attn_stream = -1;       // 0: never equal splits per group, > 0: always where they fit (tests)
     int attn_cluster = 0;       // > 0: CTAs per cluster (tests)
+    int attn_even_rounds = 0;   // > 0: rounds of equal splits (tests)
     int attn_rounds = 0;        // > 0: the work list is cut for 1/n of the clusters (tests)
     int attn_max_items = 0;
     int attn_max_groups = 0;

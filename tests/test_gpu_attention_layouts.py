@@ -1,6 +1,6 @@
-"""The ways a layer's attention is laid out (clusters of every size, equal splits, ranges over all groups), forced
-by the test-only overrides on shapes where each can go wrong: more CTAs than key tiles, groups whose size does not
-divide a row tile, a single token, fewer groups than clusters and more."""
+"""The ways a layer's attention is laid out (clusters of every size; equal splits in one round of items and in
+several; ranges over all groups), forced by the test-only overrides on shapes where each can go wrong: more CTAs than key
+tiles, groups whose size does not divide a row tile, a single token, fewer groups than clusters and more."""
 import pytest
 
 from test_gpu_edges import _attention_case, _imports
@@ -20,3 +20,17 @@ def test_layouts(shape, cluster, equal_splits):
     if equal_splits is not None:
         debug.append((binding.RESPS_DEBUG_ATTN_SINGLE, equal_splits))
     _attention_case(**SHAPES[shape], cap=1664, seed=cluster, poison=True, debug=debug)
+
+
+TILES = [dict(n=[43, 128, 1, 86], Hq=24, Hkv=8, D=128, L=[1000, 63, 1500, 0], B=4),  # 2 row tiles (the second of 1 row), 3, 1, 3
+         dict(n=96, Hq=14, Hkv=2, D=64, L=1400),                                      # 6, Q by plain loads
+         dict(n=[128, 65, 2, 20], Hq=16, Hkv=1, D=128, L=[130, 1, 5, 1536], B=4)]     # 16, 9, 1, 3
+
+
+@pytest.mark.parametrize("rounds", [1, 2, 3, 4])
+@pytest.mark.parametrize("shape", range(len(TILES)))
+def test_equal_splits_in_rounds(shape, rounds):
+    _, binding, _ = _imports()
+    debug = [(binding.RESPS_DEBUG_ATTN_CLUSTER, 1), (binding.RESPS_DEBUG_ATTN_SINGLE, 1), (binding.RESPS_DEBUG_ATTN_EVEN_ROUNDS, rounds)]
+    for cut_for in (0, 12):  # all CTAs; a twelfth of them, so that the rounds are full
+        _attention_case(**TILES[shape], cap=1664, seed=rounds, poison=True, debug=debug + [(binding.RESPS_DEBUG_ATTN_ROUNDS, cut_for)])
