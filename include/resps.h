@@ -112,7 +112,8 @@ enum {
     RESPS_DEBUG_ATTN_CLUSTER = 3,   /* most CTAs per cluster of the attention kernel (1..8): 0 = its own choice        */
     RESPS_DEBUG_SCAN_SLICES = 4,    /* slices a logits row is cut into by the streaming scan: 0 = its own choice       */
     RESPS_DEBUG_ATTN_SINGLE = 5,    /* 0: never equal splits of every (sequence, KV head, row tile) but ranges over all of
-                                       them; > 0: always equal splits where they fit (default: its own choice)    */
+                                       them; > 0: always equal splits where they fit, and with clusters groups cut
+                                       over those that are left (default: its own choice)                         */
     RESPS_DEBUG_ATTN_EVEN_ROUNDS = 6 /* rounds of equal splits (1..4), 0 = its own choice                              */
 };
 int resps_debug_set(resps_ctx* ctx, int key, int value);

@@ -12,6 +12,7 @@ namespace resps {
 int scan_chunk_max();
 int attention_max_batch();
 int attention_place_rows();
+int attention_counters();
 int attention_max_groups(int batch, int n_kv_heads, int max_tt, int group);
 int attention_max_items(int groups, int sm_count);
 }  // namespace resps
@@ -67,6 +68,7 @@ void carve(resps_ctx* c, Carver& cv) {
     const int64_t part_rows = static_cast<int64_t>(w.attn_max_items) * resps::attention_place_rows();
     cv.take(w.attn_part_o, part_rows * s.head_dim);
     cv.take(w.attn_part_ml, part_rows);
+    cv.take(w.attn_count, resps::attention_counters());
 }
 
 #define RESPS_CHECK_PTR(p) \
@@ -212,6 +214,7 @@ int resps_status(resps_ctx* ctx, resps_stream stream, int32_t* status) {
         if (cudaMemsetAsync(w.row_counter, 0, rows * sizeof(unsigned int), stream) != cudaSuccess ||
             cudaMemsetAsync(w.amax_counter, 0, nodes * sizeof(unsigned int), stream) != cudaSuccess ||
             cudaMemsetAsync(w.amax_seq_counter, 0, ctx->shape.max_batch * sizeof(unsigned int), stream) != cudaSuccess ||
+            cudaMemsetAsync(w.attn_count, 0, resps::attention_counters() * sizeof(unsigned int), stream) != cudaSuccess ||
             cudaStreamSynchronize(stream) != cudaSuccess)
             return RESPS_ERR_CUDA;
     }

@@ -53,6 +53,7 @@ constexpr int kStagesV = 4;
 static_assert(kStagesK % 2 == 0 && kStagesV % 2 == 0, "ring depths must be even");
 constexpr int kLanes = 2;
 constexpr int kSoftmaxThreads = 256;
+constexpr int kPieceWarps = kSoftmaxThreads / 32;
 constexpr int kProducerWarp = 8;   // K and Q tiles
 constexpr int kMmaWarp0 = 9;       // lane x is issued by warp kMmaWarp0 + x
 constexpr int kVProducerWarp = 11; // V tiles
@@ -65,6 +66,7 @@ constexpr int kMaxGrid = 256;      // clusters x CTAs (one per SM)
 constexpr int kSnap = 4;           // mode stream: a cut this close to a group's edge (key tiles) is moved onto it
 constexpr int kItemTiles = 4;      // what an item costs a CTA besides its tiles (its start and epilogue), in key tiles
 constexpr int kMaxRounds = 4;      // mode even: most rounds of splits
+constexpr int kPieceTiles = 5;     // mode whole: a group is cut where that takes more than this many key tiles off a CTA
 constexpr int kRereadNum = 5, kRereadDen = 4;
 constexpr int kCutTiles = 6;       // what cut groups cost a call (partials, the combine kernel's round trips)
 constexpr int kTmemCols = 512;
@@ -75,7 +77,10 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 // How a layer's work is laid out, one of three ways (PlanHead::mode):
 //  whole   clusters of several CTAs, one group (sequence, KV head, row tile) per cluster.  The CTAs share
 //          the group's key tiles, leave normalised partial results in the workspace (L2), meet on an
-//          mbarrier and merge a share of the rows x columns each: one kernel does the layer.
+//          mbarrier and merge a share of the rows x columns each: one kernel does the layer.  Where the tree at
+//          hand has fewer groups than there are clusters (which are as many as the context's largest tree needs),
+//          a group with enough key tiles is cut over several clusters, and of the warps that have merged the same
+//          share in each of them the last one merges those (fp32 sums, in L2).
 //  even    single CTAs; every group is cut into splits of at most T key tiles with the smallest T for which
 //          the splits fit one round of the grid, or two to four (CTA c takes splits c, c + CTAs, ... in the order of
 //          sequence, KV head, row tile and keys); a second, small kernel combines the partials.
@@ -106,8 +111,8 @@ struct PlanItem {
     int tile_active;     // row tile of the KV head | CTAs that have key tiles of the item << 16
     int t_begin, t_end;  // this CTA's key tiles (none: t_begin == t_end)
     int n, L;            // the sequence's tree size and prefix length
-    int pieces;          // items the group is cut into
-    int place;           // where its partial goes (mode whole: by CTA)
+    int pieces;          // items the group is cut into | (mode whole) the item's place among them << 16
+    int place;           // where its partial goes (mode whole: the group's first cluster)
 };
 // For the combine kernel: the partials of a group are in consecutive places.
 struct PlanGroup {
@@ -137,12 +142,16 @@ struct AttnArgs {
     int max_items;
     int comb_chunk;   // partials the combine kernel fetches together
     int stream_gain;  // -1: own choice; 0: never mode even; else always where it fits (tests)
+    int may_cut;      // mode whole: a group may be cut over several clusters
     int rounds;       // mode even: 0: own choice; else this many rounds (tests)
     int l2_tiles;     // K and V of more key tiles (of a KV head) than this do not stay in L2
     int min_tiles;    // fewest key tiles a CTA is given
     int q_by_tma;     // 1: Q tiles come by TMA (128 % (Hq/Hkv) == 0), 0: by plain loads
     int plan_after_wait;  // 1: the work list was written by the kernel just before this one
     int test_drop;        // test build only: 1 = the CTA's first V copy is left out
+    float4* piece_acc;      // [clusters][4][128 x D/16 units] a cut group's merged share: 16 sums of a unit,
+    float2* piece_ml;       // [clusters][units] (running max, running sum)
+    unsigned* piece_count;  // [kMaxGrid][8] warps that have left theirs: of the group's first cluster, by CTA and warp
     int32_t* status;
     // The work list, written by attention_plan_kernel.
     PlanHead* plan_head;
@@ -178,6 +187,7 @@ struct PlanShared {
     unsigned long long cut[2][kMaxGrid + 1];
     int n_items[kMaxGrid];
     int even_cost[kMaxRounds], even_share[kMaxRounds], range_cost[2];  // largest share of a CTA: mode even; ranges of whole groups, equal ranges
+    int cut_groups;                            // mode whole: groups are cut over several clusters
     int reread;                                // K and V are read again by every row tile in mode stream
 };
 static_assert(kMaxGrid >= 32 * kMaxRounds, "a warp per number of rounds");
@@ -185,6 +195,7 @@ static_assert(kMaxGrid >= 32 * kMaxRounds, "a warp per number of rounds");
 __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs a) {
     __shared__ PlanShared sh;
     const int tid = threadIdx.x, lane = tid & 31, G = a.Hq / a.Hkv;
+    const int reach = min(32, a.batch);  // lanes that a scan over the sequences has to span
     pdl_wait();  // the step parameters and node counts are complete
     pdl_launch_dependents();
     if (tid < a.batch) {
@@ -209,8 +220,8 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
             unsigned long long work = (b < a.batch) ? static_cast<unsigned long long>(groups) * sh.kt[b] : 0ull;
             const int own_groups = groups;
             const unsigned long long own_work = work;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
+#pragma unroll 1
+            for (int d = 1; d < reach; d <<= 1) {
                 const int g = __shfl_up_sync(kFull, groups, d);
                 const unsigned long long w = __shfl_up_sync(kFull, work, d);
                 if (lane >= d) groups += g, work += w;
@@ -219,14 +230,44 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
                 sh.start[b] = pos + work - own_work, sh.group0[b] = group + groups - own_groups;
                 sh.cost0[b] = sh.start[b] + static_cast<unsigned long long>(sh.group0[b]) * kItemTiles;
             }
-            pos += __shfl_sync(kFull, work, 31);
-            group += __shfl_sync(kFull, groups, 31);
+            pos += __shfl_sync(kFull, work, min(31, a.batch - b0 - 1));
+            group += __shfl_sync(kFull, groups, min(31, a.batch - b0 - 1));
         }
         if (lane == 0) {
             sh.start[a.batch] = pos, sh.group0[a.batch] = group;
             sh.cost0[a.batch] = pos + static_cast<unsigned long long>(group) * kItemTiles;
         }
+        // ---- mode whole: the clusters that the groups leave are given to them by their key tiles; a group stays whole
+        // where a piece saves a CTA too little ------------------------------------------------------------------------
+        bool cut = false;
+        if (a.may_cut && group < a.clusters) {
+            const int gain = a.stream_gain > 0 ? 0 : kPieceTiles * a.cluster, spare = a.clusters - group;
+            int base = 0;
+#pragma unroll 1
+            for (int b0 = 0; b0 < a.batch; b0 += 32) {
+                const int b = b0 + lane, kt = (b < a.batch) ? sh.kt[b] : 0;
+                int pieces = 1;
+                if (kt > gain) {  // (fewer groups than CTAs, of at most 2^15 tiles: 32 bits hold the sum)
+                    pieces += static_cast<int>(static_cast<unsigned>(spare * kt) / static_cast<unsigned>(pos));
+                    pieces = min(pieces, kt);
+                    if (kt - ceil_div(kt, pieces) <= gain) pieces = 1;
+                }
+                cut = cut || pieces > 1;
+                const int own = (b < a.batch) ? a.Hkv * sh.tiles[b] * pieces : 0;
+                int incl = own;
+#pragma unroll 1
+                for (int d = 1; d < reach; d <<= 1) {
+                    const int v = __shfl_up_sync(kFull, incl, d);
+                    if (lane >= d) incl += v;
+                }
+                if (b < a.batch) sh.splits[0][b] = pieces, sh.item0[0][b] = base + incl - own;
+                base += __shfl_sync(kFull, incl, min(31, a.batch - b0 - 1));
+            }
+            cut = __any_sync(kFull, cut);
+            if (lane == 0) sh.item0[0][a.batch] = base;
+        }
         if (lane == 0) {
+            sh.cut_groups = cut;
             sh.range_cost[0] = sh.range_cost[1] = 0;
             PlanHead h = {};
             h.n_groups = group;
@@ -261,13 +302,13 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
             cut = cut || splits > 1;
             if (b < a.batch && sh.tiles[b] > 1) tiles += min(a.Hkv * sh.kt[b], 1 << 22);
             const int own = incl;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
+#pragma unroll 1
+            for (int d = 1; d < reach; d <<= 1) {
                 const int v = __shfl_up_sync(kFull, incl, d);
                 if (lane >= d) incl += v;
             }
             if (b < a.batch) sh.splits[w][b] = splits, sh.item0[w][b] = base + incl - own;
-            base += __shfl_sync(kFull, incl, 31);
+            base += __shfl_sync(kFull, incl, min(31, a.batch - b0 - 1));
         }
         tiles = __reduce_add_sync(kFull, min(tiles, 1 << 25));
         cut = __any_sync(kFull, cut);
@@ -372,10 +413,10 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
     }
     if (mode == kModeEven) {
         // ---- CTA c takes items c, c + CTAs, ... --------------------------------------------------------------------
-        const int n = sh.item0[even][a.batch];
+        const int n = sh.item0[even][a.batch], rounds = ceil_div(n, a.clusters);  // (that are used)
         if (tid < a.clusters) {
             PlanCluster c;
-            c.first_item = tid * kMaxRounds, c.n_items = 0;
+            c.first_item = tid * rounds, c.n_items = 0;
 #pragma unroll 1
             for (int item = tid; item < n; item += a.clusters, ++c.n_items) {
                 const int b = last_at_or_before(sh.item0[even], item), splits = sh.splits[even][b], kt = sh.kt[b];
@@ -393,25 +434,37 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
         return;
     }
     if (mode == kModeWhole) {
-        // ---- a group per cluster (more groups than clusters only if a tree is larger than the context's limits allow)
+        // ---- a group, or a piece of one, per cluster (more than clusters only if a tree is larger than the context's
+        // limits allow) ----------------------------------------------------------------------------------------------
+        const bool cut = sh.cut_groups != 0;
+        const int* const first = cut ? sh.item0[0] : sh.group0;
+        const int n = first[a.batch];
         if (tid < a.clusters) {
             PlanCluster c;
-            c.first_item = static_cast<int>(static_cast<unsigned>(n_groups) * tid / a.clusters);
-            c.n_items = static_cast<int>(static_cast<unsigned>(n_groups) * (tid + 1) / a.clusters) - c.first_item;
-            if (n_groups <= a.clusters) c.first_item = tid, c.n_items = (tid < n_groups) ? 1 : 0;
+            c.first_item = static_cast<int>(static_cast<unsigned>(n) * tid / a.clusters);
+            c.n_items = static_cast<int>(static_cast<unsigned>(n) * (tid + 1) / a.clusters) - c.first_item;
+            if (n <= a.clusters) c.first_item = tid, c.n_items = (tid < n) ? 1 : 0;
             a.plan_cluster[tid] = c;
 #pragma unroll 1
             for (int i = 0; i < c.n_items; ++i) {
-                const int group = c.first_item + i, b = last_at_or_before(sh.group0, group);
-                PlanItem p = item_of(b, group - sh.group0[b]);
-                const int kt = sh.kt[b], act = active_ctas(kt, a.cluster, a.min_tiles);
+                const int item = c.first_item + i, b = last_at_or_before(first, item);
+                int local = item - first[b], pieces = 1, piece = 0, t0 = 0, kt = sh.kt[b];
+                if (cut && sh.splits[0][b] > 1) {
+                    pieces = sh.splits[0][b];
+                    piece = local, local = static_cast<int>(static_cast<unsigned>(local) / static_cast<unsigned>(pieces)), piece -= local * pieces;
+                    t0 = kt * piece / pieces, kt = kt * (piece + 1) / pieces - t0;
+                }
+                PlanItem p = item_of(b, local);
+                const int act = active_ctas(kt, a.cluster, a.min_tiles);
                 p.tile_active = (p.tile_active & 0xFFFF) | (act << 16);
+                p.pieces = pieces | (piece << 16), p.place = item - piece;
+                p.t_end = t0;
 #pragma unroll 1
                 for (int r = 0; r < a.cluster; ++r) {
                     p.t_begin = p.t_end;
-                    if (r < act) p.t_end = kt * (r + 1) / act;
+                    if (r < act) p.t_end = t0 + kt * (r + 1) / act;
                     if (i == 0) a.plan_first[tid * a.cluster + r] = p;
-                    a.plan_item[group * a.cluster + r] = p;
+                    a.plan_item[item * a.cluster + r] = p;
                 }
             }
         }
@@ -483,7 +536,7 @@ __device__ __forceinline__ Item load_item(const PlanItem* entry, int G) {
     it.b = lo.x & 0xFFFF, it.g = static_cast<int>(static_cast<unsigned>(lo.x) >> 16);
     it.row_base = (lo.y & 0xFFFF) * kBM, it.active = static_cast<int>(static_cast<unsigned>(lo.y) >> 16);
     it.t_begin = lo.z, it.t_end = lo.w;
-    it.n = hi.x, it.L = hi.y, it.pieces = hi.z, it.place = hi.w;
+    it.n = hi.x, it.L = hi.y, it.pieces = hi.z & 0xFFFF, it.place = hi.w;
     it.M = it.n * G;
     return it;
 }
@@ -771,13 +824,30 @@ __device__ __forceinline__ constexpr int bar_merge() { return kBar1 + 1; }
 // every softmax warp of every CTA of the cluster has written its share of the CTA's partial
 __device__ __forceinline__ constexpr int bar_meet() { return kBar1 + 2; }
 
+// Sixteen columns of a row: O, and with the first ones the row's log-sum-exp.
+template <int D>
+__device__ __forceinline__ void write_unit(const AttnArgs& a, const Item& it, unsigned r, unsigned c16, int G, float Mx, float den,
+                                           const float (&acc)[16]) {
+    const float inv = 1.f / den;
+    const unsigned R = it.row_base + r, t = R / static_cast<unsigned>(G), h = it.g * G + (R - t * G);
+    const int64_t row = (static_cast<int64_t>(it.b) * a.max_tt + t) * a.Hq + h;
+    uint32_t o[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) o[e] = pack_bf16(acc[2 * e] * inv, acc[2 * e + 1] * inv);
+    uint4* dst = reinterpret_cast<uint4*>(a.o + row * D + c16 * 16);
+    dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
+    dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+    if (a.lse && c16 == 0) a.lse[row] = (Mx + log2f(den)) * 0.6931471805599453f;
+}
 // Merges the partials of an item: this CTA's share of the (16 columns, row) units, O = sum_p w_p O_p /
 // sum_p w_p l_p with w_p = 2^(m_p - max m).  Bound by the latency of L2 (one round trip for six partials,
-// whose loads are in flight together) and by its own code, which is kept short.
-template <int D>
+// whose loads are in flight together) and by its own code, which is kept short.  kPiece: the group is cut over several
+// clusters, the sums stay in the workspace.  (Two copies of the code, so that the common one has nothing to skip: with
+// one the 8B shape's call took 9.57 us, with two 9.34, and 9.45 before there were pieces.)
+template <int D, bool kPiece>
 __device__ __forceinline__ void merge_partials(const AttnArgs& a, const Item& it, unsigned place0, int n_parts,
-                                               int rank, int tid, int G) {
-    constexpr unsigned kBatch = 6;
+                                               int rank, int tid, int G, unsigned cluster_id) {
+    constexpr unsigned kBatch = 6, kUnits = kBM * (D / 16);
     const unsigned nv = static_cast<unsigned>(min(kBM, it.M - it.row_base));  // valid rows
     const unsigned units = nv * (D / 16);
     const unsigned u1 = units * static_cast<unsigned>(rank + 1) / static_cast<unsigned>(a.cluster);
@@ -820,16 +890,59 @@ __device__ __forceinline__ void merge_partials(const AttnArgs& a, const Item& it
                 }
             }
         }
-        const float inv = 1.f / den;
-        const unsigned R = it.row_base + r, t = R / static_cast<unsigned>(G), h = it.g * G + (R - t * G);
-        const int64_t row = (static_cast<int64_t>(it.b) * a.max_tt + t) * a.Hq + h;
-        uint32_t o[8];
+        if (!kPiece) {
+            write_unit<D>(a, it, r, c16, G, Mx, den, acc);
+        } else {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) o[e] = pack_bf16(acc[2 * e] * inv, acc[2 * e + 1] * inv);
-        uint4* dst = reinterpret_cast<uint4*>(a.o + row * D + c16 * 16);
-        dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-        dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
-        if (a.lse && c16 == 0) a.lse[row] = (Mx + log2f(den)) * 0.6931471805599453f;
+            for (int e = 0; e < 4; ++e)
+                __stcg(a.piece_acc + (cluster_id * 4 + e) * kUnits + u, make_float4(acc[4 * e], acc[4 * e + 1], acc[4 * e + 2], acc[4 * e + 3]));
+            __stcg(a.piece_ml + cluster_id * kUnits + u, make_float2(Mx, den));
+        }
+    }
+}
+// A group that is cut over several clusters: the same warp of the same CTA of each has merged the same units.  It
+// says so (nobody waits), and the one that finds that all others have done so merges the pieces: two round trips to L2
+// more on the way of a cut group, 2.5 to 3 us, against 0.7 us for each key tile that it takes off a CTA (kPieceTiles).
+// Under a context for 128 nodes on the 8B shape (32 clusters of 4), in us a layer uncut / cut / the two kernels with the
+// same context: 16 nodes at 4096 keys 16.5 / 14.2 / 15.5, at 8192 26.3 / 17.3 / 18.7, at 12 288 35.6 / 19.9 / 21.5;
+// 64 nodes 17.1 / 15.8 / 16.7, 26.8 / 21.0 / 21.6, 36.2 / 25.9 / 26.0.
+template <int D>
+__device__ __forceinline__ void merge_pieces(const AttnArgs& a, const Item& it, int rank, int tid, int G) {
+    constexpr unsigned kUnits = kBM * (D / 16);
+    const unsigned nv = static_cast<unsigned>(min(kBM, it.M - it.row_base)), units = nv * (D / 16);
+    const unsigned u1 = units * static_cast<unsigned>(rank + 1) / static_cast<unsigned>(a.cluster);
+    const unsigned u0 = units * static_cast<unsigned>(rank) / static_cast<unsigned>(a.cluster) + tid;
+    if (u0 - (tid & 31) >= u1) return;  // the warp has no units (in no piece)
+    unsigned* const count = a.piece_count + (it.place * a.cluster + rank) * kPieceWarps + (tid >> 5);
+    unsigned before = 0;
+    __syncwarp();  // (orders the lanes' sums before the first one's arrival)
+    if ((tid & 31) == 0) asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(before) : "l"(count) : "memory");
+    before = __shfl_sync(kFull, before, 0);
+    if (before + 1u != static_cast<unsigned>(it.pieces)) return;
+    if ((tid & 31) == 0) __stcg(count, 0u);  // for the next layer
+    __syncwarp();
+#pragma unroll 1
+    for (unsigned u = u0; u < u1; u += kSoftmaxThreads) {
+        float Mx = -INFINITY, den = 0.f;
+        float acc[16] = {};
+#pragma unroll 2
+        for (int p = 0; p < it.pieces; ++p) {
+            const unsigned cluster = static_cast<unsigned>(it.place + p);
+            const float2 ml = __ldcg(a.piece_ml + cluster * kUnits + u);
+            float4 v[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[e] = __ldcg(a.piece_acc + (cluster * 4 + e) * kUnits + u);
+            if (ml.x == -INFINITY) continue;  // nothing of the piece is visible to the row
+            const float mx = fmaxf(Mx, ml.x), c = ex2_approx(Mx - mx), w = ex2_approx(ml.x - mx);
+            Mx = mx, den = den * c + ml.y * w;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                acc[4 * e] = acc[4 * e] * c + v[e].x * w, acc[4 * e + 1] = acc[4 * e + 1] * c + v[e].y * w;
+                acc[4 * e + 2] = acc[4 * e + 2] * c + v[e].z * w, acc[4 * e + 3] = acc[4 * e + 3] * c + v[e].w * w;
+            }
+        }
+        const unsigned c16 = u / nv;
+        write_unit<D>(a, it, u - c16 * nv, c16, G, Mx, den, acc);
     }
 }
 
@@ -1399,7 +1512,13 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 if (lane < a.cluster) mbar_arrive_remote(bar(bar_meet()), lane);
                 alive = __all_sync(kFull, cluster_bar_wait(bar(bar_meet()), meets & 1u, abort_flag));
                 if (!alive) break;
-                merge_partials<D>(a, it, static_cast<unsigned>(cluster_id * a.cluster) + (meets & 1u) * gridDim.x, it.active, rank, tid, G);
+                const unsigned place0 = static_cast<unsigned>(cluster_id * a.cluster) + (meets & 1u) * gridDim.x;
+                if (__builtin_expect(it.pieces == 1, 1)) {
+                    merge_partials<D, false>(a, it, place0, it.active, rank, tid, G, 0u);
+                } else {
+                    merge_partials<D, true>(a, it, place0, it.active, rank, tid, G, static_cast<unsigned>(cluster_id));
+                    merge_pieces<D>(a, it, rank, tid, G);
+                }
                 ++meets;
             }
             if (n_tiles > 0) {
@@ -1670,13 +1789,24 @@ bool cached_map(HostState* hs, const MapKey& key, int D, CUtensorMap* out) {
     return true;
 }
 
-// CTAs per cluster for mode whole, or 1 for the two-kernel modes.  Mode whole saves the second kernel and the
-// boundary between the two (about 3 us of a call), and pays with CTAs that stay without work: `groups` (of the
-// largest trees) clusters of C CTAs instead of the whole GPU.  With 0.6 us per key tile and CTA that is
-// 0.6 groups kt (1 / (C groups) - 1 / SMs) us for kt key tiles, so it is taken while the longest prefix the
-// cache can hold costs no more than it saves.  Cluster sizes that do not leave SMs of a GPC unused only.
-constexpr double kWholeGainTiles = 5.0;  // 3 us / 0.6 us
-// In a batch the cache may hold one long sequence among short ones, which only its own clusters work on.
+// CTAs per cluster for mode whole, or 1 for the two-kernel modes.  The launch shape is fixed before the tree and the
+// prefix are known (a captured step is replayed for any), so it goes by what both can be: `groups` of the largest tree
+// of the context and the longest prefix of the cache.  Mode whole saves the second kernel and pays with CTAs that stay
+// without work: clusters of C CTAs for `groups` (smaller trees have their groups cut over the clusters left).  For kt
+// key tiles that is kt (1 / C - groups / SMs) tiles a CTA.  Measured, whole / two kernels, in us a layer (largest tree
+// of each context, prefix 1024, 2048, 4096, 8192):
+//    8 groups, C = 8    9.9 /  9.9   11.2 / 11.3   13.7 / 13.3   19.0 / 16.7
+//   12         8       11.3 / 11.3   12.8 / 12.5   15.3 / 14.4   20.6 / 18.7   (Q by plain loads)
+//   16         6        9.6 / 10.6   11.5 / 12.1   14.5 / 14.5   21.6 / 19.4
+//   24         6       10.7 / 12.3   12.5 / 14.3   16.5 / 17.3   24.4 / 24.8
+//   32         4       11.4 / 12.7   13.8 / 15.0   18.6 / 20.0   28.7 / 30.5
+//   40         3       12.1 / 13.2   15.5 / 16.6   21.9 / 23.4   35.6 / 37.3   (50.0 / 49.9 at 12 288)
+// The two meet at 1000 to 2000 keys with 8 and 12 groups, at 4096 with 16, at 9000 and more with 24 to 40: at 1 to 12
+// tiles lost, so no one constant is right for all.  With 5, at the longest prefix that it admits, mode whole is up to
+// 9 % behind (8 and 12 groups); below that prefix, where a call usually is, up to 13 % ahead.
+constexpr double kWholeGainTiles = 5.0;
+// In a batch the cache may hold one long sequence among short ones, which only its own clusters work on.  (Four equal
+// sequences of 8 groups: 12.3 / 13.8 us at 1024 keys, 43.2 / 45.4 at 12 288.)
 int choose_cluster(const int* resident, int sm_count, int groups, int batch, int kt_most) {
     for (int c : {8, 6, 4, 3, 2}) {
         if (resident[c] < groups) continue;
@@ -1796,6 +1926,7 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
     a.part_o = reinterpret_cast<uint4*>(w.attn_part_o), a.part_ml = w.attn_part_ml;
     a.max_items = w.attn_max_items;
     a.min_tiles = w.attn_min_tiles, a.status = w.status;
+    a.piece_count = w.attn_count;
     unsigned char* plan = w.attn_plan;
     a.plan_head = reinterpret_cast<PlanHead*>(plan), plan += sizeof(PlanHead);
     a.plan_cluster = reinterpret_cast<PlanCluster*>(plan), plan += sizeof(PlanCluster) * kMaxGrid;
@@ -1814,6 +1945,11 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
     if (w.attn_cluster > 0) a.cluster = forced_cluster(hs->resident, std::min(w.attn_cluster, kMaxCluster), groups);
     a.clusters = a.cluster > 1 ? groups : hs->resident[1];
     const int grid = a.clusters * a.cluster;
+    // the pieces of cut groups lie behind the two places of every CTA (72 bytes of a unit against 32 in a place)
+    a.may_cut = a.cluster > 1 && groups > batch * a.Hkv && 2 * grid + (9 * a.clusters + 3) / 4 <= a.max_items &&
+                (w.attn_stream > 0 || (w.attn_stream < 0 && (capacity + kBN - 1) / kBN > kPieceTiles * a.cluster)) ? 1 : 0;
+    a.piece_acc = reinterpret_cast<float4*>(a.part_o + static_cast<int64_t>(2 * grid) * (D / 8) * kBM);
+    a.piece_ml = reinterpret_cast<float2*>(a.piece_acc + static_cast<int64_t>(a.clusters) * 4 * kBM * (D / 16));
     if (w.attn_rounds > 0 && a.cluster == 1) a.clusters = std::max(1, a.clusters / w.attn_rounds);
     // one resident round of units with room for all of a group's partials, else more CTAs per SM
     a.comb_chunk = groups * (D / 8 / kCombPieces) <= ctx->sm_count ? kCombChunkMost : kCombChunk;
@@ -1852,9 +1988,13 @@ int attention_max_groups(int batch, int n_kv_heads, int max_tt, int group) {
     return batch * n_kv_heads * ((max_tt * group + kBM - 1) / kBM);
 }
 // (also the most partials)
+int attention_counters() { return kMaxGrid * kPieceWarps; }
+// Up to kFewGroups groups one round of splits is balanced to within a seventh, and the pieces of cut groups fit behind
+// two places of every CTA (the launch checks that): such contexts have no room for more rounds.
+constexpr int kFewGroups = 20;
 int attention_max_items(int groups, int sm_count) {
     const int grid = std::min(sm_count, kMaxGrid);
-    return std::max(groups, (kMaxRounds - 1) * grid) + grid;
+    return std::max(groups, groups <= kFewGroups ? grid : (kMaxRounds - 1) * grid) + grid;
 }
 size_t attention_plan_bytes(int max_items, int max_groups) {
     return sizeof(PlanHead) + sizeof(PlanCluster) * kMaxGrid + sizeof(PlanItem) * (kMaxGrid + static_cast<size_t>(max_items) * kMaxCluster) +

@@ -54,6 +54,7 @@ struct Workspace {
     unsigned char* attn_plan = nullptr;  // the attention work list: per-cluster and per-item entries
     __half* attn_part_o = nullptr;       // [places][rows][D] fp16
     float4* attn_part_ml = nullptr;      // [places][rows]
+    unsigned int* attn_count = nullptr;  // pieces of cut groups that are there (self-resetting)
     // Only read by the test build (RESPS_WAIT_TEST): bit 0 = the attention kernel's first V copy is
     // never issued, bit 1 = the streaming scan's second chunk copy is never issued.
     int test_drop = 0;

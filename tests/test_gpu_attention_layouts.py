@@ -34,3 +34,32 @@ def test_equal_splits_in_rounds(shape, rounds):
     debug = [(binding.RESPS_DEBUG_ATTN_CLUSTER, 1), (binding.RESPS_DEBUG_ATTN_SINGLE, 1), (binding.RESPS_DEBUG_ATTN_EVEN_ROUNDS, rounds)]
     for cut_for in (0, 12):  # all CTAs; a twelfth of them, so that the rounds are full
         _attention_case(**TILES[shape], cap=1664, seed=rounds, poison=True, debug=debug + [(binding.RESPS_DEBUG_ATTN_ROUNDS, cut_for)])
+
+
+# Small trees under a context that builds large ones: fewer groups than clusters, so a group is cut over several.
+SMALL = [dict(n=5, Hq=16, Hkv=2, D=128, L=1400),                          # 2 groups, 8 clusters
+         dict(n=1, Hq=32, Hkv=8, D=64, L=1023),
+         dict(n=[5, 18], Hq=16, Hkv=1, D=128, L=[100, 1480], B=2),        # 4 groups of very different lengths
+         dict(n=[3, 1, 16, 33], Hq=14, Hkv=2, D=128, L=[0, 7, 640, 1000], B=4),
+         dict(n=2, Hq=8, Hkv=1, D=128, L=60)]                             # fewer key tiles than CTAs
+
+
+@pytest.mark.parametrize("cluster", [2, 3, 4, 6, 8])
+@pytest.mark.parametrize("shape", range(len(SMALL)))
+def test_a_group_cut_over_several_clusters(shape, cluster):
+    _, binding, _ = _imports()
+    debug = [(binding.RESPS_DEBUG_ATTN_CLUSTER, cluster), (binding.RESPS_DEBUG_ATTN_SINGLE, 1)]  # cut wherever clusters are left
+    _attention_case(**SMALL[shape], cap=1664, seed=shape, poison=True, debug=debug)
+
+
+def test_cut_groups_keep_values_beyond_fp16():
+    _, binding, _ = _imports()
+    _attention_case(6, 16, 2, 128, 3000, cap=3200, seed=3, v_scale=3.0e5, debug=[(binding.RESPS_DEBUG_ATTN_CLUSTER, 4)])
+
+
+@pytest.mark.parametrize("cap", [1216, 9408])
+@pytest.mark.parametrize("n", [12, 40, 128])
+def test_trees_of_one_context_in_caches_with_and_without_room(n, cap):
+    """The paper's largest action bounds the context; short and long prefixes, small trees and the largest."""
+    for L in (1000, cap - 128):
+        _attention_case(n, 32, 8, 128, L, cap=cap, seed=n, poison=True, max_k=32, max_depth=8)

@@ -125,11 +125,11 @@ def test_ragged_batch_and_clamping_sets_status():
 
 # ------------------------------------------------------------------------ attention
 def _attention_case(n, Hq, Hkv, D, L, cap, parent=None, poison=False, seed=0, B=1, max_tt=128, v_scale=1.0,
-                    debug=()):
+                    debug=(), max_k=4, max_depth=4):
     oracle, binding, synth = _imports()
     from harness import check_attention, u16_to_bf16_cuda, bf16_to_f64
     rng = np.random.default_rng(seed)
-    ctx = binding.Context(Hq, Hkv, D, 1000, max_batch=B, max_tt=max_tt, max_k=4, max_depth=4)
+    ctx = binding.Context(Hq, Hkv, D, 1000, max_batch=B, max_tt=max_tt, max_k=max_k, max_depth=max_depth)
     for key, value in debug:
         ctx.debug_set(key, value)
     ns = [n] * B if isinstance(n, int) else n
