@@ -53,7 +53,6 @@ struct SampledArgs {
     int64_t dld_b, dld_level, dld_row;
     const int32_t* node_row;  // [batch][max_tt]: level * RESPS_MAX_K + slot of the row a node's children came from
     double inv_t;             // 1 / temperature
-    double temperature;
     const int32_t *tokens, *parent;
     const double *u_accept, *u_sample;
     int vocab, max_tt, max_depth, max_k;
@@ -464,7 +463,7 @@ cudaError_t launch_accept_sampled(const resps_ctx* ctx, const resps_step* d_step
     a.target = target, a.ld_b = ld_b, a.ld_row = ld_row;
     a.draft = draft, a.dld_b = dld_b, a.dld_level = dld_level, a.dld_row = dld_row;
     a.node_row = ctx->ws.node_row;
-    a.temperature = temperature, a.inv_t = 1.0 / temperature;
+    a.inv_t = 1.0 / temperature;
     a.tokens = tokens, a.parent = parent, a.u_accept = u_accept, a.u_sample = u_sample;
     a.vocab = ctx->shape.vocab, a.max_tt = ctx->shape.max_tt, a.max_depth = ctx->shape.max_depth;
     a.max_k = ctx->shape.max_k;

@@ -83,7 +83,7 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
 // Keys are (ordered value, ~id) pairs, unique, so that "larger key" is exactly the method's order
 // (value descending, token id ascending).  The log-sum-exp partial is a per-thread
 // (max, sum 2^(y - max)) reduced over the CTA.
-template <bool VEC>
+// (For rows that the streaming kernel below cannot take: not 16-byte aligned, or of a length that is no multiple of 4.)
 __global__ void __launch_bounds__(kScanThreads, 4) row_scan_kernel(const ScanArgs a) {
     pdl_wait();  // the kernel before this one in the stream has completed
     pdl_launch_dependents();
@@ -108,22 +108,15 @@ __global__ void __launch_bounds__(kScanThreads, 4) row_scan_kernel(const ScanArg
     const int begin = sp * a.chunk;
     const int end = min(a.vocab, begin + a.chunk);
 
-    // ---- the chunk into registers: 8 independent 128-bit loads per thread ------------------
+    // ---- the chunk into registers: 32 independent loads per thread --------------------------
     float v[kScanPerThread];
 #pragma unroll
     for (int u = 0; u < kScanPerThread / 4; ++u) {
         const int e0 = begin + (u * kScanThreads + tid) * 4;
         v[4 * u] = v[4 * u + 1] = v[4 * u + 2] = v[4 * u + 3] = -INFINITY;
-        if (VEC) {
-            if (e0 < end) {  // vocab and chunk are multiples of 4 on this path
-                const float4 x = __ldcs(reinterpret_cast<const float4*>(row + e0));
-                v[4 * u] = x.x, v[4 * u + 1] = x.y, v[4 * u + 2] = x.z, v[4 * u + 3] = x.w;
-            }
-        } else {
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
-                if (e0 + c < end) v[4 * u + c] = __ldcs(row + e0 + c);
-        }
+        for (int c = 0; c < 4; ++c)
+            if (e0 + c < end) v[4 * u + c] = __ldcs(row + e0 + c);
     }
     if (tid == 0) s_count = 0;
     // position i of a thread is logit begin + ((i / 4) * 256 + tid) * 4 + i % 4: ids ascend with i
@@ -1064,9 +1057,9 @@ cudaError_t launch_row_scan(const resps_ctx* ctx, const resps_step* d_steps, int
     const int most_slices = max(1, min(w.scan_slices_hint > 0 ? w.scan_slices_hint : a.splits, kStreamList / a.max_k - 2));
     a.least = (a.splits + most_slices - 1) / most_slices;
     a.test_drop = w.test_drop;
-    if (!(vec_ok(logits, ld_b, ld_level, ld_row, a.vocab, a.chunk) && w.scan_chunk == kScanChunkMax)) {
+    if (!vec_ok(logits, ld_b, ld_level, ld_row, a.vocab, a.chunk)) {
         const size_t smem = sizeof(unsigned long long) * ctx->shape.max_k * max(kQuadElems, w.scan_splits);
-        return launch_pdl(row_scan_kernel<false>, dim3(w.scan_splits, rows, batch), dim3(kScanThreads), smem, st, a);
+        return launch_pdl(row_scan_kernel, dim3(w.scan_splits, rows, batch), dim3(kScanThreads), smem, st, a);
     }
     for (int b0 = 0; b0 < batch; b0 += kStreamMaxBatch) {
         a.batch = min(kStreamMaxBatch, batch - b0);
@@ -1098,7 +1091,7 @@ cudaError_t launch_row_argmax(const resps_ctx* ctx, const int32_t* d_n_nodes, in
     a.key_out = key_out;
     a.status = w.status;
     if (walked) *walked = false;
-    if (vec_ok(logits, ld_b, ld_row, 0, a.vocab, a.chunk) && w.scan_chunk == kScanChunkMax) {
+    if (vec_ok(logits, ld_b, ld_row, 0, a.vocab, a.chunk)) {
         // Slices per row as in the scan: a row is cut only as far as all CTAs still run at once.
         const int want = max(1, 2 * ctx->sm_count / max(ctx->shape.max_tt * batch, 1));
         const int slices0 = max(1, min(w.scan_splits, want));
@@ -1110,12 +1103,7 @@ cudaError_t launch_row_argmax(const resps_ctx* ctx, const int32_t* d_n_nodes, in
         dim3 grid(a.slices, ctx->shape.max_tt, batch);
         return launch_pdl(row_argmax_stream_kernel, grid, dim3(kStreamThreads), kStreamSmem, st, a, wa, walk ? 1 : 0);
     }
-    dim3 grid(w.scan_splits, ctx->shape.max_tt, batch);
-    if (vec_ok(logits, ld_b, ld_row, 0, a.vocab, a.chunk))
-        return launch_pdl(row_argmax_kernel<true>, grid, dim3(kScanThreads), 0, st, a);
-    else
-        return launch_pdl(row_argmax_kernel<false>, grid, dim3(kScanThreads), 0, st, a);
-    return cudaGetLastError();
+    return launch_pdl(row_argmax_kernel<false>, dim3(w.scan_splits, ctx->shape.max_tt, batch), dim3(kScanThreads), 0, st, a);
 }
 
 cudaError_t launch_shard_merge_rows(const resps_ctx* ctx, const resps_step* d_steps, int batch, int n_levels, int n_slots,
