@@ -35,6 +35,7 @@
 #include <cmath>
 
 #include "common.cuh"
+#include "exp_le0.cuh"
 
 namespace resps {
 namespace {
@@ -66,28 +67,6 @@ struct SampledArgs {
 struct Pair {
     double x, y;
 };
-
-// e^t for t <= 0 (below -700: 0), to about one unit in the last place: table-driven (P. Tang, "Table-driven
-// implementation of the exponential function in IEEE floating-point arithmetic", 1989).  t = k ln2/64 + r,
-// |r| <= ln2/128, e^t = 2^(k/64) e^r with 2^(i/64) from a table in shared memory and five terms of the series
-// for e^r - 1 (the next one is below 4e-17).  11 fp64 operations, half of what exp() takes for its full range.
-constexpr int kExpTable = 64;
-__device__ __forceinline__ double exp_le0(double t, const double* table) {
-    constexpr double kMagic = 6755399441055744.0;  // 1.5 * 2^52: the sum's low word is the rounded integer
-    const double biased = fma(t, 92.33248261689366, kMagic);  // 64 / ln 2
-    const int k = __double2loint(biased);
-    const double kd = biased - kMagic;
-    double r = fma(kd, -0.010830424696249145, t);  // ln 2 / 64, rounded,
-    r = fma(kd, -3.623510646634843e-19, r);        // and the rest of it
-    double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
-    q = fma(q, r, 1.0 / 6.0);
-    q = fma(q, r, 0.5);
-    q = fma(q, r, 1.0) * r;
-    const double head = table[k & (kExpTable - 1)];
-    const double y = fma(head, q, head);  // about 2^(k/64 mod 1) e^r: 2^(k >> 6) goes into its exponent
-    const double v = __hiloint2double(__double2hiint(y) + ((k >> 6) << 20), __double2loint(y));
-    return t > -700.0 ? v : 0.0;
-}
 
 // What the stored target-side value of a token still lacks: the division by the softmax sum, or one
 // rejection round (Section 3.2, "Acceptance Criterion": target side -> normalised max(0, p - q)).  The
