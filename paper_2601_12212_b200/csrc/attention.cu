@@ -966,8 +966,9 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
     // The work list was written once for the whole step.  From the second layer on it is at least
     // two kernels old: this kernel can only have started after its predecessor had started, which
     // can only have started after every CTA of the kernel before that one had passed its own
-    // dependency wait, i.e. after the kernel that wrote the list had completed and flushed.  (Every
-    // kernel of the library signals its dependents only after its own wait, or never.)  So the
+    // dependency wait, i.e. after the kernel that wrote the list had completed and flushed.  (That kernel before
+    // is an attention kernel, or comes behind one: the first call's follows the list's writer at once and signals
+    // its dependents only after its own wait.  The combine kernel signals before its wait.)  So the
     // list is read before the wait, under the tail of the preceding kernel; only when the list was
     // written by the kernel immediately before this one does the read have to follow the wait.
     // Every thread reads the CTA's first item for itself: no role waits for another.

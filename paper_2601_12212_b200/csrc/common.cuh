@@ -276,7 +276,6 @@ __device__ __forceinline__ void accept_walk_device(const AcceptArgs& a, int b, i
     }
 }
 
-// Step parameters clamped into the extents the caller supplied.
 // Thread-block clusters: this CTA's rank, the barrier over all threads, a peer's copy of a shared variable.
 __device__ __forceinline__ unsigned cluster_rank() {
     unsigned r;
@@ -297,6 +296,7 @@ __device__ __forceinline__ uint32_t peer_address(const void* local, unsigned pee
     return remote;
 }
 
+// Step parameters clamped into the extents the caller supplied.
 struct StepDims {
     int tt, d, k, L;
     bool clamped;

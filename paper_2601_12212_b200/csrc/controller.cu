@@ -16,7 +16,8 @@
 // Bound by the first layer's weights through L2 into 16 SMs per sequence (0.4 MB each, about 3 us), around it
 // a chain of three exchanges; a step whose cached action is still valid is bound by its launch.  With a CTA
 // per hidden unit and the last one to arrive running both small layers and, by one thread, the softmax, a step
-// that asks took 40 us at 8 sequences of the 3 x 4096 state and 180 actions (now 15), one that does not the same 2.2.
+// that asks took 40 us at 8 sequences of the 3 x 4096 state and 180 actions (now 18.4, and 28.6 with the weights in
+// HBM, as between the questions of a decode loop); one that does not takes 1.8.
 #include <cmath>
 
 #include "common.cuh"

@@ -40,7 +40,11 @@
 namespace resps {
 namespace {
 
-constexpr int kClu = 16;            // CTAs per sequence (more than 8: not portable, sm_100 has it)
+// CTAs per sequence (more than 8: not portable, sm_100 has it).  Seven clusters of 16 are resident, so a batch of 8
+// takes two turns; the clusters of 8 CTAs before were 15.  In us a call, single calls behind an L2 flush, before / now, at
+// V = 128256, TT=60 d=7 k=10: 1 sequence 139 / 56, 7 175 / 69, 8 184 / 78, 12 179 / 106, 15 201 / 130, 16 214 / 133,
+// 24 266 / 180, 32 352 / 227; at V = 32000: 1 86 / 40, 8 99 / 60, 15 113 / 83, 32 195 / 156.  No batch is slower.
+constexpr int kClu = 16;
 constexpr int kSampThreads = 512;
 constexpr int kWarps = kSampThreads / 32;
 constexpr unsigned kFull = 0xFFFFFFFFu;

@@ -1,12 +1,13 @@
 // Vocabulary scans: fused top-k + log-sum-exp over draft rows (tree expansion,
 // Section 3.2 "Draft Tree Expansion") and arg-max over target rows (greedy
-// verification, Section 3.1).  Both are single-pass, HBM-bound streaming
-// kernels: every logit is read exactly once with 128-bit coalesced loads.
+// verification, Section 3.1), bound by HBM where there are many rows.
 //
-// A row is cut into `splits` chunks, one CTA each.  A CTA reduces its chunk to a
-// partial result in the context workspace; the last CTA of a row to arrive
-// (atomic arrival counter, self-resetting) merges the partials and writes the
-// row's final result, so no second launch is needed.
+// 16-byte aligned rows go through the streaming kernels: bulk copies of 8192-logit chunks through a ring
+// of stages.  The scan cuts the chunks of all rows into equal ranges, one per CTA, reads every logit once from
+// HBM and the chunks that can hold one of a slice's k best a second time (from the stages, or L2); the arg-max
+// reads every logit once.  Other rows are cut into chunks of 8192 logits, one CTA each, which is read by plain
+// loads.  In both, a CTA leaves partial results in the context workspace, and the last CTA of a row (arg-max:
+// of a sequence) to arrive (atomic arrival counter, self-resetting) merges them, so no second launch is needed.
 #include <cmath>
 #include <mutex>
 
