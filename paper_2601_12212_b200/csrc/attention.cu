@@ -67,6 +67,9 @@ constexpr int kSnap = 4;           // mode stream: a cut this close to a group's
 constexpr int kItemTiles = 4;      // what an item costs a CTA besides its tiles (its start and epilogue), in key tiles
 constexpr int kMaxRounds = 4;      // mode even: most rounds of splits
 constexpr int kPieceTiles = 5;     // mode whole: a group is cut where that takes more than this many key tiles off a CTA
+// Two and more rounds are looked at from this many key tiles a CTA on, about 15 us a layer: below that they gain under
+// 3 us a layer, and looking at them takes a step 3 us.
+constexpr int kLongTiles = 24;
 constexpr int kRereadNum = 5, kRereadDen = 4;
 constexpr int kCutTiles = 6;       // what cut groups cost a call (partials, the combine kernel's round trips)
 constexpr int kTmemCols = 512;
@@ -74,7 +77,7 @@ constexpr uint32_t kWaitLimitCycles = kWaitTest ? 2000000u : 0x70000000u;  // bo
 constexpr float kRescaleSlack = 8.0f;  // O is rescaled only when the running max grows by > 2^8
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
-// How a layer's work is laid out, one of three ways (PlanHead::mode):
+// How a layer's work is laid out, one of three ways:
 //  whole   clusters of several CTAs, one group (sequence, KV head, row tile) per cluster.  The CTAs share
 //          the group's key tiles, leave normalised partial results in the workspace (L2), meet on an
 //          mbarrier and merge a share of the rows x columns each: one kernel does the layer.  Where the tree at
@@ -89,24 +92,25 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 //          groups.
 // Of even (each number of rounds) and stream the one with the smallest largest share is taken (tiles, items, cut
 // groups).  In mode even the row tiles of a KV head go through the same keys at the same time, in mode stream at
-// different times: where K and V do not stay in L2 meanwhile, every row tile reads them from HBM again.  Measured per
-// unit of the largest share, several row tiles per head: K and V of a call up to 67 MB 0.75-0.80 us in all modes; from
-// 131 MB on even 0.65-0.78, stream 0.88-0.95.  So the share of mode stream counts kRereadNum / kRereadDen times as much
-// beyond `l2_tiles` key tiles (all KV heads of the sequences with several row tiles).  In us a call, stream against
-// the best of even: 8 x 24 000 keys, 80 nodes, 8B shape 464 / 408; 5 x 28 000 keys, 40-96 nodes, 56 query heads
-// 528 / 459; 4 x 8192 keys, 96 nodes, 70B shape 162 / 151; 16 x 4096 keys, 64 nodes, 8B shape 120 / 112; 12 ragged
-// sequences up to 16 000 keys, 28 query heads 126 / 107; one round against two: 32 000 keys, 128 nodes, 8B shape 108 / 98.
+// different times: where K and V do not stay in L2 meanwhile, every row tile reads them from HBM again, and 148 CTAs
+// with 32 KB per 0.62 us ask for more than HBM has.  So the share of mode stream counts kRereadNum / kRereadDen times as
+// much beyond `l2_tiles` key tiles (all KV heads of the sequences with several row tiles; head dimension 128).  In us a
+// call, stream against the best of even: 8 x 24 000 keys, 80 nodes, 8B shape 445 / 378 (four rounds); 5 x 28 000 keys, 40-96
+// nodes, 56 query heads 504 / 423 (four); 4 x 8192 keys, 96 nodes, 70B shape 151 / 138 (four); 16 x 4096 keys, 64 nodes, 8B
+// shape 112 / 102 (two); 32 000 keys, 128 nodes 97 / 92 (two; one round 102); 12 ragged sequences up to 16 000 keys, 28 query
+// heads 127 / 109 (three).  With K and V of up to 67 MB the modes are within 3 %: 8192 keys, 128 nodes 31.2 / 29.9, 8 x 2048
+// keys, 64 nodes 29.6 / 29.7.
 constexpr int kModeWhole = 0, kModeEven = 1, kModeStream = 2;
 
-struct PlanHead {
+struct alignas(16) PlanHead {
     int n_groups, pad[3];
 };
 // A cluster's (or CTA's) first item and its number of items.
-struct PlanCluster {
+struct alignas(8) PlanCluster {
     int first_item, n_items;
 };
 // For every item and CTA of the cluster everything the CTA needs to start.
-struct PlanItem {
+struct alignas(16) PlanItem {
     int b_g;             // sequence | KV head << 16
     int tile_active;     // row tile of the KV head | CTAs that have key tiles of the item << 16
     int t_begin, t_end;  // this CTA's key tiles (none: t_begin == t_end)
@@ -115,7 +119,7 @@ struct PlanItem {
     int place;           // where its partial goes (mode whole: the group's first cluster)
 };
 // For the combine kernel: the partials of a group are in consecutive places.
-struct PlanGroup {
+struct alignas(16) PlanGroup {
     int b_g, tile, n, first_place, pieces, pad[3];
 };
 static_assert(sizeof(PlanHead) == 16 && sizeof(PlanCluster) == 8 && sizeof(PlanItem) == 32 && sizeof(PlanGroup) == 32, "vector loads");
@@ -143,6 +147,7 @@ struct AttnArgs {
     int comb_chunk;   // partials the combine kernel fetches together
     int stream_gain;  // -1: own choice; 0: never mode even; else always where it fits (tests)
     int may_cut;      // mode whole: a group may be cut over several clusters
+    int most_rounds;  // mode even: rounds that are looked at
     int rounds;       // mode even: 0: own choice; else this many rounds (tests)
     int l2_tiles;     // K and V of more key tiles (of a KV head) than this do not stay in L2
     int min_tiles;    // fewest key tiles a CTA is given
@@ -156,8 +161,8 @@ struct AttnArgs {
     // The work list, written by attention_plan_kernel.
     PlanHead* plan_head;
     PlanCluster* plan_cluster;  // [kMaxGrid]
-    PlanItem* plan_first;       // [kMaxGrid] every CTA's first item once more (one load instead of two in a row)
-    PlanItem* plan_item;        // [max_items x cluster]
+    PlanItem* plan_first;       // [kMaxGrid] every CTA's first item (one load instead of two in a row)
+    PlanItem* plan_item;        // [max_items x cluster] the others
     PlanGroup* plan_group;      // [groups]
 };
 
@@ -186,7 +191,8 @@ struct PlanShared {
     int splits[kMaxRounds][kMaxBatch];        // items a group is cut into
     unsigned long long cut[2][kMaxGrid + 1];
     int n_items[kMaxGrid];
-    int even_cost[kMaxRounds], even_share[kMaxRounds], range_cost[2];  // largest share of a CTA: mode even; ranges of whole groups, equal ranges
+    int even_share[kMaxRounds], even_cost[kMaxRounds];  // mode even: largest share of a CTA, and what comes on top
+    int range_cost[2];                         // largest share of a CTA: ranges of whole groups, equal ranges
     int cut_groups;                            // mode whole: groups are cut over several clusters
     int reread;                                // K and V are read again by every row tile in mode stream
 };
@@ -210,7 +216,8 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
         sh.kt[tid] = (n > 0) ? ceil_div(L + n, kBN) : 0;
     }
     __syncthreads();
-    if (tid < 32) {
+    if (tid < 32 * kMaxRounds) {  // (each of these warps scans for itself, the first one keeps what it finds)
+        const int w = tid >> 5;
         unsigned long long pos = 0;
         int group = 0;
 #pragma unroll 1
@@ -223,24 +230,24 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
 #pragma unroll 1
             for (int d = 1; d < reach; d <<= 1) {
                 const int g = __shfl_up_sync(kFull, groups, d);
-                const unsigned long long w = __shfl_up_sync(kFull, work, d);
-                if (lane >= d) groups += g, work += w;
+                const unsigned long long before = __shfl_up_sync(kFull, work, d);
+                if (lane >= d) groups += g, work += before;
             }
-            if (b < a.batch) {
+            if (w == 0 && b < a.batch) {
                 sh.start[b] = pos + work - own_work, sh.group0[b] = group + groups - own_groups;
                 sh.cost0[b] = sh.start[b] + static_cast<unsigned long long>(sh.group0[b]) * kItemTiles;
             }
             pos += __shfl_sync(kFull, work, min(31, a.batch - b0 - 1));
             group += __shfl_sync(kFull, groups, min(31, a.batch - b0 - 1));
         }
-        if (lane == 0) {
+        if (tid == 0) {
             sh.start[a.batch] = pos, sh.group0[a.batch] = group;
             sh.cost0[a.batch] = pos + static_cast<unsigned long long>(group) * kItemTiles;
         }
         // ---- mode whole: the clusters that the groups leave are given to them by their key tiles; a group stays whole
         // where a piece saves a CTA too little ------------------------------------------------------------------------
         bool cut = false;
-        if (a.may_cut && group < a.clusters) {
+        if (w == 0 && a.may_cut && group < a.clusters) {
             const int gain = a.stream_gain > 0 ? 0 : kPieceTiles * a.cluster, spare = a.clusters - group;
             int base = 0;
 #pragma unroll 1
@@ -266,60 +273,65 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
             cut = __any_sync(kFull, cut);
             if (lane == 0) sh.item0[0][a.batch] = base;
         }
-        if (lane == 0) {
+        if (tid == 0) {
             sh.cut_groups = cut;
             sh.range_cost[0] = sh.range_cost[1] = 0;
             PlanHead h = {};
             h.n_groups = group;
             *a.plan_head = h;
         }
+        if (a.cluster == 1) {
+            // ---- mode even: the smallest T (in steps of T/16) for which the splits fit the rounds ----------------------
+            const int rounds = w + 1, room = rounds * a.clusters;
+            const bool is_long = pos >= static_cast<unsigned long long>(kLongTiles) * a.clusters;
+            const bool looked_at = a.stream_gain != 0 &&
+                (a.rounds > 0 ? a.rounds == rounds : rounds == 1 || (rounds <= a.most_rounds && is_long));
+            int T = max(static_cast<int>(min((pos + room - 1) / room, 1ull << 24)), 1);
+            bool fits = false;
+#pragma unroll 1
+            for (int tries = 0; tries < 40 && looked_at && !fits; ++tries) {
+                unsigned count = 0;
+#pragma unroll 1
+                for (int b = lane; b < a.batch; b += 32)
+                    count += static_cast<unsigned>(a.Hkv * sh.tiles[b] * ceil_div(sh.kt[b], max(T, a.min_tiles)));
+                count = __reduce_add_sync(kFull, min(count, 1u << 20));
+                fits = count <= static_cast<unsigned>(room);
+                if (!fits) T += max(1, T >> 4);
+            }
+            T = max(T, a.min_tiles);
+            int base = 0, tiles = 0, most = 0;
+            bool split = false;
+#pragma unroll 1
+            for (int b0 = 0; b0 < a.batch && (fits || w == 0); b0 += 32) {
+                const int b = b0 + lane, splits = (b < a.batch) ? ceil_div(sh.kt[b], T) : 0;
+                int incl = (b < a.batch && fits) ? a.Hkv * sh.tiles[b] * splits : 0;
+                split = split || splits > 1;
+                most = max(most, splits > 0 ? ceil_div(sh.kt[b], splits) + kItemTiles : 0);
+                if (b < a.batch && sh.tiles[b] > 1) tiles += min(a.Hkv * sh.kt[b], 1 << 22);
+                const int own = incl;
+#pragma unroll 1
+                for (int d = 1; d < reach; d <<= 1) {
+                    const int v = __shfl_up_sync(kFull, incl, d);
+                    if (lane >= d) incl += v;
+                }
+                if (b < a.batch) sh.splits[w][b] = splits, sh.item0[w][b] = base + incl - own;
+                base += __shfl_sync(kFull, incl, min(31, a.batch - b0 - 1));
+            }
+            tiles = __reduce_add_sync(kFull, min(tiles, 1 << 25));
+            most = __reduce_max_sync(kFull, most);
+            split = __any_sync(kFull, split);
+            if (lane == 0) {
+                sh.item0[w][a.batch] = base;
+                const bool allowed = fits && base <= a.max_items;
+                // (one item, or items of one sequence, the same to a tile; else the CTAs' sums are looked at below)
+                sh.even_share[w] = (a.batch == 1 || rounds == 1) ? ceil_div(base, a.clusters) * most : 0;
+                sh.even_cost[w] = !allowed ? 1 << 30 : (split ? kCutTiles : 0) - (a.stream_gain > 0 ? 1 << 28 : 0);  // besides the share
+                if (w == 0) sh.reread = tiles > a.l2_tiles;
+            }
+        }
     }
     __syncthreads();
     const int n_groups = sh.group0[a.batch];
-    if (a.cluster == 1 && tid < 32 * kMaxRounds) {
-        // ---- mode even: the smallest T (in steps of T/16) for which the splits fit the rounds ----------------------
-        const int w = tid >> 5, rounds = w + 1, room = rounds * a.clusters;
-        const unsigned long long work = sh.start[a.batch];
-        int T = max(static_cast<int>(min((work + room - 1) / room, 1ull << 24)), 1);
-        bool fits = false;
-#pragma unroll 1
-        for (int tries = 0; tries < 40 && !fits; ++tries) {
-            unsigned count = 0;
-#pragma unroll 1
-            for (int b = lane; b < a.batch; b += 32)
-                count += static_cast<unsigned>(a.Hkv * sh.tiles[b] * ceil_div(sh.kt[b], max(T, a.min_tiles)));
-            count = __reduce_add_sync(kFull, min(count, 1u << 20));
-            fits = count <= static_cast<unsigned>(room);
-            if (!fits) T += max(1, T >> 4);
-        }
-        T = max(T, a.min_tiles);
-        int base = 0, tiles = 0;
-        bool cut = false;
-#pragma unroll 1
-        for (int b0 = 0; b0 < a.batch; b0 += 32) {
-            const int b = b0 + lane, splits = (b < a.batch) ? ceil_div(sh.kt[b], T) : 0;
-            int incl = (b < a.batch && fits) ? a.Hkv * sh.tiles[b] * splits : 0;
-            cut = cut || splits > 1;
-            if (b < a.batch && sh.tiles[b] > 1) tiles += min(a.Hkv * sh.kt[b], 1 << 22);
-            const int own = incl;
-#pragma unroll 1
-            for (int d = 1; d < reach; d <<= 1) {
-                const int v = __shfl_up_sync(kFull, incl, d);
-                if (lane >= d) incl += v;
-            }
-            if (b < a.batch) sh.splits[w][b] = splits, sh.item0[w][b] = base + incl - own;
-            base += __shfl_sync(kFull, incl, min(31, a.batch - b0 - 1));
-        }
-        tiles = __reduce_add_sync(kFull, min(tiles, 1 << 25));
-        cut = __any_sync(kFull, cut);
-        if (lane == 0) {
-            sh.item0[w][a.batch] = base;
-            const bool allowed = fits && base <= a.max_items && a.stream_gain != 0 && (a.rounds == 0 || a.rounds == rounds);
-            sh.even_share[w] = 0;
-            sh.even_cost[w] = !allowed ? 1 << 30 : (cut ? kCutTiles : 0) - (a.stream_gain > 0 ? 1 << 28 : 0);  // besides the share
-            if (w == 0) sh.reread = tiles > a.l2_tiles;
-        }
-    }
     auto last_at_or_before = [&](const int* first, int x) {  // the last sequence whose entry is <= x
         int lo = 0, hi = a.batch;
 #pragma unroll 1
@@ -385,16 +397,15 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
                 const int items = sh.group0[b1] + local1 - sh.group0[b] - local + 1;
                 atomicMax(&sh.range_cost[w], static_cast<int>(end - begin) + items * kItemTiles + (w ? kCutTiles : 0));
             }
-            // (sequences of different lengths give items of different lengths: a CTA's real sum counts.  One sequence's
-            // are the same to a tile.)
+            // (sequences of different lengths give items of different lengths: a CTA's real sum counts)
 #pragma unroll 1
-            for (int w = 0; w < kMaxRounds; ++w) {
+            for (int w = 1; w < kMaxRounds && a.batch > 1; ++w) {
                 if (sh.even_cost[w] == 1 << 30) continue;
                 const int n = sh.item0[w][a.batch];
                 int share = 0;
 #pragma unroll 1
                 for (int item = tid; item < n; item += a.clusters) {
-                    const int b = a.batch > 1 ? last_at_or_before(sh.item0[w], item) : 0;
+                    const int b = last_at_or_before(sh.item0[w], item);
                     share += ceil_div(sh.kt[b], sh.splits[w][b]) + kItemTiles;
                 }
                 atomicMax(&sh.even_share[w], share);
@@ -425,8 +436,7 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
                 PlanItem p = item_of(b, local);
                 p.t_begin = kt * sp / splits, p.t_end = kt * (sp + 1) / splits;  // (kt <= 2^15, splits <= 2^10)
                 p.pieces = splits, p.place = item;
-                if (c.n_items == 0) a.plan_first[tid] = p;
-                a.plan_item[c.first_item + c.n_items] = p;
+                *(c.n_items == 0 ? a.plan_first + tid : a.plan_item + c.first_item + c.n_items) = p;
                 if (sp == 0) write_group(sh.group0[b] + local, p);
             }
             a.plan_cluster[tid] = c;
@@ -451,7 +461,8 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
                 int local = item - first[b], pieces = 1, piece = 0, t0 = 0, kt = sh.kt[b];
                 if (cut && sh.splits[0][b] > 1) {
                     pieces = sh.splits[0][b];
-                    piece = local, local = static_cast<int>(static_cast<unsigned>(local) / static_cast<unsigned>(pieces)), piece -= local * pieces;
+                    piece = local, local = static_cast<int>(static_cast<unsigned>(local) / static_cast<unsigned>(pieces));
+                    piece -= local * pieces;
                     t0 = kt * piece / pieces, kt = kt * (piece + 1) / pieces - t0;
                 }
                 PlanItem p = item_of(b, local);
@@ -463,8 +474,7 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
                 for (int r = 0; r < a.cluster; ++r) {
                     p.t_begin = p.t_end;
                     if (r < act) p.t_end = t0 + kt * (r + 1) / act;
-                    if (i == 0) a.plan_first[tid * a.cluster + r] = p;
-                    a.plan_item[item * a.cluster + r] = p;
+                    *(i == 0 ? a.plan_first + tid * a.cluster + r : a.plan_item + item * a.cluster + r) = p;
                 }
             }
         }
@@ -505,8 +515,7 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
             const int c0 = (g0 >= begin) ? tid : cluster_of(g0), c1 = (g1 <= end) ? tid : cluster_of(g1 - 1);
             PlanItem p = item_of(b, local);
             p.t_begin = t, p.t_end = static_cast<int>(stop - g0), p.pieces = c1 - c0 + 1, p.place = first + i;
-            if (i == 0) a.plan_first[tid] = p;
-            a.plan_item[first + i] = p;
+            *(i == 0 ? a.plan_first + tid : a.plan_item + first + i) = p;
             if (t == 0) write_group(sh.group0[b] + local, p);
             // on to the next group
             pos = stop, t = 0;
@@ -895,7 +904,8 @@ __device__ __forceinline__ void merge_partials(const AttnArgs& a, const Item& it
         } else {
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-                __stcg(a.piece_acc + (cluster_id * 4 + e) * kUnits + u, make_float4(acc[4 * e], acc[4 * e + 1], acc[4 * e + 2], acc[4 * e + 3]));
+                __stcg(a.piece_acc + (cluster_id * 4 + e) * kUnits + u,
+                       make_float4(acc[4 * e], acc[4 * e + 1], acc[4 * e + 2], acc[4 * e + 3]));
             __stcg(a.piece_ml + cluster_id * kUnits + u, make_float2(Mx, den));
         }
     }
@@ -1817,6 +1827,9 @@ int choose_cluster(const int* resident, int sm_count, int groups, int batch, int
     return 1;
 }
 // K and V of this many bytes are taken to stay in L2 between the row tiles of a head (measured between 67 and 131 MB).
+// With a head dimension of 64 it does not matter where they are: 148 CTAs with 16 KB per 0.6 us ask for 3.9 TB/s, below
+// HBM's rate, where 32 KB ask for 7.8.  (16 sequences up to 32 000 keys, 546 MB: ranges 214 us, equal splits in one to
+// four rounds 215, 247, 240, 234; of twelve such shapes two gain 2 to 4 % by rounds, so they are not looked at there.)
 constexpr int64_t kL2Bytes = 96 << 20;
 int forced_cluster(const int* resident, int cluster, int groups) {
     while (cluster > 1 && resident[cluster] < groups) --cluster;
@@ -1955,7 +1968,8 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
     // one resident round of units with room for all of a group's partials, else more CTAs per SM
     a.comb_chunk = groups * (D / 8 / kCombPieces) <= ctx->sm_count ? kCombChunkMost : kCombChunk;
     a.stream_gain = w.attn_stream, a.rounds = w.attn_even_rounds;
-    a.l2_tiles = static_cast<int>(kL2Bytes / (2 * 2 * kBN * D));
+    a.most_rounds = D == 128 ? kMaxRounds : 1;
+    a.l2_tiles = D == 128 ? static_cast<int>(kL2Bytes / (2 * 2 * kBN * D)) : 1 << 30;
     MapKey kk = {k_cache, stride_tok, stride_head, stride_seq, capacity, a.Hkv, batch, 0};
     MapKey kv = kk;
     kv.base = v_cache;
