@@ -63,3 +63,51 @@ def test_trees_of_one_context_in_caches_with_and_without_room(n, cap):
     """The paper's largest action bounds the context; short and long prefixes, small trees and the largest."""
     for L in (1000, cap - 128):
         _attention_case(n, 32, 8, 128, L, cap=cap, seed=n, poison=True, max_k=32, max_depth=8)
+
+
+def test_replayed_for_small_and_large_trees():
+    """One capture of three layers, replayed while the tree shrinks and grows under it: groups are cut, whole and cut
+    again.  (bf16 result of fp32 sums: 2^-9 of the largest output, doubled.)"""
+    import math
+
+    import torch
+    _, binding, _ = _imports()
+    hq, hkv, D, cap, T, NL = 32, 8, 128, 6016, 128, 3
+    ctx = binding.Context(hq, hkv, D, 1000, max_batch=1, max_tt=T, max_k=32, max_depth=8)
+    r = dict(generator=torch.Generator(device="cuda").manual_seed(8), device="cuda", dtype=torch.bfloat16)
+    q, k, v = torch.randn(NL, 1, T, hq, D, **r), torch.randn(NL, 1, hkv, cap, D, **r), torch.randn(NL, 1, hkv, cap, D, **r)
+    o = torch.zeros_like(q)
+    steps, nodes = torch.zeros(1, 4, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    chain = [(1 << (i + 1)) - 1 for i in range(T)]  # node i sees nodes 0 to i
+    mask = torch.tensor([[[m & (2 ** 63 - 1) | -(m & 2 ** 63) for m in (c & (2 ** 64 - 1), c >> 64)] for c in chain]], device="cuda")
+
+    def set_tree(n, L):
+        steps.copy_(torch.tensor([[n, 8, 32, L]], dtype=torch.int32))
+        nodes.fill_(n)
+
+    def layers():
+        for i in range(NL):
+            binding.resps_tree_attention(ctx, steps, nodes, 1, q[i], o[i], None, k[i], v[i], hkv * cap * D, cap * D, D, cap, mask,
+                                         1 / math.sqrt(D))
+
+    set_tree(16, 100)
+    layers()
+    ctx.attention_replan()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        layers()
+    for n, L in ((12, 5800), (128, 5800), (40, 5800), (40, 700), (64, 4000), (3, 5900)):
+        set_tree(n, L)
+        o.zero_()
+        graph.replay()
+        graph.replay()
+        assert ctx.status() == 0
+        seen = torch.ones(n, L + n, dtype=torch.bool, device="cuda")
+        seen[:, L:] = torch.tril(seen[:, L:])
+        for i in range(NL):
+            s = torch.einsum("nhgd,hkd->hgnk", q[i, 0, :n].float().view(n, hkv, hq // hkv, D), k[i, 0, :, :L + n].float())
+            p = (s / math.sqrt(D)).masked_fill(~seen, float("-inf")).softmax(-1)
+            want = torch.einsum("hgnk,hkd->nhgd", p, v[i, 0, :, :L + n].float()).reshape(n, hq, D)
+            assert (o[i, 0, :n].float() - want).abs().max() <= 2 ** -8 * want.abs().max()
+    del graph
+    ctx.close()
