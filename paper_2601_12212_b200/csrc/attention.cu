@@ -79,8 +79,8 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 
 // How a layer's work is laid out, one of three ways:
 //  whole   clusters of several CTAs, one group (sequence, KV head, row tile) per cluster.  The CTAs share
-//          the group's key tiles, leave normalised partial results in the workspace (L2), meet on an
-//          mbarrier and merge a share of the rows x columns each: one kernel does the layer.  Where the tree at
+//          the group's key tiles, send each other normalised partial results through the cluster's shared
+//          memory and merge a share of the rows x columns each: one kernel does the layer.  Where the tree at
 //          hand has fewer groups than there are clusters (which are as many as the context's largest tree needs),
 //          a group with enough key tiles is cut over several clusters, and of the warps that have merged the same
 //          share in each of them the last one merges those (fp32 sums, in L2).
@@ -135,13 +135,15 @@ struct AttnArgs {
     const uint64_t* mask;
     float scale_log2;
     int Hq, Hkv, max_tt;
-    // Partials.  O is stored normalised (O / l, a convex combination of V rows) as
+    // Partials of the two-kernel modes (in mode whole the same goes into the cluster's shared memory).  O is stored normalised (O / l, a convex combination of V rows) as
     // fp16 times a power of two per half row that only differs from 1 when a value would leave the fp16
     // range: half the bytes of fp32, and 11 significant bits per element (2^-11, against the 2^-9
-    // of the final bf16 rounding).  Place = item x cluster size + CTA.
+    // of the final bf16 rounding).
     uint4* part_o;    // [places][D/8][128 rows]  eight fp16 each
     float4* part_ml;  // [places][128 rows]   (running max m, running sum l, l * scale of each half row)
     int cluster;      // CTAs per cluster (1: modes even and stream)
+    unsigned long long chunk_first;  // mode whole: first_chunk of every rank, 7 bits each
+    int chunk_step;   // ... and the bytes a CTA's part takes in a stage
     int clusters;     // clusters the work list is cut for (at most gridDim / cluster)
     int max_items;
     int comb_chunk;   // partials the combine kernel fetches together
@@ -152,6 +154,7 @@ struct AttnArgs {
     int l2_tiles;     // K and V of more key tiles (of a KV head) than this do not stay in L2
     int min_tiles;    // fewest key tiles a CTA is given
     int q_by_tma;     // 1: Q tiles come by TMA (128 % (Hq/Hkv) == 0), 0: by plain loads
+    int log2_group;   // of Hq/Hkv, where Q tiles come by TMA
     int plan_after_wait;  // 1: the work list was written by the kernel just before this one
     int test_drop;        // test build only: 1 = the CTA's first V copy is left out
     float4* piece_acc;      // [clusters][4][128 x D/16 units] a cut group's merged share: 16 sums of a unit,
@@ -331,7 +334,6 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
         }
     }
     __syncthreads();
-    const int n_groups = sh.group0[a.batch];
     auto last_at_or_before = [&](const int* first, int x) {  // the last sequence whose entry is <= x
         int lo = 0, hi = a.batch;
 #pragma unroll 1
@@ -606,6 +608,17 @@ __device__ __forceinline__ void mbar_arrive_remote(uint32_t bar, int rank) {
         "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [remote];\n\t}" ::"r"(bar), "r"(rank)
         : "memory");
 }
+// Sixteen bytes into the shared memory of a CTA of the cluster; they count on the mbarrier beside them there.
+__device__ __forceinline__ void store_async(uint32_t dst, uint4 v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(dst), "r"(v.x),
+                 "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ uint32_t at_rank(uint32_t local, int rank) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
+    return remote;
+}
 // Bounded wait: false when this wait ran out (about a second of SM clocks) or another thread of
 // the CTA has given up.  Kept to a few instructions, because it is inlined at every wait: a role runs
 // through its code once per launch, most of it cold, and what it costs to fetch is about a cycle per 4
@@ -666,37 +679,33 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
-// Shared-memory matrix descriptor, 128-byte swizzle (layout type 2), descriptor version 1.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-    uint64_t d = static_cast<uint64_t>((addr & 0x3FFFFu) >> 4);
-    d |= static_cast<uint64_t>(lbo_bytes >> 4) << 16;
-    d |= static_cast<uint64_t>(sbo_bytes >> 4) << 32;
-    d |= 1ull << 46;
-    d |= 2ull << 61;
-    return d;
-}
+// Shared-memory matrix descriptor, 128-byte swizzle (layout type 2), descriptor version 1: the low word has the start
+// address (in 16 bytes; in a cluster an address has more bits than the field) and the leading offset, the high word
+// never changes (8 rows of 128 bytes from group to group).
+__device__ __forceinline__ constexpr uint32_t desc_lo(uint32_t addr, uint32_t lbo_bytes) { return (addr & 0x3FFFFu) >> 4 | (lbo_bytes >> 4) << 16; }
+constexpr uint32_t kDescHi = (1024u >> 4) | 1u << 14 | 2u << 29;
 // Instruction descriptor: bf16 x bf16 -> fp32, M = 128, A K-major.
 __host__ __device__ constexpr uint32_t instr_desc(int n, bool b_mn_major) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (b_mn_major ? (1u << 16) : 0u) |
            (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(kBM >> 4) << 24);
 }
-__device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                     uint32_t accumulate) {
+template <uint32_t kIdesc, bool kAccumulate>
+__device__ __forceinline__ void umma(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+        "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\tsetp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_lo), "r"(b_lo), "n"(kDescHi), "n"(kIdesc), "n"(kAccumulate ? 1 : 0)
         : "memory");
 }
 // A operand from tensor memory (lane = row, two bf16 per 32-bit column).
-__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
-                                        uint32_t accumulate) {
+template <uint32_t kIdesc>
+__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\t"
+        "mov.b64 b, {%2, %3};\n\tsetp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %4, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "r"(b_lo), "n"(kDescHi), "n"(kIdesc), "r"(accumulate)
         : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
@@ -704,7 +713,6 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
                  : "memory");
 }
 
-#define RESPS_R8(a, o) "%" #a "0" #o
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
@@ -715,16 +723,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
           "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
           "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
           "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr)
-        : "memory");
-}
-#undef RESPS_R8
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr)
         : "memory");
 }
@@ -782,6 +780,30 @@ __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
 }
 
 
+// ---------------------------------------------------------------------------- merge in a cluster
+// A partial (128 rows x D columns) is cut into chunks of 32 rows x 16 columns, row block by row block, and CTA `rank` of
+// the cluster merges the chunks [first_chunk(rank), first_chunk(rank + 1)), a warp a chunk.  All CTAs send them their parts
+// of these chunks: the warp that holds rows and columns stores fp16 pairs and the rows' (max, sum, sum x scale) into the
+// merging CTA's shared memory (st.async, bytes counted by its mbarrier), so that nobody reads what is far away and no
+// fence waits for stores.
+// Bound by the way between SMs: 32 KB from each of 6 CTAs to the others are there 1480 clocks after the first store (8
+// CTAs 1300, 3 1540); plain remote stores behind a releasing arrival 2740 (3100, 2120), bulk copies 2950.  Through
+// L2 (partials written, a meeting, read back) the 8B shape spent 3.5 us between its merged lanes and O.
+__host__ __device__ constexpr int chunks_of(int D) { return kBM / 32 * (D / 16); }
+__host__ __device__ constexpr int first_chunk(int D, int cluster, int rank) { return (chunks_of(D) * rank + cluster - 1) / cluster; }
+static_assert(chunks_of(128) < 128 && 7 * (kMaxCluster + 1) <= 64, "AttnArgs::chunk_first");
+// (from the launch's table: a division by the cluster's size takes a hundred clocks, and there were a dozen on the way)
+__device__ __forceinline__ int chunk_at(const AttnArgs& a, int rank) { return static_cast<int>(a.chunk_first >> (7 * rank)) & 127; }
+// a chunk's place: 32 rows x 2 units of eight fp16, then the rows' (max, sum, sum x scale) where it is the first chunk of
+// its rows and half of the columns that the CTA merges
+constexpr int kChunkBytes = 32 * 32, kRowBytes = 32 * 16, kSlotBytes = kChunkBytes + kRowBytes;
+__host__ __device__ constexpr int chunks_most(int D, int cluster) { return (chunks_of(D) + cluster - 1) / cluster; }
+constexpr int most_staged(int D) {
+    int most = 0;
+    for (int c = 2; c <= kMaxCluster; ++c) most = most < c * chunks_most(D, c) ? c * chunks_most(D, c) : most;
+    return most;
+}
+
 // ---------------------------------------------------------------------------- shared memory map
 template <int D>
 struct Smem {
@@ -794,15 +816,20 @@ struct Smem {
     static constexpr int kOffK = kOffQ + kQTile;
     static constexpr int kOffV = kOffK + kStagesK * kKVTile;
     static constexpr int kOffBar = kOffV + kStagesV * kKVTile;
-    static constexpr int kNumBars = 2 * (kStagesK + kStagesV) + 2 + kLanes * 6 + 3;
+    static constexpr int kNumBars = 2 * (kStagesK + kStagesV) + 2 + kLanes * 6 + 4;
     static constexpr int kOffMisc = kOffBar + 8 * 40;
     static constexpr int kOffMerge = kOffMisc + 64;          // (max, sum) of every row of both lanes
-    static constexpr int kUsed = kOffMerge + kLanes * kBM * 8 + 1024;  // + slack to align the base to 1024
+    static constexpr int kUsed = kOffMerge + kLanes * kBM * 8;
+    // Mode whole: what the CTAs of the cluster send for this CTA's share of the merge, [CTA][chunk of the share].
+    static constexpr int kOffStage = kOffMerge + kLanes * kBM * 8;
+    static constexpr int kStage = most_staged(D) * kSlotBytes;
     // Never less than 120 KB, more than half of an SM's shared memory: one CTA per SM, so the
     // 512-column TMEM allocation can never wait for a neighbour.
     static constexpr int kBytes = kUsed > 120 * 1024 ? kUsed : 120 * 1024;
     static_assert(kNumBars <= 40, "barrier area");
     static_assert(2 * kBytes > 228 * 1024, "two CTAs must not fit on one SM");
+    static constexpr int kClusterBytes = kUsed + kStage > kBytes ? kUsed + kStage : kBytes;
+    static_assert(kClusterBytes <= 227 * 1024, "shared memory of a CTA");
 };
 
 // barrier indices
@@ -830,16 +857,25 @@ constexpr int kBar1 = kBar0 + 2 + kLanes * 6;
 __device__ __forceinline__ constexpr int bar_item() { return kBar1; }
 // both softmax warpgroups have their partial result (and its PV completions) behind them
 __device__ __forceinline__ constexpr int bar_merge() { return kBar1 + 1; }
-// every softmax warp of every CTA of the cluster has written its share of the CTA's partial
+// everything the CTA merges is in its shared memory: its own warps' arrivals, the other CTAs' bytes
 __device__ __forceinline__ constexpr int bar_meet() { return kBar1 + 2; }
+// every warp of the cluster has merged its share of the item: the next item's may be sent
+__device__ __forceinline__ constexpr int bar_free() { return kBar1 + 3; }
 
 // Sixteen columns of a row: O, and with the first ones the row's log-sum-exp.
+// (row of a KV head -> token; heads in a group: a power of two where Q comes by TMA)
+template <bool kPow2>
+__device__ __forceinline__ unsigned token_of(const AttnArgs& a, unsigned R, int G) {
+    return kPow2 ? R >> a.log2_group : R / static_cast<unsigned>(G);
+}
+template <bool kPow2>
+__device__ __forceinline__ int64_t output_row(const AttnArgs& a, const Item& it, int r, int G) {
+    const unsigned R = it.row_base + r, t = token_of<kPow2>(a, R, G), h = it.g * G + (R - t * G);
+    return (static_cast<int64_t>(it.b) * a.max_tt + t) * a.Hq + h;
+}
 template <int D>
-__device__ __forceinline__ void write_unit(const AttnArgs& a, const Item& it, unsigned r, unsigned c16, int G, float Mx, float den,
-                                           const float (&acc)[16]) {
+__device__ __forceinline__ void write_unit(const AttnArgs& a, int64_t row, int c16, float Mx, float den, const float (&acc)[16]) {
     const float inv = 1.f / den;
-    const unsigned R = it.row_base + r, t = R / static_cast<unsigned>(G), h = it.g * G + (R - t * G);
-    const int64_t row = (static_cast<int64_t>(it.b) * a.max_tt + t) * a.Hq + h;
     uint32_t o[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) o[e] = pack_bf16(acc[2 * e] * inv, acc[2 * e + 1] * inv);
@@ -848,66 +884,61 @@ __device__ __forceinline__ void write_unit(const AttnArgs& a, const Item& it, un
     dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
     if (a.lse && c16 == 0) a.lse[row] = (Mx + log2f(den)) * 0.6931471805599453f;
 }
-// Merges the partials of an item: this CTA's share of the (16 columns, row) units, O = sum_p w_p O_p /
-// sum_p w_p l_p with w_p = 2^(m_p - max m).  Bound by the latency of L2 (one round trip for six partials,
-// whose loads are in flight together) and by its own code, which is kept short.  kPiece: the group is cut over several
-// clusters, the sums stay in the workspace.  (Two copies of the code, so that the common one has nothing to skip: with
-// one the 8B shape's call took 9.57 us, with two 9.34, and 9.45 before there were pieces.)
+// The chunk that a warp merges, and where the row of the lane goes.
+struct MergeAt {
+    int q, r;       // chunk; row of the tile (past the valid ones: nothing to do)
+    int data, rows; // its places in the stage
+    int64_t out;    // row of O
+};
+template <int D, bool kPow2>
+__device__ __forceinline__ MergeAt merge_at(const AttnArgs& a, const Item& it, int q, int q0, int lane, int G) {
+    MergeAt m;
+    m.q = q, m.r = q / (D / 16) * 32 + lane;
+    m.data = (q - q0) * kSlotBytes + lane * 16;
+    m.rows = (max(q / (D / 32) * (D / 32), q0) - q0) * kSlotBytes + kChunkBytes + lane * 16;
+    m.out = output_row<kPow2>(a, it, m.r, G);
+    return m;
+}
+// Merges a chunk of the partials in the CTA's shared memory, O = sum_p w_p O_p / sum_p w_p l_p with
+// w_p = 2^(m_p - max m).  kPiece: the group is cut over several
+// clusters, the sums go to the workspace.  (Copies of the code, so that the common ones have nothing to skip.)
 template <int D, bool kPiece>
-__device__ __forceinline__ void merge_partials(const AttnArgs& a, const Item& it, unsigned place0, int n_parts,
-                                               int rank, int tid, int G, unsigned cluster_id) {
-    constexpr unsigned kBatch = 6, kUnits = kBM * (D / 16);
-    const unsigned nv = static_cast<unsigned>(min(kBM, it.M - it.row_base));  // valid rows
-    const unsigned units = nv * (D / 16);
-    const unsigned u1 = units * static_cast<unsigned>(rank + 1) / static_cast<unsigned>(a.cluster);
-#pragma unroll 1
-    for (unsigned u = units * static_cast<unsigned>(rank) / static_cast<unsigned>(a.cluster) + tid; u < u1; u += kSoftmaxThreads) {
-        const unsigned c16 = u / nv, r = u - c16 * nv;
-        float Mx = -INFINITY, den = 0.f;
-        float acc[16] = {};
-#pragma unroll 1
-        for (unsigned p0 = 0; p0 < static_cast<unsigned>(n_parts); p0 += kBatch) {
-            float4 ml[kBatch];
-            uint4 v[kBatch][2];
+__device__ __forceinline__ void merge_chunk(const AttnArgs& a, const Item& it, const unsigned char* stage, const MergeAt& m, int lane,
+                                            unsigned cluster_id) {
+    constexpr int kUnits = kBM * (D / 16);
+    if (it.row_base + m.r >= it.M) return;
+    float Mx = -INFINITY, den = 0.f;
 #pragma unroll
-            for (unsigned i = 0; i < kBatch; ++i) {
-                const unsigned place = place0 + min(p0 + i, static_cast<unsigned>(n_parts) - 1u);
-                ml[i] = __ldcg(a.part_ml + place * kBM + r);
-                const uint4* src = a.part_o + ((place * (D / 8) + 2 * c16) * kBM + r);
-                v[i][0] = __ldcg(src), v[i][1] = __ldcg(src + kBM);
-            }
-            float mx = Mx;
+    for (int p = 0; p < kMaxCluster; ++p)
+        Mx = fmaxf(Mx, *reinterpret_cast<const float*>(stage + m.rows + min(p, it.active - 1) * a.chunk_step));
+    unsigned long long acc2[8] = {};
+#pragma unroll 2
+    for (int p = 0; p < it.active; ++p) {
+        const unsigned char* const src = stage + p * a.chunk_step;
+        const float4 ml = *reinterpret_cast<const float4*>(src + m.rows);
+        const uint4 v0 = *reinterpret_cast<const uint4*>(src + m.data), v1 = *reinterpret_cast<const uint4*>(src + m.data + 512);
+        const float w = ml.x == -INFINITY ? 0.f : ex2_approx(ml.x - Mx);  // an empty partial is zeros
+        den += ml.y * w;
+        const float wo = ml.z * w;  // O_p = Ohat * l * scale
+        const uint32_t hw[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
 #pragma unroll
-            for (unsigned i = 0; i < kBatch; ++i) mx = fmaxf(mx, ml[i].x);
-            if (mx == -INFINITY) continue;
-            const float corr = ex2_approx(Mx - mx);  // 0 on the first batch
-            den *= corr;
-#pragma unroll
-            for (int e = 0; e < 16; ++e) acc[e] *= corr;
-            Mx = mx;
-#pragma unroll
-            for (unsigned i = 0; i < kBatch; ++i) {
-                // 0 for an empty partial, which stores zeros, and past the end
-                const float w = p0 + i < static_cast<unsigned>(n_parts) ? ex2_approx(ml[i].x - Mx) : 0.f;
-                den += ml[i].y * w;
-                const float wo = (c16 < D / 32 ? ml[i].z : ml[i].w) * w;  // O_p = Ohat * l * scale of this half of the row
-                const uint32_t hw[8] = {v[i][0].x, v[i][0].y, v[i][0].z, v[i][0].w, v[i][1].x, v[i][1].y, v[i][1].z, v[i][1].w};
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hw[e]));
-                    acc[2 * e] += f.x * wo, acc[2 * e + 1] += f.y * wo;
-                }
-            }
+        for (int e = 0; e < 8; ++e) {
+            const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hw[e]));
+            acc2[e] = fma2(pack2(f.x, f.y), pack2(wo, wo), acc2[e]);
         }
-        if (!kPiece) {
-            write_unit<D>(a, it, r, c16, G, Mx, den, acc);
-        } else {
+    }
+    float acc[16];
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-                __stcg(a.piece_acc + (cluster_id * 4 + e) * kUnits + u,
-                       make_float4(acc[4 * e], acc[4 * e + 1], acc[4 * e + 2], acc[4 * e + 3]));
-            __stcg(a.piece_ml + cluster_id * kUnits + u, make_float2(Mx, den));
-        }
+    for (int e = 0; e < 8; ++e) unpack2(acc2[e], acc[2 * e], acc[2 * e + 1]);
+    if (!kPiece) {
+        write_unit<D>(a, m.out, m.q % (D / 16), Mx, den, acc);
+    } else {
+        const unsigned u = m.q * 32 + lane;
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            __stcg(a.piece_acc + (cluster_id * 4 + e) * kUnits + u,
+                   make_float4(acc[4 * e], acc[4 * e + 1], acc[4 * e + 2], acc[4 * e + 3]));
+        __stcg(a.piece_ml + cluster_id * kUnits + u, make_float2(Mx, den));
     }
 }
 // A group that is cut over several clusters: the same warp of the same CTA of each has merged the same units.  It
@@ -916,13 +947,14 @@ __device__ __forceinline__ void merge_partials(const AttnArgs& a, const Item& it
 // Under a context for 128 nodes on the 8B shape (32 clusters of 4), in us a layer uncut / cut / the two kernels with the
 // same context: 16 nodes at 4096 keys 16.5 / 14.2 / 15.5, at 8192 26.3 / 17.3 / 18.7, at 12 288 35.6 / 19.9 / 21.5;
 // 64 nodes 17.1 / 15.8 / 16.7, 26.8 / 21.0 / 21.6, 36.2 / 25.9 / 26.0.
-template <int D>
+template <int D, bool kPow2>
 __device__ __forceinline__ void merge_pieces(const AttnArgs& a, const Item& it, int rank, int tid, int G) {
     constexpr unsigned kUnits = kBM * (D / 16);
-    const unsigned nv = static_cast<unsigned>(min(kBM, it.M - it.row_base)), units = nv * (D / 16);
-    const unsigned u1 = units * static_cast<unsigned>(rank + 1) / static_cast<unsigned>(a.cluster);
-    const unsigned u0 = units * static_cast<unsigned>(rank) / static_cast<unsigned>(a.cluster) + tid;
-    if (u0 - (tid & 31) >= u1) return;  // the warp has no units (in no piece)
+    const int lane = tid & 31, nv = min(kBM, it.M - it.row_base);
+    const int q0 = chunk_at(a, rank) + (tid >> 5), q1 = chunk_at(a, rank + 1);
+    bool any = false;
+    for (int q = q0; q < q1; q += kPieceWarps) any = any || q / (D / 16) * 32 < nv;
+    if (!any) return;  // the warp has no units (in no piece)
     unsigned* const count = a.piece_count + (it.place * a.cluster + rank) * kPieceWarps + (tid >> 5);
     unsigned before = 0;
     __syncwarp();  // (orders the lanes' sums before the first one's arrival)
@@ -932,7 +964,10 @@ __device__ __forceinline__ void merge_pieces(const AttnArgs& a, const Item& it, 
     if ((tid & 31) == 0) __stcg(count, 0u);  // for the next layer
     __syncwarp();
 #pragma unroll 1
-    for (unsigned u = u0; u < u1; u += kSoftmaxThreads) {
+    for (int q = q0; q < q1; q += kPieceWarps) {
+        const int r = q / (D / 16) * 32 + lane;
+        if (r >= nv) continue;
+        const unsigned u = q * 32 + lane;
         float Mx = -INFINITY, den = 0.f;
         float acc[16] = {};
 #pragma unroll 2
@@ -951,23 +986,36 @@ __device__ __forceinline__ void merge_pieces(const AttnArgs& a, const Item& it, 
                 acc[4 * e + 2] = acc[4 * e + 2] * c + v[e].z * w, acc[4 * e + 3] = acc[4 * e + 3] * c + v[e].w * w;
             }
         }
-        const unsigned c16 = u / nv;
-        write_unit<D>(a, it, u - c16 * nv, c16, G, Mx, den, acc);
+        write_unit<D>(a, output_row<kPow2>(a, it, r, G), q % (D / 16), Mx, den, acc);
     }
 }
 
-template <int D>
+__device__ __forceinline__ int cluster_index() {
+    int c;
+    asm("mov.u32 %0, %%clusterid.x;" : "=r"(c));
+    return c;
+}
+// What of the kernel a launch needs: the two-kernel modes, mode whole, mode whole where groups may be cut; Q by TMA or
+// by plain loads.  A launch runs through most of its code once, and an SM keeps 32 KB of it: straight code of up to
+// 24 KB takes a clock an instruction, in the next launch too, of 48 KB and more 2.1 clocks wherever it is in its loops.  One
+// kernel for all forms had 76 KB (head dimension 128); these have 39, 55 and 64 with uniform warp indexes, constant base
+// addresses and 32-bit descriptor words.  In us a call before / now, the cluster's exchange included: 8B shape at 1024
+// keys 9.34 / 8.43, 128 nodes at 2048 keys 13.5 / 11.9, 13B shape 15.1 / 14.1, 28 heads of two users 12.6 / 11.3, 70B
+// shape 22.5 / 20.6, 8 ragged sequences 61.3 / 57.4, 32 000 keys 31.3 / 29.8, 4 heads of 64 5.09 / 4.81.
+enum Form { kSingles, kWhole, kCut };
+template <int D, int kForm, bool kQByTma>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_k,
                       const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_q) {
     using S = Smem<D>;
-    extern __shared__ unsigned char smem_raw[];
-    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    unsigned char* base_ptr = smem_raw + (base - smem_u32(smem_raw));
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    const uint32_t base = smem_u32(smem_raw);
+    unsigned char* base_ptr = smem_raw;
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(kFull, tid >> 5, 0);  // (known to be the same for the warp)
     const int G = a.Hq / a.Hkv;
-    const int cluster_id = static_cast<int>(static_cast<unsigned>(blockIdx.x) / static_cast<unsigned>(a.cluster));
-    const int rank = static_cast<int>(blockIdx.x) - cluster_id * a.cluster;
+    constexpr bool kClusters = kForm != kSingles;
+    const int cluster_id = kClusters ? cluster_index() : static_cast<int>(blockIdx.x);
+    const int rank = kClusters ? static_cast<int>(cluster_rank()) : 0;
     const uint32_t bars = base + S::kOffBar;
     auto bar = [&](int i) { return bars + 8u * i; };
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + S::kOffMisc);
@@ -991,7 +1039,8 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
             first_item = c.x, n_items = c.y;
         }
     };
-    if (!a.plan_after_wait) read_plan();
+    if (a.plan_after_wait) pdl_wait();
+    read_plan();
 
     // ---- one-time set-up ---------------------------------------------------------------
     // (the producers' barriers by the producers themselves: their first copies go out before the CTA meets)
@@ -1003,7 +1052,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
             mbar_init(bar(is_v ? bar_vempty(s) : bar_kempty(s)), 1);
         }
         if (!is_v) {
-            mbar_init(bar(bar_qfull()), a.q_by_tma ? 1 : kSoftmaxThreads);
+            mbar_init(bar(bar_qfull()), kQByTma ? 1 : kSoftmaxThreads);
             mbar_init(bar(bar_qempty()), kLanes);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1022,7 +1071,8 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
         }
         mbar_init(bar(bar_item()), kSoftmaxThreads);
         mbar_init(bar(bar_merge()), kSoftmaxThreads);
-        mbar_init(bar(bar_meet()), a.cluster * (kSoftmaxThreads / 32));
+        mbar_init(bar(bar_meet()), kPieceWarps);
+        mbar_init(bar(bar_free()), a.cluster * kPieceWarps);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kMmaWarp0) {
@@ -1045,7 +1095,6 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
     cluster_arrive();
     pdl_wait();
     pdl_launch_dependents();
-    if (a.plan_after_wait) read_plan();
     auto load_q = [&](const Item& it) {
         mbar_expect_tx(bar(bar_qfull()), S::kQTile);
         tma_load_5d(base + S::kOffQ, &map_q, bar(bar_qfull()), 0, 0, it.g, it.b * a.max_tt + it.row_base / G, 0);
@@ -1063,12 +1112,12 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
         const bool is_v = warp == kVProducerWarp;
         // (in the wait test's build the CTA's first V copy may be left out)
         if (!(kWaitTest && is_v && (a.test_drop & 1))) load_tile(first_it, first_it.t_begin, 0, is_v);
-        if (!is_v && a.q_by_tma) load_q(first_it);
+        if (!is_v && kQByTma) load_q(first_it);
     }
     __syncwarp();
     cluster_wait();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    constexpr uint32_t tmem = 0;  // all columns are allocated: they begin at 0
     // The list must still describe the step parameters it is used with (the caller changes them only
     // through the library, or asks for a new list): one thread compares its item's sequence.
     bool stale = false;
@@ -1076,7 +1125,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
         const int n_live = min(max(a.n_nodes[first_it.b], 0), a.max_tt), L_live = max(a.steps[first_it.b].prefix_len, 0);
         stale = (n_live != first_it.n) || (L_live != first_it.L);
     }
-    auto get_item = [&](int i) { return i == 0 ? first_it : load_item(a.plan_item + (first_item + i) * a.cluster + rank, G); };
+    auto get_item = [&](int i) { return i == 0 ? first_it : load_item(a.plan_item + (first_item + i) * (kClusters ? a.cluster : 1) + rank, G); };
 
     // Running use counts of the barrier families.  Every role walks the same items and tiles in
     // the same order, so each keeps its own copy.
@@ -1110,7 +1159,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                         break;
                     }
                     load_tile(it, t, kt_run, is_v);
-                    if (t == it.t_begin && !is_v && a.q_by_tma) {
+                    if (t == it.t_begin && !is_v && kQByTma) {
                         // Q follows the first K tile: K and Q are what the first MMA needs.  The Q
                         // tile of the previous item is free once its last QK^T has completed.
                         if (!mbar_wait(bar(bar_qempty()), (items_run & 1u) ^ 1u, abort_flag)) {
@@ -1125,7 +1174,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
             }
             // Drain: every copy this thread issued has landed before the CTA may exit (each one is
             // waited for, also after an earlier wait has run out).
-            bool landed = is_v || !(a.q_by_tma && items_run > 0) || drain_wait(bar(bar_qfull()), (items_run - 1u) & 1u);
+            bool landed = is_v || !(kQByTma && items_run > 0) || drain_wait(bar(bar_qfull()), (items_run - 1u) & 1u);
             const uint32_t issued = kt_run;
 #pragma unroll 1
             for (uint32_t u = (issued > kStagesK ? issued - kStagesK : 0u); u < issued; ++u)
@@ -1146,11 +1195,8 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
         const int x = warp - kMmaWarp0;
         constexpr uint32_t kIdescQK = instr_desc(kBN, false);
         constexpr uint32_t kIdescPV = instr_desc(D, true);
-        // Descriptors differ only in the (16-byte granular) start address, the low 14 bits.
-        const uint64_t qdesc = smem_desc(base + S::kOffQ, 16, 1024);
-        const uint64_t kdesc0 = smem_desc(base + S::kOffK, 16, 1024);
-        const uint64_t vdesc0 = smem_desc(base + S::kOffV, S::kKVPanel, 1024);
-        const uint32_t o_t = tmem + x * 256 + 128;
+        const uint32_t q_lo = desc_lo(base + S::kOffQ, 16), k_lo0 = desc_lo(base + S::kOffK, 16), v_lo0 = desc_lo(base + S::kOffV, S::kKVPanel);
+        const uint32_t s_t0 = tmem + x * 256, o_t = s_t0 + 128;
         uint32_t k_seen = 0xFFFFFFFFu;  // ring use whose K tile this warp has already seen arrive
 #pragma unroll 1
         for (int i = 0; i < n_items && alive; ++i) {
@@ -1161,7 +1207,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
             bool first_pv = true;
             // The lane's tiles are t_begin + x, + 2, ...; one round issues Q K^T of a tile and P V of the one
             // before (the last round P V only).
-            const int mine = (it.t_end - it.t_begin - x + 1) >> 1;
+            const int n_tiles = __shfl_sync(kFull, it.t_end - it.t_begin, 0), mine = (n_tiles - x + 1) >> 1;
             const uint32_t use0 = kt_run + static_cast<uint32_t>(x);
 #pragma unroll 1
             for (int j = 0; j <= mine && mine > 0 && alive; ++j) {
@@ -1174,12 +1220,12 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                     }
                     tc_fence_after();
                     if (elect_one()) {
-                        const uint64_t kdesc = kdesc0 + static_cast<uint64_t>(s * (S::kKVTile >> 4));
-                        const uint32_t s_t = tmem + x * 256 + (jx & 1u) * kBN;
+                        const uint32_t k_lo = k_lo0 + s * (S::kKVTile >> 4), s_t = s_t0 + (jx & 1u) * kBN;
+                        umma<kIdescQK, false>(s_t, q_lo, k_lo);
 #pragma unroll
-                        for (int ks = 0; ks < D / 16; ++ks)
-                            umma(s_t, qdesc + ((ks >> 2) * (S::kQPanel >> 4) + (ks & 3) * 2),
-                                 kdesc + ((ks >> 2) * (S::kKVPanel >> 4) + (ks & 3) * 2), kIdescQK, ks > 0 ? 1u : 0u);
+                        for (int ks = 1; ks < D / 16; ++ks)
+                            umma<kIdescQK, true>(s_t, q_lo + (ks >> 2) * (S::kQPanel >> 4) + (ks & 3) * 2,
+                                                 k_lo + (ks >> 2) * (S::kKVPanel >> 4) + (ks & 3) * 2);
                         umma_commit(bar(bar_sfull(x, jx & 1u)));
                         umma_commit(bar(bar_kempty(s)));
                     }
@@ -1204,14 +1250,14 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                     if (!alive) break;
                     tc_fence_after();
                     if (elect_one()) {
-                        const uint64_t vdesc = vdesc0 + static_cast<uint64_t>(s * (S::kKVTile >> 4));
+                        const uint32_t v_lo = v_lo0 + s * (S::kKVTile >> 4);
                         // P of keys 32h .. 32h+31: hi in columns 32h .. 32h+15, lo in 32h+16 .. 32h+31
-                        const uint32_t p_t = tmem + x * 256 + (prev_j & 1u) * kBN;
+                        const uint32_t p_t = s_t0 + (prev_j & 1u) * kBN;
 #pragma unroll
                         for (int kk = 0; kk < kBN / 16; ++kk) {
                             const uint32_t a_t = p_t + (kk >> 1) * 32 + (kk & 1) * 8;
-                            umma_ts(o_t, a_t, vdesc + kk * (2048 >> 4), kIdescPV, (first_pv && kk == 0) ? 0u : 1u);
-                            umma_ts(o_t, a_t + 16, vdesc + kk * (2048 >> 4), kIdescPV, 1u);
+                            umma_ts<kIdescPV>(o_t, a_t, v_lo + kk * (2048 >> 4), (first_pv && kk == 0) ? 0u : 1u);
+                            umma_ts<kIdescPV>(o_t, a_t + 16, v_lo + kk * (2048 >> 4), 1u);
                         }
                         umma_commit(bar(bar_pvdone(x, prev_j & 1u)));
                         umma_commit(bar(bar_vempty(s)));
@@ -1225,18 +1271,24 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
             }
             if (alive && mine == 0 && elect_one()) umma_commit(bar(bar_qempty()));
             __syncwarp();
-            kt_run += static_cast<uint32_t>(it.t_end - it.t_begin);
+            kt_run += static_cast<uint32_t>(n_tiles);
             ++items_run;
         }
     }
     } else {
         // ================================ softmax warpgroup of lane x =====================
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
+        constexpr int kHalf = D / 2;                   // columns of a row that a lane merges
         const int x = warp >> 2;
         const int r = (warp & 3) * 32 + lane;          // row inside the tile = TMEM lane
         const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
         const uint32_t s_t = tmem + lane_sel + x * 256, o_t = s_t + 128;
-        uint32_t merges = 0, meets = 0;                // uses of the end-of-item barriers
+        uint32_t merges = 0, meets = 0, frees = 0;     // uses of the end-of-item barriers
+        bool in_use = false;                           // the cluster may still be merging the item before
+        auto wait_free = [&]() {
+            if (in_use) alive = __all_sync(kFull, cluster_bar_wait(bar(bar_free()), frees++ & 1u, abort_flag));
+            in_use = false;
+        };
 #pragma unroll 1
         for (int i = 0; i < n_items && alive; ++i) {
             const Item it = get_item(i);
@@ -1246,7 +1298,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 // ---- Q tile -> shared memory in the swizzled K-major layout (only when the group size does not
                 // allow the TMA view): every thread's pieces are in flight together (one at a time they
                 // took 8 us) --------------------------------------------------------------------------
-                if (!a.q_by_tma) {
+                if constexpr (!kQByTma) {
                     constexpr int kChunks = D / 8, kPer = kBM * kChunks / kSoftmaxThreads;  // 16-byte pieces of a row, of a thread
                     uint4 v[kPer];
                     const int c = tid % kChunks;
@@ -1273,7 +1325,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 const bool row_ok = R < it.M;
                 unsigned long long mlo = 0ull, mhi = 0ull;
                 if (row_ok) {
-                    const int t = R / G;
+                    const int t = token_of<kQByTma>(a, R, G);
                     mlo = a.mask[(static_cast<int64_t>(it.b) * a.max_tt + t) * 2 + 0];
                     mhi = a.mask[(static_cast<int64_t>(it.b) * a.max_tt + t) * 2 + 1];
                     // only nodes of this tree can be visible
@@ -1435,109 +1487,170 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 xch[x * kBM + r] = make_float2(m_self, l_run);
                 tc_fence_before();
                 mbar_arrive(bar(bar_merge()));
+                // The half row stays in registers: its largest magnitude decides the scale of a partial before
+                // anything is sent.  (In pieces, in a rolled loop, with such rows sent again through the workspace:
+                // 8B shape 9.0 us, 13B shape 14.9.)
+                // (a lane without tiles has nothing in tensor memory: the other's is read in its place, with weight 0)
+                const uint32_t both_t = tmem + lane_sel + 128 + x * kHalf;
+                const uint32_t self_t = both_t + (use_self ? x : x ^ 1) * 256, oth_t = both_t + (use_oth ? x ^ 1 : x) * 256;
+                // (while the other lane's result is waited for) where the chunks of the warp's rows and columns go
+                uint32_t there[kHalf / 16], meet[kHalf / 16];
+                if constexpr (kClusters) {
+                    const uint32_t stage = base + S::kOffStage + lane * 16 + rank * a.chunk_step;
+#pragma unroll
+                    for (int i = 0; i < kHalf / 16; ++i) {
+                        const int q = (warp & 3) * (D / 16) + x * (D / 32) + i, to = static_cast<unsigned>(q * a.cluster) / chunks_of(D);
+                        there[i] = at_rank(stage + (q - chunk_at(a, to)) * kSlotBytes, to);
+                        meet[i] = at_rank(bar(bar_meet()), to);
+                    }
+                }
                 alive = warp_wait(bar(bar_merge()), merges & 1u, abort_flag);
                 ++merges;
                 if (!alive) break;
                 tc_fence_after();
                 const float2 oth = xch[(x ^ 1) * kBM + r];
                 const float m_tot = fmaxf(m_self, oth.x);
-                const float w_self = (m_self == -INFINITY) ? 0.f : ex2_approx(m_self - m_tot);
-                const float w_oth = (oth.x == -INFINITY) ? 0.f : ex2_approx(oth.x - m_tot);
+                float w_self = (m_self == -INFINITY) ? 0.f : ex2_approx(m_self - m_tot);
+                float w_oth = (oth.x == -INFINITY) ? 0.f : ex2_approx(oth.x - m_tot);
                 const float l_tot = l_run * w_self + oth.y * w_oth;
                 const float inv = (l_tot > 0.f) ? 1.f / l_tot : 0.f;
-                const int tok = R / G, h = it.g * G + R % G;
-                const int64_t out_row = (static_cast<int64_t>(it.b) * a.max_tt + tok) * a.Hq + h;
-                // (two places per CTA of a cluster, in turn: an item's partials are read behind the meeting of the
-                // CTAs, and the next but one item's are written behind the next meeting)
-                const int64_t place = a.cluster > 1 ? static_cast<int>(blockIdx.x + (meets & 1u) * gridDim.x) : it.place;
-                __nv_bfloat16* dst = a.o + out_row * D;
-                uint4* po = a.part_o + place * (D / 8) * kBM + r;
-                // (a lane without tiles has nothing in tensor memory: the other's is read in its place, with weight 0)
-                const uint32_t both_t = tmem + lane_sel + 128;
-                const uint32_t self_t = both_t + (use_self ? x : x ^ 1) * 256, oth_t = both_t + (use_oth ? x ^ 1 : x) * 256;
-                if (row_ok && direct && a.lse && x == 0)
-                    a.lse[out_row] = (m_tot + log2f(l_tot)) * 0.6931471805599453f;
-                // The half row leaves tensor memory in 16-column pieces, in a loop of few instructions: it runs
-                // once per item, and unrolled over the row its 14 KB of code took 3600 cycles to fetch.
-                // Partials assume a scale of 1 and keep the largest magnitude; when a row of the warp would
-                // leave the fp16 range, a second pass writes such rows again with their scale (a scale per
-                // half of the columns: the halves come from different lanes).
-                float amax = 0.f, scale = 1.f;  // O = Ohat * l * scale
+                w_self *= inv, w_oth *= inv;
+                float scale = 1.f;  // O = Ohat * l * scale, a scale for each half of the columns
+                uint32_t g[kHalf / 32][32];
+                // (a second time where |O / l| of a partial would leave fp16's range: the weights take a scale then)
 #pragma unroll 1
-                for (int pass = 0; pass < 2; ++pass) {
-                    const float mul = (pass == 0) ? inv : inv / scale;
-                    const unsigned long long ws2 = pack2(w_self * mul, w_self * mul), wo2 = pack2(w_oth * mul, w_oth * mul);
-                    const bool store = row_ok && (pass == 0 || scale != 1.f);
-#pragma unroll 1
-                    for (int c = x * (D / 2); c < (x + 1) * (D / 2); c += 16) {
-                        uint32_t r0[16], r1[16];
-                        tmem_ld16(self_t + c, r0);
-                        tmem_ld16(oth_t + c, r1);
+                while (true) {
+                    const unsigned long long ws2 = pack2(w_self, w_self), wo2 = pack2(w_oth, w_oth);
+                    float amax = 0.f;
+#pragma unroll
+                    for (int c = 0; c < kHalf / 32; ++c) {
+                        uint32_t other[32];
+                        tmem_ld32(self_t + 32 * c, g[c]);
+                        tmem_ld32(oth_t + 32 * c, other);
                         tmem_wait_ld();
-                        float g[16];
 #pragma unroll
-                        for (int e = 0; e < 16; e += 2) {
-                            const unsigned long long s2 = pack2(__uint_as_float(r0[e]), __uint_as_float(r0[e + 1]));
-                            const unsigned long long o2 = pack2(__uint_as_float(r1[e]), __uint_as_float(r1[e + 1]));
-                            unpack2(fma2(o2, wo2, fma2(s2, ws2, pack2(0.f, 0.f))), g[e], g[e + 1]);
-                            amax = max3(amax, fabsf(g[e]), fabsf(g[e + 1]));
-                        }
-                        uint32_t v[8];
-                        if (direct) {
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) v[e] = pack_bf16(g[2 * e], g[2 * e + 1]);
-                        } else {
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) v[e] = pack_half2(g[2 * e], g[2 * e + 1]);
-                        }
-                        uint4* to = direct ? reinterpret_cast<uint4*>(dst + c) : po + (c / 8) * kBM;
-                        if (store) {
-                            __stcg(to, make_uint4(v[0], v[1], v[2], v[3]));
-                            __stcg(to + (direct ? 1 : kBM), make_uint4(v[4], v[5], v[6], v[7]));
+                        for (int e = 0; e < 32; e += 2) {
+                            const unsigned long long s2 = pack2(__uint_as_float(g[c][e]), __uint_as_float(g[c][e + 1]));
+                            const unsigned long long o2 = pack2(__uint_as_float(other[e]), __uint_as_float(other[e + 1]));
+                            float g0, g1;
+                            unpack2(fma2(o2, wo2, fma2(s2, ws2, pack2(0.f, 0.f))), g0, g1);
+                            g[c][e] = __float_as_uint(g0), g[c][e + 1] = __float_as_uint(g1);
+                            amax = fmaxf(fmaxf(amax, fabsf(g0)), fabsf(g1));
                         }
                     }
-                    if (direct || pass == 1) break;
-                    // scale: 1 unless |O / l| would exceed 2^14 (fp16 holds up to 65504)
-                    if (row_ok && amax > 16384.f) scale = exp2f(ceilf(log2f(amax)) - 14.f);
-                    // (the loads from tensor memory are warp-wide: the whole warp goes round again)
-                    if (!__any_sync(kFull, scale != 1.f)) break;
+                    const bool large = row_ok && !direct && amax > 16384.f && scale == 1.f;
+                    if (!__any_sync(kFull, large)) break;
+                    if (large) {  // the next power of two above |O / l|, 2^14 down; its reciprocal by the exponent too
+                        scale = __uint_as_float((__float_as_uint(amax) & 0x7F800000u) - (13u << 23));
+                        const float down = __uint_as_float((254u << 23) - __float_as_uint(scale));
+                        w_self *= down, w_oth *= down;
+                    }
                 }
                 // O has been read: the next item's P V may overwrite it
                 tc_fence_before();
                 mbar_arrive(bar(bar_item()));
-                if (row_ok && !direct) {
-                    float* ml = reinterpret_cast<float*>(a.part_ml + place * kBM + r);
-                    if (x == 0) {
-                        __stcg(reinterpret_cast<float2*>(ml), make_float2(m_tot, l_tot));
-                        __stcg(ml + 2, l_tot * scale);
-                    } else {
-                        __stcg(ml + 3, l_tot * scale);
+                if (kClusters && !direct) wait_free();
+                if (!alive) break;
+                if (direct) {
+                    const int64_t out_row = output_row<kQByTma>(a, it, r, G);
+                    uint4* const to = reinterpret_cast<uint4*>(a.o + out_row * D + x * kHalf);
+                    if (row_ok && a.lse && x == 0) a.lse[out_row] = (m_tot + log2f(l_tot)) * 0.6931471805599453f;
+#pragma unroll
+                    for (int i = 0; i < kHalf / 8; ++i) {
+                        uint32_t v[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            v[e] = pack_bf16(__uint_as_float(g[i >> 2][(i & 3) * 8 + 2 * e]), __uint_as_float(g[i >> 2][(i & 3) * 8 + 2 * e + 1]));
+                        if (row_ok) __stcg(to + i, make_uint4(v[0], v[1], v[2], v[3]));
+                    }
+                } else {
+                    uint32_t v[kHalf / 2];
+#pragma unroll
+                    for (int e = 0; e < kHalf / 2; ++e)
+                        v[e] = pack_half2(__uint_as_float(g[e >> 4][(2 * e) & 31]), __uint_as_float(g[e >> 4][(2 * e + 1) & 31]));
+                    if constexpr (!kClusters) {
+                        uint4* const po = a.part_o + static_cast<int64_t>(it.place) * (D / 8) * kBM + r + x * (kHalf / 8) * kBM;
+                        float* const ml = reinterpret_cast<float*>(a.part_ml + static_cast<int64_t>(it.place) * kBM + r);
+                        if (row_ok) {
+#pragma unroll
+                            for (int i = 0; i < kHalf / 8; ++i)
+                                __stcg(po + i * kBM, make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
+                            if (x == 0) {
+                                __stcg(reinterpret_cast<float2*>(ml), make_float2(m_tot, l_tot));
+                                __stcg(ml + 2, l_tot * scale);
+                            } else {
+                                __stcg(ml + 3, l_tot * scale);
+                            }
+                        }
+                    } else if (it.row_base + (r & ~31) < it.M) {
+                        const uint4 ml = make_uint4(__float_as_uint(m_tot), __float_as_uint(l_tot), __float_as_uint(l_tot * scale), 0u);
+#pragma unroll
+                        for (int i = 0; i < kHalf / 16; ++i) {
+                            const int q = (warp & 3) * (D / 16) + x * (D / 32) + i, to = static_cast<unsigned>(q * a.cluster) / chunks_of(D);
+                            // (with the first of the chunks that go to a CTA)
+                            const bool with_rows = i == 0 || static_cast<unsigned>((q - 1) * a.cluster) / chunks_of(D) != to;
+                            const uint4 v0 = make_uint4(v[8 * i], v[8 * i + 1], v[8 * i + 2], v[8 * i + 3]);
+                            const uint4 v1 = make_uint4(v[8 * i + 4], v[8 * i + 5], v[8 * i + 6], v[8 * i + 7]);
+                            if (to == rank) {
+                                uint4* const p = reinterpret_cast<uint4*>(base_ptr + S::kOffStage + lane * 16 + rank * a.chunk_step +
+                                                                          (q - chunk_at(a, rank)) * kSlotBytes);
+                                p[0] = v0, p[32] = v1;
+                                if (with_rows) p[64] = ml;
+                            } else {
+                                store_async(there[i], v0, meet[i]);
+                                store_async(there[i] + 512, v1, meet[i]);
+                                if (with_rows) store_async(there[i] + kChunkBytes, ml, meet[i]);
+                            }
+                        }
                     }
                 }
             }
 
-            if (a.cluster > 1 && !direct) {
-                // ---- every CTA of the cluster says that its partial is written (a warp at a time), and merges
-                // a share of all of them ------------------------------------------------------------------
+            if (kClusters && !direct) {
+                // ---- the CTA's warps have left their own parts, the other CTAs' bytes are counted; then it merges its
+                // share of all of them ----------------------------------------------------------------------
+                wait_free();  // (a CTA without tiles has not waited yet)
+                if (!alive) break;
                 __syncwarp();
-                if (lane < a.cluster) mbar_arrive_remote(bar(bar_meet()), lane);
+                const int q0 = chunk_at(a, rank), q1 = chunk_at(a, rank + 1);
+                if (warp == 0) {
+                    const int q = q0 + lane;
+                    const bool own = q < q1 && it.row_base + q / (D / 16) * 32 < it.M;
+                    const bool rows = own && (lane == 0 || q % (D / 32) == 0);
+                    const int senders = it.active - (n_tiles > 0 ? 1 : 0);
+                    const int bytes = senders * __reduce_add_sync(kFull, (own ? kChunkBytes : 0) + (rows ? kRowBytes : 0));
+                    if (lane == 0) mbar_expect_tx(bar(bar_meet()), static_cast<uint32_t>(bytes));
+                } else if (lane == 0) {
+                    mbar_arrive(bar(bar_meet()));
+                }
+                MergeAt m = merge_at<D, kQByTma>(a, it, q0 + warp, q0, lane, G);
+                asm volatile("" ::"r"(m.data), "r"(m.rows), "l"(m.out));  // (computed while the bytes are on their way)
                 alive = __all_sync(kFull, cluster_bar_wait(bar(bar_meet()), meets & 1u, abort_flag));
                 if (!alive) break;
-                const unsigned place0 = static_cast<unsigned>(cluster_id * a.cluster) + (meets & 1u) * gridDim.x;
-                if (__builtin_expect(it.pieces == 1, 1)) {
-                    merge_partials<D, false>(a, it, place0, it.active, rank, tid, G, 0u);
-                } else {
-                    merge_partials<D, true>(a, it, place0, it.active, rank, tid, G, static_cast<unsigned>(cluster_id));
-                    merge_pieces<D>(a, it, rank, tid, G);
+                const unsigned char* const stage = base_ptr + S::kOffStage;
+                const bool whole = kForm == kWhole || it.pieces == 1;
+#pragma unroll 1
+                while (m.q < q1) {
+                    if (kForm == kCut && !whole) merge_chunk<D, true>(a, it, stage, m, lane, static_cast<unsigned>(cluster_id));
+                    else merge_chunk<D, false>(a, it, stage, m, lane, 0u);
+                    if (m.q + kPieceWarps >= q1) break;
+                    m = merge_at<D, kQByTma>(a, it, m.q + kPieceWarps, q0, lane, G);
                 }
+                if (kForm == kCut && !whole) merge_pieces<D, kQByTma>(a, it, rank, tid, G);
                 ++meets;
+                if (i + 1 < n_items) {
+                    __syncwarp();
+                    if (lane < a.cluster) mbar_arrive_remote(bar(bar_free()), lane);
+                    in_use = true;
+                }
             }
             if (n_tiles > 0) {
                 // (long complete: only keeps a thread from running an item ahead of the others)
-                alive = warp_wait(bar(bar_item()), items_run & 1u, abort_flag);
+                if (i + 1 < n_items) alive = warp_wait(bar(bar_item()), items_run & 1u, abort_flag);
                 ++items_run;
             }
         }
+        if (kClusters && alive) wait_free();  // (nobody arrives at a CTA that has left)
     }
 
     // ---- tear-down: every role arrives here, whatever happened ------------------------------
@@ -1555,7 +1668,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
     }
     // A CTA that has met the others has received their last arrival and may leave.  Where a wait has run
     // out, nobody leaves while another CTA of the cluster may still arrive on its barriers.
-    if (a.cluster > 1 && !alive) {
+    if (kClusters && !alive) {
         cluster_arrive();
         cluster_wait();
     }
@@ -1849,18 +1962,32 @@ struct Residency {
 std::mutex g_residency_mu;
 Residency g_residency[2][64];  // [head dim 64, 128][device]
 
+// Q tiles come by TMA where a row tile is whole tokens.
+bool group_by_tma(int G) { return G <= kBM && kBM % G == 0; }
+
+using AttnKernel = void (*)(AttnArgs, CUtensorMap, CUtensorMap, CUtensorMap);
+template <int D>
+AttnKernel form_of(int form, bool q_by_tma) {
+    switch (form) {
+        case kSingles: return q_by_tma ? tree_attention_kernel<D, kSingles, true> : tree_attention_kernel<D, kSingles, false>;
+        case kWhole: return q_by_tma ? tree_attention_kernel<D, kWhole, true> : tree_attention_kernel<D, kWhole, false>;
+        default: return q_by_tma ? tree_attention_kernel<D, kCut, true> : tree_attention_kernel<D, kCut, false>;
+    }
+}
+
 template <int D>
 cudaError_t launch_for_dim(const resps_ctx* ctx, const AttnArgs& a, int grid, const CUtensorMap& mk, const CUtensorMap& mv,
                            const CUtensorMap& mq, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid), cfg.blockDim = dim3(kAttnThreads), cfg.dynamicSmemBytes = Smem<D>::kBytes, cfg.stream = st;
+    cfg.gridDim = dim3(grid), cfg.blockDim = dim3(kAttnThreads), cfg.stream = st;
+    cfg.dynamicSmemBytes = a.cluster > 1 ? Smem<D>::kClusterBytes : Smem<D>::kBytes;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = static_cast<unsigned>(a.cluster), attr[1].val.clusterDim.y = 1, attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr, cfg.numAttrs = a.cluster > 1 ? 2 : 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, tree_attention_kernel<D>, a, mk, mv, mq);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, form_of<D>(a.cluster == 1 ? kSingles : a.may_cut ? kCut : kWhole, a.q_by_tma != 0), a, mk, mv, mq);
     if (e != cudaSuccess || a.cluster > 1) return e;
     // the units of work of the largest trees, at most one resident round of CTAs
     const int64_t units = static_cast<int64_t>(a.batch) * a.Hkv * ((a.max_tt * (a.Hq / a.Hkv) + kBM - 1) / kBM) * (D / 8 / kCombPieces);
@@ -1869,9 +1996,12 @@ cudaError_t launch_for_dim(const resps_ctx* ctx, const AttnArgs& a, int grid, co
 }
 
 template <int D>
-cudaError_t setup_for_dim(int device, int sm_count, int* clusters) {
-    cudaError_t e = cudaFuncSetAttribute(tree_attention_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<D>::kBytes);
-    if (e != cudaSuccess) return e;
+cudaError_t setup_for_dim(int device, int sm_count, bool q_by_tma, int* clusters) {
+    cudaError_t e = cudaSuccess;
+    for (int form : {kSingles, kWhole, kCut}) {
+        e = cudaFuncSetAttribute(form_of<D>(form, q_by_tma), cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<D>::kClusterBytes);
+        if (e != cudaSuccess) return e;
+    }
     e = cudaFuncSetAttribute(attention_combine_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombChunkMost * kCombSlotBytes);
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lock(g_residency_mu);
@@ -1882,13 +2012,13 @@ cudaError_t setup_for_dim(int device, int sm_count, int* clusters) {
         for (int c = 2; c <= kMaxCluster; ++c) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(static_cast<unsigned>(sm_count / c * c)), cfg.blockDim = dim3(kAttnThreads);
-            cfg.dynamicSmemBytes = Smem<D>::kBytes;
+            cfg.dynamicSmemBytes = Smem<D>::kClusterBytes;
             cudaLaunchAttribute attr[1];
             attr[0].id = cudaLaunchAttributeClusterDimension;
             attr[0].val.clusterDim.x = static_cast<unsigned>(c), attr[0].val.clusterDim.y = 1, attr[0].val.clusterDim.z = 1;
             cfg.attrs = attr, cfg.numAttrs = 1;
             int n = 0;
-            e = cudaOccupancyMaxActiveClusters(&n, tree_attention_kernel<D>, &cfg);
+            e = cudaOccupancyMaxActiveClusters(&n, form_of<D>(kWhole, q_by_tma), &cfg);
             if (e != cudaSuccess) return e;
             r.clusters[c] = std::min(n, kMaxGrid / c);
         }
@@ -1904,8 +2034,9 @@ cudaError_t attention_setup(resps_ctx* ctx) {
     HostState* hs = new (std::nothrow) HostState();
     if (!hs) return cudaErrorMemoryAllocation;
     ctx->attn_host = hs;
-    return ctx->shape.head_dim == 128 ? setup_for_dim<128>(ctx->device, ctx->sm_count, hs->resident)
-                                      : setup_for_dim<64>(ctx->device, ctx->sm_count, hs->resident);
+    const bool q_by_tma = group_by_tma(ctx->shape.n_q_heads / ctx->shape.n_kv_heads);
+    return ctx->shape.head_dim == 128 ? setup_for_dim<128>(ctx->device, ctx->sm_count, q_by_tma, hs->resident)
+                                      : setup_for_dim<64>(ctx->device, ctx->sm_count, q_by_tma, hs->resident);
 }
 
 void attention_teardown(resps_ctx* ctx) {
@@ -1950,7 +2081,9 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
     a.test_drop = w.test_drop;
     const int D = ctx->shape.head_dim;
     const int G = a.Hq / a.Hkv;
-    a.q_by_tma = (G <= kBM && kBM % G == 0) ? 1 : 0;
+    a.q_by_tma = group_by_tma(G) ? 1 : 0;
+    a.log2_group = 0;
+    while ((2 << a.log2_group) <= G) ++a.log2_group;
     HostState* hs = host_state(ctx);
     std::lock_guard<std::mutex> lock(hs->mu);
     // the most groups of a tree this context builds (attention over larger ones is correct, and slower)
@@ -1959,10 +2092,12 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
     if (w.attn_cluster > 0) a.cluster = forced_cluster(hs->resident, std::min(w.attn_cluster, kMaxCluster), groups);
     a.clusters = a.cluster > 1 ? groups : hs->resident[1];
     const int grid = a.clusters * a.cluster;
-    // the pieces of cut groups lie behind the two places of every CTA (72 bytes of a unit against 32 in a place)
-    a.may_cut = a.cluster > 1 && groups > batch * a.Hkv && 2 * grid + (9 * a.clusters + 3) / 4 <= a.max_items &&
+    a.chunk_first = 0, a.chunk_step = chunks_most(D, a.cluster) * kSlotBytes;
+    for (int c = 0; c <= a.cluster; ++c) a.chunk_first |= static_cast<unsigned long long>(first_chunk(D, a.cluster, c)) << (7 * c);
+    // the pieces of cut groups lie where the two-kernel modes have partials (72 bytes a unit against 32)
+    a.may_cut = a.cluster > 1 && groups > batch * a.Hkv && (9 * a.clusters + 3) / 4 <= a.max_items &&
                 (w.attn_stream > 0 || (w.attn_stream < 0 && (capacity + kBN - 1) / kBN > kPieceTiles * a.cluster)) ? 1 : 0;
-    a.piece_acc = reinterpret_cast<float4*>(a.part_o + static_cast<int64_t>(2 * grid) * (D / 8) * kBM);
+    a.piece_acc = reinterpret_cast<float4*>(a.part_o);
     a.piece_ml = reinterpret_cast<float2*>(a.piece_acc + static_cast<int64_t>(a.clusters) * 4 * kBM * (D / 16));
     if (w.attn_rounds > 0 && a.cluster == 1) a.clusters = std::max(1, a.clusters / w.attn_rounds);
     // one resident round of units with room for all of a group's partials, else more CTAs per SM

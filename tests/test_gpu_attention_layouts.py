@@ -57,6 +57,25 @@ def test_cut_groups_keep_values_beyond_fp16():
     _attention_case(6, 16, 2, 128, 3000, cap=3200, seed=3, v_scale=3.0e5, debug=[(binding.RESPS_DEBUG_ATTN_CLUSTER, 4)])
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("cluster", [2, 3, 5, 7, 8])
+def test_clusters_with_several_items(cluster, D):
+    """Trees larger than the context's limits: a cluster takes row tile after row tile, its CTAs' staging is used again
+    (full tiles, a tile of 4 rows, a group of a single key tile, which one CTA of the cluster does alone)."""
+    _, binding, _ = _imports()
+    debug = [(binding.RESPS_DEBUG_ATTN_CLUSTER, cluster)]
+    _attention_case(n=[128, 33, 3], Hq=8, Hkv=2, D=D, L=[700, 1100, 20], B=3, cap=1280, seed=cluster, poison=True, debug=debug, max_k=2,
+                    max_depth=2)
+    _attention_case(n=[90, 19], Hq=7, Hkv=1, D=D, L=[300, 64], B=2, cap=448, seed=cluster, poison=True, debug=debug, max_k=2, max_depth=2)
+
+
+@pytest.mark.parametrize("cluster", [2, 3, 6, 8])
+@pytest.mark.parametrize("n,Hq", [(5, 12), (60, 16)])
+def test_clusters_keep_values_beyond_fp16(n, Hq, cluster):
+    _, binding, _ = _imports()
+    _attention_case(n, Hq, 4, 128, 900, cap=1024, seed=cluster, v_scale=3.0e5, debug=[(binding.RESPS_DEBUG_ATTN_CLUSTER, cluster)])
+
+
 @pytest.mark.parametrize("cap", [1216, 9408])
 @pytest.mark.parametrize("n", [12, 40, 128])
 def test_trees_of_one_context_in_caches_with_and_without_room(n, cap):
