@@ -1043,37 +1043,29 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
     read_plan();
 
     // ---- one-time set-up ---------------------------------------------------------------
-    // (the producers' barriers by the producers themselves: their first copies go out before the CTA meets)
-    if (warp >= kProducerWarp && lane == 0 && (warp == kProducerWarp || warp == kVProducerWarp)) {
-        const bool is_v = warp == kVProducerWarp;
-#pragma unroll 1
-        for (int s = 0; s < kStagesK; ++s) {  // a tile belongs to one lane
-            mbar_init(bar(is_v ? bar_vfull(s) : bar_kfull(s)), 1);
-            mbar_init(bar(is_v ? bar_vempty(s) : bar_kempty(s)), 1);
+    // A lane a barrier, by several warps side by side (one thread after the other took 450 clocks longer); the producers'
+    // barriers by the producers themselves: their first copies go out before the cluster meets.
+    const bool is_producer = warp == kProducerWarp || warp == kVProducerWarp;
+    {
+        static_assert(kStagesK == 4 && kStagesV == 4 && kLanes == 2, "places by lane");
+        int i = -1;
+        uint32_t count = 1;
+        if (is_producer) {
+            if (lane < 8) i = (lane & 3) + (lane >> 2) * 8 + (warp == kVProducerWarp ? 4 : 0);  // full and empty, K's and V's in turn
+            if (warp == kProducerWarp && (lane >> 1) == 4) i = bar_qfull() + (lane & 1), count = lane & 1 ? kLanes : kQByTma ? 1 : kSoftmaxThreads;
+        } else if (warp == 5) {
+            if (lane < 8) i = bar_sfull(lane >> 2, lane & 1) + (lane & 2) * 2;  // S, P V
+        } else if (warp == 6) {
+            if (lane < 4) i = bar_pfull(lane >> 1, lane & 1), count = kBM / 32;  // one arrival per warp
+        } else if (warp == 7) {
+            if (lane < 4) i = bar_item() + lane, count = lane < 2 ? kSoftmaxThreads : lane == 2 ? kPieceWarps : a.cluster * kPieceWarps;
         }
-        if (!is_v) {
-            mbar_init(bar(bar_qfull()), kQByTma ? 1 : kSoftmaxThreads);
-            mbar_init(bar(bar_qempty()), kLanes);
+        if (i >= 0) {
+            mbar_init(bar(i), count);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        fence_proxy_async();
-    }
-    if (tid == 0) {
-        *abort_flag = 0;
-#pragma unroll 1
-        for (int m = 0; m < kLanes; ++m) {
-#pragma unroll 1
-            for (int bf = 0; bf < 2; ++bf) {
-                mbar_init(bar(bar_sfull(m, bf)), 1);
-                mbar_init(bar(bar_pfull(m, bf)), kBM / 32);  // one arrival per warp
-                mbar_init(bar(bar_pvdone(m, bf)), 1);
-            }
-        }
-        mbar_init(bar(bar_item()), kSoftmaxThreads);
-        mbar_init(bar(bar_merge()), kSoftmaxThreads);
-        mbar_init(bar(bar_meet()), kPieceWarps);
-        mbar_init(bar(bar_free()), a.cluster * kPieceWarps);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if (is_producer) fence_proxy_async();
+        if (tid == 0) *abort_flag = 0;
     }
     if (warp == kMmaWarp0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -1082,17 +1074,21 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    if (warp == kProducerWarp && lane == 0) {
+    if (warp == kMmaWarp0 + 1 && lane == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_k) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_v) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_q) : "memory");
     }
-    // Barriers and the TMEM address are visible to the whole cluster behind this pair (other CTAs
-    // arrive on this one's barriers).  Everything so far touches no global memory but the work list, so
-    // under programmatic dependent launch it overlaps the tail of the preceding kernel.
+    // Everything so far touches no global memory but the work list, so under programmatic dependent launch it overlaps the
+    // tail of the preceding kernel.  The barriers are visible in the cluster behind the pair of arrival and wait (other CTAs
+    // arrive on this one's barriers), what else there is in the CTA behind its own barrier: the arrival need not release
+    // anything (one that does waits for the work list's loads, 500 to 900 clocks; from a CTA's first instruction to here
+    // 1800 clocks before, for the CTAs that start last on the way of every call).
     tc_fence_before();
     __syncwarp();
-    cluster_arrive();
+    if constexpr (kClusters) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+    __syncthreads();
+    tc_fence_after();
     pdl_wait();
     pdl_launch_dependents();
     auto load_q = [&](const Item& it) {
@@ -1115,8 +1111,7 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
         if (!is_v && kQByTma) load_q(first_it);
     }
     __syncwarp();
-    cluster_wait();
-    tc_fence_after();
+    if constexpr (kClusters) cluster_wait();
     constexpr uint32_t tmem = 0;  // all columns are allocated: they begin at 0
     // The list must still describe the step parameters it is used with (the caller changes them only
     // through the library, or asks for a new list): one thread compares its item's sequence.
