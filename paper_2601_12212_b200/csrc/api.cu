@@ -183,7 +183,7 @@ int resps_debug_set(resps_ctx* ctx, int key, int value) {
     resps::Workspace& w = ctx->ws;
     switch (key) {
         case RESPS_DEBUG_ATTN_ROUNDS: w.attn_rounds = std::max(0, value); break;
-        case RESPS_DEBUG_ATTN_MIN_TILES: w.attn_min_tiles = std::max(1, value); break;
+        case RESPS_DEBUG_ATTN_MIN_TILES: w.attn_min_tiles = std::max(0, value); break;
         case RESPS_DEBUG_ATTN_SINGLE: w.attn_stream = std::min(1 << 26, std::max(0, value)); break;
         case RESPS_DEBUG_ATTN_CLUSTER: w.attn_cluster = std::max(0, value); break;
         case RESPS_DEBUG_ATTN_EVEN_ROUNDS: w.attn_even_rounds = std::max(0, value); break;

@@ -153,6 +153,7 @@ struct AttnArgs {
     int rounds;       // mode even: 0: own choice; else this many rounds (tests)
     int l2_tiles;     // K and V of more key tiles (of a KV head) than this do not stay in L2
     int min_tiles;    // fewest key tiles a CTA is given
+    int alone_tiles;  // mode whole: up to so many key tiles of an item stay in one CTA
     int q_by_tma;     // 1: Q tiles come by TMA (128 % (Hq/Hkv) == 0), 0: by plain loads
     int log2_group;   // of Hq/Hkv, where Q tiles come by TMA
     int plan_after_wait;  // 1: the work list was written by the kernel just before this one
@@ -173,12 +174,15 @@ __host__ __device__ __forceinline__ int ceil_div(int a, int b) {  // a >= 0, b >
     return static_cast<int>((static_cast<unsigned>(a) + static_cast<unsigned>(b) - 1u) / static_cast<unsigned>(b));
 }
 
-// CTAs of a cluster that get key tiles of an item with `tiles` of them.  A lane that takes one tile more
-// costs about 1 us, the exchange between the CTAs about 2.5 us: up to five tiles stay in one CTA, beyond
-// that a CTA gets at least one tile per lane (min_tiles).
-__device__ __forceinline__ int active_ctas(int tiles, int cluster, int min_tiles) {
-    if (tiles <= 2 * min_tiles + 1) return 1;
-    return min(cluster, ceil_div(tiles, min_tiles));
+// CTAs of a cluster that get key tiles of an item with `tiles` of them: the fewest among which the fullest has as few
+// tiles as it can.  Splitting costs the exchange, about 1.2 us, and saves a tile's 0.5 to 1 us; in a CTA with one tile,
+// whose second lane is idle, that one takes less.  In us a layer, one CTA / as many as there are tiles, 8B shape: 32 nodes
+// (clusters of 8) 2 tiles 6.75 / 5.75, 3 7.17 / 5.94, 4 7.7 / 5.95, 5 8.2 / 6.1; 60 nodes (6) 6.6 / 6.2, 7.0 / 6.4,
+// 7.7 / 6.6, 8.4 / 6.9; 128 nodes (4) 3 tiles 8.15 / 7.2; 13B shape (3) 6.7 / 7.0, 7.2 / 7.6, 8.0 / 7.8 (4); head dimension 64
+// (8) 4.87 / 5.05, 5.3 / 5.2, 5.8 / 5.2.  7 tiles in a cluster of 6: four CTAs 7.4, six 7.6.
+__device__ __forceinline__ int active_ctas(int tiles, int cluster, int min_tiles, int alone_tiles) {
+    if (tiles <= alone_tiles) return 1;
+    return ceil_div(tiles, max(ceil_div(tiles, cluster), min_tiles));
 }
 
 // ---------------------------------------------------------------------------- work list
@@ -468,7 +472,7 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
                     t0 = kt * piece / pieces, kt = kt * (piece + 1) / pieces - t0;
                 }
                 PlanItem p = item_of(b, local);
-                const int act = active_ctas(kt, a.cluster, a.min_tiles);
+                const int act = active_ctas(kt, a.cluster, a.min_tiles, a.alone_tiles);
                 p.tile_active = (p.tile_active & 0xFFFF) | (act << 16);
                 p.pieces = pieces | (piece << 16), p.place = item - piece;
                 p.t_end = t0;
@@ -1914,16 +1918,15 @@ bool cached_map(HostState* hs, const MapKey& key, int D, CUtensorMap* out) {
 // without work: clusters of C CTAs for `groups` (smaller trees have their groups cut over the clusters left).  For kt
 // key tiles that is kt (1 / C - groups / SMs) tiles a CTA.  Measured, whole / two kernels, in us a layer (largest tree
 // of each context, prefix 1024, 2048, 4096, 8192):
-//    8 groups, C = 8    9.9 /  9.9   11.2 / 11.3   13.7 / 13.3   19.0 / 16.7
-//   12         8       11.3 / 11.3   12.8 / 12.5   15.3 / 14.4   20.6 / 18.7   (Q by plain loads)
-//   16         6        9.6 / 10.6   11.5 / 12.1   14.5 / 14.5   21.6 / 19.4
-//   24         6       10.7 / 12.3   12.5 / 14.3   16.5 / 17.3   24.4 / 24.8
-//   32         4       11.4 / 12.7   13.8 / 15.0   18.6 / 20.0   28.7 / 30.5
-//   40         3       12.1 / 13.2   15.5 / 16.6   21.9 / 23.4   35.6 / 37.3   (50.0 / 49.9 at 12 288)
-// The two meet at 1000 to 2000 keys with 8 and 12 groups, at 4096 with 16, at 9000 and more with 24 to 40: at 1 to 12
-// tiles lost, so no one constant is right for all.  With 5, at the longest prefix that it admits, mode whole is up to
-// 9 % behind (8 and 12 groups); below that prefix, where a call usually is, up to 13 % ahead.
-constexpr double kWholeGainTiles = 5.0;
+//    8 groups, C = 8    7.8 /  9.1    9.1 / 10.5   11.4 / 12.4   16.0 / 14.9
+//   12         8        9.5 / 10.6   10.7 / 11.6   12.6 / 13.3   16.9 / 16.4   (Q by plain loads)
+//   16         6        8.3 /  9.7    9.8 / 11.0   12.6 / 13.2   18.5 / 17.0
+//   24         5        9.0 / 11.4   10.5 / 13.3   14.3 / 16.0   20.7 / 21.7   (28.4 / 28.3 at 12 288)
+//   32         4        9.4 / 11.8   11.5 / 13.8   15.8 / 17.9   24.8 / 26.1   (35.0 / 36.2)
+//   40         3       11.1 / 11.9   14.0 / 14.9   20.1 / 21.1   33.7 / 35.3   (47.8 / 48.0)
+// The two meet at 5 tiles lost with 12 and 16 groups, at 6 to 7 with 8, 24 and 32, at 12 with 40.  With 7, at the longest
+// prefix that it admits, mode whole is up to 5 % behind; below that prefix, where a call usually is, up to 24 % ahead.
+constexpr double kWholeGainTiles = 7.0;
 // In a batch the cache may hold one long sequence among short ones, which only its own clusters work on.  (Four equal
 // sequences of 8 groups: 12.3 / 13.8 us at 1024 keys, 43.2 / 45.4 at 12 288.)
 int choose_cluster(const int* resident, int sm_count, int groups, int batch, int kt_most) {
@@ -2065,7 +2068,7 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
     a.Hq = ctx->shape.n_q_heads, a.Hkv = ctx->shape.n_kv_heads, a.max_tt = ctx->shape.max_tt;
     a.part_o = reinterpret_cast<uint4*>(w.attn_part_o), a.part_ml = w.attn_part_ml;
     a.max_items = w.attn_max_items;
-    a.min_tiles = w.attn_min_tiles, a.status = w.status;
+    a.status = w.status;
     a.piece_count = w.attn_count;
     unsigned char* plan = w.attn_plan;
     a.plan_head = reinterpret_cast<PlanHead*>(plan), plan += sizeof(PlanHead);
@@ -2086,6 +2089,8 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
     a.cluster = choose_cluster(hs->resident, ctx->sm_count, groups, batch, static_cast<int>((capacity + kBN - 1) / kBN));
     if (w.attn_cluster > 0) a.cluster = forced_cluster(hs->resident, std::min(w.attn_cluster, kMaxCluster), groups);
     a.clusters = a.cluster > 1 ? groups : hs->resident[1];
+    a.min_tiles = w.attn_min_tiles > 0 ? w.attn_min_tiles : a.cluster > 1 ? 1 : 2;
+    a.alone_tiles = a.cluster < 4 ? 3 : D == 64 ? 2 : 1;
     const int grid = a.clusters * a.cluster;
     a.chunk_first = 0, a.chunk_step = chunks_most(D, a.cluster) * kSlotBytes;
     for (int c = 0; c <= a.cluster; ++c) a.chunk_first |= static_cast<unsigned long long>(first_chunk(D, a.cluster, c)) << (7 * c);

@@ -44,7 +44,7 @@ struct Workspace {
     double* samp_scratch = nullptr;          // acceptance under sampling: partial sums, then (p, q) of every token and sequence
     unsigned int* amax_seq_counter = nullptr;  // [max_batch] arg-max CTAs of a sequence that have delivered (self-resetting)
     // attention
-    int attn_min_tiles = 2;     // fewest key tiles a CTA of a cluster is given
+    int attn_min_tiles = 0;     // > 0: fewest key tiles a CTA is given (tests)
     int attn_stream = -1;       // 0: never equal splits per group, > 0: always where they fit (tests)
     int attn_cluster = 0;       // > 0: CTAs per cluster (tests)
     int attn_even_rounds = 0;   // > 0: rounds of equal splits (tests)

@@ -69,6 +69,18 @@ def test_clusters_with_several_items(cluster, D):
     _attention_case(n=[90, 19], Hq=7, Hkv=1, D=D, L=[300, 64], B=2, cap=448, seed=cluster, poison=True, debug=debug, max_k=2, max_depth=2)
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("cluster", [2, 3, 4, 8])
+def test_few_key_tiles_in_a_cluster(cluster, D):
+    """One to nine key tiles: in one CTA, a tile a CTA, CTAs without any; the last tile full and with a single key."""
+    _, binding, _ = _imports()
+    for tiles in (1, 2, 3, 4, 5, 9):
+        for last in (1, 64):
+            n = 9 if tiles > 1 else 1
+            _attention_case(n, 16, 2, D, 64 * (tiles - 1) + last - n, cap=640, seed=tiles, poison=True,
+                            debug=[(binding.RESPS_DEBUG_ATTN_CLUSTER, cluster)])
+
+
 @pytest.mark.parametrize("cluster", [2, 3, 6, 8])
 @pytest.mark.parametrize("n,Hq", [(5, 12), (60, 16)])
 def test_clusters_keep_values_beyond_fp16(n, Hq, cluster):
