@@ -95,11 +95,11 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 // different times: where K and V do not stay in L2 meanwhile, every row tile reads them from HBM again, and 148 CTAs
 // with 32 KB per 0.62 us ask for more than HBM has.  So the share of mode stream counts kRereadNum / kRereadDen times as
 // much beyond `l2_tiles` key tiles (all KV heads of the sequences with several row tiles; head dimension 128).  In us a
-// call, stream against the best of even: 8 x 24 000 keys, 80 nodes, 8B shape 445 / 378 (four rounds); 5 x 28 000 keys, 40-96
-// nodes, 56 query heads 504 / 423 (four); 4 x 8192 keys, 96 nodes, 70B shape 151 / 138 (four); 16 x 4096 keys, 64 nodes, 8B
-// shape 112 / 102 (two); 32 000 keys, 128 nodes 97 / 92 (two; one round 102); 12 ragged sequences up to 16 000 keys, 28 query
-// heads 127 / 109 (three).  With K and V of up to 67 MB the modes are within 3 %: 8192 keys, 128 nodes 31.2 / 29.9, 8 x 2048
-// keys, 64 nodes 29.6 / 29.7.
+// call, stream against the best of even: 8 x 24 000 keys, 80 nodes, 8B shape 416 / 351 (four rounds); 5 x 28 000 keys, 40-96
+// nodes, 56 query heads 469 / 391 (four); 4 x 8192 keys, 96 nodes, 70B shape 141 / 128 (four); 16 x 4096 keys, 64 nodes, 8B
+// shape 108 / 94 (two); 32 000 keys, 128 nodes 92 / 82 (one); 12 ragged sequences up to 16 000 keys, 28 query
+// heads 108 / 88 (three).  With K and V that stay in L2: 8192 keys, 128 nodes 28.0 / 26.3, 8 x 2048 keys,
+// 64 nodes 27.4 / 27.6.
 constexpr int kModeWhole = 0, kModeEven = 1, kModeStream = 2;
 
 struct alignas(16) PlanHead {
@@ -947,10 +947,10 @@ __device__ __forceinline__ void merge_chunk(const AttnArgs& a, const Item& it, c
 }
 // A group that is cut over several clusters: the same warp of the same CTA of each has merged the same units.  It
 // says so (nobody waits), and the one that finds that all others have done so merges the pieces: two round trips to L2
-// more on the way of a cut group, 2.5 to 3 us, against 0.7 us for each key tile that it takes off a CTA (kPieceTiles).
+// more on the way of a cut group, 2.5 to 3 us, against 0.6 us for each key tile that it takes off a CTA (kPieceTiles).
 // Under a context for 128 nodes on the 8B shape (32 clusters of 4), in us a layer uncut / cut / the two kernels with the
-// same context: 16 nodes at 4096 keys 16.5 / 14.2 / 15.5, at 8192 26.3 / 17.3 / 18.7, at 12 288 35.6 / 19.9 / 21.5;
-// 64 nodes 17.1 / 15.8 / 16.7, 26.8 / 21.0 / 21.6, 36.2 / 25.9 / 26.0.
+// same context: 16 nodes at 4096 keys 14.6 / 12.9 / 14.1, at 8192 22.7 / 15.4 / 16.7, at 12 288 30.9 / 17.7 / 19.2;
+// 64 nodes 15.0 / 13.7 / 15.6, 23.1 / 18.4 / 19.4, 31.2 / 22.6 / 23.2.
 template <int D, bool kPow2>
 __device__ __forceinline__ void merge_pieces(const AttnArgs& a, const Item& it, int rank, int tid, int G) {
     constexpr unsigned kUnits = kBM * (D / 16);
@@ -1928,7 +1928,7 @@ bool cached_map(HostState* hs, const MapKey& key, int D, CUtensorMap* out) {
 // prefix that it admits, mode whole is up to 5 % behind; below that prefix, where a call usually is, up to 24 % ahead.
 constexpr double kWholeGainTiles = 7.0;
 // In a batch the cache may hold one long sequence among short ones, which only its own clusters work on.  (Four equal
-// sequences of 8 groups: 12.3 / 13.8 us at 1024 keys, 43.2 / 45.4 at 12 288.)
+// sequences of 8 groups: 10.4 / 12.9 us at 1024 keys, 40.5 / 43.6 at 12 288.)
 int choose_cluster(const int* resident, int sm_count, int groups, int batch, int kt_most) {
     for (int c : {8, 6, 4, 3, 2}) {
         if (resident[c] < groups) continue;
