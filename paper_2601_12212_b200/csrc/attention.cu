@@ -153,7 +153,6 @@ struct AttnArgs {
     int rounds;       // mode even: 0: own choice; else this many rounds (tests)
     int l2_tiles;     // K and V of more key tiles (of a KV head) than this do not stay in L2
     int min_tiles;    // fewest key tiles a CTA is given
-    int alone_tiles;  // mode whole: up to so many key tiles of an item stay in one CTA
     int q_by_tma;     // 1: Q tiles come by TMA (128 % (Hq/Hkv) == 0), 0: by plain loads
     int log2_group;   // of Hq/Hkv, where Q tiles come by TMA
     int plan_after_wait;  // 1: the work list was written by the kernel just before this one
@@ -175,13 +174,13 @@ __host__ __device__ __forceinline__ int ceil_div(int a, int b) {  // a >= 0, b >
 }
 
 // CTAs of a cluster that get key tiles of an item with `tiles` of them: the fewest among which the fullest has as few
-// tiles as it can.  Splitting costs the exchange, about 1.2 us, and saves a tile's 0.5 to 1 us; in a CTA with one tile,
-// whose second lane is idle, that one takes less.  In us a layer, one CTA / as many as there are tiles, 8B shape: 32 nodes
-// (clusters of 8) 2 tiles 6.75 / 5.75, 3 7.17 / 5.94, 4 7.7 / 5.95, 5 8.2 / 6.1; 60 nodes (6) 6.6 / 6.2, 7.0 / 6.4,
-// 7.7 / 6.6, 8.4 / 6.9; 128 nodes (4) 3 tiles 8.15 / 7.2; 13B shape (3) 6.7 / 7.0, 7.2 / 7.6, 8.0 / 7.8 (4); head dimension 64
-// (8) 4.87 / 5.05, 5.3 / 5.2, 5.8 / 5.2.  7 tiles in a cluster of 6: four CTAs 7.4, six 7.6.
-__device__ __forceinline__ int active_ctas(int tiles, int cluster, int min_tiles, int alone_tiles) {
-    if (tiles <= alone_tiles) return 1;
+// tiles as it can (7 tiles in a cluster of 6: four CTAs 7.4 us a layer, six 7.6).  Up to kAloneTiles tiles stay in one CTA,
+// which rounds nothing before O: split, a layer of the 8B shape with 32 nodes takes 5.9 to 6.1 us instead of 7.2 to 8.2, but
+// its partials would be rounded to fp16; as fp32 they need more code than the calls of all other lengths can bear
+// (8B shape at 1024 keys 8.3 / 8.7).
+constexpr int kAloneTiles = 5;
+__device__ __forceinline__ int active_ctas(int tiles, int cluster, int min_tiles) {
+    if (tiles <= kAloneTiles) return 1;
     return ceil_div(tiles, max(ceil_div(tiles, cluster), min_tiles));
 }
 
@@ -472,7 +471,7 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
                     t0 = kt * piece / pieces, kt = kt * (piece + 1) / pieces - t0;
                 }
                 PlanItem p = item_of(b, local);
-                const int act = active_ctas(kt, a.cluster, a.min_tiles, a.alone_tiles);
+                const int act = active_ctas(kt, a.cluster, a.min_tiles);
                 p.tile_active = (p.tile_active & 0xFFFF) | (act << 16);
                 p.pieces = pieces | (piece << 16), p.place = item - piece;
                 p.t_end = t0;
@@ -1930,7 +1929,7 @@ constexpr double kWholeGainTiles = 7.0;
 // In a batch the cache may hold one long sequence among short ones, which only its own clusters work on.  (Four equal
 // sequences of 8 groups: 10.4 / 12.9 us at 1024 keys, 40.5 / 43.6 at 12 288.)
 int choose_cluster(const int* resident, int sm_count, int groups, int batch, int kt_most) {
-    for (int c : {8, 6, 4, 3, 2}) {
+    for (int c : {8, 6, 5, 4, 3, 2}) {
         if (resident[c] < groups) continue;
         const double lost = 1.0 / c - static_cast<double>(groups / batch) / sm_count;
         if (lost * kt_most <= kWholeGainTiles) return c;
@@ -2090,7 +2089,6 @@ cudaError_t launch_tree_attention(const resps_ctx* ctx, const resps_step* d_step
     if (w.attn_cluster > 0) a.cluster = forced_cluster(hs->resident, std::min(w.attn_cluster, kMaxCluster), groups);
     a.clusters = a.cluster > 1 ? groups : hs->resident[1];
     a.min_tiles = w.attn_min_tiles > 0 ? w.attn_min_tiles : a.cluster > 1 ? 1 : 2;
-    a.alone_tiles = a.cluster < 4 ? 3 : D == 64 ? 2 : 1;
     const int grid = a.clusters * a.cluster;
     a.chunk_first = 0, a.chunk_step = chunks_most(D, a.cluster) * kSlotBytes;
     for (int c = 0; c <= a.cluster; ++c) a.chunk_first |= static_cast<unsigned long long>(first_chunk(D, a.cluster, c)) << (7 * c);
