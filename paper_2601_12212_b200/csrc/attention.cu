@@ -729,6 +729,15 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         : "r"(taddr)
         : "memory");
 }
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+}
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
@@ -1513,6 +1522,36 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 const float l_tot = l_run * w_self + oth.y * w_oth;
                 const float inv = (l_tot > 0.f) ? 1.f / l_tot : 0.f;
                 w_self *= inv, w_oth *= inv;
+                if (direct) {
+                    // (in 16-column pieces, a loop of few instructions: through the registers of the other case a call of one
+                    // CTA a group took 0.6 us longer)
+                    const int64_t out_row = output_row<kQByTma>(a, it, r, G);
+                    if (row_ok && a.lse && x == 0) a.lse[out_row] = (m_tot + log2f(l_tot)) * 0.6931471805599453f;
+                    const unsigned long long ws2 = pack2(w_self, w_self), wo2 = pack2(w_oth, w_oth);
+                    uint4* to = reinterpret_cast<uint4*>(a.o + out_row * D + x * kHalf);
+#pragma unroll 1
+                    for (int c = 0; c < kHalf; c += 16, to += 2) {
+                        uint32_t r0[16], r1[16], v[8];
+                        tmem_ld16(self_t + c, r0);
+                        tmem_ld16(oth_t + c, r1);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            const unsigned long long s2 = pack2(__uint_as_float(r0[2 * e]), __uint_as_float(r0[2 * e + 1]));
+                            const unsigned long long o2 = pack2(__uint_as_float(r1[2 * e]), __uint_as_float(r1[2 * e + 1]));
+                            float g0, g1;
+                            unpack2(fma2(o2, wo2, fma2(s2, ws2, pack2(0.f, 0.f))), g0, g1);
+                            v[e] = pack_bf16(g0, g1);
+                        }
+                        if (row_ok) {
+                            __stcg(to, make_uint4(v[0], v[1], v[2], v[3]));
+                            __stcg(to + 1, make_uint4(v[4], v[5], v[6], v[7]));
+                        }
+                    }
+                    // O has been read: the next item's P V may overwrite it
+                    tc_fence_before();
+                    mbar_arrive(bar(bar_item()));
+                } else {
                 float scale = 1.f;  // O = Ohat * l * scale, a scale for each half of the columns
                 uint32_t g[kHalf / 32][32];
                 // (a second time where |O / l| of a partial would leave fp16's range: the weights take a scale then)
@@ -1549,19 +1588,6 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                 mbar_arrive(bar(bar_item()));
                 if (kClusters && !direct) wait_free();
                 if (!alive) break;
-                if (direct) {
-                    const int64_t out_row = output_row<kQByTma>(a, it, r, G);
-                    uint4* const to = reinterpret_cast<uint4*>(a.o + out_row * D + x * kHalf);
-                    if (row_ok && a.lse && x == 0) a.lse[out_row] = (m_tot + log2f(l_tot)) * 0.6931471805599453f;
-#pragma unroll
-                    for (int i = 0; i < kHalf / 8; ++i) {
-                        uint32_t v[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            v[e] = pack_bf16(__uint_as_float(g[i >> 2][(i & 3) * 8 + 2 * e]), __uint_as_float(g[i >> 2][(i & 3) * 8 + 2 * e + 1]));
-                        if (row_ok) __stcg(to + i, make_uint4(v[0], v[1], v[2], v[3]));
-                    }
-                } else {
                     uint32_t v[kHalf / 2];
 #pragma unroll
                     for (int e = 0; e < kHalf / 2; ++e)
