@@ -1012,8 +1012,8 @@ __device__ __forceinline__ int cluster_index() {
 // 24 KB takes a clock an instruction, in the next launch too, of 48 KB and more 2.1 clocks wherever it is in its loops.  One
 // kernel for all forms had 76 KB (head dimension 128); these have 39, 55 and 64 with uniform warp indexes, constant base
 // addresses and 32-bit descriptor words.  In us a call before / now, the cluster's exchange included: 8B shape at 1024
-// keys 9.34 / 8.43, 128 nodes at 2048 keys 13.5 / 11.9, 13B shape 15.1 / 14.1, 28 heads of two users 12.6 / 11.3, 70B
-// shape 22.5 / 20.6, 8 ragged sequences 61.3 / 57.4, 32 000 keys 31.3 / 29.8, 4 heads of 64 5.09 / 4.81.
+// keys 9.35 / 7.9, 128 nodes at 2048 keys 13.4 / 11.6, 13B shape 15.1 / 13.6, 28 heads of two users 12.6 / 10.0, 70B
+// shape 22.4 / 20.4, 8 ragged sequences 60.1 / 55.8, 32 000 keys 31.6 / 29.5, 4 heads of 64 5.06 / 4.5.
 enum Form { kSingles, kWhole, kCut };
 template <int D, int kForm, bool kQByTma>
 __global__ void __launch_bounds__(kAttnThreads, 1)
