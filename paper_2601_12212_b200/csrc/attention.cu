@@ -1033,27 +1033,6 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + S::kOffMisc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + S::kOffMisc + 8);
 
-    // The work list was written once for the whole step.  From the second layer on it is at least
-    // two kernels old: this kernel can only have started after its predecessor had started, which
-    // can only have started after every CTA of the kernel before that one had passed its own
-    // dependency wait, i.e. after the kernel that wrote the list had completed and flushed.  (That kernel before
-    // is an attention kernel, or comes behind one: the first call's follows the list's writer at once and signals
-    // its dependents only after its own wait.  The combine kernel signals before its wait.)  So the
-    // list is read before the wait, under the tail of the preceding kernel; only when the list was
-    // written by the kernel immediately before this one does the read have to follow the wait.
-    // Every thread reads the CTA's first item for itself: no role waits for another.
-    int first_item = 0, n_items = 0;
-    Item first_it = {};
-    auto read_plan = [&]() {
-        if (cluster_id < a.clusters) {
-            const int2 c = __ldcg(reinterpret_cast<const int2*>(a.plan_cluster + cluster_id));
-            first_it = load_item(a.plan_first + blockIdx.x, G);
-            first_item = c.x, n_items = c.y;
-        }
-    };
-    if (a.plan_after_wait) pdl_wait();
-    read_plan();
-
     // ---- one-time set-up ---------------------------------------------------------------
     // A lane a barrier, by several warps side by side (one thread after the other took 450 clocks longer); the producers'
     // barriers by the producers themselves: their first copies go out before the cluster meets.
@@ -1090,6 +1069,27 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_k) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_v) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_q) : "memory");
+    }
+    // The work list was written once for the whole step.  From the second layer on it is at least
+    // two kernels old: this kernel can only have started after its predecessor had started, which
+    // can only have started after every CTA of the kernel before that one had passed its own
+    // dependency wait, i.e. after the kernel that wrote the list had completed and flushed.  (That kernel before
+    // is an attention kernel, or comes behind one: the first call's follows the list's writer at once and signals
+    // its dependents only after its own wait.  The combine kernel signals before its wait.)  So the
+    // list is read before the wait, under the tail of the preceding kernel; only when the list was
+    // written by the kernel immediately before this one does the read have to follow the wait.
+    // Behind the set-up, which then overlaps the list's writer too: work list and first layer of the 8B shape at 1024 keys
+    // 10.8 us a call with the wait in front of the set-up, 10.5 so; 4 heads of 64 7.55 / 7.05, 70B shape 24.8 / 24.45; layers
+    // that find the list made 8.0 / 8.0, 4.7 / 4.7, 20.7 / 20.7.  (Read twice, in front of the set-up where the list is old: 10.55,
+    // 7.2, 24.6, and 28 heads 9.4 / 9.3 with a list made.)
+    // Every thread reads the CTA's first item for itself: no role waits for another.
+    if (a.plan_after_wait) pdl_wait();
+    int first_item = 0, n_items = 0;
+    Item first_it = {};
+    if (cluster_id < a.clusters) {
+        const int2 c = __ldcg(reinterpret_cast<const int2*>(a.plan_cluster + cluster_id));
+        first_it = load_item(a.plan_first + blockIdx.x, G);
+        first_item = c.x, n_items = c.y;
     }
     // Everything so far touches no global memory but the work list, so under programmatic dependent launch it overlaps the
     // tail of the preceding kernel.  The barriers are visible in the cluster behind the pair of arrival and wait (other CTAs
