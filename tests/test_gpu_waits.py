@@ -1,9 +1,10 @@
 """Every device-side wait of the library is bounded: when it runs out the kernel flags
 RESPS_STATUS_WAIT_TIMEOUT, finishes its protocol and returns, and the context serves the next call.
 Exercised with the test build of the library (millisecond limits; one copy can be left out so that
-a wait for it really runs out) on tiny single-CTA cases.  Nothing here faults or waits without a
-limit: the skipped copy is simply never issued, every wait for it gives up after about a
-millisecond, and every copy that was issued is waited for before the CTA leaves."""
+a wait for it really runs out) on tiny cases: a single CTA, and clusters whose CTAs wait for one another's
+results.  Nothing here faults or waits without a limit: the skipped copy is simply never issued, every wait
+for it gives up after about a millisecond, every copy that was issued is waited for before the CTA leaves,
+and no CTA leaves while another of its cluster may still send to it."""
 import ctypes
 
 import numpy as np
@@ -65,6 +66,49 @@ def test_attention_wait_runs_out_and_the_context_recovers(waitlib):
     assert ctx.status() == 0
     ref = oracle.tree_attention(q[0, :n], kc[0], vc[0], L, masks[0, :n], 0.125)
     check_attention(bf16_to_f64(do)[0, :n], ref)
+    ctx.close()
+
+
+# A cluster of eight.  Both cases leave out the first V copy of every CTA that has key tiles in its cluster's first item.
+#  meet: one group of 128 rows and nine key tiles, two a CTA: five CTAs wait for the copy; the other three have rows to
+#        merge and wait for bytes that nobody sends.
+#  free: four groups on two clusters.  The first item of the first cluster has 16 rows, so the CTAs without key tiles have
+#        nothing to merge either: they go on to the second item, where the shared memory for it is never released.
+CLUSTERS = {"meet": dict(ns=[8], Ls=[530], Hq=16, max_k=4, max_depth=4), "free": dict(ns=[2, 33], Ls=[520, 1000], Hq=8, max_k=2, max_depth=2)}
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("wait", list(CLUSTERS))
+def test_cluster_waits_run_out_and_the_context_recovers(waitlib, wait, D):
+    import oracle
+    from harness import bf16_to_f64, check_attention, u16_to_bf16_cuda
+    from paper_2601_12212_b200 import synth
+    binding = waitlib
+    ns, Ls, Hq, max_k, max_depth = (CLUSTERS[wait][x] for x in ("ns", "Ls", "Hq", "max_k", "max_depth"))
+    B, Hkv, cap, T = len(ns), 1, 1088, 40
+    ctx = binding.Context(Hq, Hkv, D, 100, max_batch=B, max_tt=T, max_k=max_k, max_depth=max_depth)
+    ctx.debug_set(binding.RESPS_DEBUG_ATTN_CLUSTER, 8)
+    q, kc, vc, masks = (np.concatenate(x) for x in zip(*(_attention_inputs(binding, synth, n, Hq, Hkv, D, L, cap, T)
+                                                         for n, L in zip(ns, Ls))))
+    steps = torch.tensor([[n, 1, 1, L] for n, L in zip(ns, Ls)], dtype=torch.int32, device="cuda")
+    nn = torch.tensor(ns, dtype=torch.int32, device="cuda")
+    dq, dk, dv = u16_to_bf16_cuda(q), u16_to_bf16_cuda(kc), u16_to_bf16_cuda(vc)
+    dm = torch.from_numpy(masks.view(np.int64)).cuda()
+    do = torch.zeros_like(dq)
+
+    def call():
+        binding.resps_tree_attention(ctx, steps, nn, B, dq, do, None, dk, dv, Hkv * cap * D, cap * D, D, cap, dm, 0.125)
+
+    ctx.debug_set(DROP_KEY, DROP_ATTENTION_V)
+    call()
+    torch.cuda.synchronize()                      # the call returns
+    assert ctx.status() & binding.RESPS_STATUS_WAIT_TIMEOUT
+    ctx.debug_set(DROP_KEY, 0)
+    do.fill_(float("nan"))
+    call()                                        # the same context, a complete call
+    assert ctx.status() == 0
+    for b, (n, L) in enumerate(zip(ns, Ls)):
+        check_attention(bf16_to_f64(do)[b, :n], oracle.tree_attention(q[b, :n], kc[b], vc[b], L, masks[b, :n], 0.125))
     ctx.close()
 
 
