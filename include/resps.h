@@ -108,7 +108,8 @@ int64_t resps_workspace_bytes(const resps_ctx* ctx);
  */
 enum {
     RESPS_DEBUG_ATTN_ROUNDS = 1,    /* the attention work list is cut for 1/value of the CTAs: 0 = for all             */
-    RESPS_DEBUG_ATTN_MIN_TILES = 2, /* fewest 64-key tiles a CTA is given: 0 = its own choice                          */
+    RESPS_DEBUG_ATTN_MIN_TILES = 2, /* fewest 64-key tiles a CTA is given where a group is cut into equal splits or (from
+                                       six tiles on; fewer stay in one CTA) shared by a cluster: 0 = its own choice    */
     RESPS_DEBUG_ATTN_CLUSTER = 3,   /* most CTAs per cluster of the attention kernel (1..8): 0 = its own choice        */
     RESPS_DEBUG_SCAN_SLICES = 4,    /* slices a logits row is cut into by the streaming scan: 0 = its own choice       */
     RESPS_DEBUG_ATTN_SINGLE = 5,    /* 0: never equal splits of every (sequence, KV head, row tile) but ranges over all of

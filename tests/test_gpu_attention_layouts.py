@@ -72,13 +72,27 @@ def test_clusters_with_several_items(cluster, D):
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("cluster", [2, 3, 4, 8])
 def test_few_key_tiles_in_a_cluster(cluster, D):
-    """One to nine key tiles: in one CTA, a tile a CTA, CTAs without any; the last tile full and with a single key."""
+    """One to nine key tiles: up to five stay in one CTA; six to eight are a tile a CTA in a cluster of eight, with two,
+    one and no CTAs left over, and more a CTA in smaller ones; nine take five CTAs of eight, two each.  The last tile
+    full and with a single key."""
     _, binding, _ = _imports()
-    for tiles in (1, 2, 3, 4, 5, 9):
+    for tiles in range(1, 10):
         for last in (1, 64):
             n = 9 if tiles > 1 else 1
             _attention_case(n, 16, 2, D, 64 * (tiles - 1) + last - n, cap=640, seed=tiles, poison=True,
                             debug=[(binding.RESPS_DEBUG_ATTN_CLUSTER, cluster)])
+
+
+@pytest.mark.parametrize("least", [1, 4, 1000])
+@pytest.mark.parametrize("cluster", [1, 3, 8])
+def test_fewest_key_tiles_of_a_cta(cluster, least):
+    """Shares of at least so many key tiles, up to whole groups in one CTA (3, 9 and 23 key tiles; in clusters and in equal
+    splits).  Results do not depend on it."""
+    _, binding, _ = _imports()
+    debug = [(binding.RESPS_DEBUG_ATTN_CLUSTER, cluster), (binding.RESPS_DEBUG_ATTN_MIN_TILES, least)]
+    if cluster == 1:
+        debug.append((binding.RESPS_DEBUG_ATTN_SINGLE, 1))
+    _attention_case(n=[9, 33, 70], Hq=14, Hkv=2, D=128, L=[130, 520, 1400], B=3, cap=1536, seed=least, poison=True, debug=debug)
 
 
 @pytest.mark.parametrize("cluster", [2, 3, 6, 8])
