@@ -152,7 +152,7 @@ struct AttnArgs {
     int most_rounds;  // mode even: rounds that are looked at
     int rounds;       // mode even: 0: own choice; else this many rounds (tests)
     int l2_tiles;     // K and V of more key tiles (of a KV head) than this do not stay in L2
-    int min_tiles;    // fewest key tiles a CTA is given
+    int min_tiles;    // fewest key tiles a CTA is given (clusters: of items of more than kAloneTiles)
     int q_by_tma;     // 1: Q tiles come by TMA (128 % (Hq/Hkv) == 0), 0: by plain loads
     int log2_group;   // of Hq/Hkv, where Q tiles come by TMA
     int plan_after_wait;  // 1: the work list was written by the kernel just before this one
@@ -1030,7 +1030,6 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
     const int rank = kClusters ? static_cast<int>(cluster_rank()) : 0;
     const uint32_t bars = base + S::kOffBar;
     auto bar = [&](int i) { return bars + 8u * i; };
-    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + S::kOffMisc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + S::kOffMisc + 8);
 
     // ---- one-time set-up ---------------------------------------------------------------
@@ -1552,42 +1551,44 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                     tc_fence_before();
                     mbar_arrive(bar(bar_item()));
                 } else {
-                float scale = 1.f;  // O = Ohat * l * scale, a scale for each half of the columns
-                uint32_t g[kHalf / 32][32];
-                // (a second time where |O / l| of a partial would leave fp16's range: the weights take a scale then)
+                    float scale = 1.f;  // O = Ohat * l * scale, a scale for each half of the columns
+                    uint32_t g[kHalf / 32][32];
+                    // (a second time where |O / l| of a partial would leave fp16's range: the weights take a scale then)
 #pragma unroll 1
-                while (true) {
-                    const unsigned long long ws2 = pack2(w_self, w_self), wo2 = pack2(w_oth, w_oth);
-                    float amax = 0.f;
+                    while (true) {
+                        const unsigned long long ws2 = pack2(w_self, w_self), wo2 = pack2(w_oth, w_oth);
+                        float amax = 0.f;
 #pragma unroll
-                    for (int c = 0; c < kHalf / 32; ++c) {
-                        uint32_t other[32];
-                        tmem_ld32(self_t + 32 * c, g[c]);
-                        tmem_ld32(oth_t + 32 * c, other);
-                        tmem_wait_ld();
+                        for (int c = 0; c < kHalf / 32; ++c) {
+                            uint32_t other[32];
+                            tmem_ld32(self_t + 32 * c, g[c]);
+                            tmem_ld32(oth_t + 32 * c, other);
+                            tmem_wait_ld();
 #pragma unroll
-                        for (int e = 0; e < 32; e += 2) {
-                            const unsigned long long s2 = pack2(__uint_as_float(g[c][e]), __uint_as_float(g[c][e + 1]));
-                            const unsigned long long o2 = pack2(__uint_as_float(other[e]), __uint_as_float(other[e + 1]));
-                            float g0, g1;
-                            unpack2(fma2(o2, wo2, fma2(s2, ws2, pack2(0.f, 0.f))), g0, g1);
-                            g[c][e] = __float_as_uint(g0), g[c][e + 1] = __float_as_uint(g1);
-                            amax = fmaxf(fmaxf(amax, fabsf(g0)), fabsf(g1));
+                            for (int e = 0; e < 32; e += 2) {
+                                const unsigned long long s2 = pack2(__uint_as_float(g[c][e]), __uint_as_float(g[c][e + 1]));
+                                const unsigned long long o2 = pack2(__uint_as_float(other[e]), __uint_as_float(other[e + 1]));
+                                float g0, g1;
+                                unpack2(fma2(o2, wo2, fma2(s2, ws2, pack2(0.f, 0.f))), g0, g1);
+                                g[c][e] = __float_as_uint(g0), g[c][e + 1] = __float_as_uint(g1);
+                                amax = fmaxf(fmaxf(amax, fabsf(g0)), fabsf(g1));
+                            }
+                        }
+                        // (`!direct` holds here and only steers the compiler: without it head dimension 64 in single CTAs
+                        // spills 36 bytes for 24, 16 sequences of up to 8000 keys 86.9 -> 89.1 us)
+                        const bool large = row_ok && !direct && amax > 16384.f && scale == 1.f;
+                        if (!__any_sync(kFull, large)) break;
+                        if (large) {  // the next power of two above |O / l|, 2^14 down; its reciprocal by the exponent too
+                            scale = __uint_as_float((__float_as_uint(amax) & 0x7F800000u) - (13u << 23));
+                            const float down = __uint_as_float((254u << 23) - __float_as_uint(scale));
+                            w_self *= down, w_oth *= down;
                         }
                     }
-                    const bool large = row_ok && !direct && amax > 16384.f && scale == 1.f;
-                    if (!__any_sync(kFull, large)) break;
-                    if (large) {  // the next power of two above |O / l|, 2^14 down; its reciprocal by the exponent too
-                        scale = __uint_as_float((__float_as_uint(amax) & 0x7F800000u) - (13u << 23));
-                        const float down = __uint_as_float((254u << 23) - __float_as_uint(scale));
-                        w_self *= down, w_oth *= down;
-                    }
-                }
-                // O has been read: the next item's P V may overwrite it
-                tc_fence_before();
-                mbar_arrive(bar(bar_item()));
-                if (kClusters && !direct) wait_free();
-                if (!alive) break;
+                    // O has been read: the next item's P V may overwrite it
+                    tc_fence_before();
+                    mbar_arrive(bar(bar_item()));
+                    if (kClusters) wait_free();
+                    if (!alive) break;
                     uint32_t v[kHalf / 2];
 #pragma unroll
                     for (int e = 0; e < kHalf / 2; ++e)
