@@ -1696,6 +1696,9 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
     if (kClusters && !alive) {
         cluster_arrive();
         cluster_wait();
+        // (what the last of them sent just before it left may still be on its way: 17 us, 1500 clocks are usual)
+        const uint32_t t0 = static_cast<uint32_t>(clock());
+        while (static_cast<uint32_t>(clock()) - t0 < 32768u) {}
     }
 }
 
