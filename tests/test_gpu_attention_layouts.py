@@ -12,7 +12,7 @@ SHAPES = [dict(n=7, Hq=12, Hkv=4, D=64, L=5), dict(n=33, Hq=14, Hkv=2, D=128, L=
           dict(n=[20, 128], Hq=16, Hkv=4, D=128, L=[5, 1400], B=2)]  # a cluster: a short item, then a long one
 
 
-@pytest.mark.parametrize("cluster,equal_splits", [(1, 0), (1, 1000), (2, None), (3, None), (4, None), (6, None), (8, None)])
+@pytest.mark.parametrize("cluster,equal_splits", [(1, 0), (1, 1000), (2, None), (3, None), (4, None), (6, None), (8, None), (5, None), (7, None)])
 @pytest.mark.parametrize("shape", range(len(SHAPES)))
 def test_layouts(shape, cluster, equal_splits):
     _, binding, _ = _imports()
@@ -44,7 +44,7 @@ SMALL = [dict(n=5, Hq=16, Hkv=2, D=128, L=1400),                          # 2 gr
          dict(n=2, Hq=8, Hkv=1, D=128, L=60)]                             # fewer key tiles than CTAs
 
 
-@pytest.mark.parametrize("cluster", [2, 3, 4, 6, 8])
+@pytest.mark.parametrize("cluster", [2, 3, 4, 6, 8, 5, 7])
 @pytest.mark.parametrize("shape", range(len(SMALL)))
 def test_a_group_cut_over_several_clusters(shape, cluster):
     _, binding, _ = _imports()
@@ -55,6 +55,13 @@ def test_a_group_cut_over_several_clusters(shape, cluster):
 def test_cut_groups_keep_values_beyond_fp16():
     _, binding, _ = _imports()
     _attention_case(6, 16, 2, 128, 3000, cap=3200, seed=3, v_scale=3.0e5, debug=[(binding.RESPS_DEBUG_ATTN_CLUSTER, 4)])
+
+
+@pytest.mark.parametrize("cluster", [5, 7])
+def test_groups_cut_over_uneven_clusters_keep_values_beyond_fp16(cluster):
+    """The 32 chunks of a partial in shares of 7 and 6, of 5 and 4; two groups in four pieces each."""
+    _, binding, _ = _imports()
+    _attention_case(6, 16, 2, 128, 4000, cap=4200, seed=cluster, v_scale=3.0e5, debug=[(binding.RESPS_DEBUG_ATTN_CLUSTER, cluster)])
 
 
 @pytest.mark.parametrize("D", [64, 128])

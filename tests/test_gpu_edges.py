@@ -209,9 +209,9 @@ def test_attention_work_list_of_several_rounds(rounds):
 
 @pytest.mark.parametrize("single_units", [0, 100000])
 def test_attention_both_groupings_of_the_work_list(single_units):
-    """The work list cuts a call into single row tiles (both halves of a CTA on one tile) while it is small and
-    into pairs of row tiles otherwise; the test-only override forces each grouping on shapes that take the
-    other one by themselves: a short GQA sequence with several row tiles per KV head, a long one, a ragged batch."""
+    """The work list of single CTAs is made of equal splits of every group or of ranges over all groups; the test-only
+    override never takes, or always takes, the equal splits (a short GQA sequence with several row tiles per KV head, a
+    long one, a ragged batch).  In clusters it never cuts a group, or cuts one wherever clusters are left."""
     _, binding, _ = _imports()
     dbg = ((binding.RESPS_DEBUG_ATTN_SINGLE, single_units),)
     _attention_case(60, 32, 8, 128, 700, cap=1024, seed=11, debug=dbg)
