@@ -1686,6 +1686,9 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
     if (stale) atomicOr(a.status, RESPS_STATUS_STALE_PLAN);
     tc_fence_before();
     __syncthreads();
+    // (the addresses count on it: the test build looks whether the swizzled tiles and tensor memory begin where they do)
+    if (kWaitTest && tid == 0 && ((base & 1023u) != 0 || *reinterpret_cast<volatile uint32_t*>(base_ptr + S::kOffMisc) != tmem))
+        atomicOr(a.status, RESPS_STATUS_WAIT_TIMEOUT);
     if (warp == kMmaWarp0) {
         __syncwarp();
         tc_fence_after();

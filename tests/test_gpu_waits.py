@@ -112,6 +112,27 @@ def test_cluster_waits_run_out_and_the_context_recovers(waitlib, wait, D):
     ctx.close()
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("Hq", [16, 14])             # Q by TMA, by plain loads
+@pytest.mark.parametrize("cluster", [1, 2, 8])       # single CTAs, clusters with cut groups, one group a cluster
+def test_addresses_begin_where_every_kernel_takes_them_to(waitlib, cluster, Hq, D):
+    """The test build's kernels look at what their constant addresses rest on (shared memory at a multiple of 1024,
+    tensor memory at column 0) and would set a status bit."""
+    from harness import u16_to_bf16_cuda
+    from paper_2601_12212_b200 import synth
+    binding = waitlib
+    n, Hkv, L, cap, T = 5, 2, 1000, 1088, 40
+    ctx = binding.Context(Hq, Hkv, D, 100, max_batch=1, max_tt=T, max_k=4, max_depth=4)
+    ctx.debug_set(binding.RESPS_DEBUG_ATTN_CLUSTER, cluster)
+    q, kc, vc, masks = _attention_inputs(binding, synth, n, Hq, Hkv, D, L, cap, T)
+    steps, nn = (torch.tensor(x, dtype=torch.int32, device="cuda") for x in ([[n, 1, 1, L]], [n]))
+    dq, dk, dv = u16_to_bf16_cuda(q), u16_to_bf16_cuda(kc), u16_to_bf16_cuda(vc)
+    dm, do = torch.from_numpy(masks.view(np.int64)).cuda(), torch.zeros_like(dq)
+    binding.resps_tree_attention(ctx, steps, nn, 1, dq, do, None, dk, dv, Hkv * cap * D, cap * D, D, cap, dm, 0.125)
+    assert ctx.status() == 0 and do[0, :n].abs().max() > 0
+    ctx.close()
+
+
 def test_scan_wait_runs_out_and_the_context_recovers(waitlib):
     import oracle
     binding = waitlib
