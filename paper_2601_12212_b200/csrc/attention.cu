@@ -93,7 +93,7 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 // Of even (each number of rounds) and stream the one with the smallest largest share is taken (tiles, items, cut
 // groups).  In mode even the row tiles of a KV head go through the same keys at the same time, in mode stream at
 // different times: where K and V do not stay in L2 meanwhile, every row tile reads them from HBM again, and 148 CTAs
-// with 32 KB per 0.62 us ask for more than HBM has.  So the share of mode stream counts kRereadNum / kRereadDen times as
+// with 32 KB per 0.57 us ask for more than HBM has.  So the share of mode stream counts kRereadNum / kRereadDen times as
 // much beyond `l2_tiles` key tiles (all KV heads of the sequences with several row tiles; head dimension 128).  In us a
 // call, stream against the best of even: 8 x 24 000 keys, 80 nodes, 8B shape 416 / 351 (four rounds); 5 x 28 000 keys, 40-96
 // nodes, 56 query heads 469 / 391 (four); 4 x 8192 keys, 96 nodes, 70B shape 141 / 128 (four); 16 x 4096 keys, 64 nodes, 8B
@@ -135,10 +135,10 @@ struct AttnArgs {
     const uint64_t* mask;
     float scale_log2;
     int Hq, Hkv, max_tt;
-    // Partials of the two-kernel modes (in mode whole the same goes into the cluster's shared memory).  O is stored normalised (O / l, a convex combination of V rows) as
-    // fp16 times a power of two per half row that only differs from 1 when a value would leave the fp16
-    // range: half the bytes of fp32, and 11 significant bits per element (2^-11, against the 2^-9
-    // of the final bf16 rounding).
+    // Partials of the two-kernel modes (in mode whole the same goes into the cluster's shared memory).  O is stored
+    // normalised (O / l, a convex combination of V rows) as fp16 times a power of two per half row that only differs
+    // from 1 when a value would leave the fp16 range: half the bytes of fp32, and 11 significant bits per element
+    // (2^-11, against the 2^-9 of the final bf16 rounding).
     uint4* part_o;    // [places][D/8][128 rows]  eight fp16 each
     float4* part_ml;  // [places][128 rows]   (running max m, running sum l, l * scale of each half row)
     int cluster;      // CTAs per cluster (1: modes even and stream)
@@ -1956,8 +1956,15 @@ bool cached_map(HostState* hs, const MapKey& key, int D, CUtensorMap* out) {
 //   24         5        9.0 / 11.4   10.5 / 13.3   14.3 / 16.0   20.7 / 21.7   (28.4 / 28.3 at 12 288)
 //   32         4        9.4 / 11.8   11.5 / 13.8   15.8 / 17.9   24.8 / 26.1   (35.0 / 36.2)
 //   40         3       11.1 / 11.9   14.0 / 14.9   20.1 / 21.1   33.7 / 35.3   (47.8 / 48.0)
-// The two meet at 5 tiles lost with 12 and 16 groups, at 6 to 7 with 8, 24 and 32, at 12 with 40.  With 7, at the longest
-// prefix that it admits, mode whole is up to 5 % behind; below that prefix, where a call usually is, up to 24 % ahead.
+// At the longest prefix that 5, 6 and 7 lost tiles admit (a cache without room beyond it), whole / two kernels:
+//    8 groups   11.0 / 12.7   12.1 / 13.3   13.1 / 14.0  (6240 keys)
+//   12          15.8 / 15.9   17.0 / 17.0   18.5 / 18.0  (10 129)
+//   16          14.6 / 14.4   16.0 / 15.5   17.8 / 16.7  (7556; Q by plain loads 15.9 / 15.5, 17.1 / 16.6, 18.7 / 17.6)
+//   24          21.4 / 22.1   24.3 / 24.9   28.2 / 27.5  (11 744)
+//   32          27.5 / 28.7   32.3 / 34.1   37.1 / 38.6  (13 120)
+//   40          23.7 / 25.8   26.6 / 30.0   29.6 / 33.8  (7056)
+// With 7 a call at that limit takes up to 6 % longer than the two kernels would (16 groups), and one of 1024 keys in such a
+// cache, where calls usually are well below its end, 11 to 21 % less (16 groups 8.2 / 9.6, 24 9.1 / 11.5).
 constexpr double kWholeGainTiles = 7.0;
 // In a batch the cache may hold one long sequence among short ones, which only its own clusters work on.  (Four equal
 // sequences of 8 groups: 10.4 / 12.9 us at 1024 keys, 40.5 / 43.6 at 12 288.)
@@ -1970,9 +1977,10 @@ int choose_cluster(const int* resident, int sm_count, int groups, int batch, int
     return 1;
 }
 // K and V of this many bytes are taken to stay in L2 between the row tiles of a head (measured between 67 and 131 MB).
-// With a head dimension of 64 it does not matter where they are: 148 CTAs with 16 KB per 0.6 us ask for 3.9 TB/s, below
-// HBM's rate, where 32 KB ask for 7.8.  (16 sequences up to 32 000 keys, 546 MB: ranges 214 us, equal splits in one to
-// four rounds 215, 247, 240, 234; of twelve such shapes two gain 2 to 4 % by rounds, so they are not looked at there.)
+// With a head dimension of 64 it does not matter where they are: 148 CTAs with 16 KB per 0.6 us ask for 4 TB/s, below
+// HBM's rate, where 32 KB per 0.57 us ask for 8.5.  (16 sequences up to 32 000 keys, 546 MB, ranges / the best of two to four
+// rounds of equal splits: trees of up to 32 nodes 135.7 / 138.5, 135.6 / 143.8, 135.2 / 146 us, up to 96 nodes 248 / 244,
+// 279 / 307, 314 / 302.  Four of six lose 2 to 10 %, two gain 2 to 4 %, so rounds are not looked at there.)
 constexpr int64_t kL2Bytes = 96 << 20;
 int forced_cluster(const int* resident, int cluster, int groups) {
     while (cluster > 1 && resident[cluster] < groups) --cluster;
@@ -1984,7 +1992,8 @@ int most_nodes(const resps_shape& s) {
 }
 
 // Clusters of C CTAs that are resident at once with this kernel's shared memory (index C; the GPCs are not
-// multiples of every size), asked for once per device.
+// multiples of every size), asked for once per device.  One answer serves all forms of a head dimension: they have the
+// same threads, registers (the launch bound's) and shared memory, of which one CTA takes more than half an SM's.
 struct Residency {
     int clusters[kMaxCluster + 1] = {};
     bool known = false;
@@ -2168,10 +2177,11 @@ int attention_place_rows() { return kBM; }
 int attention_max_groups(int batch, int n_kv_heads, int max_tt, int group) {
     return batch * n_kv_heads * ((max_tt * group + kBM - 1) / kBM);
 }
-// (also the most partials)
 int attention_counters() { return kMaxGrid * kPieceWarps; }
-// Up to kFewGroups groups one round of splits is balanced to within a seventh, and the pieces of cut groups fit behind
-// two places of every CTA (the launch checks that): such contexts have no room for more rounds.
+// Items of the two-kernel modes, also the most partials: a round of splits or a range a CTA (which may begin inside a
+// group), and up to kMaxRounds rounds.  Up to kFewGroups groups one round is balanced to within a seventh: such contexts have
+// no room for more.  (The sums of cut groups in clusters, 9/4 places a cluster, lie in the same memory; the launch checks that
+// they fit.)
 constexpr int kFewGroups = 20;
 int attention_max_items(int groups, int sm_count) {
     const int grid = std::min(sm_count, kMaxGrid);

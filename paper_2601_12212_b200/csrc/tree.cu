@@ -81,8 +81,8 @@ struct FastDiv {
 
 __global__ void __launch_bounds__(kTreeThreads, 1) tree_build_kernel(const TreeArgs a) {
     // The step parameters were written at least two kernels ago (a scan or a merge kernel of the same
-    // call always sits between their writer and this kernel, and every kernel of the library signals its
-    // dependents only after its own wait), so they are read, and everything that follows from them is
+    // call always sits between their writer and this kernel, and signals its dependents only after its
+    // own wait), so they are read, and everything that follows from them is
     // set up, before the wait for the rows: under the tail of the kernel that scans them.  (Where no such
     // kernel precedes this one -- the last call of the level form -- the wait comes first.)
     if (!a.setup_before_wait) pdl_wait();
