@@ -385,8 +385,9 @@ __global__ void __launch_bounds__(kMaxGrid) attention_plan_kernel(const AttnArgs
                 const int behind = sh.kt[b] - t;
                 const unsigned long long g0 = sh.start[b] + static_cast<unsigned long long>(local) * sh.kt[b];
                 whole = g0 + (t <= behind ? 0 : sh.kt[b]);
-                // a piece shorter than its own epilogue is not worth a cut
-                equal = (min(t, behind) <= kSnap) ? whole : g0 + t;
+                // a piece shorter than its own epilogue is not worth a cut; nor are ranges of less than a tile (several CTAs
+                // would begin at one place, and the pieces of a group are counted by its CTAs)
+                equal = (min(t, behind) <= kSnap || cost < static_cast<unsigned long long>(a.clusters)) ? whole : g0 + t;
             }
             sh.cut[0][tid] = whole, sh.cut[1][tid] = equal;
         }

@@ -22,6 +22,14 @@ def test_layouts(shape, cluster, equal_splits):
     _attention_case(**SHAPES[shape], cap=1664, seed=cluster, poison=True, debug=debug)
 
 
+@pytest.mark.parametrize("n,Hq,Hkv,L,B", [(12, 16, 2, 900, 1), (1, 8, 1, 2000, 1), ([30, 3], 8, 2, [1000, 700], 2)])
+def test_ranges_over_fewer_tiles_than_ctas(n, Hq, Hkv, L, B):
+    """15 to 32 key tiles a group, a few groups: most of the 148 CTAs have no range."""
+    _, binding, _ = _imports()
+    debug = [(binding.RESPS_DEBUG_ATTN_CLUSTER, 1), (binding.RESPS_DEBUG_ATTN_SINGLE, 0)]
+    _attention_case(n, Hq, Hkv, 128, L, cap=2048, seed=B, B=B, poison=True, debug=debug)
+
+
 TILES = [dict(n=[43, 128, 1, 86], Hq=24, Hkv=8, D=128, L=[1000, 63, 1500, 0], B=4),  # 2 row tiles (the second of 1 row), 3, 1, 3
          dict(n=96, Hq=14, Hkv=2, D=64, L=1400),                                      # 6, Q by plain loads
          dict(n=[128, 65, 2, 20], Hq=16, Hkv=1, D=128, L=[130, 1, 5, 1536], B=4)]     # 16, 9, 1, 3
