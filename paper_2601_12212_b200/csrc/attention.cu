@@ -1577,7 +1577,8 @@ tree_attention_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap map_
                         }
                         // (`!direct` holds here and only steers the compiler: without it head dimension 64 in single CTAs
                         // spills 36 bytes for 24, 16 sequences of up to 8000 keys 86.9 -> 89.1 us)
-                        const bool large = row_ok && !direct && amax > 16384.f && scale == 1.f;
+                        // (not behind an infinity: a scale for it would take the row's other values out of fp16 at the lower end)
+                        const bool large = row_ok && !direct && amax > 16384.f && amax < INFINITY && scale == 1.f;
                         if (!__any_sync(kFull, large)) break;
                         if (large) {  // the next power of two above |O / l|, 2^14 down; its reciprocal by the exponent too
                             scale = __uint_as_float((__float_as_uint(amax) & 0x7F800000u) - (13u << 23));

@@ -171,3 +171,40 @@ def test_replayed_for_small_and_large_trees():
             assert (o[i, 0, :n].float() - want).abs().max() <= 2 ** -8 * want.abs().max()
     del graph
     ctx.close()
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("cluster,equal_splits", [(1, 0), (1, 1), (2, None), (5, None), (8, None)])
+def test_an_infinity_in_v_stays_in_its_column(cluster, equal_splits, D):
+    """One V of a visible key is infinite: its column is infinite (or not a number) in every row of that KV head, and the
+    other columns are what they are without it, also where a partial's scale goes by the row's largest magnitude."""
+    import numpy as np
+    import torch
+    import oracle
+    _, binding, synth = _imports()
+    from harness import bf16_to_f64, check_attention, u16_to_bf16_cuda
+    n, Hq, Hkv, L, cap, T, head, key, col = 12, 16, 2, 900, 1024, 16, 1, 333, 5
+    ctx = binding.Context(Hq, Hkv, D, 1000, max_batch=1, max_tt=T, max_k=4, max_depth=4)
+    ctx.debug_set(binding.RESPS_DEBUG_ATTN_CLUSTER, cluster)
+    if equal_splits is not None:
+        ctx.debug_set(binding.RESPS_DEBUG_ATTN_SINGLE, equal_splits)
+    rng = np.random.default_rng(D + cluster)
+    q, kc, vc = (synth.to_bf16_bits(rng.normal(size=s).astype(np.float32).ravel()).reshape(s)
+                 for s in ((1, T, Hq, D), (1, Hkv, cap, D), (1, Hkv, cap, D)))
+    masks = np.zeros((1, T, 2), np.uint64)
+    for i in range(n):
+        masks[0, i, 0] = (1 << (i + 1)) - 1
+    vc[0, head, key, col] = 0
+    want = oracle.tree_attention(q[0, :n], kc[0], vc[0], L, masks[0, :n], 0.125)
+    vc[0, head, key, col] = 0x7F80
+    dq, dk, dv = u16_to_bf16_cuda(q), u16_to_bf16_cuda(kc), u16_to_bf16_cuda(vc)
+    do, dm = torch.zeros_like(dq), torch.from_numpy(masks.view(np.int64)).cuda()
+    steps, nn = (torch.tensor(x, dtype=torch.int32, device="cuda") for x in ([[n, 1, 1, L]], [n]))
+    binding.resps_tree_attention(ctx, steps, nn, 1, dq, do, None, dk, dv, Hkv * cap * D, cap * D, D, cap, dm, 0.125)
+    assert ctx.status() == 0
+    got = bf16_to_f64(do)[0, :n]
+    rows = slice(head * Hq // Hkv, (head + 1) * Hq // Hkv)
+    assert not np.isfinite(got[:, rows, col]).any()
+    got[:, rows, col] = want[:, rows, col]
+    check_attention(got, want)
+    ctx.close()
